@@ -122,7 +122,7 @@ int seq_tree_mask_from_parents(const int32_t* parent, int32_t n, uint32_t* mask_
  * launch; a parent[i] outside {-1} u [0,i) raises SEQ_DEV_BAD_PARENT and is
  * read as -1, as there.  The results are those of a call with the mask_bits of
  * seq_tree_mask_from_parents(parent).  The CUDA-core kernel has no such mode:
- * a request that needs it (fp32, a group size that does not divide 128,
+ * a request that needs it (fp32, a group of more than 128 heads,
  * kernel == 1) without mask_bits returns SEQ_ERR_UNSUPPORTED.  When mask_bits
  * is given, parent is ignored.
  * workspace: at least seq_tree_attention_workspace_bytes(p) bytes, 256-byte

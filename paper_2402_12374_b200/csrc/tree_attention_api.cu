@@ -70,7 +70,7 @@ static int choose_kernel(const seq_tree_attention_params& p) {
   // Measured on B200: even with a single query row per kv head (127 of the tile's 128 rows padding) the
   // tensor-core kernel is faster than the CUDA-core one, because it streams K/V once per kv head with
   // TMA while the CUDA-core kernel re-reads them for every (node, head).  The CUDA-core kernel is kept
-  // for fp32 inputs and for group sizes that do not divide 128.
+  // for fp32 inputs and for groups of more than 128 heads.
   return 2;
 }
 

@@ -107,6 +107,7 @@ static_assert(offsetof(UmmaSmem, v) == offsetof(UmmaSmem, k) + sizeof(UmmaSmem::
 
 struct UmmaArgs {
   int32_t n, L_host, Hq, Hkv, group, mask_wpr, splits, nodes_per_tile, tiles;
+  int32_t rows;           // query rows of a full tile: nodes_per_tile * group, 128 when the group divides it
   const int32_t* L_dev;   // nullable: the prefix length in device memory (<= L_host)
   int32_t L_count;        // > 1: one length per request, requests stacked as heads (grid schedule only: a CTA has one kv head)
   int32_t zero_tail;      // the K/V maps cover the whole cache: rows past the tree are cleared in shared memory
@@ -251,6 +252,15 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
+// The Q tile of nodes [i0, i0 + nodes_per_tile) of kv head g.  When the group divides 128 the tile has 128 rows and one
+// copy brings both 64-element halves; otherwise it has fewer (the halves of one copy would then lie rows * 128 bytes
+// apart, off the swizzle's 1024-byte boundary), and each half is a copy of its own to its fixed place.
+__device__ __forceinline__ void load_q(uint8_t* dst, const CUtensorMap* map, uint64_t* bar, int rows, int i0, int g) {
+  mbar_expect_tx(bar, (uint32_t)rows * 256u);
+  tma_load_5d(dst, map, bar, 0, 0, i0, 0, g);
+  if (rows < kTileM) tma_load_5d(dst + kHalfBytes, map, bar, 0, 0, i0, 1, g);
+}
+
 // Two single-precision values in one 64-bit register, for the packed fused multiply-add and add: half the issue slots.
 __device__ __forceinline__ uint64_t pair_of(float lo, float hi) {
   uint64_t d;
@@ -420,8 +430,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
   if (!kStream && threadIdx.x == 0) {
     const Seg s0 = seg_at(range_lo);
     if (s0.nblk > 0) {
-      mbar_expect_tx(&sm->q_full, kTileBytes);
-      tma_load_5d(sm->q, &q_map, &sm->q_full, 0, 0, s0.i0, 0, s0.g);
+      load_q(sm->q, &q_map, &sm->q_full, a.rows, s0.i0, s0.g);
       for (int jj = 0; jj < 2 && jj < s0.nblk; ++jj) {
         mbar_expect_tx(&sm->k_full[jj][0], kKvBytes);
         tma_load_4d(sm->k[jj][0], &k_map, &sm->k_full[jj][0], 0, (s0.blk_lo + jj) * kBlockN, 0, s0.g);
@@ -430,6 +439,13 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
   }
   if (a.mask_bits == nullptr)
     for (int t = threadIdx.x; t < a.n; t += kUmmaThreads) sm->parent[t] = a.parent[t];
+  if (a.rows < kTileM) {  // rows no copy writes (the group does not divide 128): zeros, so that their scores are finite
+    for (int t = a.rows * 8 + (int)threadIdx.x; t < kTileM * 8; t += kUmmaThreads) {
+      reinterpret_cast<uint4*>(sm->q)[t] = make_uint4(0u, 0u, 0u, 0u);
+      reinterpret_cast<uint4*>(sm->q + kHalfBytes)[t] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    fence_async_smem();
+  }
   if (kStream && warp == 2) {  // blocks of a kv head before each place of its layout: four places per lane, then a warp scan
     const int per = (a.tiles + 31) / 32;
     int local[kMaxStreamTiles / 32], sum = 0;
@@ -488,8 +504,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
         // barrier within one phase of its arrivers)
         if (!is_v && seg > 0 && !mbar_wait(sm, &sm->o_free, (seg - 1) & 1, a.dev_status)) break;
         if (kStream && !is_v && elect_one()) {  // (grid schedule: requested before the roles split, see above)
-          mbar_expect_tx(&sm->q_full, kTileBytes);
-          tma_load_5d(sm->q, &q_map, &sm->q_full, 0, 0, i0, 0, g);  // both 64-element halves by one copy
+          load_q(sm->q, &q_map, &sm->q_full, a.rows, i0, g);
         }
         __syncwarp();
         if (kStream && !is_v) { issued |= 16u; issued_parity = (issued_parity & ~16u) | ((uint32_t)(seg & 1) << 4); }
@@ -647,7 +662,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
   const int seg = kStream ? seg_n : 0, base = kStream ? base_n : 0;  // grid mode: constants
   const int i = i0 + r / a.group;             // node of this row
   const int h = g * a.group + r % a.group;
-  const bool row_valid = i < a.n;
+  const bool row_valid = i < sg.i1;           // (a row past the tile's nodes may be one of the next tile's)
   // The row's ancestor bits: the caller's mask, or rows derived from the parent array at the start of the
   // segment by the first thread of each node (0 <= parent[j] < j, so a walk ends; anything else is flagged and
   // read as "no parent").  In grid mode the row threads are idle at this point, waiting for the first tiles.
@@ -678,7 +693,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
   // A warp whose 32 rows all lie past the tile's last node (small trees fill only part of a 128-row tile) leaves
   // the special-function unit and the issue slots to the warps with real rows; its P rows stay whatever they are
   // (rows of the product are independent).
-  const bool warp_live = i0 + (quad * 32) / a.group < a.n;
+  const bool warp_live = i0 + (quad * 32) / a.group < sg.i1;
   for (int u = 0; u < n_mine && ok; ++u) {
     const int jj = 2 * u + chain, b = (base + u) & 1, w = (base + u) >> 1;
     const uint32_t tmem_s = tmem + 128u * chain + 64u * b + lane_sel;
@@ -1063,9 +1078,7 @@ CUresult encode_cached(EncodeTiledFn encode, CUtensorMap* out, CUtensorMapDataTy
 
 bool umma_supported(const seq_tree_attention_params& p) {
   if (p.dtype != SEQ_F16 && p.dtype != SEQ_BF16) return false;
-  const int G = p.num_q_heads / p.num_kv_heads;
-  if (G > kTileM || kTileM % G != 0) return false;
-  return true;
+  return p.num_q_heads / p.num_kv_heads <= kTileM;  // a tile holds at least one node's group of heads
 }
 
 // How the tiles are spread over the SMs.  Grid schedule: one CTA (or a cluster of `splits` CTAs along the key
@@ -1146,7 +1159,7 @@ int launch_attention_umma(const seq_tree_attention_params& p, int splits, cudaSt
     cuuint64_t dims[5] = {64, (cuuint64_t)G, (cuuint64_t)p.n_tree, 2, (cuuint64_t)p.num_kv_heads};
     cuuint64_t strides[4] = {(cuuint64_t)p.q_stride_head * 2, (cuuint64_t)p.q_stride_tok * 2, 128,
                              (cuuint64_t)p.q_stride_head * 2 * G};
-    cuuint32_t box[5] = {64, (cuuint32_t)G, (cuuint32_t)nodes_per_tile, 2, 1};
+    cuuint32_t box[5] = {64, (cuuint32_t)G, (cuuint32_t)nodes_per_tile, kTileM % G == 0 ? 2u : 1u, 1};  // (see load_q)
     if (encode_cached(encode, &q_map, dt, 5, p.q, dims, strides, box) != CUDA_SUCCESS) return SEQ_ERR_CUDA;
   }
   for (int which = 0; which < 2; ++which) {
@@ -1162,6 +1175,7 @@ int launch_attention_umma(const seq_tree_attention_params& p, int splits, cudaSt
   UmmaArgs a;
   a.n = p.n_tree; a.L_host = p.prefix_len; a.Hq = p.num_q_heads; a.Hkv = p.num_kv_heads; a.group = G;
   a.mask_wpr = p.mask_words_per_row; a.splits = splits; a.nodes_per_tile = nodes_per_tile; a.tiles = tiles;
+  a.rows = nodes_per_tile * G;
   const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 0.08838834764831845f;
   a.scale_log2 = scale * kLog2e;
   const uint32_t fmt = p.dtype == SEQ_BF16 ? 1u : 0u;
