@@ -147,9 +147,22 @@ def _dev(t: torch.Tensor | None, name: str, dtype=None) -> int | None:
     return t.data_ptr()
 
 
+# torch.cuda.current_stream() builds a Stream object, 3.1 us a call; the handle alone is 0.1 us.  (A torch without these
+# two functions takes the long way.)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+if _raw_stream is None or _raw_device is None:
+    def _raw_stream(_device):
+        return torch.cuda.current_stream().cuda_stream
+
+    def _raw_device():
+        return 0
+
+
 def _stream(stream) -> int:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream if hasattr(s, "cuda_stream") else int(s)
+    if stream is None:
+        return _raw_stream(_raw_device())
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def _check(fn: str, code: int) -> None:
@@ -203,23 +216,24 @@ def seq_tree_draft_sample(draft_logits, temperature: float, uniforms, k: int, *,
     """k tokens per row drawn without replacement from softmax(draft_logits / temperature) by exponential
     sort with the supplied uniforms; returns int32 [rows, k] (device), -1 where nothing was left to draw."""
     rows, V = draft_logits.shape
-    if uniforms.shape != draft_logits.shape or draft_logits.stride(1) != 1 or uniforms.stride(1) != 1:
+    ls, lc = draft_logits.stride()
+    us, uc = uniforms.stride()
+    if uniforms.shape != draft_logits.shape or lc != 1 or uc != 1:
         raise ValueError("draft_logits and uniforms must be [rows, vocab] with contiguous rows")
     if tokens_out is None:
         tokens_out = torch.empty((rows, k), dtype=torch.int32, device=draft_logits.device)
-    p = DraftSampleParams()
-    p.n_rows, p.vocab, p.k = rows, V, k
-    p.draft_logits, p.logits_row_stride = _dev(draft_logits, "draft_logits", torch.float32), (draft_logits.stride(0) if rows > 1 else V)
-    p.uniforms, p.uniforms_row_stride = _dev(uniforms, "uniforms", torch.float32), (uniforms.stride(0) if rows > 1 else V)
-    p.temperature = temperature
-    p.tokens_out = _dev(tokens_out, "tokens_out", torch.int32)
-    p.dev_status = _dev(dev_status, "dev_status", torch.int32)
-    need = load().seq_tree_draft_sample_workspace_bytes(C.byref(p))
-    if workspace is None and need:
-        workspace = torch.empty(need, dtype=torch.uint8, device=draft_logits.device)
-    p.workspace = _dev(workspace, "workspace") if workspace is not None else None
-    p.workspace_bytes = workspace.numel() * workspace.element_size() if workspace is not None else 0
-    _check("seq_tree_draft_sample", load().seq_tree_draft_sample(C.byref(p), _stream(stream)))
+    lib = load()
+    p = DraftSampleParams(rows, V, k, _dev(draft_logits, "draft_logits", torch.float32), ls if rows > 1 else V,
+                          _dev(uniforms, "uniforms", torch.float32), us if rows > 1 else V, temperature,
+                          _dev(tokens_out, "tokens_out", torch.int32), _dev(dev_status, "dev_status", torch.int32))
+    ref = C.byref(p)
+    if workspace is None:
+        need = lib.seq_tree_draft_sample_workspace_bytes(ref)
+        if need:
+            workspace = torch.empty(need, dtype=torch.uint8, device=draft_logits.device)
+    if workspace is not None:
+        p.workspace, p.workspace_bytes = _dev(workspace, "workspace"), workspace.numel() * workspace.element_size()
+    _check("seq_tree_draft_sample", lib.seq_tree_draft_sample(ref, _stream(stream)))
     return tokens_out
 
 
@@ -273,14 +287,16 @@ class AttentionCall:
         p.workspace = _dev(workspace, "workspace") if workspace is not None else None
         p.workspace_bytes = workspace.numel() * workspace.element_size() if workspace is not None else 0
         self.params, self.out, self.lse, self.workspace_bytes_needed = p, out, lse, need
+        self._ref = C.byref(p)
+        self._name = "seq_tree_attention_noalloc" if noalloc else "seq_tree_attention"
+        self._fn = getattr(load(), self._name)
         self.workspace = workspace
         self._keep = (q, k_cache, v_cache, mask_bits, parent, out, lse, workspace, dev_status, prefix_len_dev)
 
     def run(self, stream=None):
-        if self.noalloc:
-            _check("seq_tree_attention_noalloc", load().seq_tree_attention_noalloc(C.byref(self.params), _stream(stream)))
-        else:
-            _check("seq_tree_attention", load().seq_tree_attention(C.byref(self.params), _stream(stream)))
+        rc = self._fn(self._ref, _raw_stream(_raw_device()) if stream is None else _stream(stream))
+        if rc:
+            _check(self._name, rc)
         return self.out
 
 
@@ -344,13 +360,15 @@ class VerifyCall:
         if workspace is not None:
             p.workspace, p.workspace_bytes = _dev(workspace, "workspace"), workspace.numel() * workspace.element_size()
         self.workspace, self.workspace_bytes_needed = workspace, need
-        self.params = p
+        self.params, self._ref, self._fn = p, C.byref(p), load().seq_tree_verify
         self.path, self.path_len, self.bonus_token = path, path_len, bonus_token
         self.residual_out, self.next_child_out = residual_out, next_child_out
         self._keep = (parent, tokens, target_logits, draft_logits, uniforms, dev_status)
 
     def run(self, stream=None):
-        _check("seq_tree_verify", load().seq_tree_verify(C.byref(self.params), _stream(stream)))
+        rc = self._fn(self._ref, _raw_stream(_raw_device()) if stream is None else _stream(stream))
+        if rc:
+            _check("seq_tree_verify", rc)
         return self.path, self.path_len, self.bonus_token
 
     def rows_read(self):
@@ -375,28 +393,31 @@ def seq_tree_verify_batch(parent, tokens, target_logits, draft_logits, temperatu
     residual_out [R, V] and next_child_out [R, n] optional.  Returns path [R, n], path_len [R], bonus_token [R]."""
     R, n, V = target_logits.shape
     dev = target_logits.device
-    path = torch.empty((R, n), dtype=torch.int32, device=dev)
-    path_len = torch.zeros(R, dtype=torch.int32, device=dev)
-    bonus = torch.full((R,), -1, dtype=torch.int32, device=dev)
     for t, nm in ((parent, "parent"), (tokens, "tokens"), (uniforms, "uniforms"), (target_logits, "target_logits"),
                   (draft_logits, "draft_logits"), (residual_out, "residual_out"), (next_child_out, "next_child_out")):
         if t is not None and (t.shape[0] != R or t.stride(-1) != 1):
             raise ValueError(f"{nm}: one entry per request, innermost dimension contiguous")
-    if draft_logits is not None and draft_logits.stride(0) != target_logits.stride(0):
+    request, row, _ = target_logits.stride()
+    draft_request, draft_row, _ = draft_logits.stride() if draft_logits is not None else (request, 0, 1)
+    if draft_request != request:
         raise ValueError("target_logits and draft_logits must have the same stride between requests")
     if parent.stride(0) != tokens.stride(0) or parent.stride(0) != n or (next_child_out is not None and next_child_out.stride(0) != n):
         raise ValueError("parent, tokens and next_child_out must be [R, n] contiguous")
-    one = VerifyCall(parent[0], tokens[0], target_logits[0], None if draft_logits is None else draft_logits[0], temperature,
-                     uniforms[0], path=path[0], path_len=path_len, bonus_token=bonus,
-                     residual_out=None if residual_out is None else residual_out[0],
-                     next_child_out=None if next_child_out is None else next_child_out[0], dev_status=dev_status,
-                     specinfer=specinfer, target_sample=target_sample)
-    p = VerifyBatchParams()
-    p.request0 = one.params
-    p.batch = R
-    p.tree_stride, p.logits_stride = n, target_logits.stride(0)
-    p.uniforms_stride = uniforms.stride(0)
-    p.residual_stride = residual_out.stride(0) if residual_out is not None else 0
+    ldt = target_logits.dtype
+    if ldt is not torch.float32 and ldt is not torch.bfloat16:
+        raise ValueError("target_logits must be float32 or bfloat16")
+    path = torch.empty((R, n), dtype=torch.int32, device=dev)
+    path_len, bonus = torch.empty((2, R), dtype=torch.int32, device=dev).unbind(0)  # (every launch writes both)
+    flags = ((SEQ_VERIFY_SPECINFER if specinfer else 0) | (SEQ_VERIFY_TARGET_SAMPLE if target_sample else 0) |
+             (SEQ_VERIFY_LOGITS_BF16 if ldt is torch.bfloat16 else 0))
+    p = VerifyBatchParams(
+        VerifyParams(n, V, _dev(parent, "parent", torch.int32), _dev(tokens, "tokens", torch.int32),
+                     _dev(target_logits, "target_logits", ldt), row, _dev(draft_logits, "draft_logits", ldt), draft_row,
+                     temperature, _dev(uniforms, "uniforms", torch.float32), path.data_ptr(), path_len.data_ptr(),
+                     bonus.data_ptr(), _dev(residual_out, "residual_out", torch.float32),
+                     _dev(next_child_out, "next_child_out", torch.int32), None, 0,
+                     _dev(dev_status, "dev_status", torch.int32), flags),
+        R, n, request, uniforms.stride(0), residual_out.stride(0) if residual_out is not None else 0)
     _check("seq_tree_verify_batch", load().seq_tree_verify_batch(C.byref(p), _stream(stream)))
     return path, path_len, bonus
 
@@ -424,16 +445,14 @@ def seq_tree_top_p_filter(logits, temperature: float, top_p: float, *, out=None,
     rows, V = logits.shape
     if out is None:
         out = torch.empty_like(logits)
-    for t, nm in ((logits, "logits"), (out, "out")):
-        if t.shape != logits.shape or t.stride(1) != 1:
+    ls, lc = logits.stride()
+    os_, oc = out.stride()
+    for t, c, nm in ((logits, lc, "logits"), (out, oc, "out")):
+        if c != 1 or t.shape != logits.shape:
             raise ValueError(f"{nm} must be [rows, vocab] with contiguous rows")
-    p = TopPParams()
-    p.n_rows, p.vocab = rows, V
-    p.logits, p.logits_row_stride = _dev(logits, "logits", torch.float32), (logits.stride(0) if rows > 1 else (V + 3) // 4 * 4)
-    p.out, p.out_row_stride = _dev(out, "out", torch.float32), (out.stride(0) if rows > 1 else (V + 3) // 4 * 4)
-    p.temperature, p.top_p = temperature, top_p
-    p.kept_out = _dev(kept_out, "kept_out", torch.int32)
-    p.dev_status = _dev(dev_status, "dev_status", torch.int32)
+    p = TopPParams(rows, V, _dev(logits, "logits", torch.float32), ls if rows > 1 else (V + 3) // 4 * 4,
+                   _dev(out, "out", torch.float32), os_ if rows > 1 else (V + 3) // 4 * 4, temperature, top_p,
+                   _dev(kept_out, "kept_out", torch.int32), _dev(dev_status, "dev_status", torch.int32))
     _check("seq_tree_top_p_filter", load().seq_tree_top_p_filter(C.byref(p), _stream(stream)))
     return out
 
@@ -490,19 +509,15 @@ def seq_tree_kv_commit(k_cache, v_cache, prefix_len: int, n_tree: int, path, pat
     seq_tree_verify wrote them).  k_cache / v_cache: [planes, rows, head_dim] (v_cache may be None), rows
     contiguous."""
     planes, rows, d = k_cache.shape
-    for t in (k_cache, v_cache):
-        if t is not None and (t.shape != k_cache.shape or t.stride() != k_cache.stride() or t.stride(2) != 1):
-            raise ValueError("k_cache and v_cache must be [planes, rows, head_dim] with the same strides, rows contiguous")
+    strides = k_cache.stride()
+    if strides[2] != 1 or (v_cache is not None and (v_cache.shape != k_cache.shape or v_cache.stride() != strides)):
+        raise ValueError("k_cache and v_cache must be [planes, rows, head_dim] with the same strides, rows contiguous")
     e = k_cache.element_size()
-    p = KvCommitParams()
-    p.num_planes, p.row_bytes, p.prefix_len, p.n_tree = planes, d * e, prefix_len, n_tree
-    p.k_cache, p.v_cache = _dev(k_cache, "k_cache"), _dev(v_cache, "v_cache")
-    p.plane_stride_bytes = (k_cache.stride(0) if planes > 1 else rows * k_cache.stride(1)) * e
-    p.row_stride_bytes = k_cache.stride(1) * e
-    p.path, p.path_len = _dev(path, "path", torch.int32), _dev(path_len, "path_len", torch.int32)
-    p.new_prefix_len = _dev(new_prefix_len, "new_prefix_len", torch.int32)
-    p.prefix_len_dev = _dev(prefix_len_dev, "prefix_len_dev", torch.int32)
-    p.dev_status = _dev(dev_status, "dev_status", torch.int32)
+    p = KvCommitParams(planes, d * e, prefix_len, n_tree, _dev(k_cache, "k_cache"), _dev(v_cache, "v_cache"),
+                       (strides[0] if planes > 1 else rows * strides[1]) * e, strides[1] * e,
+                       _dev(path, "path", torch.int32), _dev(path_len, "path_len", torch.int32),
+                       _dev(new_prefix_len, "new_prefix_len", torch.int32), _dev(dev_status, "dev_status", torch.int32),
+                       _dev(prefix_len_dev, "prefix_len_dev", torch.int32))
     _check("seq_tree_kv_commit", load().seq_tree_kv_commit(C.byref(p), _stream(stream)))
 
 
