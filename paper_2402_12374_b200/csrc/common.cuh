@@ -103,6 +103,8 @@ inline int once_per_device(int* done, F setup) {
 int validate_attention_params(const seq_tree_attention_params* p);
 int launch_attention_simt(const seq_tree_attention_params& p, int splits, cudaStream_t stream);
 int simt_default_splits(const seq_tree_attention_params& p);
+int launch_attention_f32(const seq_tree_attention_params& p, size_t max_workspace, cudaStream_t stream);
+int f32_splits(const seq_tree_attention_params& p);
 int launch_combine_splits(const seq_tree_attention_params& p, int splits, cudaStream_t stream);
 
 }  // namespace seqtree

@@ -60,8 +60,9 @@ int validate_attention_params(const seq_tree_attention_params* p) {
   return SEQ_OK;
 }
 
-// 1 = CUDA cores, 2 = tensor cores
+// 1 = CUDA cores (16-bit inputs), 2 = tensor cores, 3 = CUDA cores in single precision
 static int choose_kernel(const seq_tree_attention_params& p) {
+  if (p.dtype == SEQ_F32) return p.mask_bits != nullptr && p.kernel <= 1 ? 3 : 0;
   const bool ok = umma_supported(p);
   if (p.mask_bits == nullptr) return ok && p.kernel != 1 ? 2 : 0;  // only the tensor-core kernel derives the mask itself
   if (p.kernel == 1) return 1;
@@ -70,7 +71,7 @@ static int choose_kernel(const seq_tree_attention_params& p) {
   // Measured on B200: even with a single query row per kv head (127 of the tile's 128 rows padding) the
   // tensor-core kernel is faster than the CUDA-core one, because it streams K/V once per kv head with
   // TMA while the CUDA-core kernel re-reads them for every (node, head).  The CUDA-core kernel is kept
-  // for fp32 inputs and for groups of more than 128 heads.
+  // for callers that ask for it and for groups of more than 128 heads.
   return 2;
 }
 
@@ -83,7 +84,7 @@ extern "C" size_t seq_tree_attention_workspace_bytes(const seq_tree_attention_pa
   const int which = choose_kernel(*p);
   if (which == 0) return 0;
   if (which == 2) return umma_workspace_bytes(*p);  // only its stream mode (more units than SMs) needs one
-  const int splits = simt_default_splits(*p);
+  const int splits = which == 3 ? f32_splits(*p) : simt_default_splits(*p);
   size_t bytes = splits > 1 ? split_workspace_bytes(splits, p->num_q_heads, p->n_tree) : 0;
   return (bytes + 255) & ~(size_t)255;
 }
@@ -94,11 +95,12 @@ extern "C" int seq_tree_attention(const seq_tree_attention_params* p, void* stre
   const int which = choose_kernel(*p);
   if (which == 0) return SEQ_ERR_UNSUPPORTED;
   if (which == 2) return launch_attention_umma(*p, umma_default_splits(*p), (cudaStream_t)stream);
-  const int splits = simt_default_splits(*p);
+  const int splits = which == 3 ? f32_splits(*p) : simt_default_splits(*p);
   if (splits > 1) {
     if (p->workspace == nullptr || p->workspace_bytes < split_workspace_bytes(splits, p->num_q_heads, p->n_tree))
       return SEQ_ERR_WORKSPACE;
     if (reinterpret_cast<uintptr_t>(p->workspace) % 256 != 0) return SEQ_ERR_INVALID_ARG;
   }
+  if (which == 3) return launch_attention_f32(*p, ~(size_t)0, (cudaStream_t)stream);
   return launch_attention_simt(*p, splits, (cudaStream_t)stream);
 }

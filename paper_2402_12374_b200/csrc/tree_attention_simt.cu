@@ -1,5 +1,5 @@
-// Tree-masked attention on CUDA cores: the path for small trees, for the fp32 mode and for
-// shapes the tensor-core kernel does not take; plus the split-KV combine used by both kernels.
+// Tree-masked attention of 16-bit inputs on CUDA cores: for callers that ask for it (kernel = 1, or no scratch memory
+// to lend) and for groups of more than 128 heads; plus the split-KV combine, which the fp32 kernel uses too.
 //
 // One CTA per (node i, query head h, split).  Keys are taken in chunks of 32: in a chunk lane l
 // scores key l (a full 128-term dot product, q broadcast from shared memory), the warp agrees on
@@ -15,14 +15,6 @@ constexpr int kSimtWarps = 4;
 
 template <typename T>
 struct Vec16;  // 16-byte vector load of T
-template <>
-struct Vec16<float> {
-  static constexpr int kElems = 4;
-  __device__ static void load(const float* p, float* out) {
-    float4 v = *reinterpret_cast<const float4*>(p);
-    out[0] = v.x; out[1] = v.y; out[2] = v.z; out[3] = v.w;
-  }
-};
 template <>
 struct Vec16<__half> {
   static constexpr int kElems = 8;
@@ -52,11 +44,6 @@ struct Vec16<__nv_bfloat16> {
 
 template <typename T>
 __device__ __forceinline__ void load4(const T* p, float* out);
-template <>
-__device__ __forceinline__ void load4<float>(const float* p, float* out) {
-  float4 v = *reinterpret_cast<const float4*>(p);
-  out[0] = v.x; out[1] = v.y; out[2] = v.z; out[3] = v.w;
-}
 template <>
 __device__ __forceinline__ void load4<__half>(const __half* p, float* out) {
   uint2 v = *reinterpret_cast<const uint2*>(p);
@@ -234,6 +221,8 @@ combine_splits_kernel(const float* __restrict__ o_part, const float2* __restrict
                       float* __restrict__ lse) {
   const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   if (row >= Hq * n) return;
   const int h = row / n, i = row - h * n;
   const size_t rows = (size_t)Hq * n;
@@ -287,22 +276,25 @@ static int launch_simt_t(const seq_tree_attention_params& p, int splits, cudaStr
 }
 
 int launch_attention_simt(const seq_tree_attention_params& p, int splits, cudaStream_t stream) {
-  switch (p.dtype) {
-    case SEQ_F16: return launch_simt_t<__half>(p, splits, stream);
-    case SEQ_BF16: return launch_simt_t<__nv_bfloat16>(p, splits, stream);
-    case SEQ_F32: return launch_simt_t<float>(p, splits, stream);
-  }
-  return SEQ_ERR_INVALID_ARG;
+  if (p.dtype == SEQ_F16) return launch_simt_t<__half>(p, splits, stream);
+  return launch_simt_t<__nv_bfloat16>(p, splits, stream);
 }
 
 template <typename T>
 static int launch_combine_t(const seq_tree_attention_params& p, int splits, cudaStream_t stream) {
   SplitLayout sl = split_layout(p.workspace, splits, p.num_q_heads, p.n_tree);
   const int rows = p.num_q_heads * p.n_tree;
-  combine_splits_kernel<T><<<(rows + 3) / 4, 128, 0, stream>>>(
-      sl.o_part, sl.ml, splits, p.num_q_heads, p.n_tree, reinterpret_cast<T*>(p.out), p.o_stride_tok,
-      p.o_stride_head, p.lse);
-  SEQ_CUDA_OK(cudaGetLastError());
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((rows + 3) / 4);
+  cfg.blockDim = dim3(128);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // scheduled under the attention kernel's tail
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  SEQ_CUDA_OK(cudaLaunchKernelEx(&cfg, combine_splits_kernel<T>, (const float*)sl.o_part, (const float2*)sl.ml, splits,
+                                 p.num_q_heads, p.n_tree, reinterpret_cast<T*>(p.out), p.o_stride_tok, p.o_stride_head, p.lse));
   return SEQ_OK;
 }
 
@@ -354,5 +346,6 @@ extern "C" int seq_tree_attention_noalloc(const seq_tree_attention_params* p, vo
   q.workspace = g_noalloc_ptr[dev];
   q.workspace_bytes = SEQ_NOALLOC_SCRATCH_BYTES;
   q.kernel = 1;
+  if (p->dtype == SEQ_F32) return launch_attention_f32(q, SEQ_NOALLOC_SCRATCH_BYTES, (cudaStream_t)stream);
   return launch_attention_simt(q, splits, (cudaStream_t)stream);
 }

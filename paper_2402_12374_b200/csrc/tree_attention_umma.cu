@@ -54,9 +54,9 @@
 #include <cstddef>
 #include <cuda.h>
 #include <stdlib.h>
-#include <string.h>
 
 #include "common.cuh"
+#include "tensor_map.cuh"
 #include "trace_attention.cuh"
 
 namespace cg = cooperative_groups;
@@ -1016,66 +1016,6 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
 }
 
 // ---------------------------------------------------------------- host side ---------------------
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static EncodeTiledFn encode_fn() {
-  static void* cached = nullptr;  // the driver's entry point, looked up once (the same answer from every thread)
-  void* p = __atomic_load_n(&cached, __ATOMIC_ACQUIRE);
-  if (p == nullptr) {
-    cudaDriverEntryPointQueryResult qres;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres) != cudaSuccess ||
-        qres != cudaDriverEntryPointSuccess || p == nullptr)
-      return nullptr;
-    __atomic_store_n(&cached, p, __ATOMIC_RELEASE);
-  }
-  return reinterpret_cast<EncodeTiledFn>(p);
-}
-
-// Encoded tensor maps are kept: a caller that launches directly (no CUDA graph) passes the same pointers and shapes
-// step after step, and an encode is a driver call of a microsecond or two.  A map depends on nothing but the
-// arguments of the encode (the swizzle, interleave, promotion and fill are the same for every map of this file), so
-// the key is those arguments, compared byte for byte; 16 entries, replaced in turn; one lock around the table.
-namespace {
-struct MapKey {
-  const void* base;
-  cuuint64_t dims[5], strides[4];
-  cuuint32_t box[5];
-  int32_t rank, dtype;
-};
-struct MapEntry { MapKey key; CUtensorMap map; bool used; };
-MapEntry g_maps[16];
-unsigned g_maps_next = 0;
-int g_maps_lock = 0;
-
-CUresult encode_cached(EncodeTiledFn encode, CUtensorMap* out, CUtensorMapDataType dt, cuuint32_t rank, const void* base,
-                       const cuuint64_t* dims, const cuuint64_t* strides, const cuuint32_t* box) {
-  MapKey key;
-  memset(&key, 0, sizeof(key));
-  key.base = base; key.rank = (int32_t)rank; key.dtype = (int32_t)dt;
-  for (cuuint32_t i = 0; i < rank; ++i) { key.dims[i] = dims[i]; key.box[i] = box[i]; }
-  for (cuuint32_t i = 0; i + 1 < rank; ++i) key.strides[i] = strides[i];
-  while (__atomic_exchange_n(&g_maps_lock, 1, __ATOMIC_ACQUIRE) != 0) { }
-  for (MapEntry& e : g_maps)
-    if (e.used && memcmp(&e.key, &key, sizeof(key)) == 0) {
-      *out = e.map;
-      __atomic_store_n(&g_maps_lock, 0, __ATOMIC_RELEASE);
-      return CUDA_SUCCESS;
-    }
-  __atomic_store_n(&g_maps_lock, 0, __ATOMIC_RELEASE);
-  const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-  const CUresult r = encode(out, dt, rank, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) return r;
-  while (__atomic_exchange_n(&g_maps_lock, 1, __ATOMIC_ACQUIRE) != 0) { }
-  MapEntry& e = g_maps[g_maps_next++ % 16];
-  e.key = key; e.map = *out; e.used = true;
-  __atomic_store_n(&g_maps_lock, 0, __ATOMIC_RELEASE);
-  return CUDA_SUCCESS;
-}
-}  // namespace
-
 bool umma_supported(const seq_tree_attention_params& p) {
   if (p.dtype != SEQ_F16 && p.dtype != SEQ_BF16) return false;
   return p.num_q_heads / p.num_kv_heads <= kTileM;  // a tile holds at least one node's group of heads
@@ -1144,8 +1084,6 @@ size_t umma_workspace_bytes(const seq_tree_attention_params& p) {
 }
 
 int launch_attention_umma(const seq_tree_attention_params& p, int splits, cudaStream_t stream) {
-  EncodeTiledFn encode = encode_fn();
-  if (encode == nullptr) return SEQ_ERR_CUDA;
   const int G = p.num_q_heads / p.num_kv_heads;
   const int nodes_per_tile = kTileM / G;
   const int tiles = (p.n_tree + nodes_per_tile - 1) / nodes_per_tile;
@@ -1160,7 +1098,7 @@ int launch_attention_umma(const seq_tree_attention_params& p, int splits, cudaSt
     cuuint64_t strides[4] = {(cuuint64_t)p.q_stride_head * 2, (cuuint64_t)p.q_stride_tok * 2, 128,
                              (cuuint64_t)p.q_stride_head * 2 * G};
     cuuint32_t box[5] = {64, (cuuint32_t)G, (cuuint32_t)nodes_per_tile, kTileM % G == 0 ? 2u : 1u, 1};  // (see load_q)
-    if (encode_cached(encode, &q_map, dt, 5, p.q, dims, strides, box) != CUDA_SUCCESS) return SEQ_ERR_CUDA;
+    if (!tensor_map(&q_map, dt, 5, p.q, dims, strides, box)) return SEQ_ERR_CUDA;
   }
   for (int which = 0; which < 2; ++which) {
     // only the live rows [0, prefix_len + n_tree) are mapped: anything past them reads as zero.  (With the prefix
@@ -1168,8 +1106,7 @@ int launch_attention_umma(const seq_tree_attention_params& p, int splits, cudaSt
     cuuint64_t dims[4] = {64, (cuuint64_t)(p.prefix_len_dev != nullptr ? p.kv_capacity : p.prefix_len + p.n_tree), 2, (cuuint64_t)p.num_kv_heads};
     cuuint64_t strides[3] = {(cuuint64_t)p.kv_stride_tok * 2, 128, (cuuint64_t)p.kv_stride_head * 2};
     cuuint32_t box[4] = {64, (cuuint32_t)kBlockN, 2, 1};
-    if (encode_cached(encode, which == 0 ? &k_map : &v_map, dt, 4, which == 0 ? p.k_cache : p.v_cache, dims, strides, box) != CUDA_SUCCESS)
-      return SEQ_ERR_CUDA;
+    if (!tensor_map(which == 0 ? &k_map : &v_map, dt, 4, which == 0 ? p.k_cache : p.v_cache, dims, strides, box)) return SEQ_ERR_CUDA;
   }
 
   UmmaArgs a;

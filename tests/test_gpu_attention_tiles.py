@@ -1,0 +1,50 @@
+"""Attention at the sizes where a tile can go wrong, every output against the oracle: groups of heads that do not divide a
+tile of 128 rows on the tensor cores, and the single-precision kernel at the edges of its row tiles (8, 16, 32, 64 rows),
+of its groups of 32 keys and of its key-range splits."""
+from __future__ import annotations
+
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as O
+from paper_2402_12374_b200 import binding as B
+from paper_2402_12374_b200 import workloads as W
+from tests import gpu_util as G
+
+pytestmark = pytest.mark.gpu
+
+
+def _inputs(hkv, group, n, L, dtype, seed=3):
+    cfg = dataclasses.replace(W.CONFIGS["tiny"], num_q_heads=hkv * group, num_kv_heads=hkv, prefix_len=L, n_tree=n, max_depth=14, max_fanout=8)
+    return W.make_attention_inputs(cfg, seed, dtype=dtype, extra_capacity=9)
+
+
+@pytest.mark.parametrize("kernel", [B.KERNEL_AUTO, B.KERNEL_TENSOR_CORE_STREAM, B.KERNEL_TENSOR_CORE_GRID])
+@pytest.mark.parametrize("hkv,group,n,L", [(1, 3, 42, 33), (1, 3, 43, 0), (2, 5, 25, 64), (2, 5, 101, 150), (1, 6, 1, 20), (2, 7, 36, 300),
+                                           (1, 12, 25, 63), (1, 100, 3, 50), (1, 127, 2, 65)])
+def test_groups_that_do_not_divide_the_tile(hkv, group, n, L, kernel):
+    G.check_attention(_inputs(hkv, group, n, L, "bf16"), kernel=kernel)
+
+
+@pytest.mark.parametrize("hkv,group,n,L", [(1, 1, 1, 0), (2, 1, 8, 31), (1, 1, 9, 119), (1, 2, 8, 128), (2, 3, 11, 97), (1, 1, 32, 96), (1, 1, 33, 224),
+                                           (2, 4, 16, 255), (1, 5, 13, 64), (3, 1, 65, 63), (1, 150, 2, 40), (1, 1, 1, 3000)])
+def test_single_precision_tiles(hkv, group, n, L):
+    G.check_attention(_inputs(hkv, group, n, L, "fp32"))
+
+
+def test_single_precision_with_the_length_in_device_memory():
+    """Rows behind the tree hold NaN: they are fetched in this mode and must not reach a result."""
+    d = G.dev()
+    n, L, slack = 21, 75, 60
+    ai = _inputs(2, 3, n, L, "fp32")
+    pad = torch.full((2, slack, 128), float("nan"))
+    k, v = (torch.cat([t[:, :L + n], pad], dim=1).contiguous().to(d) for t in (ai.k_cache, ai.v_cache))
+    mask, _, st = G.gpu_mask(ai.parent.numpy())
+    out = B.seq_tree_attention(ai.q.to(d), k, v, mask, L + slack - 1, dev_status=st, prefix_len_dev=torch.tensor([L], dtype=torch.int32, device=d))
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    ref, _, _ = O.tree_attention(ai.q, ai.k_cache[:, :L + n], ai.v_cache[:, :L + n], ai.parent, L)
+    assert np.abs(out.double().cpu().numpy() - ref).max() < 1e-5
