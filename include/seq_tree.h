@@ -342,11 +342,10 @@ int seq_tree_verify_batch(const seq_tree_verify_batch_params* p, void* stream);
  *   tokens_out     int32 [n_rows][k], device: the drawn tokens in draw order, -1 where no token with
  *                  positive probability was left.
  *   dev_status     nullable.
- *   workspace      seq_tree_draft_sample_workspace_bytes(p) bytes, 8-byte aligned, device, contents
- *                  undefined before and after: the k best (score, token) pairs of every 4096-token chunk
- *                  of every row (two launches: per-chunk draws, then the row's draws among them).
+ *   workspace      seq_tree_draft_sample_workspace_bytes(p) bytes, which is 0: a row's candidates meet in shared
+ *                  memory.  The fields stay in the struct and are not read.
  * The decision is taken in fp32 (on the logarithm of the inverse key): two keys closer than fp32 resolves
- * may come out in either order.  Returns SEQ_OK, SEQ_ERR_INVALID_ARG, SEQ_ERR_WORKSPACE, or
+ * may come out in either order.  Returns SEQ_OK, SEQ_ERR_INVALID_ARG, SEQ_ERR_CUDA, or
  * SEQ_ERR_UNSUPPORTED (vocab/4096 * k above 25600).
  */
 typedef struct {

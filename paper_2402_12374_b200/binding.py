@@ -222,18 +222,12 @@ def seq_tree_draft_sample(draft_logits, temperature: float, uniforms, k: int, *,
         raise ValueError("draft_logits and uniforms must be [rows, vocab] with contiguous rows")
     if tokens_out is None:
         tokens_out = torch.empty((rows, k), dtype=torch.int32, device=draft_logits.device)
-    lib = load()
     p = DraftSampleParams(rows, V, k, _dev(draft_logits, "draft_logits", torch.float32), ls if rows > 1 else V,
                           _dev(uniforms, "uniforms", torch.float32), us if rows > 1 else V, temperature,
                           _dev(tokens_out, "tokens_out", torch.int32), _dev(dev_status, "dev_status", torch.int32))
-    ref = C.byref(p)
-    if workspace is None:
-        need = lib.seq_tree_draft_sample_workspace_bytes(ref)
-        if need:
-            workspace = torch.empty(need, dtype=torch.uint8, device=draft_logits.device)
-    if workspace is not None:
+    if workspace is not None:  # (none is needed)
         p.workspace, p.workspace_bytes = _dev(workspace, "workspace"), workspace.numel() * workspace.element_size()
-    _check("seq_tree_draft_sample", lib.seq_tree_draft_sample(ref, _stream(stream)))
+    _check("seq_tree_draft_sample", load().seq_tree_draft_sample(C.byref(p), _stream(stream)))
     return tokens_out
 
 

@@ -7,32 +7,44 @@
 // every token of a row and drops out), and take the k largest in descending order, ties to the lower
 // token.  No pass for a maximum or a sum is needed: a row is read once.
 //
-// Two launches.  (1) One CTA per (row, chunk of 4096 tokens): every thread computes the scores of its 16
-// tokens (16-byte loads when the rows allow them) into shared memory and remembers its best; a draw is one
-// block-wide arg-max over the threads' bests, after which only the thread that owned the winner looks through
-// its tokens again; the chunk's k best (score, token) pairs go to the workspace.  The k best of a row are
-// among the k best of its chunks.  (2) One CTA per row draws k times from those candidates the same way.
-// Many small CTAs per SM keep the special-function and load latencies of step (1) covered.
+// One CTA takes a part of a row - all of it when there are enough rows - in steps of 4096 tokens, the next step's loads in
+// flight while one is worked on.  Almost every token only has to be shown to be out of the running, and for that an upper
+// bound of its score will do: -log u >= 1 - u, so score <= logit/T - log(1 - u), one logarithm and a handful of
+// instructions, tight where the winners are (u near 1).  The first step finds a threshold that k tokens are known to reach
+// (each thread scores the token with its best bound; the k-th largest of the bests of 64 or 128 groups of threads); after
+// that only tokens whose bound passes the threshold are listed.  Whenever the steps done have doubled (about k tokens pass
+// in that time), and at the end, the listed tokens are scored and ranked against each other, the k best stay and the
+// threshold becomes the k-th score itself.  A list that overflows (long runs of equal scores) sends the part through the
+// same ranking 256 tokens at a time.  The parts of a row are a thread-block cluster (up to 8): each pushes its k best into
+// the first CTA's shared memory, which ranks them in the same way.  No workspace, one launch.
+//
+// What bounds it: the two streams of logits and uniforms from HBM.  378 rows of 128256 tokens, k = 9: k block-wide arg-max
+// rounds per 4096 tokens and two logarithms and a series per token took 213 us; this takes 62 (95 % of the copy
+// bandwidth of 6.55 TB/s; k = 32: 72).  A few short rows are bound by the chain of steps, rankings and the cluster: 5 us.
+#include <cooperative_groups.h>
 #include <float.h>
 #include <math.h>
 
 #include "common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace seqtree {
 
 constexpr int kDsThreads = 256;
 constexpr int kDsWarps = kDsThreads / 32;
 constexpr int kDsMaxK = 64;
-constexpr int kDsChunk = 4096;                  // tokens per CTA of the first launch
-constexpr int kDsPerThread = kDsChunk / kDsThreads;  // 16: four groups of four consecutive tokens
+constexpr int kDsStep = 4096;            // tokens per step of a CTA
+constexpr int kDsE = kDsStep / kDsThreads;  // 16 per thread
+constexpr int kDsList = 1024;            // tokens in the running
+constexpr int kDsMaxParts = 8;           // CTAs per row: a portable cluster
 
 struct DraftSampleArgs {
-  int32_t n_rows, V, k, vec_ok, chunks;
+  int32_t n_rows, V, k, parts, part_tokens;  // part_tokens: a multiple of the step
   const float* logits; int64_t logits_stride;
   const float* uniforms; int64_t uniforms_stride;
   float inv_T;
   int32_t* out;
-  float2* cand;  // [n_rows][chunks][k] (score, token bits)
   int32_t* dev_status;
 };
 
@@ -58,133 +70,265 @@ __device__ __forceinline__ float ds_score(float logit, float u, float inv_T, boo
   return logit * inv_T - __logf(ds_neg_log(u));
 }
 
-__device__ __forceinline__ void ds_better(float& bs, int& bi, float s, int i) {
-  if (s > bs || (s == bs && i < bi)) { bs = s; bi = i; }
-}
+struct DsShared {
+  float2 list[kDsList];  // (score, token bits); behind the ranked ones, tokens not scored yet
+  __align__(16) float top[128];  // the first step's group maxima
+  float2 cand[kDsMaxParts * kDsMaxK];  // the first CTA of a cluster: every part's k best, in order
+  float tau;             // a score that k tokens reach, -inf before there are k
+  int count;
+};
 
-// Warp-wide arg-max of (s, i): larger score, then lower index, in two redux instructions (scores mapped to
-// integers in the same order).  Result in every lane.
-__device__ __forceinline__ void ds_warp_argmax(float& s, int& i) {
-  int b = __float_as_int(s);
-  b ^= (b >> 31) & 0x7fffffff;
-  const int m = __reduce_max_sync(0xffffffffu, b);
-  i = __reduce_min_sync(0xffffffffu, b == m ? i : 0x7fffffff);
-  b = m ^ ((m >> 31) & 0x7fffffff);
-  s = __int_as_float(b);
-}
-// Block-wide arg-max.  Result in every thread.  The per-warp results go through one of two shared buffers,
-// alternating from call to call (`round`), so that one barrier per call is enough: a thread can be at most one
-// call ahead of the slowest reader, which then still reads the other buffer.
-__device__ __forceinline__ void ds_block_argmax(float& s, int& i, float (*w_s)[kDsWarps], int (*w_i)[kDsWarps], int round) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, buf = round & 1;
-  ds_warp_argmax(s, i);
-  if (lane == 0) { w_s[buf][warp] = s; w_i[buf][warp] = i; }
-  __syncthreads();
-  s = lane < kDsWarps ? w_s[buf][lane] : -INFINITY;
-  i = lane < kDsWarps ? w_i[buf][lane] : 0x7fffffff;
-  ds_warp_argmax(s, i);
-}
-
-// (1) the k best of one chunk of one row, best first; slots past the last token with a chance: (-inf, -1)
-__global__ void __launch_bounds__(kDsThreads) draft_sample_chunk_kernel(const DraftSampleArgs a) {
-  __shared__ float sc[kDsChunk];
-  __shared__ float w_s[2][kDsWarps];
-  __shared__ int w_i[2][kDsWarps];
-  const int chunk = blockIdx.x, row = blockIdx.y, tid = threadIdx.x;
-  const int base = chunk * kDsChunk, cnt = min(kDsChunk, a.V - base);
-  const float* lrow = a.logits + (int64_t)row * a.logits_stride + base;
-  const float* urow = a.uniforms + (int64_t)row * a.uniforms_stride + base;
-  bool bad = false;
-  float bs = -INFINITY;
-  int bi = 0x7fffffff;
-  // group g of four tokens belongs to thread g % 256
+// Ranks the first `count` entries of the list against each other - larger score first, then lower token -, leaves the k
+// best in order at its front, their number in sh.count and, once there are k, the last one's score in sh.tau.  Entries
+// without a chance (-inf) drop out.  All threads call it after a barrier behind the last write to the list.
+__device__ __forceinline__ void ds_compact(DsShared& sh, int count, int k) {
+  const int tid = threadIdx.x;
+  if (count <= kDsThreads / 2) {
+    // a short list: two, four or eight threads share an entry's comparisons
+    const int share = count <= kDsThreads / 8 ? 8 : count <= kDsThreads / 4 ? 4 : 2;
+    const int j = tid / share;
+    float2 mine = make_float2(-INFINITY, 0.f);
+    int rank = 0;
+    if (j < count) mine = sh.list[j];
+    const bool live = mine.x > -INFINITY;
+    const int mi = __float_as_int(mine.y);
+    for (int o = tid % share; o < count; o += share) {
+      const float2 x = sh.list[o];
+      rank += x.x > mine.x || (x.x == mine.x && __float_as_int(x.y) < mi);
+    }
+    for (int d = 1; d < share; d <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, d);
+    const int total = __syncthreads_count(live && tid % share == 0);  // (also: everyone has read the list)
+    if (live && tid % share == 0 && rank < k) {
+      sh.list[rank] = mine;
+      if (rank == k - 1) sh.tau = mine.x;
+    }
+    if (tid == 0) sh.count = min(total, k);
+    __syncthreads();
+    return;
+  }
+  float2 mine[kDsList / kDsThreads];
+  int rank[kDsList / kDsThreads];
+  int live = 0;
 #pragma unroll
-  for (int j = 0; j < kDsPerThread / 4; ++j) {
-    const int t0 = 4 * (tid + kDsThreads * j);
-    float s[4];
-    if (a.vec_ok && t0 + 3 < cnt) {
-      const float4 x = *reinterpret_cast<const float4*>(lrow + t0);
-      const float4 u = *reinterpret_cast<const float4*>(urow + t0);
-      s[0] = ds_score(x.x, u.x, a.inv_T, bad); s[1] = ds_score(x.y, u.y, a.inv_T, bad);
-      s[2] = ds_score(x.z, u.z, a.inv_T, bad); s[3] = ds_score(x.w, u.w, a.inv_T, bad);
+  for (int q = 0; q < kDsList / kDsThreads; ++q) {
+    const int j = tid + q * kDsThreads;
+    rank[q] = k;
+    if (j >= count) continue;
+    mine[q] = sh.list[j];
+    if (!(mine[q].x > -INFINITY)) continue;
+    ++live;
+    const int mi = __float_as_int(mine[q].y);
+    int r = 0;
+#pragma unroll 4
+    for (int o = 0; o < count; ++o) {
+      const float2 x = sh.list[o];
+      r += x.x > mine[q].x || (x.x == mine[q].x && __float_as_int(x.y) < mi);
+    }
+    rank[q] = r;
+  }
+  int total = __syncthreads_count(live > 0);  // (also: everyone has read the list)
+  if (count > kDsThreads)
+    for (int extra = 2; extra <= kDsList / kDsThreads; ++extra) total += __syncthreads_count(live >= extra);
+#pragma unroll
+  for (int q = 0; q < kDsList / kDsThreads; ++q)
+    if (rank[q] < k) {
+      sh.list[rank[q]] = mine[q];
+      if (rank[q] == k - 1) sh.tau = mine[q].x;
+    }
+  if (tid == 0) sh.count = min(total, k);
+  __syncthreads();
+}
+
+// The bound a token has to pass: the threshold less what the bounds' rounding may cost (31 ulp of place in the first step,
+// a few ulp of the approximations).
+__device__ __forceinline__ float ds_cut(float tau) { return fminf(tau - 1e-3f - 1e-5f * fminf(fabsf(tau), 1e30f), 3e38f); }
+
+template <bool kVec>
+__global__ void __launch_bounds__(kDsThreads) draft_sample_kernel(const DraftSampleArgs a) {
+  __shared__ DsShared sh;
+  const int part = blockIdx.x, row = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (a.parts > 1) cg::this_cluster().barrier_arrive();  // waited for before the first remote store
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int lo = part * a.part_tokens, cnt = min(a.part_tokens, a.V - lo);
+  const float* lrow = a.logits + (int64_t)row * a.logits_stride + lo;
+  const float* urow = a.uniforms + (int64_t)row * a.uniforms_stride + lo;
+  // a thread's tokens of a step: groups of four consecutive ones (kVec), else every 256th
+  auto token_of = [&](int t0, int e) { return t0 + (kVec ? 4 * (tid + kDsThreads * (e >> 2)) + (e & 3) : tid + kDsThreads * e); };
+  float x[kDsE], u[kDsE];
+  auto fetch = [&](int t0) {  // tokens past the part: no chance
+    if (kVec) {
+#pragma unroll
+      for (int j = 0; j < kDsE / 4; ++j) {
+        const int t = token_of(t0, 4 * j);
+        const bool in = t < cnt;  // (cnt is a multiple of 4 here)
+        const float4 xv = in ? __ldg(reinterpret_cast<const float4*>(lrow + t)) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+        const float4 uv = in ? __ldg(reinterpret_cast<const float4*>(urow + t)) : make_float4(0.5f, 0.5f, 0.5f, 0.5f);
+        x[4 * j] = xv.x; x[4 * j + 1] = xv.y; x[4 * j + 2] = xv.z; x[4 * j + 3] = xv.w;
+        u[4 * j] = uv.x; u[4 * j + 1] = uv.y; u[4 * j + 2] = uv.z; u[4 * j + 3] = uv.w;
+      }
     } else {
 #pragma unroll
-      for (int e = 0; e < 4; ++e) s[e] = t0 + e < cnt ? ds_score(lrow[t0 + e], urow[t0 + e], a.inv_T, bad) : -INFINITY;
-    }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      sc[t0 + e] = s[e];
-      if (t0 + e < cnt) ds_better(bs, bi, s[e], t0 + e);
-    }
-  }
-  if (bad) dev_flag(a.dev_status, SEQ_DEV_NONFINITE);
-
-  float2* cand = a.cand + ((int64_t)row * a.chunks + chunk) * a.k;
-  for (int r = 0; r < a.k; ++r) {
-    float s = bs;
-    int i = bi;
-    ds_block_argmax(s, i, w_s, w_i, r);
-    if (!(s > -INFINITY)) {  // nothing with a chance is left in this chunk
-      for (int j = r + tid; j < a.k; j += kDsThreads) cand[j] = make_float2(-INFINITY, __int_as_float(-1));
-      return;
-    }
-    if (tid == 0) cand[r] = make_float2(s, __int_as_float(base + i));
-    if (((i >> 2) % kDsThreads) == tid) {  // the owner of the winner finds its next best
-      sc[i] = -INFINITY;
-      bs = -INFINITY;
-      bi = 0x7fffffff;
-#pragma unroll
-      for (int j = 0; j < kDsPerThread / 4; ++j) {
-        const int t0 = 4 * (tid + kDsThreads * j);
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-          if (t0 + e < cnt) ds_better(bs, bi, sc[t0 + e], t0 + e);
+      for (int e = 0; e < kDsE; ++e) {
+        const int t = token_of(t0, e);
+        x[e] = t < cnt ? __ldg(lrow + t) : -INFINITY;
+        u[e] = t < cnt ? __ldg(urow + t) : 0.5f;
       }
     }
-  }
-}
-
-// (2) the k best of a row from its chunks' candidates (chunks * k of them), in draw order
-__global__ void __launch_bounds__(kDsThreads) draft_sample_merge_kernel(const DraftSampleArgs a) {
-  __shared__ float w_s[2][kDsWarps];
-  __shared__ int w_i[2][kDsWarps];
-  extern __shared__ float2 cs[];  // the row's candidates
-  const int row = blockIdx.x, tid = threadIdx.x;
-  const int n = a.chunks * a.k;
-  const float2* cand = a.cand + (int64_t)row * n;
-  for (int j = tid; j < n; j += kDsThreads) cs[j] = cand[j];
-  __syncthreads();
-  // candidate j belongs to thread j % 256; a thread's best is (score, token), compared like everywhere else
-  auto rescan = [&](float& bs, int& bi, int& bj) {
-    bs = -INFINITY; bi = 0x7fffffff; bj = -1;
-    for (int j = tid; j < n; j += kDsThreads) {
-      const float s = cs[j].x;
-      const int t = __float_as_int(cs[j].y);
-      if (t >= 0 && (s > bs || (s == bs && t < bi))) { bs = s; bi = t; bj = j; }
-    }
   };
-  float bs; int bi, bj;
-  rescan(bs, bi, bj);
-  int32_t* out = a.out + (int64_t)row * a.k;
-  for (int r = 0; r < a.k; ++r) {
-    float s = bs;
-    int i = bi;
-    ds_block_argmax(s, i, w_s, w_i, r);
-    if (!(s > -INFINITY)) {  // the remaining draws do not exist
-      for (int j = r + tid; j < a.k; j += kDsThreads) out[j] = -1;
-      return;
+  bool bad = false, unused = false;
+  // The bounds of the fetched tokens into ub, their largest returned.  A bound that is not a number stands for "look at the score".
+  float ub[kDsE];
+  auto bounds = [&](bool place) -> float {
+    float best = -INFINITY;
+#pragma unroll
+    for (int e = 0; e < kDsE; ++e) {
+      bad |= !(x[e] < INFINITY);  // NaN or +inf logit: flagged, never drawn
+      float b = fminf(fmaf(__log2f(1.f - u[e]), -kLn2, x[e] * a.inv_T), FLT_MAX);
+      if (place && b > -INFINITY) b = __uint_as_float((__float_as_uint(b) & ~31u) | (uint32_t)e);  // the token's place in the lowest bits
+      ub[e] = b;
+      best = fmaxf(best, b);
     }
-    if (tid == 0) out[r] = i;
-    if (bi == i && bj >= 0) {  // tokens are unique among the candidates: this thread held the winner
-      cs[bj] = make_float2(-INFINITY, __int_as_float(-1));
-      rescan(bs, bi, bj);
+    return best;
+  };
+  auto list_passing = [&](int t0, float cut) {
+#pragma unroll
+    for (int e = 0; e < kDsE; ++e)
+      if (ub[e] > cut) {
+        const int pos = atomicAdd(&sh.count, 1);
+        if (pos < kDsList) sh.list[pos].y = __int_as_float(token_of(t0, e));
+      }
+  };
+
+  // ---- first step: the threshold
+  fetch(0);
+  {
+    const float best = bounds(true);
+    fetch(kDsStep);
+    float top = -INFINITY;
+    if (best > -INFINITY) {
+      const int t = token_of(0, (int)(__float_as_uint(best) & 31u) % kDsE);
+      if (t < cnt) top = ds_score(lrow[t], urow[t], a.inv_T, unused);
+    }
+    const int share = a.k > 16 ? 2 : 4, groups = kDsThreads / share;
+    top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 1));
+    if (share == 4) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, 2));
+    if (tid % share == 0) sh.top[tid / share] = top;
+    if (tid == 0) { sh.tau = -INFINITY; sh.count = 0; }
+    __syncthreads();
+    if (tid < groups) {
+      const float mine = sh.top[tid];
+      int above = 0, reach = 0;
+#pragma unroll 8
+      for (int o = 0; o < groups; o += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(&sh.top[o]);
+        above += (v.x > mine) + (v.y > mine) + (v.z > mine) + (v.w > mine);
+        reach += (v.x >= mine) + (v.y >= mine) + (v.z >= mine) + (v.w >= mine);
+      }
+      if (above < a.k && a.k <= reach) sh.tau = mine;  // (equal ones write the same value)
+    }
+    __syncthreads();
+  }
+  float cut = ds_cut(sh.tau);
+  list_passing(0, cut);
+
+  // ---- the other steps: bounds against the threshold, a ranking every few of them
+  int ranked = 0;  // entries at the list's front that carry their score
+  bool overflow = false;
+  auto rank_list = [&]() {
+    __syncthreads();
+    const int count = sh.count;
+    overflow |= count > kDsList;
+    if (overflow) return;
+    for (int j = ranked + tid; j < count; j += kDsThreads) {
+      const int t = __float_as_int(sh.list[j].y);
+      sh.list[j].x = ds_score(lrow[t], urow[t], a.inv_T, unused);
+    }
+    __syncthreads();
+    ds_compact(sh, count, a.k);
+    ranked = sh.count;
+    cut = ds_cut(sh.tau);
+  };
+  for (int t0 = kDsStep, step = 1; t0 < cnt; t0 += kDsStep, ++step) {
+    const float best = bounds(false);
+    if (t0 + kDsStep < cnt) fetch(t0 + kDsStep);
+    if (best > cut) list_passing(t0, cut);
+    if ((step & (step + 1)) == 0) rank_list();
+  }
+  rank_list();
+  if (bad) dev_flag(a.dev_status, SEQ_DEV_NONFINITE);
+  if (overflow) {
+    __syncthreads();
+    if (tid == 0) { sh.count = 0; sh.tau = -INFINITY; }
+    __syncthreads();
+    for (int t0 = 0; t0 < cnt; t0 += kDsThreads) {
+      const int t = t0 + tid;
+      const float s = t < cnt ? ds_score(lrow[t], urow[t], a.inv_T, unused) : -INFINITY;
+      if (s > -INFINITY && s >= sh.tau) sh.list[atomicAdd(&sh.count, 1)] = make_float2(s, __int_as_float(t));
+      __syncthreads();
+      const int count = sh.count;
+      __syncthreads();
+      ds_compact(sh, count, a.k);
     }
   }
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  int have = sh.count;
+  if (a.parts > 1) {
+    cg::this_cluster().barrier_wait();  // the first CTA runs: its shared memory may be written
+    float2* to = cg::this_cluster().map_shared_rank(sh.cand, 0) + part * a.k;
+    for (int j = tid; j < a.k; j += kDsThreads) {
+      const float2 e = j < have ? sh.list[j] : make_float2(-INFINITY, 0.f);
+      to[j] = make_float2(e.x, __int_as_float(lo + __float_as_int(e.y)));
+    }
+    cg::this_cluster().sync();
+    if (part != 0) return;
+    // Threshold: warp w looks at the d-th candidate of every part, d = 2^w and k at last; the ceil(k / d)-th largest of
+    // them is reached by d candidates of each of ceil(k / d) parts, hence by k.  The largest such bound lets few more than
+    // k pass, however the row's best spread over the parts.
+    float kth = -INFINITY;
+    if (warp < 7) {
+      const int d = min(1 << warp, a.k), need = (a.k + d - 1) / d;
+      const float mine = lane < a.parts ? sh.cand[lane * a.k + d - 1].x : -INFINITY;
+      int above = 0, reach = 0;
+#pragma unroll
+      for (int o = 0; o < kDsMaxParts; ++o) {
+        const float v = __shfl_sync(0xffffffffu, mine, o);
+        above += v > mine;
+        reach += v >= mine;
+      }
+      kth = warp_max(lane < a.parts && above < need && need <= reach ? mine : -INFINITY);
+    }
+    if (tid == 0) sh.count = 0;
+    if (lane == 0) sh.top[warp] = kth;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kDsWarps; ++w) kth = fmaxf(kth, sh.top[w]);
+    for (int j = tid; j < a.parts * a.k; j += kDsThreads) {
+      const float2 c = sh.cand[j];
+      if (c.x > -INFINITY && c.x >= kth) sh.list[atomicAdd(&sh.count, 1)] = c;
+    }
+    __syncthreads();
+    const int count = sh.count;
+    __syncthreads();
+    ds_compact(sh, count, a.k);
+    have = sh.count;
+  }
+  for (int j = tid; j < a.k; j += kDsThreads) a.out[(int64_t)row * a.k + j] = j < have ? __float_as_int(sh.list[j].y) : -1;
 }
 
 }  // namespace seqtree
 
 using namespace seqtree;
+
+// Parts per row: as many as give every SM three CTAs (about what its memory pipeline needs in flight), of at least one
+// step each, eight at most (the CTAs of a row are a portable cluster).
+static int ds_part_tokens(const seq_tree_draft_sample_params* p) {
+  const int steps = (p->vocab + kDsStep - 1) / kDsStep;
+  const int want = (int)(((int64_t)device_sm_count() * 3 + p->n_rows / 2) / p->n_rows);
+  const int most = steps < kDsMaxParts ? steps : kDsMaxParts;
+  const int parts = want < 1 ? 1 : want > most ? most : want;
+  return (steps + parts - 1) / parts * kDsStep;
+}
+static int ds_parts(const seq_tree_draft_sample_params* p) { return (p->vocab + ds_part_tokens(p) - 1) / ds_part_tokens(p); }
 
 static int ds_validate(const seq_tree_draft_sample_params* p) {
   if (p == nullptr || p->draft_logits == nullptr || p->uniforms == nullptr || p->tokens_out == nullptr)
@@ -198,36 +342,38 @@ static int ds_validate(const seq_tree_draft_sample_params* p) {
 }
 
 extern "C" size_t seq_tree_draft_sample_workspace_bytes(const seq_tree_draft_sample_params* p) {
-  if (ds_validate(p) != SEQ_OK) return 0;
-  const size_t chunks = (p->vocab + kDsChunk - 1) / kDsChunk;
-  return (((size_t)p->n_rows * chunks * p->k * sizeof(float2)) + 255) & ~(size_t)255;
+  (void)p;
+  return 0;  // the candidates of a row's parts meet in shared memory
 }
 
 extern "C" int seq_tree_draft_sample(const seq_tree_draft_sample_params* p, void* stream) {
   const int rc = ds_validate(p);
   if (rc != SEQ_OK) return rc;
-  const int chunks = (p->vocab + kDsChunk - 1) / kDsChunk;
-  const size_t need = (size_t)p->n_rows * chunks * p->k * sizeof(float2);
-  if (p->workspace == nullptr || p->workspace_bytes < need) return SEQ_ERR_WORKSPACE;
-  if (reinterpret_cast<uintptr_t>(p->workspace) % 8 != 0) return SEQ_ERR_INVALID_ARG;
+  if ((int64_t)(p->vocab + kDsStep - 1) / kDsStep * p->k > 25600) return SEQ_ERR_UNSUPPORTED;  // vocabularies beyond 1.6 M tokens at k = 64
+  const int parts = ds_parts(p);
   DraftSampleArgs a;
-  a.n_rows = p->n_rows; a.V = p->vocab; a.k = p->k; a.chunks = chunks;
+  a.n_rows = p->n_rows; a.V = p->vocab; a.k = p->k; a.parts = parts; a.part_tokens = ds_part_tokens(p);
   a.logits = p->draft_logits; a.logits_stride = p->logits_row_stride;
   a.uniforms = p->uniforms; a.uniforms_stride = p->uniforms_row_stride;
   a.inv_T = 1.f / p->temperature;
   a.out = p->tokens_out;
-  a.cand = static_cast<float2*>(p->workspace);
   a.dev_status = p->dev_status;
-  // a chunk starts at a multiple of 4096 tokens, so 16-byte alignment of the rows carries over to the chunks
-  a.vec_ok = reinterpret_cast<uintptr_t>(p->draft_logits) % 16 == 0 && reinterpret_cast<uintptr_t>(p->uniforms) % 16 == 0 &&
-             p->logits_row_stride % 4 == 0 && p->uniforms_row_stride % 4 == 0;
-  const size_t smem = (size_t)chunks * p->k * sizeof(float2);
-  if (smem > 200 * 1024) return SEQ_ERR_UNSUPPORTED;  // vocabularies beyond 1.6 M tokens at k = 64
-  draft_sample_chunk_kernel<<<dim3(chunks, p->n_rows), kDsThreads, 0, (cudaStream_t)stream>>>(a);
-  SEQ_CUDA_OK(cudaGetLastError());
-  if (smem > 48 * 1024)
-    SEQ_CUDA_OK(cudaFuncSetAttribute(draft_sample_merge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  draft_sample_merge_kernel<<<p->n_rows, kDsThreads, smem, (cudaStream_t)stream>>>(a);
-  SEQ_CUDA_OK(cudaGetLastError());
+  // a part starts at a multiple of 4096 tokens, so 16-byte alignment of the rows carries over to the parts
+  const bool vec = reinterpret_cast<uintptr_t>(p->draft_logits) % 16 == 0 && reinterpret_cast<uintptr_t>(p->uniforms) % 16 == 0 &&
+             p->logits_row_stride % 4 == 0 && p->uniforms_row_stride % 4 == 0 && p->vocab % 4 == 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(parts, p->n_rows);
+  cfg.blockDim = dim3(kDsThreads);
+  cfg.stream = (cudaStream_t)stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = parts;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // scheduled under the tail of the launch before
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  SEQ_CUDA_OK(vec ? cudaLaunchKernelEx(&cfg, draft_sample_kernel<true>, a) : cudaLaunchKernelEx(&cfg, draft_sample_kernel<false>, a));
   return SEQ_OK;
 }

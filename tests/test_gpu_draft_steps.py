@@ -1,0 +1,57 @@
+"""seq_tree_draft_sample where its steps, parts and lists end: vocabularies around multiples of a step (4096 tokens) and of a
+part, one to eight CTAs per row, up to 64 draws, rows whose best tokens all come last, rows of equal keys and rows with
+fewer tokens in the running than draws (the list overflows or the threshold stays open).  Tokens against the oracle, rows
+with keys closer than fp32 resolves left out as in the other tests of this call."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as O
+from paper_2402_12374_b200 import binding as B
+from tests.test_gpu_draft_sample import _check_rows, _dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("rows,V,k", [(3, 4095, 16), (3, 4096, 17), (3, 4097, 64), (2, 8192, 9), (150, 12289, 3), (60, 32769, 8), (500, 8193, 5),
+                                      (1, 131072, 64), (2, 65541, 33)])
+def test_vocabularies_at_the_edges_of_steps_and_parts(rows, V, k):
+    rng = np.random.default_rng(V + k)
+    logits = (3 * rng.standard_normal((rows, V))).astype(np.float32)
+    u = rng.random((rows, V)).astype(np.float32)
+    ok, excl, st = _check_rows(logits, u, 0.6, k)
+    assert st == 0 and ok >= 0.7 * rows, (ok, excl)
+
+
+@pytest.mark.parametrize("rows,V", [(1, 40000), (450, 9000)])
+def test_rows_whose_best_tokens_come_last(rows, V):
+    """Every step's tokens beat all earlier ones: the list overflows and the row is ranked 256 tokens at a time."""
+    logits = np.tile(np.linspace(0.0, 400.0, V, dtype=np.float32), (rows, 1))
+    u = np.full((rows, V), 0.5, np.float32)
+    d = _dev()
+    got = B.seq_tree_draft_sample(torch.from_numpy(logits).to(d), 0.5, torch.from_numpy(u).to(d), 64).cpu().numpy()
+    assert (got == np.arange(V - 1, V - 65, -1)[None]).all()
+
+
+@pytest.mark.parametrize("rows,V,k", [(1, 3000, 64), (2, 70000, 7), (450, 5000, 64)])
+def test_equal_keys_go_in_token_order(rows, V, k):
+    d = _dev()
+    got = B.seq_tree_draft_sample(torch.zeros((rows, V), device=d), 1.0, torch.full((rows, V), 0.3, device=d), k).cpu().numpy()
+    assert (got == np.arange(k)[None]).all()
+
+
+@pytest.mark.parametrize("finite", [0, 1, 5, 40, 3000])
+def test_rows_with_few_tokens_in_the_running(finite):
+    rng = np.random.default_rng(finite)
+    rows, V, k = 4, 30001, 40
+    logits = np.full((rows, V), -np.inf, np.float32)
+    for r in range(rows):
+        logits[r, rng.choice(V, finite, replace=False)] = rng.standard_normal(finite)
+    u = rng.random((rows, V)).astype(np.float32)
+    d = _dev()
+    got = B.seq_tree_draft_sample(torch.from_numpy(logits).to(d), 1.0, torch.from_numpy(u).to(d), k).cpu().numpy()
+    for r in range(rows):
+        ref = O.draft_sample(logits[r], 1.0, u[r], k)
+        assert (got[r] >= 0).sum() == min(k, finite)
+        if finite == 0 or ref["min_rel_gap"] >= 1e-4:
+            assert got[r].tolist() == ref["tokens"].tolist()
