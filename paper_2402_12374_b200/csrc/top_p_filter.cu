@@ -1,18 +1,34 @@
 // seq_tree_top_p_filter: nucleus truncation of softmax(logits / T), row by row (the top-p hyperparameter of the
-// robustness study, Section 4.2).  One CTA per row.  A histogram of the probability MASS over 2048 equal steps of the
-// exponent argument finds the bin in which the cut falls; the tokens of that bin (a few dozen on the paper's shapes)
-// are ordered exactly in shared memory by (logit bits, token id); a flat row or a long run of equal logits, whose bin
-// holds more than 1024 tokens, takes a radix select on the logit bits (11 + 11 + 10) instead.  Masses are 2^-40 fixed
-// point in 64-bit integers: sums are exact and independent of the order of the atomic adds, so the kept set is
-// reproducible bit for bit.  A row is read four times (maximum, histogram, collect, write), once from HBM and then
-// from L2.
+// robustness study, Section 4.2).  A histogram of the probability MASS over equal steps of the exponent argument finds the
+// bin in which the cut falls; the tokens of that bin (a few dozen on the paper's shapes) are ordered exactly in shared
+// memory by (logit bits, token id).  Masses are 2^-40 fixed point in 64-bit integers: sums are exact and independent of
+// their order, so the kept set is reproducible bit for bit.
+//
+// One row is one cluster of up to 8 CTAs (vocabularies up to 131072) and is read once: each CTA's slice stays in shared
+// memory through all passes.  (In registers it would take loops unrolled over all of a thread's tokens, and the passes would
+// wait for their own instructions: 24 us for 64 rows of 32000.)  Exchanges over distributed shared memory: the row maximum,
+// the histograms with the masses' sums, the tokens of the cut's bin; every CTA then finds the cut by itself and writes its
+// slice.  The histogram covers the exponent arguments below 15 first - tokens below 2^-15 of the most probable one, most of
+// the vocabulary, only enter the sum - and the rest, in two more rounds, in the rare case that the cut is not among them.
+// One CTA takes the row through global memory instead (four passes, or seven with a radix select on the logit bits, 11 + 11
+// + 10) where the vocabulary is larger, and where more than 1024 tokens share the cut's bin (flat rows, long runs of equal
+// logits).
+//
+// What bounds it: the chain of exchanges for a few rows, HBM for many.  64 rows of 32000 tokens: 29.7 us with one CTA of
+// 1024 threads per row reading it four times and adding every token to the histogram, 13.2 so (about a dozen exchanges and
+// barriers of 0.5 to 1 us each around 4 us of passes); one row 28.6 -> 8.0; 127 rows of 128256 89 -> 81.
 #include <climits>
+#include <cstddef>
+
+#include <cooperative_groups.h>
 
 #include "common.cuh"
 
+namespace cg = cooperative_groups;
+
 namespace seqtree {
 
-constexpr int kTpThreads = 1024;
+constexpr int kTpThreads = 512;
 constexpr int kTpWarps = kTpThreads / 32;
 constexpr float kTpScale = 1099511627776.f;  // 2^40
 constexpr int kTpCand = 1024;  // tokens of the cut's bin that are ordered in shared memory (more: radix select)
@@ -27,19 +43,18 @@ struct TopPArgs {
 };
 
 struct TpShared {
-  unsigned long long hist[2048];
+  __align__(16) unsigned long long hist[2048];
   // first-level histogram as three 32-bit limbs per bin (native 32-bit shared-memory adds; a 64-bit add is a
   // compare-and-swap loop): mass = lo + hi * 2^21 + top * 2^53, carries moved up when an add wraps
   uint32_t lo[2048], hi[2048], top[2048];
   uint32_t count[1024];
-  unsigned long long warp_tot[kTpWarps];
+  __align__(16) unsigned long long warp_tot[kTpWarps];
   float warp_max[kTpWarps];
   // results of a level's search
   uint32_t sel_bin; unsigned long long sel_above; unsigned long long sel_mass; uint32_t sel_count;
   int32_t tie_limit;
   int32_t bad, kept, ncand;
   unsigned long long tau_comp;
-  unsigned long long sorted_c[kTpCand], sorted_w[kTpCand];  // the cut's bin in order: (key, ~index) and mass
 };
 
 // order-preserving map float -> uint32 (ascending)
@@ -94,7 +109,7 @@ __device__ __forceinline__ void tp_for_each(const float* row, int V, F f) {
 }
 
 // Exclusive prefix sum over the block's threads in thread order; every thread also gets the total.
-__device__ __forceinline__ unsigned long long tp_block_scan(unsigned long long v, TpShared& sh, unsigned long long& total) {
+__device__ __forceinline__ unsigned long long tp_block_scan(unsigned long long v, unsigned long long* warp_tot, unsigned long long& total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned long long inc = v;
 #pragma unroll
@@ -103,14 +118,15 @@ __device__ __forceinline__ unsigned long long tp_block_scan(unsigned long long v
     if (lane >= o) inc += up;
   }
   __syncthreads();  // warp_tot free for reuse
-  if (lane == 31) sh.warp_tot[warp] = inc;
+  if (lane == 31) warp_tot[warp] = inc;
   __syncthreads();
   unsigned long long before = 0, all = 0;
-#pragma unroll 1
-  for (int w = 0; w < kTpWarps; ++w) {
-    const unsigned long long t = sh.warp_tot[w];
-    if (w < warp) before += t;
-    all += t;
+#pragma unroll
+  for (int w = 0; w < kTpWarps; w += 2) {
+    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(&warp_tot[w]);
+    if (w < warp) before += t.x;
+    if (w + 1 < warp) before += t.y;
+    all += t.x + t.y;
   }
   total = all;
   return before + inc - v;
@@ -118,17 +134,21 @@ __device__ __forceinline__ unsigned long long tp_block_scan(unsigned long long v
 
 // Among `bins` bins of sh.hist taken from the highest index down, finds the one in which the running mass reaches
 // `target` (> 0, <= the bins' total); leaves its index, the mass above it, its own mass (and token count when
-// `with_count`) in sh.sel_*.  bins is 2048 or 1024: two or one bin per thread.
+// `with_count`) in sh.sel_*.  bins is 2048 or 1024: four or two bins per thread.
 __device__ __forceinline__ void tp_find_crossing(TpShared& sh, int bins, unsigned long long target, bool with_count) {
-  const int per = bins / kTpThreads;  // 2 or 1
+  const int per = bins / kTpThreads;
   const int hi = bins - 1 - (int)threadIdx.x * per;  // this thread's highest bin
-  unsigned long long m0 = sh.hist[hi], m1 = per == 2 ? sh.hist[hi - 1] : 0ull;
-  unsigned long long total;
-  const unsigned long long above = tp_block_scan(m0 + m1, sh, total);
-  if (above < target && target <= above + m0) {
-    sh.sel_bin = hi; sh.sel_above = above; sh.sel_mass = m0; sh.sel_count = with_count ? sh.count[hi] : 0u;
-  } else if (per == 2 && above + m0 < target && target <= above + m0 + m1) {
-    sh.sel_bin = hi - 1; sh.sel_above = above + m0; sh.sel_mass = m1; sh.sel_count = with_count ? sh.count[hi - 1] : 0u;
+  unsigned long long mine = 0, total;
+  for (int b = 0; b < per; ++b) mine += sh.hist[hi - b];
+  unsigned long long above = tp_block_scan(mine, sh.warp_tot, total);
+  if (above < target && target <= above + mine) {
+    for (int b = 0; b < per; ++b) {
+      const unsigned long long m = sh.hist[hi - b];
+      if (above < target && target <= above + m) {
+        sh.sel_bin = hi - b; sh.sel_above = above; sh.sel_mass = m; sh.sel_count = with_count ? sh.count[hi - b] : 0u;
+      }
+      above += m;
+    }
   }
   __syncthreads();
 }
@@ -141,11 +161,26 @@ __device__ __forceinline__ int tp_lbin(float x, float M, float c2) {
   return d < 40.f ? 2047 - (int)(d * 51.2f) : -1;
 }
 
-__global__ void __launch_bounds__(kTpThreads, 1) top_p_filter_kernel(const TopPArgs a) {
-  extern __shared__ __align__(16) uint8_t tp_smem[];
-  TpShared& sh = *reinterpret_cast<TpShared*>(tp_smem);
-  const float* row = a.logits + (int64_t)blockIdx.x * a.in_stride;
-  float* orow = a.out + (int64_t)blockIdx.x * a.out_stride;
+// Among n tokens of the cut's bin, (key and index, mass) each, finds the last kept one: the first, in descending order, at
+// which the running mass reaches `rest`.  No sort: a token's running mass is the sum over those before it.
+__device__ __forceinline__ void tp_cut(const ulonglong2* tokens, int n, unsigned long long rest, unsigned long long* tau_comp) {
+  for (int i = threadIdx.x; i < n; i += kTpThreads) {
+    const ulonglong2 mine = tokens[i];
+    unsigned long long before = 0;
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) {
+      const ulonglong2 t = tokens[j];
+      before += t.x > mine.x ? t.y : 0ull;
+    }
+    if (before < rest && rest <= before + mine.y) *tau_comp = mine.x;
+  }
+  __syncthreads();
+}
+
+// One row by one CTA through global memory.
+__device__ __noinline__ void top_p_row(TpShared& sh, const TopPArgs& a, int row_index) {
+  const float* row = a.logits + (int64_t)row_index * a.in_stride;
+  float* orow = a.out + (int64_t)row_index * a.out_stride;
   const int V = a.V, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
   // ---- the row maximum (NaN / +inf flagged and read as -inf), histogram cleared meanwhile
@@ -166,7 +201,7 @@ __global__ void __launch_bounds__(kTpThreads, 1) top_p_filter_kernel(const TopPA
     bad = __syncthreads_or(bad);
     if (threadIdx.x == 0) {
       dev_flag(a.dev_status, SEQ_DEV_DEGENERATE | (bad ? SEQ_DEV_NONFINITE : 0));
-      if (a.kept_out != nullptr) a.kept_out[blockIdx.x] = 0;
+      if (a.kept_out != nullptr) a.kept_out[row_index] = 0;
     }
     return;
   }
@@ -198,9 +233,9 @@ __global__ void __launch_bounds__(kTpThreads, 1) top_p_filter_kernel(const TopPA
   unsigned long long target;
   {
     // the whole mass, then the mass the nucleus has to reach (rounded up, at least one unit)
-    const unsigned long long mine = sh.hist[2 * threadIdx.x] + sh.hist[2 * threadIdx.x + 1];
-    unsigned long long S;
-    tp_block_scan(mine, sh, S);
+    unsigned long long mine = 0, S;
+    for (int i = threadIdx.x; i < 2048; i += kTpThreads) mine += sh.hist[i];
+    tp_block_scan(mine, sh.warp_tot, S);
     const double want = ceil(a.top_p * (double)S);
     target = want < 1.0 ? 1ull : (want >= (double)S ? S : (unsigned long long)want);
   }
@@ -210,16 +245,14 @@ __global__ void __launch_bounds__(kTpThreads, 1) top_p_filter_kernel(const TopPA
   __syncthreads();
 
   // ---- the tokens of that bin, as (key, ~index) so that a larger value means "earlier in the order"
-  unsigned long long* cand = sh.hist;               // [kTpCand]   (the histogram is no longer needed)
-  unsigned long long* cand_w = sh.hist + kTpCand;   // [kTpCand]
+  ulonglong2* cand = reinterpret_cast<ulonglong2*>(sh.hist);  // [kTpCand]   (the histogram is no longer needed)
   tp_for_each(row, V, [&](int i, float x) {
     int b2 = 0;
     x = tp_clean(x, b2);
     if (tp_lbin(x, M, a.c2) == B0) {
       const int pos = atomicAdd(&sh.ncand, 1);
       if (pos < kTpCand) {
-        cand[pos] = ((unsigned long long)tp_key(x) << 32) | (uint32_t)~(uint32_t)i;
-        cand_w[pos] = tp_mass(x, M, a.c2);
+        cand[pos] = make_ulonglong2(((unsigned long long)tp_key(x) << 32) | (uint32_t)~(uint32_t)i, tp_mass(x, M, a.c2));
       }
     }
   });
@@ -228,23 +261,7 @@ __global__ void __launch_bounds__(kTpThreads, 1) top_p_filter_kernel(const TopPA
   uint32_t tau = 0;          // fallback only: key of the least probable kept token
   bool exact = ncand <= kTpCand;
   if (exact) {
-    // rank every candidate among the others (all distinct), lay them out in order, scan the masses
-    unsigned long long my_w = 0, my_c = 0;
-    if ((int)threadIdx.x < ncand) {
-      my_c = cand[threadIdx.x];
-      my_w = cand_w[threadIdx.x];
-      int rank = 0;
-#pragma unroll 4
-      for (int j = 0; j < ncand; ++j) rank += cand[j] > my_c;
-      sh.sorted_c[rank] = my_c;
-      sh.sorted_w[rank] = my_w;
-    }
-    __syncthreads();
-    const unsigned long long w = (int)threadIdx.x < ncand ? sh.sorted_w[threadIdx.x] : 0ull;
-    unsigned long long total;
-    const unsigned long long before = tp_block_scan(w, sh, total);
-    if ((int)threadIdx.x < ncand && before < rest0 && rest0 <= before + w) sh.tau_comp = sh.sorted_c[threadIdx.x];
-    __syncthreads();
+    tp_cut(cand, ncand, rest0, &sh.tau_comp);
   } else {
     // ---- many tokens in one bin (a flat row, runs of equal logits): radix select on the key bits inside the bin
     __syncthreads();
@@ -305,7 +322,7 @@ __global__ void __launch_bounds__(kTpThreads, 1) top_p_filter_kernel(const TopPA
         cnt += tp_key(tp_clean(row[i], b2)) == tau;
       }
       unsigned long long total;
-      const unsigned long long before = tp_block_scan(cnt, sh, total);
+      const unsigned long long before = tp_block_scan(cnt, sh.warp_tot, total);
       if (before < need && need <= before + cnt) {
         unsigned long long seen = before;
         for (int i = lo; i < hi; ++i) {
@@ -334,9 +351,284 @@ __global__ void __launch_bounds__(kTpThreads, 1) top_p_filter_kernel(const TopPA
   if (lane == 0) atomicAdd(&sh.kept, kept);
   __syncthreads();
   if (threadIdx.x == 0) {
-    if (a.kept_out != nullptr) a.kept_out[blockIdx.x] = sh.kept;
+    if (a.kept_out != nullptr) a.kept_out[row_index] = sh.kept;
     if (sh.bad) dev_flag(a.dev_status, SEQ_DEV_NONFINITE);
   }
+}
+
+__global__ void __launch_bounds__(kTpThreads) top_p_row_kernel(const TopPArgs a) {
+  extern __shared__ __align__(16) uint8_t tp_smem[];
+  top_p_row(*reinterpret_cast<TpShared*>(tp_smem), a, blockIdx.x);
+}
+
+// One row by one cluster, the CTA's slice in shared memory.
+constexpr int kTpBins = 768;           // bins of one round of the histogram, 24 groups of 32
+constexpr int kTpRounds = 3;           // 2048 bins in rounds, most probable first (the last one is shorter)
+constexpr int kTpMaxCluster = 8, kTpMaxSlice = 16384;
+constexpr int kTpFastCand = 512;       // tokens of the cut's bin that are ordered here (more: the row goes to one CTA)
+constexpr int kTpQueue = 64;           // per warp: tokens of the round's bins waiting to be added by a full warp
+struct TpFast {
+  // Two limbs of 20 and 21 bits per bin, added without a return value; from 4096 tokens in one bin on they could wrap, and
+  // then the bins' total is not the exact sum of the round's masses any more.
+  uint32_t limb[2][kTpBins];
+  unsigned long long coarse[32];       // masses of the groups of bins; [24] all tokens' mass, [25] the round's tokens' (both exact)
+  unsigned long long stage[kTpMaxCluster][32];  // what was read from the cluster's CTAs
+  unsigned long long part[2][kTpWarps];
+  float queue[kTpWarps][kTpQueue];
+  __align__(16) ulonglong2 cand[kTpFastCand];  // this CTA's tokens of the cut's bin (read by the other CTAs)
+  __align__(16) ulonglong2 all[kTpFastCand];   // the cluster's
+  unsigned long long tau_comp;
+  int32_t max;                         // the row's maximum as an ordered integer (every CTA of the cluster adds its warps')
+  int32_t ncand;
+  __align__(16) float x[4];            // the slice (as long as it is)
+};
+
+// float <-> int of the same order
+__device__ __forceinline__ int tp_ordered(float x) { const int b = __float_as_int(x); return b ^ ((b >> 31) & 0x7fffffff); }
+__device__ __forceinline__ float tp_unordered(int b) { return __int_as_float(b ^ ((b >> 31) & 0x7fffffff)); }
+
+// Warp-wide: inclusive prefix sum over the lanes.
+__device__ __forceinline__ unsigned long long tp_warp_scan(unsigned long long v) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long up = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += up;
+  }
+  return v;
+}
+__device__ __forceinline__ unsigned long long tp_warp_sum(unsigned long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+__global__ void __launch_bounds__(kTpThreads, 2) top_p_cluster_kernel(const TopPArgs a, const int slice) {
+  extern __shared__ __align__(16) uint8_t tp_smem[];
+  TpFast& me = *reinterpret_cast<TpFast*>(tp_smem);
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = blockIdx.x, ranks = gridDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int lo = rank * slice, cnt = max(min(slice, a.V - lo), 0), cnt4 = (cnt + 3) & ~3;
+  const float* row = a.logits + (int64_t)blockIdx.y * a.in_stride + lo;
+  float* orow = a.out + (int64_t)blockIdx.y * a.out_stride + lo;
+
+  if (tid == 0) { me.ncand = 0; me.tau_comp = 0ull; me.max = tp_ordered(-INFINITY); }
+  __syncthreads();
+  cluster.barrier_arrive();  // waited for before the first remote access
+  for (int i = tid; i < 2 * kTpBins; i += kTpThreads) me.limb[0][i] = 0u;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (a.kept_out != nullptr && rank == 0 && tid == 0) a.kept_out[blockIdx.y] = 0;  // (the cluster's barriers order it before the counts)
+
+  // ---- the slice (NaN / +inf flagged and read as -inf, padded to groups of four with -inf) and the row maximum
+  int bad = 0;
+  float m = -INFINITY;
+  auto take = [&](int i, float4 v) {
+    v.x = tp_clean(v.x, bad); v.y = tp_clean(v.y, bad); v.z = tp_clean(v.z, bad); v.w = tp_clean(v.w, bad);
+    m = fmaxf(fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)), m);
+    *reinterpret_cast<float4*>(&me.x[i]) = v;
+  };
+  constexpr int kDeep = 8, kPass = 4 * kTpThreads;  // eight loads in flight per thread
+  const int full = cnt & ~3;
+  for (int i0 = 4 * tid; i0 < full; i0 += kDeep * kPass) {
+    float4 v[kDeep];
+#pragma unroll
+    for (int k = 0; k < kDeep; ++k)
+      if (i0 + k * kPass < full) v[k] = *reinterpret_cast<const float4*>(row + i0 + k * kPass);
+#pragma unroll
+    for (int k = 0; k < kDeep; ++k)
+      if (i0 + k * kPass < full) take(i0 + k * kPass, v[k]);
+  }
+  if (full < cnt && tid == 0)  // the row's last tokens
+    take(full, make_float4(row[full], full + 1 < cnt ? row[full + 1] : -INFINITY, full + 2 < cnt ? row[full + 2] : -INFINITY, -INFINITY));
+  m = warp_max(m);
+  if (bad) dev_flag(a.dev_status, SEQ_DEV_NONFINITE);
+  cluster.barrier_wait();
+  if (lane < ranks) atomicMax(&cluster.map_shared_rank(&me, lane)->max, tp_ordered(m));
+  cluster.sync();
+  const float M = tp_unordered(me.max);
+  if (M == -INFINITY) {  // no token with any mass: nothing to keep
+    for (int i = tid; i < cnt; i += kTpThreads) orow[i] = -INFINITY;
+    if (rank == 0 && tid == 0) dev_flag(a.dev_status, SEQ_DEV_DEGENERATE);
+    return;
+  }
+
+  // ---- masses: the sum of all of them (first round), the histogram of the round's bins
+  // With d = (M - x) * c2 the exponent argument, a token's bin counted from the most probable is (int)(d * 51.2).
+  unsigned long long target = 0, above_round = 0, rest0 = 0;
+  int B0 = -1;            // the bin in which the cut falls, and the mass still to find inside it
+  bool wrapped = false;
+  float* queue = me.queue[warp];
+  for (int round = 0, bin0 = 0; round < kTpRounds; ++round, bin0 += kTpBins) {
+    const float first = (float)bin0, last = fminf(first + (float)kTpBins, 2048.f);
+    unsigned long long sum = 0;
+    uint32_t small = 0;  // tokens behind the first round's bins: below 2^25 each, 32 of them at most
+    int waiting = 0;
+    auto add = [&](float x) {  // a token of the round's bins
+      const float d = (M - x) * a.c2;
+      const unsigned long long w = __float2ull_rn(tp_ex2(-d) * kTpScale);
+      const int b = (int)(d * 51.2f) - bin0;
+      sum += w;
+      atomicAdd(&me.limb[0][b], (uint32_t)w & 0xfffffu);
+      const uint32_t high = (uint32_t)(w >> 20);
+      if (high) atomicAdd(&me.limb[1][b], high);
+    };
+    // Few tokens of a warp are in the round's bins, but often one is: they queue up, and a full warp of them is added at once.
+    auto see = [&](float x) {
+      const float d = (M - x) * a.c2, p = d * 51.2f;
+      const bool in = p >= first && p < last && d < 40.f;
+      if (round == 0 && !in && d < 40.f) small += __float2uint_rn(tp_ex2(-d) * kTpScale);
+      const uint32_t who = __ballot_sync(0xffffffffu, in);
+      if (in) queue[waiting + __popc(who & ((1u << lane) - 1u))] = x;
+      waiting += __popc(who);
+      if (waiting >= 32) {
+        __syncwarp();
+        waiting -= 32;
+        add(queue[waiting + lane]);
+        __syncwarp();
+      }
+    };
+#pragma unroll 1
+    for (int i0 = 0; i0 < cnt4; i0 += 4 * kTpThreads) {  // (whole warps take part: the queue is theirs)
+      const int i = i0 + 4 * tid;
+      const float4 v = i < cnt4 ? *reinterpret_cast<const float4*>(&me.x[i]) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      see(v.x); see(v.y); see(v.z); see(v.w);
+    }
+    __syncwarp();
+    if (lane < waiting) add(queue[lane]);
+    const unsigned long long sum_all = tp_warp_sum(sum + small), sum_round = tp_warp_sum(sum);
+    if (lane == 0) { me.part[0][warp] = sum_all; me.part[1][warp] = sum_round; }
+    __syncthreads();
+    for (int grp = warp; grp < 26; grp += kTpWarps) {
+      unsigned long long v;
+      if (grp < 24) v = me.limb[0][32 * grp + lane] + ((unsigned long long)me.limb[1][32 * grp + lane] << 20);
+      else v = lane < kTpWarps ? me.part[grp - 24][lane] : 0ull;
+      v = tp_warp_sum(v);
+      if (lane == 0) me.coarse[grp] = v;
+    }
+    cluster.sync();
+    // the cluster's groups: one remote load per thread, then every warp finds the cut's group for itself
+    if (warp < ranks && lane < 26) me.stage[warp][lane] = cluster.map_shared_rank(&me, warp)->coarse[lane];
+    __syncthreads();
+    unsigned long long v = 0;
+    if (lane < 26)
+      for (int r = 0; r < ranks; ++r) v += me.stage[r][lane];
+    const unsigned long long all_mass = __shfl_sync(0xffffffffu, v, 24), exact = __shfl_sync(0xffffffffu, v, 25);
+    if (round == 0) {  // the mass the nucleus has to reach (rounded up, at least one unit)
+      const double want = ceil(a.top_p * (double)all_mass);
+      target = want < 1.0 ? 1ull : (want >= (double)all_mass ? all_mass : (unsigned long long)want);
+    }
+    if (lane >= 24) v = 0;
+    unsigned long long incl = tp_warp_scan(v);
+    wrapped = __shfl_sync(0xffffffffu, incl, 31) != exact;
+    if (wrapped) break;  // (every warp of every CTA of the cluster sees the same)
+    uint32_t hit = __ballot_sync(0xffffffffu, above_round + incl - v < target && target <= above_round + incl);
+    __syncthreads();     // the staged groups have been read
+    if (hit) {
+      const int grp = __ffs(hit) - 1;
+      const unsigned long long above = above_round + __shfl_sync(0xffffffffu, incl - v, grp);
+      if (warp < ranks) {
+        const TpFast* other = cluster.map_shared_rank(&me, warp);
+        me.stage[warp][lane] = other->limb[0][32 * grp + lane] + ((unsigned long long)other->limb[1][32 * grp + lane] << 20);
+      }
+      __syncthreads();
+      v = 0;
+      for (int r = 0; r < ranks; ++r) v += me.stage[r][lane];
+      incl = tp_warp_scan(v);
+      hit = __ballot_sync(0xffffffffu, above + incl - v < target && target <= above + incl);
+      const int b = __ffs(hit) - 1;
+      B0 = bin0 + 32 * grp + b;
+      rest0 = target - (above + __shfl_sync(0xffffffffu, incl - v, b));
+      break;
+    }
+    above_round += __shfl_sync(0xffffffffu, incl, 31);
+    cluster.sync();  // everyone has read the groups before the bins are cleared
+    for (int i = tid; i < 2 * kTpBins; i += kTpThreads) me.limb[0][i] = 0u;
+    __syncthreads();
+  }
+  const bool whole_row = wrapped || B0 < 0;
+  const float cut_lo = whole_row ? 4096.f : (float)B0, cut_hi = cut_lo + 1.f;  // (whole row: no token is collected)
+
+  // ---- the tokens of that bin, as (key, ~index) so that a larger value means "earlier in the order".  Every other token
+  // is decided by its bin: the logit itself in a more probable one, -inf in a less probable one.  It is written at once,
+  // unless the call works in place: the row may still be needed as it was.
+  const bool early = row != orow && !whole_row;
+  int kept = 0;
+  auto decide = [&](float x, int i) -> float {
+    const float d = (M - x) * a.c2, p = d * 51.2f;
+    if (p >= cut_lo && p < cut_hi && d < 40.f) {
+      const int pos = atomicAdd(&me.ncand, 1);
+      if (pos < kTpFastCand)
+        me.cand[pos] = make_ulonglong2(((unsigned long long)tp_key(x) << 32) | (uint32_t)~(uint32_t)(lo + i), __float2ull_rn(tp_ex2(-d) * kTpScale));
+    }
+    const bool keep = p < cut_lo;
+    kept += keep;
+    return keep ? x : -INFINITY;
+  };
+  auto store = [&](int i, float4 v) {
+    if (i + 3 < cnt) {
+      *reinterpret_cast<float4*>(orow + i) = v;
+    } else {
+      orow[i] = v.x;
+      if (i + 1 < cnt) orow[i + 1] = v.y;
+      if (i + 2 < cnt) orow[i + 2] = v.z;
+    }
+  };
+#pragma unroll 1
+  for (int i = 4 * tid; i < cnt4; i += 4 * kTpThreads) {
+    float4 v = *reinterpret_cast<const float4*>(&me.x[i]);
+    v.x = decide(v.x, i); v.y = decide(v.y, i + 1); v.z = decide(v.z, i + 2); v.w = decide(v.w, i + 3);
+    if (early) store(i, v);
+  }
+  cluster.sync();
+  int n;  // tokens of the whole cluster
+  {
+    const int c = lane < ranks ? cluster.map_shared_rank(&me, lane)->ncand : 0;
+    int incl = c;
+#pragma unroll
+    for (int o = 1; o < kTpMaxCluster; o <<= 1) {
+      const int up = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += up;
+    }
+    n = __shfl_sync(0xffffffffu, incl, kTpMaxCluster - 1);
+    const int mine = __shfl_sync(0xffffffffu, c, warp % kTpMaxCluster);
+    const int before = __shfl_sync(0xffffffffu, incl, warp % kTpMaxCluster) - mine;
+    if (warp < ranks && n <= kTpFastCand) {  // warp r copies CTA r's list
+      const TpFast* other = cluster.map_shared_rank(&me, warp);
+      for (int i = lane; i < mine; i += 32) me.all[before + i] = other->cand[i];
+    }
+  }
+  cluster.barrier_arrive();  // waited for at the end: nobody leaves while its list is being read
+  __syncthreads();
+  if (n > kTpFastCand || whole_row) {  // (the same for every CTA) too many to order here: the first CTA takes the row
+    cluster.barrier_wait();
+    if (rank == 0) top_p_row(*reinterpret_cast<TpShared*>(tp_smem), a, blockIdx.y);
+    return;
+  }
+  tp_cut(me.all, n, rest0, &me.tau_comp);
+  const unsigned long long tau_comp = me.tau_comp;
+
+  // ---- the tokens of the cut's bin: kept if not behind the last kept one in the order (key descending, index ascending)
+  if (!early) {
+#pragma unroll 1
+    for (int i = 4 * tid; i < cnt4; i += 4 * kTpThreads) {
+      float4 v = *reinterpret_cast<const float4*>(&me.x[i]);
+      auto inside = [&](float x) { return (M - x) * a.c2 * 51.2f < cut_lo ? x : -INFINITY; };
+      store(i, make_float4(inside(v.x), inside(v.y), inside(v.z), inside(v.w)));
+    }
+    __syncthreads();
+  }
+  for (int j = tid; j < me.ncand; j += kTpThreads)
+    if (me.cand[j].x >= tau_comp) {
+      const int i = (int)~(uint32_t)me.cand[j].x - lo;
+      orow[i] = me.x[i];
+      ++kept;
+    }
+  if (a.kept_out != nullptr) {
+    kept = __reduce_add_sync(0xffffffffu, kept);
+    if (lane == 0) atomicAdd(a.kept_out + blockIdx.y, kept);
+  }
+  cluster.barrier_wait();
 }
 
 // top_p >= 1: every token stays (rows copied when the call is not in place)
@@ -346,6 +638,53 @@ __global__ void top_p_copy_kernel(const TopPArgs a) {
   if (row != orow)
     for (int i = threadIdx.x; i < a.V; i += blockDim.x) orow[i] = row[i];
   if (threadIdx.x == 0 && a.kept_out != nullptr) a.kept_out[blockIdx.x] = a.V;
+}
+
+// CTAs per row: as many as let the rows' clusters run side by side (two CTAs per SM), of at least 4096 tokens each and 8 at
+// most; at least what keeps a slice within 16384 tokens.  A row of more than 8 x 16384 tokens goes to one CTA.
+static int launch_top_p(int rows, const TopPArgs& a, cudaStream_t stream) {
+  const int least = (a.V + kTpMaxSlice - 1) / kTpMaxSlice, most = (a.V + 4095) / 4096;
+  const bool cluster = least <= kTpMaxCluster;
+  int64_t ranks = 2 * (int64_t)device_sm_count() / rows;
+  ranks = ranks > most ? most : ranks;
+  ranks = ranks > kTpMaxCluster ? kTpMaxCluster : ranks < least ? least : ranks;
+  const int slice = (int)(((a.V + ranks - 1) / ranks + 3) & ~(int64_t)3);
+  // (the fallback's scratch takes the slice's place too)
+  const size_t fast = offsetof(TpFast, x) + (size_t)slice * 4, smem = fast > sizeof(TpShared) ? fast : sizeof(TpShared);
+  static int attr_done[64];
+  const int rc = once_per_device(attr_done, [&]() -> int {  // above the 48 KB a kernel gets without asking
+    SEQ_CUDA_OK(cudaFuncSetAttribute(top_p_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(offsetof(TpFast, x) + kTpMaxSlice * 4)));
+    SEQ_CUDA_OK(cudaFuncSetAttribute(top_p_row_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TpShared)));
+    return SEQ_OK;
+  });
+  if (rc != SEQ_OK) return rc;
+  if (!cluster) {
+    top_p_row_kernel<<<rows, kTpThreads, sizeof(TpShared), stream>>>(a);
+    SEQ_CUDA_OK(cudaGetLastError());
+    return SEQ_OK;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(kTpThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)ranks;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // set-up under the previous kernel's tail
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  TopPArgs part = a;
+  for (int first = 0; first < rows; first += 65535) {  // (a grid's y extent)
+    cfg.gridDim = dim3((unsigned)ranks, rows - first < 65535 ? rows - first : 65535);
+    part.logits = a.logits + (int64_t)first * a.in_stride;
+    part.out = a.out + (int64_t)first * a.out_stride;
+    part.kept_out = a.kept_out != nullptr ? a.kept_out + first : nullptr;
+    SEQ_CUDA_OK(cudaLaunchKernelEx(&cfg, top_p_cluster_kernel, part, slice));
+  }
+  return SEQ_OK;
 }
 
 }  // namespace seqtree
@@ -370,11 +709,8 @@ extern "C" int seq_tree_top_p_filter(const seq_tree_top_p_params* p, void* strea
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (p->top_p >= 1.f)
     top_p_copy_kernel<<<p->n_rows, 256, 0, s>>>(a);
-  else {
-    // above the 48 KB a kernel gets without asking; set on every call (cheap, and correct on every device)
-    SEQ_CUDA_OK(cudaFuncSetAttribute(top_p_filter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TpShared)));
-    top_p_filter_kernel<<<p->n_rows, kTpThreads, sizeof(TpShared), s>>>(a);
-  }
+  else
+    return launch_top_p(p->n_rows, a, s);
   SEQ_CUDA_OK(cudaGetLastError());
   return SEQ_OK;
 }
