@@ -203,11 +203,12 @@ static int verify_launch(const seq_tree_verify_params* p, int batch, int64_t tre
     __atomic_store_n(&wide_ok[dev], wide, __ATOMIC_RELEASE);
   }
   if (batch > 0) {
-    // A batch that fits the GPU as clusters of 16 side by side runs the walk with its rows in registers, one cluster
-    // per request (one request then costs what it costs alone); a larger one the shared-memory walk on clusters of 8,
-    // eighteen requests at a time.
-    if (wide == 1 && batch * 16 <= device_sm_count() && verify_walk_supported(p->vocab, p->flags, p->temperature))
-      return launch_verify_walk(a, false, s, batch);
+    // One cluster per request: the walk with its rows in registers where it is the better one (see there), else the
+    // shared-memory walk on clusters of 8.
+    if (wide == 1 && verify_walk_supported(p->vocab, p->flags, p->temperature)) {
+      const int rc = launch_verify_walk_batch(a, batch, s);
+      if (rc != SEQ_ERR_UNSUPPORTED) return rc;
+    }
     if (bf16) return SEQ_ERR_UNSUPPORTED;
     return verify_launch_with<8, vcl8::VShared, 0>(vcl8::tree_verify_kernel<true>, a, p->vocab, batch, false, s);
   }
@@ -215,7 +216,7 @@ static int verify_launch(const seq_tree_verify_params* p, int batch, int64_t tre
     return verify_launch_with<8, vcl8::VShared, 1>(vcl8::tree_verify_kernel<false>, a, p->vocab, p->n_tree < 18 ? p->n_tree : 18, false, s);
   // One request.  Vocabularies below 8192 tokens gain nothing from more CTAs.
   // the walk with its rows in registers, where a cluster of 16 can be placed and the mode is one it serves
-  if (wide == 1 && verify_walk_supported(p->vocab, p->flags, p->temperature)) return launch_verify_walk(a, false, s);
+  if (wide == 1 && verify_walk_supported(p->vocab, p->flags, p->temperature)) return launch_verify_walk(a, s);
   if (bf16) return SEQ_ERR_UNSUPPORTED;
   if (wide == 1 && p->vocab >= 8192)
     return verify_launch_with<16, vcl16::VShared, 2>(vcl16::tree_verify_kernel<false>, a, p->vocab, 1, false, s);

@@ -26,9 +26,10 @@ size_t verify_nodes_workspace_bytes(int n_tree);
 bool verify_nodes_supported(int n_tree, int vocab, int flags);
 int launch_verify_nodes(const VerifyArgs& a, void* workspace, size_t workspace_bytes, int max_clusters, cudaStream_t stream);
 
-// The walk with rows in registers (tree_verify_walk.cu): one cluster of 16 CTAs, no workspace.
+// The walk with rows in registers (tree_verify_walk.cu): one cluster of 16 CTAs (8 for large batches), no workspace.
 bool verify_walk_supported(int vocab, int flags, float temperature);
-// `requests` > 1: a batched launch, one cluster per request (the strides of VerifyArgs lead from one request to the next).
-int launch_verify_walk(const VerifyArgs& a, bool check_only, cudaStream_t stream, int requests = 1);
+int launch_verify_walk(const VerifyArgs& a, cudaStream_t stream);
+// A batched launch, one cluster per request (the strides of VerifyArgs lead from one request to the next).
+int launch_verify_walk_batch(const VerifyArgs& a, int requests, cudaStream_t stream);
 
 }  // namespace seqtree

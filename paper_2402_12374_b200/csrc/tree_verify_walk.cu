@@ -37,11 +37,11 @@ namespace cg = cooperative_groups;
 namespace seqtree {
 namespace vwk {
 
-constexpr int kCl = 16;               // CTAs in the cluster (not a portable size: asked for, and checked, at launch)
+constexpr int kCl = 16;               // CTAs in the cluster of one request (not a portable size: asked for, and checked, at launch)
+constexpr int kClBatch = 8;           // ... of each request of a batch too large for clusters of 16 side by side
 constexpr int kTh = 256;              // threads per CTA
 constexpr int kWarps = kTh / 32;
-constexpr int kParts = kCl * kWarps;  // (rank, warp) segments, in vocabulary order
-constexpr int kPPL = kParts / 32;     // table entries per lane
+// (rank, warp) segments, in vocabulary order: CL * kWarps of them; table entries per lane: CL / 4
 
 struct Shared {
   int32_t parent[SEQ_MAX_TREE];
@@ -56,7 +56,7 @@ struct Shared {
   int32_t kid_tok[2][SEQ_MAX_TREE];   // by rank: the children's tokens
   uint8_t dup[2][SEQ_MAX_TREE];       // by rank: a child that carries the token of an earlier sibling
   int32_t chunk_cnt[32];              // children among nodes [32 j, 32 j + 32)
-  float4 xbuf[2][kParts];             // cluster exchange: one entry per (rank, warp), double-buffered
+  float4 xbuf[2][kCl * kWarps];             // cluster exchange: one entry per (rank, warp), double-buffered
   int32_t node_flags;
   int32_t pick[2][4];                 // greedy walk, by hop parity: the matching child, the first child with a bad token, the first child
 };
@@ -194,28 +194,27 @@ __device__ __forceinline__ float exponentials(float* x, float m, float c2) {
 
 // Every warp of every CTA publishes one float4 to every CTA of the cluster.  On return lane l of every warp holds
 // entries l, l + 32, ... (rank-major, i.e. in vocabulary order).
-struct Exch { float4 e[kPPL]; };
+template <int CL>
+struct Exch { float4 e[CL * kWarps / 32]; };
 // ... in two halves, so that work that does not depend on the exchange can run while the barrier gathers
+template <int CL>
 __device__ __forceinline__ void exchange_push(cg::cluster_group& cluster, Ctx& c, float4 mine) {
-  if (c.lane < kCl) *cluster.map_shared_rank(&c.sh->xbuf[c.xpar][c.rank * kWarps + c.warp], c.lane) = mine;
+  if (c.lane < CL) *cluster.map_shared_rank(&c.sh->xbuf[c.xpar][c.rank * kWarps + c.warp], c.lane) = mine;
   __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
 }
-__device__ __forceinline__ void exchange_pull(Ctx& c, Exch& x) {
+template <int CL>
+__device__ __forceinline__ void exchange_pull(Ctx& c, Exch<CL>& x) {
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 #pragma unroll
-  for (int m = 0; m < kPPL; ++m) x.e[m] = c.sh->xbuf[c.xpar][c.lane + 32 * m];
+  for (int m = 0; m < CL * kWarps / 32; ++m) x.e[m] = c.sh->xbuf[c.xpar][c.lane + 32 * m];
   c.xpar ^= 1;
 }
-__device__ __forceinline__ void cluster_exchange(cg::cluster_group& cluster, Ctx& c, float4 mine, Exch& x) {
-  exchange_push(cluster, c, mine);
-  exchange_pull(c, x);
-}
-
 // A batched launch runs one request per cluster: the same code on that request's arrays.
+template <int CL>
 __device__ __forceinline__ VerifyArgs request_args(const VerifyArgs& in) {
   VerifyArgs a = in;
-  const int64_t r = blockIdx.x / kCl;
+  const int64_t r = blockIdx.x / CL;
   if (r > 0) {
     a.parent += r * in.tree_stride; a.tokens += r * in.tree_stride;
     a.target = reinterpret_cast<const float*>(reinterpret_cast<const char*>(in.target) + r * in.logits_stride * ((in.flags & SEQ_VERIFY_LOGITS_BF16) ? 2 : 4));
@@ -228,9 +227,12 @@ __device__ __forceinline__ VerifyArgs request_args(const VerifyArgs& in) {
   return a;
 }
 
-template <int NCH, bool kBf16>
-__global__ void __launch_bounds__(kTh, 1) tree_verify_walk_kernel(const VerifyArgs a_in) {
-  const VerifyArgs a = request_args(a_in);
+// (The batch's instances up to 32768 tokens keep to 128 registers: two requests' CTAs share an SM, 64 requests of 32000
+// tokens take 42 us instead of 65.)
+template <int NCH, bool kBf16, int CL>
+__global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_verify_walk_kernel(const VerifyArgs a_in) {
+  const VerifyArgs a = request_args<CL>(a_in);
+  constexpr int kPPL = CL * kWarps / 32;  // table entries per lane
   constexpr int kEsz = kBf16 ? 2 : 4;  // bytes per logit
   const char* const tbase = reinterpret_cast<const char*>(a.target);
   const char* const dbase = reinterpret_cast<const char*>(a.draft);
@@ -322,11 +324,11 @@ __global__ void __launch_bounds__(kTh, 1) tree_verify_walk_kernel(const VerifyAr
     }
     if (bad) dev_flag(a.dev_status, SEQ_DEV_NONFINITE);
     WTRACE(leader, 13);
-    Exch x;
+    Exch<CL> x;
     {
       const float Mwp = warp_max(mp), Mwq = warp_max(mq);
       const float swp = warp_sum(sp * rel_exp(mp, Mwp, c2)), swq = warp_sum(sq * rel_exp(mq, Mwq, c2));
-      exchange_push(cluster, c, make_float4(Mwp, swp, Mwq, swq));
+      exchange_push<CL>(cluster, c, make_float4(Mwp, swp, Mwq, swq));
     }
     WTRACE(leader, 40);
     // ---- while the cluster's barrier gathers: the node's children, in order, by rank among them; the two logits at
@@ -387,7 +389,7 @@ __global__ void __launch_bounds__(kTh, 1) tree_verify_walk_kernel(const VerifyAr
         }
     }
     WTRACE(leader, 12);
-    exchange_pull(c, x);
+    exchange_pull<CL>(c, x);
     WTRACE(leader, 14);
     float Mp = -INFINITY, Mq = -INFINITY;
 #pragma unroll
@@ -494,12 +496,12 @@ __global__ void __launch_bounds__(kTh, 1) tree_verify_walk_kernel(const VerifyAr
       for (int e = 0; e < kE; e += 2) { z0 += resid(p[e], q[e], Cnf, Unf); z1 += resid(p[e + 1], q[e + 1], Cnf, Unf); }
       const float zr = warp_sum(z0 + z1), zd = warp_sum(zd_mine);
       WTRACE(leader, 17);
-      exchange_push(cluster, c, make_float4(zr, zd, 0.f, 0.f));
+      exchange_push<CL>(cluster, c, make_float4(zr, zd, 0.f, 0.f));
       if (more) {
         load_row<NCH, kBf16>(c, tbase + (int64_t)nxt * a.target_stride * kEsz, pn);
         if (nxt_has_kids) load_row<NCH, kBf16>(c, dbase + (int64_t)nxt * a.draft_stride * kEsz, qn);
       }
-      exchange_pull(c, x);
+      exchange_pull<CL>(c, x);
       WTRACE(leader, 18);
       float zsum = 0.f, zdsum = 0.f;
 #pragma unroll
@@ -654,7 +656,7 @@ __device__ __forceinline__ void warp_argmax(int& key, int& idx) {
 
 template <int NCH, bool kBf16>
 __global__ void __launch_bounds__(kTh, 1) tree_verify_greedy_kernel(const VerifyArgs a_in) {
-  const VerifyArgs a = request_args(a_in);
+  const VerifyArgs a = request_args<kCl>(a_in);
   constexpr int kEsz = kBf16 ? 2 : 4;
   constexpr int kE = 4 * NCH, kSpan = 32 * kE;
   const char* const tbase = reinterpret_cast<const char*>(a.target);
@@ -720,7 +722,7 @@ __global__ void __launch_bounds__(kTh, 1) tree_verify_greedy_kernel(const Verify
       }
     }
     warp_argmax(key, idx);
-    exchange_push(cluster, c, make_float4(__int_as_float(key), __int_as_float(idx), 0.f, 0.f));
+    exchange_push<kCl>(cluster, c, make_float4(__int_as_float(key), __int_as_float(idx), 0.f, 0.f));
     // ---- while the barrier gathers: the node's first child, and its row on the way
     __syncthreads();  // pick[] is reset
 #pragma unroll
@@ -731,11 +733,11 @@ __global__ void __launch_bounds__(kTh, 1) tree_verify_greedy_kernel(const Verify
     __syncthreads();
     const int first_kid = pick[2];
     if (first_kid != 0x7fffffff) load_row<NCH, kBf16>(c, tbase + (int64_t)first_kid * a.target_stride * kEsz, pn);
-    Exch t;
-    exchange_pull(c, t);
+    Exch<kCl> t;
+    exchange_pull<kCl>(c, t);
     key = INT_MIN; idx = 0x7fffffff;
 #pragma unroll
-    for (int m = 0; m < kPPL; ++m) {  // entries in vocabulary order: the first of equal keys stays
+    for (int m = 0; m < kCl * kWarps / 32; ++m) {  // entries in vocabulary order: the first of equal keys stays
       const int k = __float_as_int(t.e[m].x), i = __float_as_int(t.e[m].y);
       if (i != 0x7fffffff && (idx == 0x7fffffff || k > key)) { key = k; idx = i; }
     }
@@ -784,19 +786,27 @@ bool verify_walk_supported(int vocab, int flags, float temperature) {
   return vocab >= 1 && (size_t)vocab <= (size_t)vwk::kCl * vwk::kTh * 4 * 8;
 }
 
-int launch_verify_walk(const VerifyArgs& a_in, bool check_only, cudaStream_t stream, int requests) {
+typedef void (*WalkKernel)(const VerifyArgs);
+template <int CL>
+static WalkKernel walk_kernel(int nch, bool bf16) {
+  return bf16 ? (nch == 2 ? vwk::tree_verify_walk_kernel<2, true, CL> : nch == 4 ? vwk::tree_verify_walk_kernel<4, true, CL> : vwk::tree_verify_walk_kernel<8, true, CL>)
+              : (nch == 2 ? vwk::tree_verify_walk_kernel<2, false, CL> : nch == 4 ? vwk::tree_verify_walk_kernel<4, false, CL> : vwk::tree_verify_walk_kernel<8, false, CL>);
+}
+
+// cl: CTAs per request, 16 or (T > 0 and a vocabulary that 8 CTAs hold) 8.  With `clusters` given nothing is launched: the
+// number of clusters that the device runs side by side is written there.
+static int walk_launch(const VerifyArgs& a_in, int cl, int requests, int* clusters, cudaStream_t stream) {
   VerifyArgs a = a_in;
-  a.slice_cap = (((a.V + vwk::kCl - 1) / vwk::kCl) + 3) & ~3;
+  a.slice_cap = (((a.V + cl - 1) / cl) + 3) & ~3;
   const int nch = a.slice_cap <= vwk::kTh * 4 * 2 ? 2 : a.slice_cap <= vwk::kTh * 4 * 4 ? 4 : 8;
   const bool bf16 = (a.flags & SEQ_VERIFY_LOGITS_BF16) != 0;
   const bool greedy = a.temperature == 0.f;
-  void (*kernel)(const VerifyArgs) =
+  const WalkKernel kernel =
       greedy ? (bf16 ? (nch == 2 ? vwk::tree_verify_greedy_kernel<2, true> : nch == 4 ? vwk::tree_verify_greedy_kernel<4, true> : vwk::tree_verify_greedy_kernel<8, true>)
                      : (nch == 2 ? vwk::tree_verify_greedy_kernel<2, false> : nch == 4 ? vwk::tree_verify_greedy_kernel<4, false> : vwk::tree_verify_greedy_kernel<8, false>))
-      : bf16 ? (nch == 2 ? vwk::tree_verify_walk_kernel<2, true> : nch == 4 ? vwk::tree_verify_walk_kernel<4, true> : vwk::tree_verify_walk_kernel<8, true>)
-             : (nch == 2 ? vwk::tree_verify_walk_kernel<2, false> : nch == 4 ? vwk::tree_verify_walk_kernel<4, false> : vwk::tree_verify_walk_kernel<8, false>);
-  const int slot = (nch == 2 ? 0 : nch == 4 ? 1 : 2) + (bf16 ? 3 : 0) + (greedy ? 6 : 0);
-  static int attr_done[12][64];
+      : cl == 16 ? walk_kernel<vwk::kCl>(nch, bf16) : walk_kernel<vwk::kClBatch>(nch, bf16);
+  const int slot = (nch == 2 ? 0 : nch == 4 ? 1 : 2) + (bf16 ? 3 : 0) + (greedy ? 6 : cl == 16 ? 0 : 12);
+  static int attr_done[18][64];
   const int rc = once_per_device(attr_done[slot], [&]() -> int {
     SEQ_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(vwk::Shared)));
     SEQ_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
@@ -804,27 +814,57 @@ int launch_verify_walk(const VerifyArgs& a_in, bool check_only, cudaStream_t str
   });
   if (rc != SEQ_OK) return rc;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(vwk::kCl * (requests > 0 ? requests : 1));
+  cfg.gridDim = dim3(cl * requests);
   cfg.blockDim = dim3(vwk::kTh);
   cfg.dynamicSmemBytes = sizeof(vwk::Shared);
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = vwk::kCl;
+  attr[0].val.clusterDim.x = cl;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // start under the previous kernel's tail
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 2;
-  if (check_only) {  // can a cluster of this size be placed on this device at all?
-    int clusters = 0;
-    cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); return SEQ_ERR_UNSUPPORTED; }
-    return clusters >= 1 ? SEQ_OK : SEQ_ERR_UNSUPPORTED;
+  cfg.numAttrs = clusters != nullptr ? 1 : 2;
+  if (clusters != nullptr) {
+    if (cudaOccupancyMaxActiveClusters(clusters, kernel, &cfg) != cudaSuccess) { cudaGetLastError(); *clusters = 0; }
+    return SEQ_OK;
   }
   SEQ_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, a));
   return SEQ_OK;
+}
+
+int launch_verify_walk(const VerifyArgs& a, cudaStream_t stream) { return walk_launch(a, vwk::kCl, 1, nullptr, stream); }
+
+// CTAs per request for a batch, 0 where the shared-memory walk is the better one.  Measured at T > 0 against that walk: up
+// to 9 requests run as clusters of 16 on SMs of their own where the device places that many (32000 tokens: 18.2 us against
+// 26); more of them, as clusters of 8 with rows of up to 65536 tokens in registers, win at any size (10 / 16 / 32 / 64
+// requests of 32000 tokens: 22 / 21 / 22 / 42 us against 31 / 29 / 28 / 57; of 50257: 24 / 30 / 46 / 72 against 43 / 51 / 54
+// / 86).  Larger vocabularies need 16 CTAs and are served in turns: 10 / 32 requests of 128256 tokens 29 / 68 us against 41
+// / 71, 48 requests 99 against 92.  Greedy walks keep 16 CTAs (64 requests of 32000 tokens: 27 us against 33).
+static int walk_batch_cluster(const VerifyArgs& a, int requests) {
+  if (a.temperature == 0.f) return vwk::kCl;
+  if (a.V > vwk::kClBatch * vwk::kTh * 32) return requests * vwk::kCl <= 4 * device_sm_count() ? vwk::kCl : 0;
+  if (requests * vwk::kCl > device_sm_count()) return vwk::kClBatch;
+  static int side_by_side[6][64];  // per kernel shape and device: clusters of 16, + 1; 0 = not asked yet
+  const int slice = (((a.V + vwk::kCl - 1) / vwk::kCl) + 3) & ~3;
+  const int shape = (slice <= vwk::kTh * 8 ? 0 : slice <= vwk::kTh * 16 ? 1 : 2) + ((a.flags & SEQ_VERIFY_LOGITS_BF16) ? 3 : 0);
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return vwk::kCl;
+  if (dev >= 0 && dev < 64) n = __atomic_load_n(&side_by_side[shape][dev], __ATOMIC_ACQUIRE);
+  if (n == 0) {
+    if (walk_launch(a, vwk::kCl, 1, &n, nullptr) != SEQ_OK) n = 0;
+    ++n;
+    if (dev >= 0 && dev < 64) __atomic_store_n(&side_by_side[shape][dev], n, __ATOMIC_RELEASE);
+  }
+  return requests <= n - 1 ? vwk::kCl : vwk::kClBatch;
+}
+
+// SEQ_ERR_UNSUPPORTED: not a batch for this schedule.
+int launch_verify_walk_batch(const VerifyArgs& a, int requests, cudaStream_t stream) {
+  const int cl = walk_batch_cluster(a, requests);
+  return cl == 0 ? SEQ_ERR_UNSUPPORTED : walk_launch(a, cl, requests, nullptr, stream);
 }
 
 }  // namespace seqtree
