@@ -5,13 +5,7 @@
 
 namespace seqtree {
 
-// Defined in tree_attention_pair.cu: two query tiles per CTA.  cost < 0: not for this shape.
-struct PairPlan { int splits; bool stream; double cost; };
-PairPlan pair_plan(const seq_tree_attention_params& p);
-size_t pair_workspace_bytes(const seq_tree_attention_params& p, const PairPlan& plan);
-int launch_attention_pair(const seq_tree_attention_params& p, const PairPlan& plan, cudaStream_t stream);
-
-// Defined in tree_attention_umma.cu: one query tile per CTA.
+// Defined in tree_attention_umma.cu.
 bool umma_supported(const seq_tree_attention_params& p);
 int umma_default_splits(const seq_tree_attention_params& p);
 int launch_attention_umma(const seq_tree_attention_params& p, int splits, cudaStream_t stream);
@@ -89,10 +83,7 @@ extern "C" size_t seq_tree_attention_workspace_bytes(const seq_tree_attention_pa
   if (validate_attention_params(p) != SEQ_OK) return 0;
   const int which = choose_kernel(*p);
   if (which == 0) return 0;
-  if (which == 2) {  // only the stream schedules need one
-    const PairPlan pair = pair_plan(*p);
-    return pair.cost >= 0 ? pair_workspace_bytes(*p, pair) : umma_workspace_bytes(*p);
-  }
+  if (which == 2) return umma_workspace_bytes(*p);  // only its stream mode (more units than SMs) needs one
   const int splits = which == 3 ? f32_splits(*p) : simt_default_splits(*p);
   size_t bytes = splits > 1 ? split_workspace_bytes(splits, p->num_q_heads, p->n_tree) : 0;
   return (bytes + 255) & ~(size_t)255;
@@ -103,11 +94,7 @@ extern "C" int seq_tree_attention(const seq_tree_attention_params* p, void* stre
   if (rc != SEQ_OK) return rc;
   const int which = choose_kernel(*p);
   if (which == 0) return SEQ_ERR_UNSUPPORTED;
-  if (which == 2) {
-    const PairPlan pair = pair_plan(*p);
-    if (pair.cost >= 0) return launch_attention_pair(*p, pair, (cudaStream_t)stream);
-    return launch_attention_umma(*p, umma_default_splits(*p), (cudaStream_t)stream);
-  }
+  if (which == 2) return launch_attention_umma(*p, umma_default_splits(*p), (cudaStream_t)stream);
   const int splits = which == 3 ? f32_splits(*p) : simt_default_splits(*p);
   if (splits > 1) {
     if (p->workspace == nullptr || p->workspace_bytes < split_workspace_bytes(splits, p->num_q_heads, p->n_tree))
