@@ -177,6 +177,12 @@ __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sy
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
+// A value that every lane of the warp holds, so that the compiler knows it is the same: what is derived from it stays on the
+// uniform datapath, where the operands of tcgen05.mma have to be (a value it cannot prove uniform is moved there for every
+// single instruction).
+template <typename T>
+__device__ __forceinline__ T uniform(T x) { return __shfl_sync(0xffffffffu, x, 0); }
+
 // True in exactly one lane of a converged warp.  Code that must be issued once per warp (MMAs, commits)
 // goes under this predicate while everything around it stays warp-uniform, which keeps descriptors and
 // addresses on the uniform datapath.
@@ -193,20 +199,41 @@ __device__ __forceinline__ bool elect_one() {
 __device__ __forceinline__ void tc_commit(uint64_t* bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
-}
+// The two products of a block, each issued as one run of MMAs.  The operands' descriptors differ in their low words only
+// (start address in 16-byte units), which the run itself steps along the contraction: descriptors worked out beside the MMAs
+// are hoisted out of the block loop by the compiler and cost the issuing warp its few registers.
+constexpr uint32_t kDescHi = (1024u >> 4) | (1u << 14) | (2u << 29);  // 1024 B between groups of 8 rows, version 1, 128-byte swizzle
+// low word of a shared-memory descriptor; lbo: bytes between 64-element blocks along MN (MN-major operands)
+__device__ __forceinline__ uint32_t desc_lo(uint32_t smem_addr, uint32_t lbo) { return ((smem_addr >> 4) & 0x3FFFu) | (((lbo >> 4) & 0x3FFFu) << 16); }
 
-__device__ __forceinline__ void tc_mma_tmem_a(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+// S = Q K^T over head_dim = 128: eight steps of 16 elements, 32 bytes apart inside a 64-element sub-tile; kQHalf, kKHalf:
+// bytes from the first sub-tile to the second
+template <uint32_t kQHalf, uint32_t kKHalf>
+__device__ __forceinline__ void mma_qk(uint32_t d_tmem, uint32_t q_lo, uint32_t k_lo, uint32_t idesc) {
+#define SEQ_STEP(qs, ks) "add.u32 q, q, " qs ";\n\tadd.u32 k, k, " ks ";\n\tmov.b64 x, {q, %3};\n\tmov.b64 y, {k, %3};\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %4, t;\n\t"
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+      "{\n\t.reg .pred p, t;\n\t.reg .b64 x, y;\n\t.reg .b32 q, k;\n\t"
+      "setp.ne.b32 p, 0, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+      "mov.b32 q, %1;\n\tmov.b32 k, %2;\n\t"
+      "mov.b64 x, {%1, %3};\n\tmov.b64 y, {%2, %3};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %4, p;\n\t"
+      SEQ_STEP("2", "2") SEQ_STEP("2", "2") SEQ_STEP("2", "2") SEQ_STEP("%5", "%6") SEQ_STEP("2", "2") SEQ_STEP("2", "2") SEQ_STEP("2", "2")
+      "}"
+      ::"r"(d_tmem), "r"(q_lo), "r"(k_lo), "r"(kDescHi), "r"(idesc), "n"((kQHalf >> 4) - 6), "n"((kKHalf >> 4) - 6) : "memory");
+#undef SEQ_STEP
+}
+// O (+)= P V over 64 keys: A = 8 packed columns of P, B = 16 key rows of V (2048 bytes) per step
+__device__ __forceinline__ void mma_pv(uint32_t d_tmem, uint32_t p_tmem, uint32_t v_lo, uint32_t idesc, uint32_t accumulate) {
+#define SEQ_STEP "add.u32 a, a, 8;\n\tadd.u32 v, v, 128;\n\tmov.b64 y, {v, %3};\n\ttcgen05.mma.cta_group::1.kind::f16 [%0], [a], y, %4, t;\n\t"
+  asm volatile(
+      "{\n\t.reg .pred p, t;\n\t.reg .b64 y;\n\t.reg .b32 a, v;\n\t"
+      "setp.ne.b32 p, %5, 0;\n\tsetp.eq.b32 t, 0, 0;\n\t"
+      "mov.b32 a, %1;\n\tmov.b32 v, %2;\n\t"
+      "mov.b64 y, {%2, %3};\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], y, %4, p;\n\t"
+      SEQ_STEP SEQ_STEP SEQ_STEP "}"
+      ::"r"(d_tmem), "r"(p_tmem), "r"(v_lo), "r"(kDescHi), "r"(idesc), "r"(accumulate) : "memory");
+#undef SEQ_STEP
 }
 
 #define SEQ_R32(a, o) \
@@ -284,15 +311,6 @@ __device__ __forceinline__ float ex2(float x) {
   return y;
 }
 
-// Shared-memory matrix descriptor, 128-byte swizzle (layout type 2), descriptor version 1.
-// lbo/sbo in bytes.  K-major operands: sbo = 1024 (8 rows of 128 B), lbo unused.
-// MN-major operands: lbo = stride between 64-element blocks along MN, sbo = 1024 between groups of 8 along K.
-__device__ __forceinline__ uint64_t make_desc(uint32_t smem_addr, uint32_t lbo, uint32_t sbo) {
-  const uint32_t lo = ((smem_addr >> 4) & 0x3FFFu) | (((lbo >> 4) & 0x3FFFu) << 16);
-  const uint32_t hi = ((sbo >> 4) & 0x3FFFu) | (1u << 14) | (2u << 29);
-  return ((uint64_t)hi << 32) | lo;
-}
-
 template <bool kBf16>
 __device__ __forceinline__ uint32_t pack2(float a, float b) {
   if (kBf16) {
@@ -322,7 +340,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
   extern __shared__ uint8_t smem_raw[];
   UmmaSmem* sm = reinterpret_cast<UmmaSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   cg::cluster_group cluster = cg::this_cluster();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform((int)threadIdx.x >> 5), lane = threadIdx.x & 31;
 #ifdef SEQ_TRACE
   int utrace_i = 0;
 #endif
@@ -410,7 +428,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
   if (a.L_dev != nullptr) {
     const int v = a.L_dev[(!kStream && a.L_count > 1) ? ((int)blockIdx.y * a.L_count) / a.Hkv : 0];
     if (v < 0 || v > a.L_host) { if (threadIdx.x == 0) dev_flag(a.dev_status, SEQ_DEV_BAD_LENGTH); }
-    L = min(max(v, 0), a.L_host);
+    L = uniform(min(max(v, 0), a.L_host));
     if (kStream) {  // the flattened block space of this prefix length (every warp for itself)
       int sum = 0;
       for (int t = lane; t < a.tiles; t += 32) sum += kStreamTileCost + (L + min((t + 1) * a.nodes_per_tile, a.n) + kBlockN - 1) / kBlockN;
@@ -478,7 +496,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = sm->tmem_base;
+  const uint32_t tmem = uniform(sm->tmem_base);
   if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 0);
 
   if (warp < 4) {
@@ -540,22 +558,16 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
       if (n_c > 0) {
         const int base = c ? base_b : base_a;
         bool go = q_here;
-        // A step along the contraction only moves a descriptor's 14-bit start-address field (16-byte units).
-        const uint64_t qd0 = make_desc(smem_u32(sm->q), 16, 1024);
+        const uint32_t q_lo = desc_lo(smem_u32(sm->q), 16);
         const uint32_t tmem_o = tmem + 256u + 128u * c;
         // S of block u of the chain: buffer u & 1
         auto issue_qk = [&](int u) -> bool {
           const int b = (base + u) & 1, w = (base + u) >> 1;
           if (!mbar_wait(sm, &sm->k_full[c][b], w & 1, a.dev_status)) return false;
           tc_fence_after();
-          const uint64_t kd0 = make_desc(smem_u32(sm->k[c][b]), 16, 1024);
           const uint32_t d = tmem + 128u * c + 64u * b;
           if (elect_one()) {
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks) {  // 16 elements of head_dim per step: 32 bytes inside a 64-element sub-tile
-              tc_mma(d, qd0 + (uint64_t)(((ks >> 2) * kHalfBytes + (ks & 3) * 32) >> 4),
-                     kd0 + (uint64_t)(((ks >> 2) * kKvHalf + (ks & 3) * 32) >> 4), a.idesc_qk, ks > 0);
-            }
+            mma_qk<kHalfBytes, kKvHalf>(d, q_lo, desc_lo(smem_u32(sm->k[c][b]), 16), a.idesc_qk);
             tc_commit(&sm->k_empty[c][b]);
             tc_commit(&sm->s_full[c][b]);
           }
@@ -590,13 +602,10 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
             }
           }
           tc_fence_after();
-          const uint64_t vd0 = make_desc(smem_u32(sm->v[c][b]), kKvHalf, 1024);
           const uint32_t pa = tmem + 128u * c + 64u * b;
           const uint32_t first = u > 0 ? 1u : 0u;
           if (elect_one()) {
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)  // A = 8 packed columns of P, B = 16 key rows of V per step
-              tc_mma_tmem_a(tmem_o, pa + 8u * ks, vd0 + (uint64_t)(ks * (2048 >> 4)), a.idesc_pv, ks > 0 ? 1u : first);
+            mma_pv(tmem_o, pa, desc_lo(smem_u32(sm->v[c][b]), kKvHalf), a.idesc_pv, first);
             tc_commit(&sm->v_empty[c][b]);
             tc_commit(&sm->pv_done[c]);
           }
