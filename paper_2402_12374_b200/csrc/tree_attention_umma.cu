@@ -568,8 +568,8 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
           const uint32_t d = tmem + 128u * c + 64u * b;
           if (elect_one()) {
             mma_qk<kHalfBytes, kKvHalf>(d, q_lo, desc_lo(smem_u32(sm->k[c][b]), 16), a.idesc_qk);
+            tc_commit(&sm->s_full[c][b]);  // the row threads wait for this one
             tc_commit(&sm->k_empty[c][b]);
-            tc_commit(&sm->s_full[c][b]);
           }
           __syncwarp();
           if (lane == 0) UTRACE(c == 0 ? 1 : 3, 2);
@@ -580,11 +580,11 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
         if (go && n_c > 1) go = issue_qk(1);
         for (int u = 0; u < n_c && go; ++u) {
           const int b = (base + u) & 1, w = (base + u) >> 1;
+          if (!mbar_wait(sm, &sm->v_full[c][b], w & 1, a.dev_status)) break;
           if (!mbar_wait(sm, &sm->p_full[c][b], w & 1, a.dev_status)) break;
           // the first P.V of a segment overwrites O: the row threads must have read the previous segment's
           if (u == 0 && seg > 0 && !mbar_wait(sm, &sm->o_free, (seg - 1) & 1, a.dev_status)) break;
           if (lane == 0) UTRACE(c == 0 ? 1 : 3, 3);
-          if (!mbar_wait(sm, &sm->v_full[c][b], w & 1, a.dev_status)) break;
           if (a.zero_tail) {
             // The tensor maps of this mode cover the whole cache, so a block that reaches past the last tree row has
             // fetched rows that may hold anything; their probabilities are exactly 0, but 0 * NaN is not: the rows are
