@@ -305,6 +305,23 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// The address of a shared-memory word of CTA `rank` of the cluster, and stores to it.
+__device__ __forceinline__ uint32_t remote_smem(uint32_t addr, int rank) {
+  uint32_t d;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(addr), "r"(rank));
+  return d;
+}
+__device__ __forceinline__ void st_cluster4(uint32_t addr, const float* x) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]) : "memory");
+}
+__device__ __forceinline__ void st_cluster2(uint32_t addr, float x, float y) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(x), "f"(y) : "memory");
+}
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -372,8 +389,8 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
       x.i1 = min(x.i0 + a.nodes_per_tile, a.n);
       // keys this tile can see end at L + i1 (a node sees no later node); blocks of this CTA
       x.nblk_tile = (L + x.i1 + kBlockN - 1) / kBlockN;
-      x.blk_lo = (int)(((long)split * x.nblk_tile) / a.splits);
-      x.nblk = (int)(((long)(split + 1) * x.nblk_tile) / a.splits) - x.blk_lo;
+      x.blk_lo = (split * x.nblk_tile) / a.splits;
+      x.nblk = ((split + 1) * x.nblk_tile) / a.splits - x.blk_lo;
       x.next = 1;
     } else {
       x.g = (int)(pos / blocks_per_head);
@@ -676,7 +693,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
   // segment by the first thread of each node (0 <= parent[j] < j, so a walk ends; anything else is flagged and
   // read as "no parent").  In grid mode the row threads are idle at this point, waiting for the first tiles.
   // (The previous segment's rows are out of use: every row thread has passed that segment's merge barrier.)
-  if (a.mask_bits == nullptr) {
+  if (a.mask_bits == nullptr && (blk_lo + nblk) * kBlockN > L) {  // (a segment of prefix keys alone needs none)
     if (chain == 0 && r % a.group == 0) {
       uint32_t* row = sm->tile_mask[r / a.group];
       const int wpr = (a.n + 31) >> 5;
@@ -760,41 +777,44 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
     // stands, and their sum tells whether that was right: a score more than the threshold above the reference gives a
     // term, hence a sum, above 2^threshold.  Only then (or without a reference) is the block maximum taken, the
     // reference moved, O rescaled, and the pass repeated (the scores are still in registers).
-    float alpha = 1.f, sum = 0.f;
+    float alpha = 1.f, sum;
     bool settle = __any_sync(0xffffffffu, m_used == -INFINITY);
-    if (!settle) {
-      sum = exponentials();
-      settle = __any_sync(0xffffffffu, !(sum <= kRescaleLimit));
-    }
-    if (settle) {
-      float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll 1
+    for (;;) {  // (a loop, so that the exponentials' code exists once)
+      if (settle) {
+        float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-      for (int e = 0; e < 64; e += 2)  // three-input maximum: two scores per instruction
-        mx[(e >> 1) & 3] = max3(mx[(e >> 1) & 3], __uint_as_float(sreg[e]), __uint_as_float(sreg[e + 1]));
-      const float m_blk = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sc;  // scale > 0
-      const bool move = m_blk > m_used + kRescaleThreshold || (m_used == -INFINITY && m_blk != -INFINITY);
-      if (__any_sync(0xffffffffu, move)) {
-        if (move) {
-          alpha = m_used == -INFINITY ? 0.f : ex2(m_used - m_blk);
-          m_used = m_blk;
-        }
-        if (u > 0) {
-          // O may still be taking the chain's previous block: wait for it, then rescale this warp's rows
-          if (!mbar_wait(sm, &sm->pv_done[chain], (base + u - 1) & 1, a.dev_status)) { ok = false; break; }
-          tc_fence_after();
+        for (int e = 0; e < 64; e += 2)  // three-input maximum: two scores per instruction
+          mx[(e >> 1) & 3] = max3(mx[(e >> 1) & 3], __uint_as_float(sreg[e]), __uint_as_float(sreg[e + 1]));
+        const float m_blk = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * sc;  // scale > 0
+        const bool move = m_blk > m_used + kRescaleThreshold || (m_used == -INFINITY && m_blk != -INFINITY);
+        if (__any_sync(0xffffffffu, move)) {
+          if (move) {
+            alpha = m_used == -INFINITY ? 0.f : ex2(m_used - m_blk);
+            m_used = m_blk;
+          }
+          if (u > 0) {
+            // O may still be taking the chain's previous block: wait for it, then rescale this warp's rows
+            if (!mbar_wait(sm, &sm->pv_done[chain], (base + u - 1) & 1, a.dev_status)) { ok = false; break; }
+            tc_fence_after();
+#pragma unroll 1
+            for (int c = 0; c < 4; ++c) {
+              uint32_t o[32];
+              tmem_ld32(tmem_o + 32u * c, o, 0);
+              tc_wait_ld();
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            uint32_t o[32];
-            tmem_ld32(tmem_o + 32u * c, o, 0);
-            tc_wait_ld();
-#pragma unroll
-            for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
-            tmem_st32(tmem_o + 32u * c, o, 0);
+              for (int e = 0; e < 32; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * alpha);
+              tmem_st32(tmem_o + 32u * c, o, 0);
+            }
           }
         }
       }
       sum = exponentials();
+      if (settle) break;
+      settle = __any_sync(0xffffffffu, !(sum <= kRescaleLimit));
+      if (!settle) break;
     }
+    if (!ok) break;
     if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 3);
     l = l * alpha + sum;
     if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 4);
@@ -828,25 +848,27 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
     M = fmaxf(mlA.x, mlB.x);
     const float fA = mlA.x == -INFINITY ? 0.f : ex2(mlA.x - M), fB = mlB.x == -INFINITY ? 0.f : ex2(mlB.x - M);
     Lc = mlA.y * fA + mlB.y * fB;
-    const int nA = nblk > 0 ? (nblk + 1) >> 1 : 0, nB = nblk >> 1;  // CTA-uniform: which accumulators were written
     const uint32_t oA = tmem + 256u + lane_sel + 64u * chain, oB = oA + 128u;
-#pragma unroll
-    for (int e = 0; e < 64; ++e) merged[e] = 0.f;
-    if (nA > 0 && ok) {
-      uint32_t o[64];
-      tmem_ld32(oA, o, 0);
-      tmem_ld32(oA + 32u, o, 32);
+    uint64_t* m2 = reinterpret_cast<uint64_t*>(merged);
+    if (nblk > 0 && ok) {
+      tmem_ld32(oA, reinterpret_cast<uint32_t*>(merged), 0);
+      tmem_ld32(oA + 32u, reinterpret_cast<uint32_t*>(merged), 32);
       tc_wait_ld();
+      const uint64_t f2 = pair_of(fA, fA);
 #pragma unroll
-      for (int e = 0; e < 64; ++e) merged[e] = __uint_as_float(o[e]) * fA;
+      for (int e = 0; e < 32; ++e) m2[e] = mul2(m2[e], f2);
+    } else {
+#pragma unroll
+      for (int e = 0; e < 64; ++e) merged[e] = 0.f;
     }
-    if (nB > 0 && ok) {
+    if (nblk > 1 && ok) {  // (a segment of one block has left O_B alone)
       uint32_t o[64];
       tmem_ld32(oB, o, 0);
       tmem_ld32(oB + 32u, o, 32);
       tc_wait_ld();
+      const uint64_t f2 = pair_of(fB, fB);
 #pragma unroll
-      for (int e = 0; e < 64; ++e) merged[e] = fmaf(__uint_as_float(o[e]), fB, merged[e]);
+      for (int e = 0; e < 32; ++e) m2[e] = fma2(pair_of(__uint_as_float(o[2 * e]), __uint_as_float(o[2 * e + 1])), f2, m2[e]);
     }
   }
   // both accumulators are in registers: the next segment's first P.V may overwrite them
