@@ -115,7 +115,7 @@ struct UmmaArgs {
   // cut into gridDim.x equal ranges, one per CTA; a tile cut by a range boundary is completed by whichever
   // of its CTAs finishes last, from partial results in the workspace.
   int32_t stream, blocks_per_head_host;
-  int64_t total_blocks_host;
+  int32_t total_blocks_host;  // (a layout of 2^31 positions and more is not streamed)
   int32_t* ws_count;   // [Hkv * tiles] arrivals per tile, zero on entry and on exit
   float2* ws_ml;       // [2 * gridDim.x][128] (m, l) of a partial result
   float4* ws_o;        // [2 * gridDim.x][2][16][128] its unnormalised accumulator, thread-major
@@ -375,13 +375,13 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
   // device memory below (the host's value is then the largest it can be, which the launch was planned for).
   int L = a.L_host;
   int blocks_per_head = a.blocks_per_head_host;
-  int64_t total_blocks = a.total_blocks_host;
-  int64_t range_lo = 0, range_hi = 1;
-  struct Seg { int g, tile, slot_in_head, i0, i1, blk_lo, nblk, nblk_tile; int64_t next; };
+  int total_blocks = a.total_blocks_host;
+  int range_lo = 0, range_hi = 1;
+  struct Seg { int g, tile, slot_in_head, i0, i1, blk_lo, nblk, nblk_tile, next; };
   // Stream mode lays the tiles of a kv head out alternating from both ends (0, T-1, 1, T-2, ...): late tiles
   // have more masked blocks, which cost more, and this way every range gets its share of them.
   auto tile_at = [&](int k) { return (k & 1) ? a.tiles - 1 - (k >> 1) : (k >> 1); };
-  auto seg_at = [&](int64_t pos) -> Seg {
+  auto seg_at = [&](int pos) -> Seg {
     Seg x;
     if (!kStream) {
       x.tile = blockIdx.x; x.g = blockIdx.y; x.slot_in_head = x.tile;
@@ -393,8 +393,8 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
       x.nblk = ((split + 1) * x.nblk_tile) / a.splits - x.blk_lo;
       x.next = 1;
     } else {
-      x.g = (int)(pos / blocks_per_head);
-      const int rem = (int)(pos % blocks_per_head);
+      x.g = pos / blocks_per_head;
+      const int rem = pos - x.g * blocks_per_head;
       int lo = 0, hi = a.tiles - 1;  // the last place in the head's layout whose first block is at or before rem
       while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -406,7 +406,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
       x.i1 = min(x.i0 + a.nodes_per_tile, a.n);
       // the tile's positions are [vs, ve): kStreamTileCost positions of overhead, then its blocks
       const int vs = sm->tile_prefix[lo], ve = sm->tile_prefix[lo + 1];
-      const int end = (int)min((int64_t)ve, (int64_t)rem + (range_hi - pos));  // where this CTA leaves the tile
+      const int end = min(ve, rem + (range_hi - pos));  // where this CTA leaves the tile
       const int from = max(rem, vs + kStreamTileCost);
       x.blk_lo = from - (vs + kStreamTileCost);
       x.nblk_tile = ve - vs - kStreamTileCost;
@@ -452,12 +452,15 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
       blocks_per_head = sum;
-      total_blocks = (int64_t)sum * a.Hkv;
+      total_blocks = sum * a.Hkv;
     }
   }
+  // where the range of CTA x starts: total_blocks * x / gridDim.x
+  const int per_cta = kStream ? total_blocks / (int)gridDim.x : 0, left_over = total_blocks - per_cta * (int)gridDim.x;
+  auto cta_lo = [&](int x) { return per_cta * x + (left_over * x) / (int)gridDim.x; };
   if (kStream) {
-    range_lo = (total_blocks * (int64_t)blockIdx.x) / (int64_t)gridDim.x;
-    range_hi = (total_blocks * (int64_t)(blockIdx.x + 1)) / (int64_t)gridDim.x;
+    range_lo = cta_lo(blockIdx.x);
+    range_hi = cta_lo(blockIdx.x + 1);
   }
   // Grid schedule: the one segment of this CTA is known from its block index, so the thread that armed the barriers
   // requests the Q tile and the first K tile of each chain right away, before the CTA-wide barrier below and the
@@ -521,7 +524,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsLight));
     int seg_n = 0, base_an = 0, base_bn = 0;  // segments done; blocks chains A, B have processed in them
     uint32_t issued = 0, issued_parity = 0;   // producers: stages (bit 2*chain + stage; bit 4: Q) this warp has requested a tile for, and the phase of the last request
-    for (int64_t pos = range_lo; pos < range_hi;) {
+    for (int pos = range_lo; pos < range_hi;) {
     const Seg sg = seg_at(pos);
     if (kStream && sg.nblk == 0) { pos = sg.next; continue; }
     const int g = sg.g, i0 = sg.i0, blk_lo = sg.blk_lo, nblk = sg.nblk;
@@ -681,7 +684,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
   const uint32_t lane_sel = (uint32_t)(quad * 32) << 16;
   const uint32_t tmem_o = tmem + 256u + 128u * chain + lane_sel;
   int seg_n = 0, base_n = 0;  // segments done; blocks this chain has processed in them
-  for (int64_t pos = range_lo; pos < range_hi;) {
+  for (int pos = range_lo; pos < range_hi;) {
   const Seg sg = seg_at(pos);
   if (kStream && sg.nblk == 0) { pos = sg.next; continue; }
   const int g = sg.g, i0 = sg.i0, blk_lo = sg.blk_lo, nblk = sg.nblk;
@@ -883,9 +886,8 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
     // if the piece opens the CTA's range, else 1), then counted; the CTA whose count completes the tile
     // adds the other pieces to its own and writes the output.  Nobody waits for anybody.
     // positions of the tile's blocks in the layout, and the CTAs whose ranges hold some of them
-    const int64_t t0 = (int64_t)g * blocks_per_head + sm->tile_prefix[sg.slot_in_head] + kStreamTileCost, t1 = t0 + sg.nblk_tile;
-    auto cta_lo = [&](int c) { return (total_blocks * (int64_t)c) / (int64_t)gridDim.x; };
-    int c_first = (int)((t0 * (int64_t)gridDim.x) / total_blocks);  // the CTA whose range holds block t0 ...
+    const int t0 = g * blocks_per_head + sm->tile_prefix[sg.slot_in_head] + kStreamTileCost, t1 = t0 + sg.nblk_tile;
+    int c_first = min((int)((float)t0 / (float)total_blocks * (float)gridDim.x), (int)gridDim.x - 1);  // the CTA whose range holds block t0 ...
     while (cta_lo(c_first + 1) <= t0) ++c_first;                      // ... exactly
     while (cta_lo(c_first) > t0) --c_first;
     int c_last = c_first;
@@ -1062,7 +1064,8 @@ static UmmaPlan umma_plan(const seq_tree_attention_params& p) {
   const int tiles = (p.n_tree + nodes_per_tile - 1) / nodes_per_tile;
   const long units = (long)tiles * p.num_kv_heads;
   const int nblk = (p.prefix_len + p.n_tree + kBlockN - 1) / kBlockN;
-  const bool can_stream = tiles <= kMaxStreamTiles && p.prefix_len_dev_count <= 1;  // (a range of the stream schedule crosses kv heads: one length)
+  // (a range of the stream schedule crosses kv heads: one length; positions are 32-bit)
+  const bool can_stream = tiles <= kMaxStreamTiles && p.prefix_len_dev_count <= 1 && (double)units * (nblk + kStreamTileCost) < 2147483648.0;
   const int kNumSMs = device_sm_count();
 #ifdef SEQ_TRACE
   if (const char* e = getenv("SEQ_DEBUG_SPLITS")) return {atoi(e), false};  // debug builds only
@@ -1168,7 +1171,7 @@ int launch_attention_umma(const seq_tree_attention_params& p, int splits, cudaSt
       const int i1 = (t + 1) * nodes_per_tile < p.n_tree ? (t + 1) * nodes_per_tile : p.n_tree;
       a.blocks_per_head_host += kStreamTileCost + (p.prefix_len + i1 + kBlockN - 1) / kBlockN;
     }
-    a.total_blocks_host = (int64_t)a.blocks_per_head_host * p.num_kv_heads;
+    a.total_blocks_host = a.blocks_per_head_host * p.num_kv_heads;
     uint8_t* ws = static_cast<uint8_t*>(p.workspace);
     a.ws_count = reinterpret_cast<int32_t*>(ws);
     a.ws_ml = reinterpret_cast<float2*>(ws + cnt_bytes);
@@ -1181,7 +1184,7 @@ int launch_attention_umma(const seq_tree_attention_params& p, int splits, cudaSt
   // Stream schedule: one CTA per SM, but never more CTAs than positions in the layout: a range must not be empty
   // (the CTAs that share a cut tile are counted from the ranges, and each of them has to arrive).
   const int sms = device_sm_count();
-  const int stream_ctas = a.total_blocks_host < sms ? (int)a.total_blocks_host : sms;
+  const int stream_ctas = a.total_blocks_host < sms ? a.total_blocks_host : sms;
   cfg.gridDim = a.stream ? dim3(stream_ctas, 1, 1) : dim3(tiles, p.num_kv_heads, splits);
   cfg.blockDim = dim3(kUmmaThreads);
   cfg.dynamicSmemBytes = smem;
