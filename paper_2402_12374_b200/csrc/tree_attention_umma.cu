@@ -389,8 +389,9 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
       x.i1 = min(x.i0 + a.nodes_per_tile, a.n);
       // keys this tile can see end at L + i1 (a node sees no later node); blocks of this CTA
       x.nblk_tile = (L + x.i1 + kBlockN - 1) / kBlockN;
-      x.blk_lo = (split * x.nblk_tile) / a.splits;
-      x.nblk = ((split + 1) * x.nblk_tile) / a.splits - x.blk_lo;
+      // (rounded up: the CTA of the last keys, which are masked, is not the one with a block more)
+      x.blk_lo = (split * x.nblk_tile + a.splits - 1) / a.splits;
+      x.nblk = ((split + 1) * x.nblk_tile + a.splits - 1) / a.splits - x.blk_lo;
       x.next = 1;
     } else {
       x.g = pos / blocks_per_head;
