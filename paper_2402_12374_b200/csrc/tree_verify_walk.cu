@@ -5,8 +5,8 @@
 // The vocabulary is cut into one contiguous slice per CTA and one contiguous segment per warp; a thread keeps its
 // 4 * NCH elements of the target row and of the draft row in registers (8 elements per row at 32000 tokens, 32 at
 // 128256), so every vocabulary-wide pass (exponentials, the residual's normaliser after a rejection) is a few
-// instructions per thread, followed by one warp reduction, one table of per-warp partials pushed into every CTA's
-// shared memory, and one cluster barrier.  What the walk will need next is known one step ahead: while child i of
+// instructions per thread, followed by one warp reduction and one table of per-warp partials, sent into every CTA's shared
+// memory and counted in there by an mbarrier.  What the walk will need next is known one step ahead: while child i of
 // the current node is being tested, child i's own rows are loaded into a second set of registers (they are needed
 // exactly if child i is accepted); on a rejection the loads for child i + 1 are issued before the residual pass, so
 // they land behind that pass and its exchange.  A visited node therefore costs its arithmetic and one exchange, not
@@ -57,6 +57,7 @@ struct Shared {
   uint8_t dup[2][SEQ_MAX_TREE];       // by rank: a child that carries the token of an earlier sibling
   int32_t chunk_cnt[32];              // children among nodes [32 j, 32 j + 32)
   float4 xbuf[2][kCl * kWarps];             // cluster exchange: one entry per (rank, warp), double-buffered
+  uint64_t xbar[2];                   // ... and the mbarrier that counts each buffer's bytes in
   int32_t node_flags;
   int32_t pick[2][4];                 // greedy walk, by hop parity: the matching child, the first child with a bad token, the first child
 };
@@ -86,7 +87,8 @@ struct Ctx {
   Shared* sh;
   int rank, lo, cnt;     // CTA in cluster, its vocabulary slice
   int tid, warp, lane;
-  int xpar;
+  uint32_t local, remote;  // shared-window addresses of this CTA's Shared and of CTA `lane`'s
+  uint32_t xn;             // exchanges done
 };
 
 // One row slice into registers: NCH independent 16-byte loads per thread, the ragged end element by element;
@@ -194,21 +196,76 @@ __device__ __forceinline__ float exponentials(float* x, float m, float c2) {
 
 // Every warp of every CTA publishes one float4 to every CTA of the cluster.  On return lane l of every warp holds
 // entries l, l + 32, ... (rank-major, i.e. in vocabulary order).
+//
+// The entries travel as asynchronous stores that count their bytes into the receiver's mbarrier, so nothing fences:
+// a cluster barrier's release would first wait for everything the warp has in flight - the next node's rows, the path's
+// stores - and it was the largest single stall of the walk (a quarter of the warps' time).  Measured, cluster barrier ->
+// this: 768 nodes x 128256 tokens 26.0 -> 21.7 us, 64 x 32000 12.0 -> 9.9, greedy 128 x 32000 7.0 -> 5.0, 16 requests of
+// 64 x 32000 24.3 -> 22.2, 64 of them 47.5 -> 42.8.
+// Buffers and mbarriers are used in turn.  Exchange k + 2 reuses those of exchange k: a warp sends for k + 2 only once it
+// has every warp's entry of k + 1, and a warp sends that only after it has read (and used) its entries of k.
 template <int CL>
 struct Exch { float4 e[CL * kWarps / 32]; };
-// ... in two halves, so that work that does not depend on the exchange can run while the barrier gathers
+constexpr uint32_t kSpinLimit = 1u << 22;
 template <int CL>
-__device__ __forceinline__ void exchange_push(cg::cluster_group& cluster, Ctx& c, float4 mine) {
-  if (c.lane < CL) *cluster.map_shared_rank(&c.sh->xbuf[c.xpar][c.rank * kWarps + c.warp], c.lane) = mine;
-  __syncwarp();
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+__device__ __forceinline__ void exchange_arm(const Ctx& c, int buf) {  // by one thread: the bytes of one exchange
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+               ::"r"(c.local + (uint32_t)offsetof(Shared, xbar) + 8u * buf), "r"((uint32_t)(CL * kWarps * sizeof(float4))) : "memory");
 }
+// Before anything else: the mbarriers, and this CTA's arrival at the one cluster barrier.  exchange_ready() waits for it:
+// from there on every CTA is resident and its mbarriers count.
 template <int CL>
-__device__ __forceinline__ void exchange_pull(Ctx& c, Exch<CL>& x) {
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+__device__ __forceinline__ void exchange_init(Ctx& c) {
+  c.local = (uint32_t)__cvta_generic_to_shared(c.sh);
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(c.remote) : "r"(c.local), "r"(c.lane & (CL - 1)));
+  c.xn = 0;
+  if (c.tid == 0) {
 #pragma unroll
-  for (int m = 0; m < CL * kWarps / 32; ++m) x.e[m] = c.sh->xbuf[c.xpar][c.lane + 32 * m];
-  c.xpar ^= 1;
+    for (int b = 0; b < 2; ++b) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(c.local + (uint32_t)offsetof(Shared, xbar) + 8u * b) : "memory");
+    }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    exchange_arm<CL>(c, 0);
+    exchange_arm<CL>(c, 1);
+  }
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void exchange_ready() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+// ... in two halves, so that work that does not depend on the exchange can run while the entries travel
+template <int CL>
+__device__ __forceinline__ void exchange_push(const Ctx& c, float4 mine) {
+  const uint32_t buf = c.xn & 1u;
+  if (c.lane < CL) {
+    const uint32_t to = c.remote + (uint32_t)offsetof(Shared, xbuf) + (buf * (kCl * kWarps) + c.rank * kWarps + c.warp) * (uint32_t)sizeof(float4);
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+                 ::"r"(to), "r"(__float_as_uint(mine.x)), "r"(__float_as_uint(mine.y)), "r"(__float_as_uint(mine.z)), "r"(__float_as_uint(mine.w)),
+                   "r"(c.remote + (uint32_t)offsetof(Shared, xbar) + 8u * buf) : "memory");
+  }
+}
+// False when the bounded wait ran out (the same for the whole warp, after SEQ_DEV_TIMEOUT and a pause that lets the stores
+// on their way to and from this CTA land): the warp leaves the kernel.
+template <int CL>
+__device__ __forceinline__ bool exchange_pull(Ctx& c, Exch<CL>& x, int32_t* dev_status) {
+  const uint32_t buf = c.xn & 1u, parity = (c.xn >> 1) & 1u;
+  const uint32_t bar = c.local + (uint32_t)offsetof(Shared, xbar) + 8u * buf;
+  uint32_t done = 0;
+#pragma unroll 1
+  for (uint32_t it = 0; it < kSpinLimit && !done; ++it) {
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    done = __all_sync(0xffffffffu, done);
+  }
+  if (!done) {
+    dev_flag(dev_status, SEQ_DEV_TIMEOUT);
+    for (int it = 0; it < 1000; ++it) __nanosleep(1000);
+    return false;
+  }
+  if (c.tid == 0) exchange_arm<CL>(c, (int)buf);  // for the exchange after the next
+#pragma unroll
+  for (int m = 0; m < CL * kWarps / 32; ++m) x.e[m] = c.sh->xbuf[buf][c.lane + 32 * m];
+  ++c.xn;
+  return true;
 }
 // A batched launch runs one request per cluster: the same code on that request's arrays.
 template <int CL>
@@ -238,16 +295,15 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
   const char* const dbase = reinterpret_cast<const char*>(a.draft);
   constexpr int kE = 4 * NCH;        // elements per thread and row
   constexpr int kSpan = 32 * kE;     // consecutive elements of the slice that one warp holds
-  cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ __align__(16) uint8_t dyn_smem[];
   Shared* sh = reinterpret_cast<Shared*>(dyn_smem);
   Ctx c;
   c.sh = sh;
-  c.rank = (int)cluster.block_rank();
+  c.rank = (int)cg::this_cluster().block_rank();
   c.lo = min(c.rank * a.slice_cap, a.V);
   c.cnt = min(a.V - c.lo, a.slice_cap);
   c.tid = threadIdx.x; c.warp = threadIdx.x >> 5; c.lane = threadIdx.x & 31;
-  c.xpar = 0;
+  exchange_init<CL>(c);
   const bool specinfer = (a.flags & SEQ_VERIFY_SPECINFER) != 0;  // D is never touched: ZD stays 1, S stays empty
   const float c2 = kLog2e / a.temperature;
   const bool leader = c.rank == 0 && c.tid == 0;
@@ -297,7 +353,8 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
     if (c.rank == 0 && a.next_child_out != nullptr)
       for (int i = c.tid; i < a.n; i += kTh) a.next_child_out[i] = -2;  // nodes the walk does not visit
   }
-  cluster.sync();  // the tree is in place; every CTA of the cluster is resident before any remote write
+  __syncthreads();  // the tree is in place
+  exchange_ready();
   widen<NCH, kBf16>(pn, p);
   widen<NCH, kBf16>(qn, q);  // (a tree of one node: never loaded, never read)
   WTRACE(leader, 2);
@@ -328,10 +385,10 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
     {
       const float Mwp = warp_max(mp), Mwq = warp_max(mq);
       const float swp = warp_sum(sp * rel_exp(mp, Mwp, c2)), swq = warp_sum(sq * rel_exp(mq, Mwq, c2));
-      exchange_push<CL>(cluster, c, make_float4(Mwp, swp, Mwq, swq));
+      exchange_push<CL>(c, make_float4(Mwp, swp, Mwq, swq));
     }
     WTRACE(leader, 40);
-    // ---- while the cluster's barrier gathers: the node's children, in order, by rank among them; the two logits at
+    // ---- while the entries travel: the node's children, in order, by rank among them; the two logits at
     // each child's token (left in flight); the first child's own rows start their way (they are needed exactly if it
     // is accepted).  (The children arrays are used in turn: a warp may still be reading the previous node's.)
     int n_kids;
@@ -389,7 +446,7 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
         }
     }
     WTRACE(leader, 12);
-    exchange_pull<CL>(c, x);
+    if (!exchange_pull<CL>(c, x, a.dev_status)) return;
     WTRACE(leader, 14);
     float Mp = -INFINITY, Mq = -INFINITY;
 #pragma unroll
@@ -458,7 +515,7 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
       WTRACE(leader, 16);
       if (accept) { accepted = ch; break; }
       // ---- rejected: the next child's rows must start their way, and the residual is updated.  The loads are issued
-      // behind the exchange's barrier arrival (its release fence would otherwise wait for them to land).
+      // behind the exchange's push: ahead of it they delay it (256 nodes x 50257 tokens 15.2 -> 15.6 us).
       const bool more = i + 1 < n_kids;
       if (more) {
         nxt = sh->kids[np][i + 1];
@@ -496,12 +553,12 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
       for (int e = 0; e < kE; e += 2) { z0 += resid(p[e], q[e], Cnf, Unf); z1 += resid(p[e + 1], q[e + 1], Cnf, Unf); }
       const float zr = warp_sum(z0 + z1), zd = warp_sum(zd_mine);
       WTRACE(leader, 17);
-      exchange_push<CL>(cluster, c, make_float4(zr, zd, 0.f, 0.f));
+      exchange_push<CL>(c, make_float4(zr, zd, 0.f, 0.f));
       if (more) {
         load_row<NCH, kBf16>(c, tbase + (int64_t)nxt * a.target_stride * kEsz, pn);
         if (nxt_has_kids) load_row<NCH, kBf16>(c, dbase + (int64_t)nxt * a.draft_stride * kEsz, qn);
       }
-      exchange_pull<CL>(c, x);
+      if (!exchange_pull<CL>(c, x, a.dev_status)) return;
       WTRACE(leader, 18);
       float zsum = 0.f, zdsum = 0.f;
 #pragma unroll
@@ -632,15 +689,15 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
   WTRACE(leader, 30);
   if (leader) *a.path_len = plen;
   if (bonus_found >= 0) *a.bonus = bonus_found;
-  // No closing cluster barrier: remote shared memory is only written before a cluster barrier that every CTA joins,
-  // so nothing can still address a CTA that has left.
+  // No closing cluster barrier: a CTA leaves after it has received every entry of the last exchange, so nothing can still
+  // address it.
 }
 
 
 // ---------------------------------------------------------------- greedy decoding (T = 0) -----------------------
 // R is the one-hot at the target arg-max (lowest index on ties), a child is accepted iff its token is that arg-max;
 // draft logits and uniforms play no part.  Per visited node: the target row in registers, one arg-max over the
-// cluster (one exchange), one look at the children.  While the exchange gathers, the row of the node's first child -
+// cluster (one exchange), one look at the children.  While the exchange is on its way, the row of the node's first child -
 // the draft's most probable token, the likeliest match - is requested; any other match is fetched when it is known.
 __device__ __forceinline__ int ordered_key(float x) {  // an integer that orders like the (non-NaN) float
   int b = __float_as_int(x);
@@ -660,16 +717,15 @@ __global__ void __launch_bounds__(kTh, 1) tree_verify_greedy_kernel(const Verify
   constexpr int kEsz = kBf16 ? 2 : 4;
   constexpr int kE = 4 * NCH, kSpan = 32 * kE;
   const char* const tbase = reinterpret_cast<const char*>(a.target);
-  cg::cluster_group cluster = cg::this_cluster();
   extern __shared__ __align__(16) uint8_t dyn_smem[];
   Shared* sh = reinterpret_cast<Shared*>(dyn_smem);
   Ctx c;
   c.sh = sh;
-  c.rank = (int)cluster.block_rank();
+  c.rank = (int)cg::this_cluster().block_rank();
   c.lo = min(c.rank * a.slice_cap, a.V);
   c.cnt = min(a.V - c.lo, a.slice_cap);
   c.tid = threadIdx.x; c.warp = threadIdx.x >> 5; c.lane = threadIdx.x & 31;
-  c.xpar = 0;
+  exchange_init<kCl>(c);
   const bool leader = c.rank == 0 && c.tid == 0;
   if (c.tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -698,7 +754,8 @@ __global__ void __launch_bounds__(kTh, 1) tree_verify_greedy_kernel(const Verify
     if (c.rank == 0 && a.next_child_out != nullptr)
       for (int i = c.tid; i < a.n; i += kTh) a.next_child_out[i] = -2;  // nodes the walk does not visit
   }
-  cluster.sync();  // the tree is in place; every CTA of the cluster is resident before any remote write
+  __syncthreads();  // the tree is in place
+  exchange_ready();
 
   int cur = 0, plen = 0, g = 0;
   bool bad = false;
@@ -722,8 +779,8 @@ __global__ void __launch_bounds__(kTh, 1) tree_verify_greedy_kernel(const Verify
       }
     }
     warp_argmax(key, idx);
-    exchange_push<kCl>(cluster, c, make_float4(__int_as_float(key), __int_as_float(idx), 0.f, 0.f));
-    // ---- while the barrier gathers: the node's first child, and its row on the way
+    exchange_push<kCl>(c, make_float4(__int_as_float(key), __int_as_float(idx), 0.f, 0.f));
+    // ---- while the entries travel: the node's first child, and its row on the way
     __syncthreads();  // pick[] is reset
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -734,7 +791,7 @@ __global__ void __launch_bounds__(kTh, 1) tree_verify_greedy_kernel(const Verify
     const int first_kid = pick[2];
     if (first_kid != 0x7fffffff) load_row<NCH, kBf16>(c, tbase + (int64_t)first_kid * a.target_stride * kEsz, pn);
     Exch<kCl> t;
-    exchange_pull<kCl>(c, t);
+    if (!exchange_pull<kCl>(c, t, a.dev_status)) return;
     key = INT_MIN; idx = 0x7fffffff;
 #pragma unroll
     for (int m = 0; m < kCl * kWarps / 32; ++m) {  // entries in vocabulary order: the first of equal keys stays
