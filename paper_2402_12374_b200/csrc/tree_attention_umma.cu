@@ -34,12 +34,12 @@
 // piece (m, l, unnormalised accumulator) in the workspace and count themselves on the tile's counter;
 // the pieces are added in CTA order, so the result does not depend on who finishes last.
 //
-// Merge.  The CTAs that share (tile, kv head) form a thread-block cluster along the key
-// range (cs = 1 .. 8); its 2*cs chains share the 16 slices of 8 output columns round-robin.  Every chain pushes,
-// for every row, each 8-column piece of its unnormalised fp32 accumulator into the shared memory of
-// the chain that owns that slice (the K/V stages, dead by then) and its (m, l) into every CTA, with
-// plain remote stores over distributed shared memory; after one cluster barrier each owner reduces
-// its slices from local shared memory and writes the final output.  No workspace, no second kernel.
+// Merge.  The CTAs that share (tile, kv head) form a thread-block cluster along the key range (cs = 1 .. 8).  Each sends
+// its rows' (m, l) into every CTA as soon as its two chains are done; that travels while it reads its accumulators out of
+// tensor memory.  Then it knows the rows' common maximum and sum, scales its partial to its share of the final output, and
+// sends each slice of 8 output columns to the CTA that owns it (the K/V stages, dead by then, receive them).  After a
+// cluster barrier an owner has only additions left.  No workspace, no second kernel.  (Against unscaled pieces, with the
+// owner working out every contributor's factor behind the barrier: 64 nodes on 1024 keys of 32 heads 9.95 -> 9.6 us.)
 //
 // Masking: key j < prefix_len is visible; key prefix_len + t is visible iff bit t of the row's
 // ancestor mask; masked scores become -inf before the maximum, so their probability is exactly 0.
@@ -131,6 +131,9 @@ struct UmmaArgs {
 // ---------------------------------------------------------------- PTX wrappers ------------------
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }
@@ -350,18 +353,20 @@ __device__ __forceinline__ uint32_t mask_window(const uint32_t* row, int wpr, in
   return bits;
 }
 
-template <bool kBf16, bool kStream>
+enum { kGrid, kCluster, kStreamed };  // the schedule: a CTA per unit; a cluster of CTAs per unit; ranges of all units' blocks
+template <bool kBf16, int kMode>
 __global__ void __launch_bounds__(kUmmaThreads, 1)
 tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                            const __grid_constant__ CUtensorMap v_map, const UmmaArgs a) {
+  constexpr bool kStream = kMode == kStreamed;
   extern __shared__ uint8_t smem_raw[];
   UmmaSmem* sm = reinterpret_cast<UmmaSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  cg::cluster_group cluster = cg::this_cluster();
   const int warp = uniform((int)threadIdx.x >> 5), lane = threadIdx.x & 31;
 #ifdef SEQ_TRACE
   int utrace_i = 0;
 #endif
-  const int split = blockIdx.z;  // the cluster spans blockIdx.z
+  const int split = kMode == kCluster ? blockIdx.z : 0;  // the cluster spans blockIdx.z
+  if (kMode == kCluster) cluster_arrive_relaxed();  // "this CTA runs": waited for before the first remote store
   if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 10);
 #ifdef SEQ_TRACE
   const unsigned cta_lin = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
@@ -390,8 +395,8 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
       // keys this tile can see end at L + i1 (a node sees no later node); blocks of this CTA
       x.nblk_tile = (L + x.i1 + kBlockN - 1) / kBlockN;
       // (rounded up: the CTA of the last keys, which are masked, is not the one with a block more)
-      x.blk_lo = (split * x.nblk_tile + a.splits - 1) / a.splits;
-      x.nblk = ((split + 1) * x.nblk_tile + a.splits - 1) / a.splits - x.blk_lo;
+      x.blk_lo = kMode == kGrid ? 0 : (split * x.nblk_tile + a.splits - 1) / a.splits;
+      x.nblk = kMode == kGrid ? x.nblk_tile : ((split + 1) * x.nblk_tile + a.splits - 1) / a.splits - x.blk_lo;
       x.next = 1;
     } else {
       x.g = pos / blocks_per_head;
@@ -647,9 +652,12 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
       }
       __syncwarp();
     }
-    if (a.splits > 1) {  // the two cluster barriers of the merge (see the row threads)
-      cluster.sync();
-      cluster.sync();
+    if (kMode == kCluster) {  // the cluster barriers of the merge (see the row threads)
+      cluster_wait();
+      cluster_arrive_relaxed();
+      cluster_wait();
+      cluster_arrive_relaxed();
+      cluster_wait();
     }
     if (threadIdx.x == 32) UTRACE(1, 9);
     pos = sg.next;
@@ -852,6 +860,16 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
     M = fmaxf(mlA.x, mlB.x);
     const float fA = mlA.x == -INFINITY ? 0.f : ex2(mlA.x - M), fB = mlB.x == -INFINITY ? 0.f : ex2(mlB.x - M);
     Lc = mlA.y * fA + mlB.y * fB;
+    if (kMode == kCluster) {
+      __syncwarp();
+      cluster_wait();  // every CTA of the cluster runs
+      if (chain == 0 && row_valid) {
+        const uint32_t to = smem_u32(&sm->ml_cta[split][r]);
+        for (int q = 0; q < a.splits; ++q) st_cluster2(remote_smem(to, q), M, Lc);
+      }
+      __syncwarp();
+      cluster_arrive_release();
+    }
     const uint32_t oA = tmem + 256u + lane_sel + 64u * chain, oB = oA + 128u;
     uint64_t* m2 = reinterpret_cast<uint64_t*>(merged);
     if (nblk > 0 && ok) {
@@ -963,7 +981,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
   }
   if (kStream && nblk < sg.nblk_tile && !sm->last_part) {
     // not the completing piece: nothing to write
-  } else if (a.splits == 1) {
+  } else if (kMode != kCluster) {
     if (row_valid) {
       const float inv = 1.f / Lc;  // the row saw at least its own key, so Lc > 0
 #pragma unroll
@@ -978,32 +996,12 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
       if (chain == 0 && a.lse != nullptr) a.lse[(size_t)h * a.n + i] = (M + log2f(Lc)) * kLn2;
     }
   } else {
-    // Step 2, across the cluster (cs = 2 .. 8 CTAs along the key range).  The 16 slices of 8 output
-    // columns are owned round-robin: slice s by CTA s % cs, as its slot s / cs.  Every CTA pushes each
-    // 8-column piece of its merged partial into the owner's receive buffer (the K and V stages, adjacent in
-    // shared memory and dead by then: cs * ceil(16 / cs) * 4 KB <= 84 KB of their 128 KB), laid out as float4
-    // planes [contributor][slot][half][row], and its (m, l) into every CTA, with plain remote stores; after a
-    // cluster barrier each owner reduces its slots locally.
-    const int cs = a.splits, slots = (16 + cs - 1) / cs;  // (any cs from 2 to 8; the last slots of some CTAs may be empty)
-    tc_fence_before();
-    cluster.sync();  // every CTA of the cluster is done with its K and V stages before anyone writes into them
+    // Step 2, across the cluster (cs = 2 .. 8 CTAs along the key range).  The 16 slices of 8 output columns are owned
+    // round-robin: slice s by CTA s % cs, as its slot s / cs.  An owner receives into its K and V stages (adjacent in
+    // shared memory: cs * ceil(16 / cs) * 4 KB <= 84 KB of their 128 KB), as float4 planes [contributor][slot][half][row].
+    const int cs = a.splits, slots = (int)((15u + (uint32_t)cs) / (uint32_t)cs);  // (any cs from 2 to 8; the last slots of some CTAs may be empty)
+    cluster_wait();  // every CTA's (m, l) is here, and every CTA is done with its K and V stages
     if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 7);
-    // (rows past the tile's last node are padding: nothing of theirs is pushed, reduced or stored)
-    if (chain == 0 && row_valid)
-      for (int q = 0; q < cs; ++q) *cluster.map_shared_rank(&sm->ml_cta[split][r], q) = make_float2(M, Lc);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (!row_valid) break;
-      const int s_idx = 8 * chain + j;
-      uint4* dst = cluster.map_shared_rank(reinterpret_cast<uint4*>(&sm->k[0][0][0]), s_idx % cs) +
-                   ((size_t)(split * slots + s_idx / cs) * 2) * kTileM + r;
-      dst[0] = make_uint4(__float_as_uint(merged[8 * j]), __float_as_uint(merged[8 * j + 1]),
-                          __float_as_uint(merged[8 * j + 2]), __float_as_uint(merged[8 * j + 3]));
-      dst[kTileM] = make_uint4(__float_as_uint(merged[8 * j + 4]), __float_as_uint(merged[8 * j + 5]),
-                               __float_as_uint(merged[8 * j + 6]), __float_as_uint(merged[8 * j + 7]));
-    }
-    cluster.sync();
-    if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 8);
     float Mg = -INFINITY;
     for (int q = 0; q < cs; ++q) Mg = fmaxf(Mg, sm->ml_cta[q][r].x);
     float Ls = 0.f;
@@ -1011,29 +1009,48 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
       const float2 mlq = sm->ml_cta[q][r];
       if (mlq.x != -INFINITY) Ls += mlq.y * ex2(mlq.x - Mg);
     }
-    const float inv = 1.f / Ls;  // some CTA saw the row's own key, so Ls > 0
-    const float4* mine = reinterpret_cast<const float4*>(&sm->k[0][0][0]);
-    for (int slot = chain; slot < slots && row_valid; slot += 2) {  // the two warp groups share this CTA's slots
-      if (slot * cs + split >= 16) break;  // (cs does not divide 16: this CTA owns one slice fewer)
-      float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      for (int q = 0; q < cs; ++q) {
-        const float mq = sm->ml_cta[q][r].x;
-        if (mq == -INFINITY) continue;
-        const float f = ex2(mq - Mg);
-        const float4* src = mine + ((size_t)(q * slots + slot) * 2) * kTileM + r;
-        const float4 x = src[0], y = src[kTileM];
-        acc[0] = fmaf(x.x, f, acc[0]); acc[1] = fmaf(x.y, f, acc[1]); acc[2] = fmaf(x.z, f, acc[2]); acc[3] = fmaf(x.w, f, acc[3]);
-        acc[4] = fmaf(y.x, f, acc[4]); acc[5] = fmaf(y.y, f, acc[5]); acc[6] = fmaf(y.z, f, acc[6]); acc[7] = fmaf(y.w, f, acc[7]);
-      }
-      if (row_valid) {
-        uint4 val;
-        val.x = pack2<kBf16>(acc[0] * inv, acc[1] * inv);
-        val.y = pack2<kBf16>(acc[2] * inv, acc[3] * inv);
-        val.z = pack2<kBf16>(acc[4] * inv, acc[5] * inv);
-        val.w = pack2<kBf16>(acc[6] * inv, acc[7] * inv);
-        *reinterpret_cast<uint4*>(out_row + 2 * (8 * (slot * cs + split))) = val;
+    const uint32_t recv = smem_u32(&sm->k[0][0][0]);
+    // (rows past the tile's last node are padding: nothing of theirs is pushed, reduced or stored)
+    if (row_valid) {
+      const float f = M == -INFINITY ? 0.f : ex2(M - Mg) / Ls;  // some CTA saw the row's own key, so Ls > 0
+      const uint64_t f2 = pair_of(f, f);
+      uint64_t* m2 = reinterpret_cast<uint64_t*>(merged);
+#pragma unroll
+      for (int e = 0; e < 32; ++e) m2[e] = mul2(m2[e], f2);
+      int slot = (int)(8u * (uint32_t)chain / (uint32_t)cs), owner = 8 * chain - slot * cs;
+      const uint32_t to = recv + 16u * (uint32_t)(split * slots * 2 * kTileM + r);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) {
+        const uint32_t dst = remote_smem(to + 16u * (uint32_t)(slot * 2 * kTileM), owner);
+        st_cluster4(dst, merged + 8 * j);
+        st_cluster4(dst + 16u * kTileM, merged + 8 * j + 4);
+        if (++owner == cs) { owner = 0; ++slot; }
       }
     }
+    if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 13);
+    __syncwarp();
+    cluster_arrive_release();
+    cluster_wait();
+    if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 8);
+    const ulonglong2* mine = reinterpret_cast<const ulonglong2*>(&sm->k[0][0][0]) + r;
+    if (row_valid)
+      for (int slot = chain; slot * cs + split < 16; slot += 2) {  // the two warp groups share this CTA's slots
+        const ulonglong2* src = mine + slot * 2 * kTileM;
+        ulonglong2 x = src[0], y = src[kTileM];
+        for (int q = 1; q < cs; ++q) {
+          src += slots * 2 * kTileM;
+          const ulonglong2 u = src[0], v = src[kTileM];
+          x.x = add2(x.x, u.x); x.y = add2(x.y, u.y); y.x = add2(y.x, v.x); y.y = add2(y.y, v.y);
+        }
+        float o[8];
+        unpair(x.x, o[0], o[1]); unpair(x.y, o[2], o[3]); unpair(y.x, o[4], o[5]); unpair(y.y, o[6], o[7]);
+        uint4 val;
+        val.x = pack2<kBf16>(o[0], o[1]);
+        val.y = pack2<kBf16>(o[2], o[3]);
+        val.z = pack2<kBf16>(o[4], o[5]);
+        val.w = pack2<kBf16>(o[6], o[7]);
+        *reinterpret_cast<uint4*>(out_row + 2 * (8 * (slot * cs + split))) = val;
+      }
     if (split == 0 && chain == 0 && row_valid && a.lse != nullptr) a.lse[(size_t)h * a.n + i] = (Mg + log2f(Ls)) * kLn2;
   }
   if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 9);
@@ -1044,7 +1061,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
 #ifdef SEQ_TRACE
   if (threadIdx.x == 128 && cta_lin < 1024) g_cta_times[cta_lin][1] = gtimer();
 #endif
-  // no remote access happens after the second cluster barrier, so CTAs may leave independently
+  // no remote access happens after the last cluster barrier, so CTAs may leave independently
   tc_fence_before();
   __syncthreads();  // pairs with warp group 0, whose MMA warp then frees the tensor memory
 }
@@ -1199,9 +1216,10 @@ int launch_attention_umma(const seq_tree_attention_params& p, int splits, cudaSt
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  // four instantiations: element type x (grid | stream) mode; the grid-mode code carries none of the stream machinery
+  // Six instantiations: element type x schedule.  None carries another's code: half of a short call's instructions run
+  // once, at the rate at which they are fetched.
   auto launch = [&](auto kernel, int which) -> int {
-    static int attr_done[4][64];  // the opt-in shared-memory size is set once per kernel and device
+    static int attr_done[6][64];  // the opt-in shared-memory size is set once per kernel and device
     const int rc = once_per_device(attr_done[which], [&]() -> int {
       SEQ_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
       return SEQ_OK;
@@ -1210,8 +1228,12 @@ int launch_attention_umma(const seq_tree_attention_params& p, int splits, cudaSt
     SEQ_CUDA_OK(cudaLaunchKernelEx(&cfg, kernel, q_map, k_map, v_map, a));
     return SEQ_OK;
   };
-  if (p.dtype == SEQ_BF16) return a.stream ? launch(tree_attention_umma_kernel<true, true>, 0) : launch(tree_attention_umma_kernel<true, false>, 1);
-  return a.stream ? launch(tree_attention_umma_kernel<false, true>, 2) : launch(tree_attention_umma_kernel<false, false>, 3);
+  const int mode = a.stream ? kStreamed : splits > 1 ? kCluster : kGrid;
+  if (p.dtype == SEQ_BF16)
+    return mode == kStreamed ? launch(tree_attention_umma_kernel<true, kStreamed>, 0)
+           : mode == kCluster ? launch(tree_attention_umma_kernel<true, kCluster>, 1) : launch(tree_attention_umma_kernel<true, kGrid>, 2);
+  return mode == kStreamed ? launch(tree_attention_umma_kernel<false, kStreamed>, 3)
+         : mode == kCluster ? launch(tree_attention_umma_kernel<false, kCluster>, 4) : launch(tree_attention_umma_kernel<false, kGrid>, 5);
 }
 
 }  // namespace seqtree
