@@ -1076,6 +1076,39 @@ bool umma_supported(const seq_tree_attention_params& p) {
 // range) per (tile, kv head), in as many waves as that takes.  Stream schedule: one CTA per SM, each with an equal range of the
 // flattened block space and share the tiles that a range boundary cuts.  p.kernel = 3 / 4 force one of them.
 struct UmmaPlan { int splits; bool stream; };
+constexpr size_t kUmmaSmemBytes = sizeof(UmmaSmem) + 1024;
+// Clusters of cs CTAs that the device runs at a time (one CTA fills an SM).  Asked once per device and size; without a
+// device, or where the question fails, what the SMs would hold.
+static int clusters_side_by_side(int cs) {
+  const int sms = device_sm_count();
+  if (cs == 1) return sms;
+  static int known[kMaxClusterSplit + 1][64];  // + 1; 0 = not asked yet
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return sms / cs; }
+  n = __atomic_load_n(&known[cs][dev], __ATOMIC_ACQUIRE);
+  if (n == 0) {
+    auto kernel = tree_attention_umma_kernel<true, kCluster>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1, 1, cs);
+    cfg.blockDim = dim3(kUmmaThreads);
+    cfg.dynamicSmemBytes = kUmmaSmemBytes;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = cs;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kUmmaSmemBytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = sms / cs;
+    }
+    ++n;
+    __atomic_store_n(&known[cs][dev], n, __ATOMIC_RELEASE);
+  }
+  return n - 1;
+}
 static UmmaPlan umma_plan(const seq_tree_attention_params& p) {
   const int G = p.num_q_heads / p.num_kv_heads;
   const int nodes_per_tile = kTileM / G;
@@ -1098,15 +1131,20 @@ static UmmaPlan umma_plan(const seq_tree_attention_params& p) {
     const bool last_wave_thin = units * 10 <= waves * kNumSMs * 6;
     if (nblk >= 32 && (last_wave_thin || nblk >= 72)) return {1, true};
   }
+  // Otherwise the split with the lowest estimate.  Microseconds per wave, fitted to launches of 72 shapes (8 to 768 nodes,
+  // prefixes of 100 to 8000 keys, 8 to 384 units) with every split forced: 0.45 per block of a CTA's key range, 4.7 fixed,
+  // and the merge across the cluster, which grows with the pieces that an owner's threads add up one after the other
+  // (ceil(ceil(16 / cs) / 2) * cs, hence 4 below 3).  What a wave holds is asked of the device: a cluster lies in one
+  // GPC, so the SMs left over in each are lost to it (74, 44, 36, 28, 21, 14 and 14 clusters of 2 to 8 CTAs were seen, where
+  // 148 / cs had been assumed; 24 units of 17 blocks 17.3 -> 10.1 us, 16 of 48 21.8 -> 12.5, 48 of 66 34.7 -> 23.3).
+  static const double kMerge[kMaxClusterSplit + 1] = {0.0, 0.0, 2.25, 3.2, 2.8, 3.5, 3.8, 4.2, 4.2};
   int best = 1;
   double best_cost = -1.0;
-  for (int cs = 1; cs <= kMaxClusterSplit; ++cs) {
-    if (cs > 1 && cs > nblk) break;
-    const long waves = (units * cs + kNumSMs - 1) / kNumSMs;
-    // microseconds per wave, fitted to measured launches of the paper's shapes with every split forced: 0.65 per
-    // block of a CTA's key range, 4.7 fixed, and 1.6 + 0.5 per CTA beyond two for the merge across the cluster
-    const double merge = cs == 1 ? 0.0 : 1.6 + 0.5 * (cs - 2);
-    const double cost = (double)waves * (0.65 * ((nblk + cs - 1) / cs) + 4.7 + merge);
+  for (int cs = 1; cs <= kMaxClusterSplit && cs <= nblk; ++cs) {
+    const int room = clusters_side_by_side(cs);
+    if (room == 0) continue;
+    const long waves = (units + room - 1) / room;
+    const double cost = (double)waves * (0.45 * ((nblk + cs - 1) / cs) + 4.7 + kMerge[cs]);
     if (best_cost < 0 || cost < best_cost - 1e-9) { best = cs; best_cost = cost; }
   }
   return {best, false};
@@ -1197,7 +1235,7 @@ int launch_attention_umma(const seq_tree_attention_params& p, int splits, cudaSt
     SEQ_CUDA_OK(cudaMemsetAsync(a.ws_count, 0, cnt_bytes, stream));  // the counters start at zero (the kernel leaves them at zero)
   }
 
-  const size_t smem = sizeof(UmmaSmem) + 1024;
+  const size_t smem = kUmmaSmemBytes;
   cudaLaunchConfig_t cfg = {};
   // Stream schedule: one CTA per SM, but never more CTAs than positions in the layout: a range must not be empty
   // (the CTAs that share a cut tile are counted from the ranges, and each of them has to arrive).

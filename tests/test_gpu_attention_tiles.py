@@ -29,6 +29,12 @@ def test_groups_that_do_not_divide_the_tile(hkv, group, n, L, kernel):
     G.check_attention(_inputs(hkv, group, n, L, "bf16"), kernel=kernel)
 
 
+@pytest.mark.parametrize("hkv,n,L", [(60, 2, 1250), (40, 3, 1100), (32, 2, 1030), (24, 3, 1590), (16, 4, 3000), (1, 5, 2200), (1, 4, 4000)])
+def test_clusters_of_every_size(hkv, n, L):
+    """Where the device runs 74, 44, 36, 28, 21, 14 and 14 clusters of 2 to 8 CTAs side by side, these take one size each."""
+    G.check_attention(_inputs(hkv, 1, n, L, "bf16"))
+
+
 @pytest.mark.parametrize("hkv,group,n,L", [(1, 1, 1, 0), (2, 1, 8, 31), (1, 1, 9, 119), (1, 2, 8, 128), (2, 3, 11, 97), (1, 1, 32, 96), (1, 1, 33, 224),
                                            (2, 4, 16, 255), (1, 5, 13, 64), (3, 1, 65, 63), (1, 150, 2, 40), (1, 1, 1, 3000)])
 def test_single_precision_tiles(hkv, group, n, L):
