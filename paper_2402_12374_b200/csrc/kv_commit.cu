@@ -1,6 +1,8 @@
 // seq_tree_kv_commit: the accepted path's key/value rows move to the front of the tree region, in place.
 // Pure data movement, bound by latency at the paper's sizes (a few rows per plane): one thread per 16 bytes of a
-// plane's rows, a batch of independent loads in flight before the batch's stores.
+// plane's rows, a batch of independent loads in flight before the batch's stores.  Launched with programmatic stream
+// serialisation, like the verification before it and the next step's attention behind it: its CTAs are in place when the
+// path is there, and the attention's set-up runs under this kernel.
 #include "common.cuh"
 
 namespace seqtree {
@@ -20,6 +22,8 @@ struct CommitArgs {
 
 __global__ void __launch_bounds__(kCommitThreads) kv_commit_kernel(const CommitArgs a) {
   __shared__ int32_t s_path[SEQ_MAX_TREE];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // everything below may read what the previous kernel wrote
   // path_len and the whole path buffer (n entries, as seq_tree_verify owns it) are fetched together: one memory
   // latency instead of two.  Every CTA checks the path for itself: 0 first, strictly ascending, below n.
   const int len = *a.path_len;
@@ -94,7 +98,15 @@ extern "C" int seq_tree_kv_commit(const seq_tree_kv_commit_params* p, void* stre
   const int64_t want = (total + kCommitThreads - 1) / kCommitThreads;
   const long cap = (long)device_sm_count() * 8;
   const int grid = (int)(want < cap ? want : cap);  // at most one wave of 8 CTAs per SM; larger caches loop
-  kv_commit_kernel<<<grid, kCommitThreads, 0, static_cast<cudaStream_t>(stream)>>>(a);
-  SEQ_CUDA_OK(cudaGetLastError());
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kCommitThreads);
+  cfg.stream = static_cast<cudaStream_t>(stream);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  SEQ_CUDA_OK(cudaLaunchKernelEx(&cfg, kv_commit_kernel, a));
   return SEQ_OK;
 }
