@@ -48,13 +48,9 @@ struct Shared {
   int32_t tokens[SEQ_MAX_TREE];
   float uniforms[SEQ_MAX_TREE + 1];
   uint32_t has_child[SEQ_MAX_TREE / 32];
-  // The current node's children, listed by warp 0 while the other warps may still be reading the previous node's:
-  // two copies, used in turn.
-  int32_t kids[2][SEQ_MAX_TREE];      // in ascending order (the order they were drawn in)
-  float2 kid_raw[2][SEQ_MAX_TREE];       // (target logit, draft logit) of the current node at each child's token, by rank;
-                                      // after the last test: scratch of the final draw's fine level
-  int32_t kid_tok[2][SEQ_MAX_TREE];   // by rank: the children's tokens
-  uint8_t dup[2][SEQ_MAX_TREE];       // by rank: a child that carries the token of an earlier sibling
+  // The current node's children in ascending order (the order they were drawn in): (node, token).  Two copies, used in
+  // turn: a warp may still be reading the previous node's.  After the last test: scratch of the final draw's fine level.
+  int2 kid[2][SEQ_MAX_TREE];
   int32_t chunk_cnt[32];              // children among nodes [32 j, 32 j + 32)
   float4 xbuf[2][kCl * kWarps];             // cluster exchange: one entry per (rank, warp), double-buffered
   uint64_t xbar[2];                   // ... and the mbarrier that counts each buffer's bytes in
@@ -69,6 +65,11 @@ __device__ __forceinline__ float fast_ex2(float x) {
 }
 __device__ __forceinline__ float rel_exp(float m, float M, float c2) { return m == -INFINITY ? 0.f : fast_ex2((m - M) * c2); }
 __device__ __forceinline__ float resid(float pn, float qn, float Cf, float Uf) { return fmaxf(fmaf(-Cf, qn, pn) - Uf, 0.f); }
+__device__ __forceinline__ float max_lanes(float v) {
+  float m;
+  asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v));
+  return m;
+}
 __device__ __forceinline__ double sum_lanes(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -333,6 +334,7 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
     load_row<NCH, kBf16>(c, tbase, pn);
     if (a.n > 1) load_row<NCH, kBf16>(c, dbase, qn);  // (a root without children: never read)
     if (c.tid < SEQ_MAX_TREE / 32) sh->has_child[c.tid] = 0u;
+    if (c.tid < 32) sh->chunk_cnt[c.tid] = 0;
     if (c.tid == 0) sh->node_flags = 0;
     __syncthreads();
 #pragma unroll
@@ -383,22 +385,22 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
     WTRACE(leader, 13);
     Exch<CL> x;
     {
-      const float Mwp = warp_max(mp), Mwq = warp_max(mq);
+      const float Mwp = max_lanes(mp), Mwq = max_lanes(mq);
       const float swp = warp_sum(sp * rel_exp(mp, Mwp, c2)), swq = warp_sum(sq * rel_exp(mq, Mwq, c2));
       exchange_push<CL>(c, make_float4(Mwp, swp, Mwq, swq));
     }
     WTRACE(leader, 40);
-    // ---- while the entries travel: the node's children, in order, by rank among them; the two logits at
-    // each child's token (left in flight); the first child's own rows start their way (they are needed exactly if it
-    // is accepted).  (The children arrays are used in turn: a warp may still be reading the previous node's.)
-    int n_kids;
-    int krank[4];
-    float2 kraw[4];
-    {
+    // ---- while the entries travel: the node's children, in order; the first child's own rows start their way (they are
+    // needed exactly if it is accepted); lane l of every warp takes child l (then l + 32, ...): its token, uniform, the two
+    // logits of the current node at it (left in flight), and whether an earlier sibling carries the same token.
+    int n_kids = 0, nxt = -1;
+    bool nxt_has_kids = false;
+    if (cur_has_kids) {
       bool k[4];
       uint32_t b[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
+        if (kTh * j >= a.n) break;  // (chunks behind the tree count no children from the start)
         const int ch = c.tid + kTh * j;
         k[j] = ch < a.n && sh->parent[ch] == cur;
         b[j] = __ballot_sync(0xffffffffu, k[j]);
@@ -406,52 +408,49 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
       }
       __syncthreads();
       const int cc = sh->chunk_cnt[c.lane];
-      int inc = cc;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int up = __shfl_up_sync(0xffffffffu, inc, o);
-        if (c.lane >= o) inc += up;
-      }
-      n_kids = __shfl_sync(0xffffffffu, inc, 31);
+      n_kids = __reduce_add_sync(0xffffffffu, cc);
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        krank[j] = -1;
-        const int r = __shfl_sync(0xffffffffu, inc - cc, kWarps * j + c.warp) + __popc(b[j] & ((1u << c.lane) - 1u));
-        if (k[j]) {
-          const int ch = c.tid + kTh * j, s = sh->tokens[ch];
-          sh->kids[np][r] = ch;
-          sh->kid_tok[np][r] = s;
-          krank[j] = r;
-          if (s >= 0 && s < a.V) kraw[j] = make_float2(load_logit<kBf16>(trow, s), load_logit<kBf16>(drow, s));
-        }
+        if (kTh * j >= a.n) break;
+        const int before = __reduce_add_sync(0xffffffffu, c.lane < kWarps * j + c.warp ? cc : 0);
+        const int ch = c.tid + kTh * j;
+        if (k[j]) sh->kid[np][before + __popc(b[j] & ((1u << c.lane) - 1u))] = make_int2(ch, sh->tokens[ch]);
       }
       __syncthreads();
-    }
-    int nxt = n_kids > 0 ? sh->kids[np][0] : -1;
-    bool nxt_has_kids = false;
-    if (nxt >= 0) {
+      nxt = sh->kid[np][0].x;
       nxt_has_kids = (sh->has_child[nxt >> 5] >> (nxt & 31)) & 1u;
       load_row<NCH, kBf16>(c, tbase + (int64_t)nxt * a.target_stride * kEsz, pn);
       if (nxt_has_kids) load_row<NCH, kBf16>(c, dbase + (int64_t)nxt * a.draft_stride * kEsz, qn);
     }
     WTRACE(leader, 44);
-    if (!specinfer) {  // does an earlier sibling carry the same token?
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (krank[j] >= 0) {
-          int d = 0;
-          const int s = sh->kid_tok[np][krank[j]];
-          for (int r = 0; r < krank[j]; ++r) d |= sh->kid_tok[np][r] == s;
-          sh->dup[np][krank[j]] = (uint8_t)d;
-        }
-    }
+    int kch = 0, ktok = -1;                 // this lane's child
+    float ku = 0.f;
+    float2 kraw = make_float2(0.f, 0.f);
+    bool kvalid = false, kdup = false;
+    auto take_kids = [&](int base) {
+      const int r = base + c.lane;
+      ktok = -1;
+      kdup = false;
+      if (r < n_kids) {
+        const int2 e = sh->kid[np][r];
+        kch = e.x; ktok = e.y;
+        ku = sh->uniforms[kch];
+      }
+      kvalid = ktok >= 0 && ktok < a.V;
+      if (kvalid) kraw = make_float2(load_logit<kBf16>(trow, ktok), load_logit<kBf16>(drow, ktok));
+      if (!specinfer) {  // (lanes past the last child come after every child: what they hold does not matter)
+        kdup = (__match_any_sync(0xffffffffu, ktok) & ((1u << c.lane) - 1u)) != 0u;
+        for (int r2 = 0; r2 < base; ++r2) kdup |= sh->kid[np][r2].y == ktok;  // (a node of more than 32 children)
+      }
+    };
+    if (n_kids > 0) take_kids(0);
     WTRACE(leader, 12);
     if (!exchange_pull<CL>(c, x, a.dev_status)) return;
     WTRACE(leader, 14);
     float Mp = -INFINITY, Mq = -INFINITY;
 #pragma unroll
     for (int m = 0; m < kPPL; ++m) { Mp = fmaxf(Mp, x.e[m].x); Mq = fmaxf(Mq, x.e[m].z); }
-    Mp = warp_max(Mp); Mq = warp_max(Mq);
+    Mp = max_lanes(Mp); Mq = max_lanes(Mq);
     // (Single precision from here on: the sums have 128 terms of like size, the scalars C, U, Z, ZD a handful of
     // updates; their rounding stays two orders of magnitude inside the 1e-5 band of the parity rule.)
     float part_sum[kPPL];   // residual mass of the (rank, warp) segments lane, lane + 32, ...: the draw's coarse level
@@ -481,44 +480,38 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
       }
       zd_mine = s0 + s1;
     }
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (krank[j] >= 0) sh->kid_raw[np][krank[j]] = kraw[j];
-    __syncthreads();  // the children's logits and repeat marks are in place
     WTRACE(leader, 15);
     float C = 0.f, U = 0.f, Z = 1.f, ZD = 1.f;
     int nS = 0, accepted = -1;
-    uint32_t dead = 0u;  // this thread's elements that were rejected (they are in S)
+    // each lane's child: its two probabilities (zero once an earlier, hence rejected, sibling carried the same token: it is
+    // in S.  Without the draft update there is no S: a repeated token is tested like any other, and its R is 0 by then)
+    float kps = 0.f, kqs = 0.f;
+    uint32_t valid_kids = 0u, dup_kids = 0u;
+    auto score_kids = [&]() {
+      kps = kvalid && !kdup ? fast_ex2((clean_logit(kraw.x) - Mp) * c2) * invSp : 0.f;
+      kqs = kvalid && !kdup ? fast_ex2((clean_logit(kraw.y) - Mq) * c2) * invSq : 0.f;
+      valid_kids = __ballot_sync(0xffffffffu, kvalid);
+      dup_kids = __ballot_sync(0xffffffffu, kdup);
+    };
+    if (n_kids > 0) score_kids();
     // ---- Algorithm 2's loop over the children, in their order
 #pragma unroll 1
     for (int i = 0; i < n_kids; ++i) {
-      const int ch = sh->kids[np][i], s = sh->kid_tok[np][i];
-      const bool valid = s >= 0 && s < a.V;
+      if (i > 0 && (i & 31) == 0) { take_kids(i); score_kids(); }
+      const bool valid = (valid_kids >> (i & 31)) & 1u, in_S = (dup_kids >> (i & 31)) & 1u;
       if (!valid) dev_flag(a.dev_status, SEQ_DEV_BAD_TOKEN);
-      // an earlier (hence rejected) sibling carried the same token: it is in S.  (Without the draft update there is
-      // no S: a repeated token is tested like any other, and its R is 0 by then.)
-      const bool in_S = !specinfer && sh->dup[np][i] != 0;
-      bool accept = false;
-      if (valid) {
-        float ps = 0.f, qs = 0.f;
-        if (!in_S) {
-          const float2 raw = sh->kid_raw[np][i];
-          ps = fast_ex2((clean_logit(raw.x) - Mp) * c2) * invSp;
-          qs = fast_ex2((clean_logit(raw.y) - Mq) * c2) * invSq;
-        }
-        // the acceptance test u < R[s]/D[s], with R[s] = rs/Z and D[s] = qs/ZD (or 1/(V-|S|)); cross-multiplied,
-        // which also covers D[s] = 0 (accept iff R[s] > 0)
-        const float rs = in_S ? 0.f : resid(ps, qs, C, U);
-        const float u = sh->uniforms[ch];
-        accept = mode == 0 ? (u * Z * qs < rs * ZD) : (u * Z < rs * (float)(a.V - nS));
-      }
+      // the acceptance test u < R[s]/D[s], with R[s] = rs/Z and D[s] = qs/ZD (or 1/(V-|S|)); cross-multiplied, which also
+      // covers D[s] = 0 (accept iff R[s] > 0).  Every lane tests its child, child i's answer counts.
+      const float rs = resid(kps, kqs, C, U);
+      const bool win = kvalid && (mode == 0 ? ku * Z * kqs < rs * ZD : ku * Z < rs * (float)(a.V - nS));
+      const bool accept = (__ballot_sync(0xffffffffu, win) >> (i & 31)) & 1u;
       WTRACE(leader, 16);
-      if (accept) { accepted = ch; break; }
+      if (accept) { accepted = __shfl_sync(0xffffffffu, kch, i & 31); break; }
       // ---- rejected: the next child's rows must start their way, and the residual is updated.  The loads are issued
       // behind the exchange's push: ahead of it they delay it (256 nodes x 50257 tokens 15.2 -> 15.6 us).
       const bool more = i + 1 < n_kids;
       if (more) {
-        nxt = sh->kids[np][i + 1];
+        nxt = sh->kid[np][i + 1].x;
         nxt_has_kids = (sh->has_child[nxt >> 5] >> (nxt & 31)) & 1u;
       }
       if (!valid) {  // (not a token: R and D untouched)
@@ -532,16 +525,19 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
       float Cn = C, Un = U;
       if (mode == 0) Cn += Z * __frcp_rn(ZD);
       else if (a.V - nS > 0) Un += Z * __frcp_rn((float)(a.V - nS));
-      // the draft update: s leaves D and joins S.  The thread that holds s marks it and re-sums its share of D
+      // the draft update: s leaves D and joins S.  The thread that holds s clears it (its R is 0 from here on, see above)
+      // and re-sums its share of D
       if (!in_S && !specinfer) {
+        const int s = __shfl_sync(0xffffffffu, ktok, i & 31);
         const int idx = s - c.lo - c.warp * kSpan;
         if (s - c.lo >= 0 && s - c.lo < c.cnt && idx >= 0 && idx < kSpan && ((idx >> 2) & 31) == c.lane) {
-          dead |= 1u << (((idx >> 7) << 2) | (idx & 3));
+          const int at = ((idx >> 7) << 2) | (idx & 3);
           float s0 = 0.f, s1 = 0.f;
 #pragma unroll
           for (int k = 0; k < kE; k += 2) {
-            s0 += ((dead >> k) & 1u) ? 0.f : q[k];
-            s1 += ((dead >> (k + 1)) & 1u) ? 0.f : q[k + 1];
+            if (k == at) p[k] = q[k] = 0.f;
+            if (k + 1 == at) p[k + 1] = q[k + 1] = 0.f;
+            s0 += q[k]; s1 += q[k + 1];
           }
           zd_mine = s0 + s1;
         }
@@ -592,10 +588,6 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
       const float Cf = C, Uf = U;
 #pragma unroll
       for (int e = 0; e < kE; ++e) p[e] = resid(p[e], use_q ? q[e] : 0.f, Cf, Uf);  // the residual replaces p
-      if (dead) {  // rejected tokens have left the residual for good
-#pragma unroll
-        for (int e = 0; e < kE; ++e) p[e] = ((dead >> e) & 1u) ? 0.f : p[e];
-      }
       const float u = sh->uniforms[a.n];
       // coarse level, every warp for itself: inclusive scan over the (rank, warp) masses, 32 at a time
       double inc[kPPL], before = 0.0;
@@ -648,7 +640,7 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
         // The segment's residual values go to shared memory in vocabulary order (one padding word per 32, so that
         // the reads below do not collide); lane l then owns elements [NCH*4*l, +NCH*4): the lanes' sums are scanned,
         // and the lane that holds the crossing walks its elements.  Rolled loops: this runs in one warp.
-        float* seg = reinterpret_cast<float*>(sh->kid_raw[np ^ 1]);
+        float* seg = reinterpret_cast<float*>(sh->kid[np ^ 1]);
 #pragma unroll
         for (int e = 0; e < kE; ++e) {
           const int idx = (e >> 2) * 128 + c.lane * 4 + (e & 3);
