@@ -824,8 +824,8 @@ def run_workload(cfg, T, args, rank, local_rank, world, dev, stream, peaks, with
     ver_sets += device_verify_sets(cfg, parent, T, nv - 1, dev, rank_seed_base(rank))
     for tok, tl, dl, u in ver_sets:
         ver_calls.append(B.VerifyCall(parent_d, tok, tl, dl, T, u, dev_status=status))
-    combine = args.kernel == B.KERNEL_CUDA_CORE and attn_calls[0].workspace_bytes_needed > 0
-    launches_per_step = (0 if fused_mask else 1) + (2 if combine else 1) + 1
+    two = attn_calls[0].workspace_bytes_needed > 0  # the pieces' counters or their sum are a launch of their own
+    launches_per_step = (0 if fused_mask else 1) + (2 if two else 1) + 1
 
     def step(i, s):
         if not fused_mask:

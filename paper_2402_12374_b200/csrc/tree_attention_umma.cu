@@ -1066,6 +1066,13 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
   __syncthreads();  // pairs with warp group 0, whose MMA warp then frees the tensor memory
 }
 
+__global__ void zero_words_kernel(int32_t* words, int n) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) words[i] = 0;
+}
+
 // ---------------------------------------------------------------- host side ---------------------
 bool umma_supported(const seq_tree_attention_params& p) {
   if (p.dtype != SEQ_F16 && p.dtype != SEQ_BF16) return false;
@@ -1232,7 +1239,20 @@ int launch_attention_umma(const seq_tree_attention_params& p, int splits, cudaSt
     a.ws_count = reinterpret_cast<int32_t*>(ws);
     a.ws_ml = reinterpret_cast<float2*>(ws + cnt_bytes);
     a.ws_o = reinterpret_cast<float4*>(ws + cnt_bytes + stream_ml_bytes());
-    SEQ_CUDA_OK(cudaMemsetAsync(a.ws_count, 0, cnt_bytes, stream));  // the counters start at zero (the kernel leaves them at zero)
+    // The counters start at zero.  A kernel of one's own, not a memset: it is scheduled under the tail of the launch before
+    // and lets the attention's set-up run under itself (768 nodes on 4096 keys of 64/8 heads 123.1 -> 120.8 us, 384 on 2048
+    // of 52 heads 43.1 -> 40.9).
+    cudaLaunchConfig_t zero = {};
+    const int words = (int)(cnt_bytes / sizeof(int32_t));
+    zero.gridDim = dim3((words + 255) / 256);
+    zero.blockDim = dim3(256);
+    zero.stream = stream;
+    cudaLaunchAttribute early[1];
+    early[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    early[0].val.programmaticStreamSerializationAllowed = 1;
+    zero.attrs = early;
+    zero.numAttrs = 1;
+    SEQ_CUDA_OK(cudaLaunchKernelEx(&zero, zero_words_kernel, a.ws_count, words));
   }
 
   const size_t smem = kUmmaSmemBytes;
