@@ -20,9 +20,9 @@
 // marks all the same.  The per-warp partial sums of the last pass are the coarse level of the final inverse CDF,
 // which the one warp that holds the crossing finishes on its own.
 //
-// Serves the default mode and the variant without the draft update at T > 0, and - with a kernel of its own at the
-// end of this file - greedy decoding (T = 0, every mode); sampling from the target at T > 0, the every-node hook and
-// batches run on the kernels of tree_verify.cu.
+// Serves the default mode and the variant without the draft update at T > 0, and - with kernels of their own at the end of
+// this file - greedy decoding (T = 0, every mode) and sampling from the target (T > 0, fp32 logits); the every-node hook and
+// what does not fit the registers run on the kernels of tree_verify.cu.
 #include <cooperative_groups.h>
 #include <float.h>
 #include <limits.h>
@@ -54,6 +54,8 @@ struct Shared {
   int32_t chunk_cnt[32];              // children among nodes [32 j, 32 j + 32)
   float4 xbuf[2][kCl * kWarps];             // cluster exchange: one entry per (rank, warp), double-buffered
   uint64_t xbar[2];                   // ... and the mbarrier that counts each buffer's bytes in
+  float4 drawn[2];                    // sampling walk: the drawn token, from the warp that found it; used in turn
+  uint64_t dbar[2];
   int32_t node_flags;
   int32_t pick[2][4];                 // greedy walk, by hop parity: the matching child, the first child with a bad token, the first child
 };
@@ -208,10 +210,32 @@ __device__ __forceinline__ float exponentials(float* x, float m, float c2) {
 template <int CL>
 struct Exch { float4 e[CL * kWarps / 32]; };
 constexpr uint32_t kSpinLimit = 1u << 22;
+__device__ __forceinline__ void bar_arm(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
 template <int CL>
 __device__ __forceinline__ void exchange_arm(const Ctx& c, int buf) {  // by one thread: the bytes of one exchange
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
-               ::"r"(c.local + (uint32_t)offsetof(Shared, xbar) + 8u * buf), "r"((uint32_t)(CL * kWarps * sizeof(float4))) : "memory");
+  bar_arm(c.local + (uint32_t)offsetof(Shared, xbar) + 8u * buf, (uint32_t)(CL * kWarps * sizeof(float4)));
+}
+__device__ __forceinline__ void send4(uint32_t to, uint32_t bar, float4 v) {  // both in the receiver
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
+               ::"r"(to), "r"(__float_as_uint(v.x)), "r"(__float_as_uint(v.y)), "r"(__float_as_uint(v.z)), "r"(__float_as_uint(v.w)), "r"(bar) : "memory");
+}
+// False when the bounded wait ran out (the same for the whole warp, after SEQ_DEV_TIMEOUT and a pause that lets the stores
+// on their way to and from this CTA land): the warp leaves the kernel.
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, int32_t* dev_status) {
+  uint32_t done = 0;
+#pragma unroll 1
+  for (uint32_t it = 0; it < kSpinLimit && !done; ++it) {
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+    done = __all_sync(0xffffffffu, done);
+  }
+  if (!done) {
+    dev_flag(dev_status, SEQ_DEV_TIMEOUT);
+    for (int it = 0; it < 1000; ++it) __nanosleep(1000);
+  }
+  return done;
 }
 // Before anything else: the mbarriers, and this CTA's arrival at the one cluster barrier.  exchange_ready() waits for it:
 // from there on every CTA is resident and its mbarriers count.
@@ -224,10 +248,13 @@ __device__ __forceinline__ void exchange_init(Ctx& c) {
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(c.local + (uint32_t)offsetof(Shared, xbar) + 8u * b) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(c.local + (uint32_t)offsetof(Shared, dbar) + 8u * b) : "memory");
     }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     exchange_arm<CL>(c, 0);
     exchange_arm<CL>(c, 1);
+#pragma unroll
+    for (int b = 0; b < 2; ++b) bar_arm(c.local + (uint32_t)offsetof(Shared, dbar) + 8u * b, sizeof(float4));
   }
   __syncwarp();
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
@@ -238,30 +265,14 @@ template <int CL>
 __device__ __forceinline__ void exchange_push(const Ctx& c, float4 mine) {
   const uint32_t buf = c.xn & 1u;
   if (c.lane < CL) {
-    const uint32_t to = c.remote + (uint32_t)offsetof(Shared, xbuf) + (buf * (kCl * kWarps) + c.rank * kWarps + c.warp) * (uint32_t)sizeof(float4);
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];"
-                 ::"r"(to), "r"(__float_as_uint(mine.x)), "r"(__float_as_uint(mine.y)), "r"(__float_as_uint(mine.z)), "r"(__float_as_uint(mine.w)),
-                   "r"(c.remote + (uint32_t)offsetof(Shared, xbar) + 8u * buf) : "memory");
+    send4(c.remote + (uint32_t)offsetof(Shared, xbuf) + (buf * (kCl * kWarps) + c.rank * kWarps + c.warp) * (uint32_t)sizeof(float4),
+          c.remote + (uint32_t)offsetof(Shared, xbar) + 8u * buf, mine);
   }
 }
-// False when the bounded wait ran out (the same for the whole warp, after SEQ_DEV_TIMEOUT and a pause that lets the stores
-// on their way to and from this CTA land): the warp leaves the kernel.
 template <int CL>
-__device__ __forceinline__ bool exchange_pull(Ctx& c, Exch<CL>& x, int32_t* dev_status) {
-  const uint32_t buf = c.xn & 1u, parity = (c.xn >> 1) & 1u;
-  const uint32_t bar = c.local + (uint32_t)offsetof(Shared, xbar) + 8u * buf;
-  uint32_t done = 0;
-#pragma unroll 1
-  for (uint32_t it = 0; it < kSpinLimit && !done; ++it) {
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
-    done = __all_sync(0xffffffffu, done);
-  }
-  if (!done) {
-    dev_flag(dev_status, SEQ_DEV_TIMEOUT);
-    for (int it = 0; it < 1000; ++it) __nanosleep(1000);
-    return false;
-  }
+__device__ __forceinline__ bool exchange_pull(Ctx& c, Exch<CL>& x, int32_t* dev_status) {  // false: see bar_wait
+  const uint32_t buf = c.xn & 1u;
+  if (!bar_wait(c.local + (uint32_t)offsetof(Shared, xbar) + 8u * buf, (c.xn >> 1) & 1u, dev_status)) return false;
   if (c.tid == 0) exchange_arm<CL>(c, (int)buf);  // for the exchange after the next
 #pragma unroll
   for (int m = 0; m < CL * kWarps / 32; ++m) x.e[m] = c.sh->xbuf[buf][c.lane + 32 * m];
@@ -283,6 +294,90 @@ __device__ __forceinline__ VerifyArgs request_args(const VerifyArgs& in) {
     if (in.next_child_out != nullptr) a.next_child_out += r * in.tree_stride;
   }
   return a;
+}
+
+// The draw by inverse CDF, coarse level, every warp for itself: an inclusive scan over the (rank, warp) masses, 32 at a time.
+// Returns the segment that holds the crossing (-1: no mass anywhere) and the target inside it; take_last: rounding left the
+// total at or below the target, the last segment with mass is returned and its last element with mass is the one.
+template <int CL>
+__device__ __forceinline__ int draw_segment(const Ctx& c, const float* part_sum, float u, double& total_mass, double& tl, bool& take_last) {
+  constexpr int kPPL = CL * kWarps / 32;
+  double inc[kPPL], before = 0.0;
+#pragma unroll
+  for (int m = 0; m < kPPL; ++m) {
+    double v = (double)part_sum[m];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double up = __shfl_up_sync(0xffffffffu, v, o);
+      if (c.lane >= o) v += up;
+    }
+    inc[m] = v + before;
+    before = __shfl_sync(0xffffffffu, inc[m], 31);
+  }
+  total_mass = before;
+  const double tgt = (double)u * total_mass;
+  int part = -1;
+  take_last = false;
+#pragma unroll
+  for (int m = 0; m < kPPL; ++m) {
+    const uint32_t hit = __ballot_sync(0xffffffffu, part_sum[m] > 0.f && inc[m] > tgt);
+    if (part < 0 && hit) part = 32 * m + __ffs(hit) - 1;
+  }
+  if (part < 0) {
+    take_last = true;
+#pragma unroll
+    for (int m = kPPL - 1; m >= 0; --m) {
+      const uint32_t pos = __ballot_sync(0xffffffffu, part_sum[m] > 0.f);
+      if (part < 0 && pos) part = 32 * m + 31 - __clz(pos);
+    }
+  }
+  tl = 0.0;
+  if (part == c.rank * kWarps + c.warp) {
+#pragma unroll
+    for (int m = 0; m < kPPL; ++m) {
+      const double i_m = __shfl_sync(0xffffffffu, inc[m], part & 31), s_m = (double)__shfl_sync(0xffffffffu, part_sum[m], part & 31);
+      if ((part >> 5) == m) tl = tgt - (i_m - s_m);
+    }
+  }
+  return part;
+}
+// ... fine level, by the one warp whose segment holds the crossing.  The segment's values go to shared memory in vocabulary
+// order (one padding word per 32, so that the reads do not collide); lane l then owns elements [4 NCH l, + 4 NCH): the lanes'
+// sums are scanned, and the lane that holds the crossing walks its elements and returns the token (the others -1).  Rolled
+// loops: this runs in one warp.
+template <int NCH>
+__device__ __forceinline__ int draw_in_segment(const Ctx& c, const float* p, float* seg, double tl, bool take_last) {
+  constexpr int kE = 4 * NCH, kSpan = 32 * kE;
+#pragma unroll
+  for (int e = 0; e < kE; ++e) {
+    const int idx = (e >> 2) * 128 + c.lane * 4 + (e & 3);
+    seg[idx + (idx >> 5)] = p[e];
+  }
+  __syncwarp();
+  const int mine0 = kE * c.lane;  // this lane's first element of the segment
+  float ls = 0.f;
+#pragma unroll 4
+  for (int k = 0; k < kE; ++k) { const int idx = mine0 + k; ls += seg[idx + (idx >> 5)]; }
+  double incl = (double)ls;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double up = __shfl_up_sync(0xffffffffu, incl, o);
+    if (c.lane >= o) incl += up;
+  }
+  const uint32_t cross = take_last ? 0u : __ballot_sync(0xffffffffu, ls > 0.f && incl > tl);
+  const uint32_t mass = __ballot_sync(0xffffffffu, ls > 0.f);
+  if (mass == 0u) return c.lane == 0 ? c.lo + c.warp * kSpan : -1;  // (a segment said to have mass has none: its first token)
+  if (c.lane != (cross ? __ffs(cross) - 1 : 31 - __clz(mass))) return -1;
+  double r = incl - (double)ls;
+  int pick = -1, last_k = 0;
+#pragma unroll 1
+  for (int k = 0; k < kE && pick < 0; ++k) {
+    const int idx = mine0 + k;
+    const float v = seg[idx + (idx >> 5)];
+    r += (double)v;
+    if (v > 0.f) { last_k = k; if (cross && r > tl) pick = k; }
+  }
+  return c.lo + c.warp * kSpan + mine0 + (pick < 0 ? last_k : pick);  // nothing crosses: the last element with mass
 }
 
 // (The batch's instances up to 32768 tokens keep to 128 registers: two requests' CTAs share an SM, 64 requests of 32000
@@ -589,35 +684,9 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
 #pragma unroll
       for (int e = 0; e < kE; ++e) p[e] = resid(p[e], use_q ? q[e] : 0.f, Cf, Uf);  // the residual replaces p
       const float u = sh->uniforms[a.n];
-      // coarse level, every warp for itself: inclusive scan over the (rank, warp) masses, 32 at a time
-      double inc[kPPL], before = 0.0;
-#pragma unroll
-      for (int m = 0; m < kPPL; ++m) {
-        double v = (double)part_sum[m];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const double up = __shfl_up_sync(0xffffffffu, v, o);
-          if (c.lane >= o) v += up;
-        }
-        inc[m] = v + before;
-        before = __shfl_sync(0xffffffffu, inc[m], 31);
-      }
-      const double total_mass = before, tgt = (double)u * total_mass;
-      int part = -1;
-      bool take_last = false;
-#pragma unroll
-      for (int m = 0; m < kPPL; ++m) {
-        const uint32_t hit = __ballot_sync(0xffffffffu, part_sum[m] > 0.f && inc[m] > tgt);
-        if (part < 0 && hit) part = 32 * m + __ffs(hit) - 1;
-      }
-      if (part < 0) {  // rounding left the total at or below the target: the last segment with mass
-        take_last = true;
-#pragma unroll
-        for (int m = kPPL - 1; m >= 0; --m) {
-          const uint32_t pos = __ballot_sync(0xffffffffu, part_sum[m] > 0.f);
-          if (part < 0 && pos) part = 32 * m + 31 - __clz(pos);
-        }
-      }
+      double total_mass, tl;
+      bool take_last;
+      const int part = draw_segment<CL>(c, part_sum, u, total_mass, tl, take_last);
       if (a.residual_out != nullptr) {
         const float inv = total_mass > 0.0 ? (float)fast_rcp(total_mass) : 0.f;
 #pragma unroll
@@ -629,51 +698,7 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
       if (part < 0) {
         if (leader) { dev_flag(a.dev_status, SEQ_DEV_DEGENERATE); bonus_found = 0; }  // no mass anywhere: token 0
       } else if (part == c.rank * kWarps + c.warp) {
-        // fine level, the one warp whose segment holds the crossing
-        double incl_part = 0.0, mass_part = 0.0;
-#pragma unroll
-        for (int m = 0; m < kPPL; ++m) {
-          const double i_m = __shfl_sync(0xffffffffu, inc[m], part & 31), s_m = (double)__shfl_sync(0xffffffffu, part_sum[m], part & 31);
-          if ((part >> 5) == m) { incl_part = i_m; mass_part = s_m; }
-        }
-        const double tl = tgt - (incl_part - mass_part);  // the target inside this segment
-        // The segment's residual values go to shared memory in vocabulary order (one padding word per 32, so that
-        // the reads below do not collide); lane l then owns elements [NCH*4*l, +NCH*4): the lanes' sums are scanned,
-        // and the lane that holds the crossing walks its elements.  Rolled loops: this runs in one warp.
-        float* seg = reinterpret_cast<float*>(sh->kid[np ^ 1]);
-#pragma unroll
-        for (int e = 0; e < kE; ++e) {
-          const int idx = (e >> 2) * 128 + c.lane * 4 + (e & 3);
-          seg[idx + (idx >> 5)] = p[e];
-        }
-        __syncwarp();
-        const int mine0 = kE * c.lane;  // this lane's first element of the segment
-        float ls = 0.f;
-#pragma unroll 4
-        for (int k = 0; k < kE; ++k) { const int idx = mine0 + k; ls += seg[idx + (idx >> 5)]; }
-        double incl = (double)ls;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const double up = __shfl_up_sync(0xffffffffu, incl, o);
-          if (c.lane >= o) incl += up;
-        }
-        const uint32_t cross = take_last ? 0u : __ballot_sync(0xffffffffu, ls > 0.f && incl > tl);
-        const uint32_t mass = __ballot_sync(0xffffffffu, ls > 0.f);
-        if (mass == 0u) {
-          if (c.lane == 0) bonus_found = c.lo + c.warp * kSpan;  // (a segment said to have mass has none: its first token)
-        } else if (c.lane == (cross ? __ffs(cross) - 1 : 31 - __clz(mass))) {
-          double r = incl - (double)ls;
-          int pick = -1, last_k = 0;
-#pragma unroll 1
-          for (int k = 0; k < kE && pick < 0; ++k) {
-            const int idx = mine0 + k;
-            const float v = seg[idx + (idx >> 5)];
-            r += (double)v;
-            if (v > 0.f) { last_k = k; if (cross && r > tl) pick = k; }
-          }
-          if (pick < 0) pick = last_k;  // nothing crosses (rounding, or by design): the last element with mass
-          bonus_found = c.lo + c.warp * kSpan + mine0 + pick;
-        }
+        bonus_found = draw_in_segment<NCH>(c, p, reinterpret_cast<float*>(sh->kid[np ^ 1]), tl, take_last);
       }
     }
     break;
@@ -824,13 +849,161 @@ __global__ void __launch_bounds__(kTh, 1) tree_verify_greedy_kernel(const Verify
   if (leader) { *a.path_len = plen; *a.bonus = g; }
 }
 
+// ---------------------------------------------------------------- sampling from the target ----------------------
+// SEQ_VERIFY_TARGET_SAMPLE at T > 0: a token is drawn from softmax(target / T) at each node with the node's uniform, and the
+// first child that carries it is taken.  Per visited node the target row in registers (its exponentials, one exchange), the
+// draw as above, and a second exchange of one entry: the warp that found the token tells every CTA.  As in the greedy walk the
+// first child's row is requested while the first exchange is on its way.
+// Bound by the chain of a node's steps, like the walk above.  Against the shared-memory walk: 768 nodes x 128256 tokens 16.0
+// -> 6.7 us, 64 x 32000 9.8 -> 4.2, 16 requests of 64 x 32000 12.9 -> 6.2.
+template <int NCH, int CL>
+__global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_verify_sample_kernel(const VerifyArgs a_in) {
+  const VerifyArgs a = request_args<CL>(a_in);
+  constexpr int kPPL = CL * kWarps / 32, kE = 4 * NCH, kSpan = 32 * kE;
+  const char* const tbase = reinterpret_cast<const char*>(a.target);
+  extern __shared__ __align__(16) uint8_t dyn_smem[];
+  Shared* sh = reinterpret_cast<Shared*>(dyn_smem);
+  Ctx c;
+  c.sh = sh;
+  c.rank = (int)cg::this_cluster().block_rank();
+  c.lo = min(c.rank * a.slice_cap, a.V);
+  c.cnt = min(a.V - c.lo, a.slice_cap);
+  c.tid = threadIdx.x; c.warp = threadIdx.x >> 5; c.lane = threadIdx.x & 31;
+  exchange_init<CL>(c);
+  const float c2 = kLog2e / a.temperature;
+  const bool leader = c.rank == 0 && c.tid == 0;
+  if (c.tid == 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  RawRow<NCH, false> pn;
+  {
+    int tp[4], tt[4];
+    float tu[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int i = c.tid + kTh * k;
+      tp[k] = i < a.n ? a.parent[i] : -1;
+      tt[k] = i < a.n ? a.tokens[i] : 0;
+      tu[k] = i < a.n ? a.uniforms[i] : 0.f;
+    }
+    load_row<NCH, false>(c, tbase, pn);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int i = c.tid + kTh * k;
+      if (i < a.n) {
+        int pp = tp[k];
+        if (i == 0) pp = -1;
+        else if (pp < -1 || pp >= i) { if (c.rank == 0) dev_flag(a.dev_status, SEQ_DEV_BAD_PARENT); pp = -1; }
+        sh->parent[i] = pp;
+        sh->tokens[i] = tt[k];
+        sh->uniforms[i] = tu[k];
+      }
+    }
+    if (c.rank == 0 && a.next_child_out != nullptr)
+      for (int i = c.tid; i < a.n; i += kTh) a.next_child_out[i] = -2;  // nodes the walk does not visit
+  }
+  __syncthreads();  // the tree is in place
+  exchange_ready();
+
+  int cur = 0, plen = 0, token = 0;
+  uint32_t dn = 0;  // tokens told
+  float p[kE];
+#pragma unroll 1
+  for (int hop = 0; hop < a.n; ++hop) {  // a walk visits at most n nodes
+    if (leader) a.path[plen] = cur;
+    ++plen;
+    int32_t* pick = sh->pick[hop & 1];
+    if (c.tid < 3) pick[c.tid] = 0x7fffffff;  // (the other set is the one the previous hop may still be reading)
+    widen<NCH, false>(pn, p);
+    bool bad = false;
+    const float mp = clean_and_max<NCH>(p, bad);
+    const float sp = exponentials<NCH>(p, mp, c2);
+    if (bad) dev_flag(a.dev_status, SEQ_DEV_NONFINITE);
+    const float Mwp = max_lanes(mp);
+    exchange_push<CL>(c, make_float4(Mwp, warp_sum(sp * rel_exp(mp, Mwp, c2)), 0.f, 0.f));
+    // ---- while the entries travel: the node's first child, and its row on the way
+    __syncthreads();  // pick[] is reset
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int i = c.tid + kTh * k;
+      if (i < a.n && sh->parent[i] == cur) atomicMin(&pick[2], i);
+    }
+    __syncthreads();
+    const int first_kid = pick[2];
+    if (first_kid != 0x7fffffff) load_row<NCH, false>(c, tbase + (int64_t)first_kid * a.target_stride * 4, pn);
+    Exch<CL> x;
+    if (!exchange_pull<CL>(c, x, a.dev_status)) return;
+    float Mp = -INFINITY;
+#pragma unroll
+    for (int m = 0; m < kPPL; ++m) Mp = fmaxf(Mp, x.e[m].x);
+    Mp = max_lanes(Mp);
+    float part_sum[kPPL], asum = 0.f;
+#pragma unroll
+    for (int m = 0; m < kPPL; ++m) {
+      part_sum[m] = x.e[m].y * rel_exp(x.e[m].x, Mp, c2);
+      asum += part_sum[m];
+    }
+    const float Sp = warp_sum(asum);
+    const float invSp = Sp > 0.f ? __frcp_rn(Sp) : 0.f;
+#pragma unroll
+    for (int m = 0; m < kPPL; ++m) part_sum[m] *= invSp;
+    const float fp = rel_exp(mp, Mp, c2) * invSp;
+#pragma unroll
+    for (int e = 0; e < kE; ++e) p[e] *= fp;
+    double total_mass, tl;
+    bool take_last;
+    const int part = draw_segment<CL>(c, part_sum, sh->uniforms[cur], total_mass, tl, take_last);
+    token = 0;
+    if (part < 0) {
+      dev_flag(a.dev_status, SEQ_DEV_DEGENERATE);  // a target row without mass: token 0
+    } else {
+      const uint32_t buf = dn & 1u, bar = (uint32_t)offsetof(Shared, dbar) + 8u * buf;
+      if (part == c.rank * kWarps + c.warp) {
+        const int mine = draw_in_segment<NCH>(c, p, reinterpret_cast<float*>(sh->kid[hop & 1]), tl, take_last);
+        const int found = __reduce_max_sync(0xffffffffu, mine);
+        if (c.lane < CL) send4(c.remote + (uint32_t)offsetof(Shared, drawn) + 16u * buf, c.remote + bar, make_float4(__int_as_float(found), 0.f, 0.f, 0.f));
+      }
+      if (!bar_wait(c.local + bar, (dn >> 1) & 1u, a.dev_status)) return;
+      if (c.tid == 0) bar_arm(c.local + bar, sizeof(float4));
+      token = __float_as_int(sh->drawn[buf].x);
+      ++dn;
+    }
+    // ---- the first child that carries the token; one with a token outside the vocabulary is reported if it comes before
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int i = c.tid + kTh * k;
+      if (i < a.n && sh->parent[i] == cur) {
+        const int s = sh->tokens[i];
+        if (s < 0 || s >= a.V) atomicMin(&pick[1], i);
+        else if (s == token) atomicMin(&pick[0], i);
+      }
+    }
+    __syncthreads();
+    const int match = pick[0];
+    if (leader) {
+      if (pick[1] < match) dev_flag(a.dev_status, SEQ_DEV_BAD_TOKEN);
+      if (a.next_child_out != nullptr) a.next_child_out[cur] = match == 0x7fffffff ? -1 : match;
+    }
+    if (match == 0x7fffffff) break;
+    if (match != first_kid) load_row<NCH, false>(c, tbase + (int64_t)match * a.target_stride * 4, pn);
+    cur = match;
+  }
+  if (a.residual_out != nullptr) {  // the distribution that the last token came from
+#pragma unroll
+    for (int e = 0; e < kE; ++e) {
+      const int local = c.warp * kSpan + (e >> 2) * 128 + c.lane * 4 + (e & 3);
+      if (local < c.cnt) a.residual_out[c.lo + local] = p[e];
+    }
+  }
+  if (leader) { *a.path_len = plen; *a.bonus = token; }
+}
+
 }  // namespace vwk
 
 // Elements a cluster of this kernel holds per row: 16 CTAs x 256 threads x 4 NCH.
 bool verify_walk_supported(int vocab, int flags, float temperature) {
   if (flags & SEQ_VERIFY_ALL_NODES) return false;
   if (temperature == 0.f) return vocab >= 1 && (size_t)vocab <= (size_t)vwk::kCl * vwk::kTh * 4 * 8;  // greedy: its own kernel, whatever the mode flags say
-  if (flags & SEQ_VERIFY_TARGET_SAMPLE) return false;
   if (!(temperature > 0.f)) return false;
   return vocab >= 1 && (size_t)vocab <= (size_t)vwk::kCl * vwk::kTh * 4 * 8;
 }
@@ -842,6 +1015,11 @@ static WalkKernel walk_kernel(int nch, bool bf16) {
               : (nch == 2 ? vwk::tree_verify_walk_kernel<2, false, CL> : nch == 4 ? vwk::tree_verify_walk_kernel<4, false, CL> : vwk::tree_verify_walk_kernel<8, false, CL>);
 }
 
+template <int CL>
+static WalkKernel sample_kernel(int nch) {
+  return nch == 2 ? vwk::tree_verify_sample_kernel<2, CL> : nch == 4 ? vwk::tree_verify_sample_kernel<4, CL> : vwk::tree_verify_sample_kernel<8, CL>;
+}
+
 // cl: CTAs per request, 16 or (T > 0 and a vocabulary that 8 CTAs hold) 8.  With `clusters` given nothing is launched: the
 // number of clusters that the device runs side by side is written there.
 static int walk_launch(const VerifyArgs& a_in, int cl, int requests, int* clusters, cudaStream_t stream) {
@@ -849,13 +1027,14 @@ static int walk_launch(const VerifyArgs& a_in, int cl, int requests, int* cluste
   a.slice_cap = (((a.V + cl - 1) / cl) + 3) & ~3;
   const int nch = a.slice_cap <= vwk::kTh * 4 * 2 ? 2 : a.slice_cap <= vwk::kTh * 4 * 4 ? 4 : 8;
   const bool bf16 = (a.flags & SEQ_VERIFY_LOGITS_BF16) != 0;
-  const bool greedy = a.temperature == 0.f;
+  const bool greedy = a.temperature == 0.f, sample = !greedy && (a.flags & SEQ_VERIFY_TARGET_SAMPLE) != 0;
   const WalkKernel kernel =
       greedy ? (bf16 ? (nch == 2 ? vwk::tree_verify_greedy_kernel<2, true> : nch == 4 ? vwk::tree_verify_greedy_kernel<4, true> : vwk::tree_verify_greedy_kernel<8, true>)
                      : (nch == 2 ? vwk::tree_verify_greedy_kernel<2, false> : nch == 4 ? vwk::tree_verify_greedy_kernel<4, false> : vwk::tree_verify_greedy_kernel<8, false>))
+      : sample ? (cl == 16 ? sample_kernel<vwk::kCl>(nch) : sample_kernel<vwk::kClBatch>(nch))
       : cl == 16 ? walk_kernel<vwk::kCl>(nch, bf16) : walk_kernel<vwk::kClBatch>(nch, bf16);
-  const int slot = (nch == 2 ? 0 : nch == 4 ? 1 : 2) + (bf16 ? 3 : 0) + (greedy ? 6 : cl == 16 ? 0 : 12);
-  static int attr_done[18][64];
+  const int slot = (nch == 2 ? 0 : nch == 4 ? 1 : 2) + (sample ? (cl == 16 ? 18 : 21) : (bf16 ? 3 : 0) + (greedy ? 6 : cl == 16 ? 0 : 12));
+  static int attr_done[24][64];
   const int rc = once_per_device(attr_done[slot], [&]() -> int {
     SEQ_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(vwk::Shared)));
     SEQ_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
@@ -891,14 +1070,17 @@ int launch_verify_walk(const VerifyArgs& a, cudaStream_t stream) { return walk_l
 // 26); more of them, as clusters of 8 with rows of up to 65536 tokens in registers, win at any size (10 / 16 / 32 / 64
 // requests of 32000 tokens: 22 / 21 / 22 / 42 us against 31 / 29 / 28 / 57; of 50257: 24 / 30 / 46 / 72 against 43 / 51 / 54
 // / 86).  Larger vocabularies need 16 CTAs and are served in turns: 10 / 32 requests of 128256 tokens 29 / 68 us against 41
-// / 71, 48 requests 99 against 92.  Greedy walks keep 16 CTAs (64 requests of 32000 tokens: 27 us against 33).
+// / 71, 48 requests 99 against 92.  Greedy walks keep 16 CTAs (64 requests of 32000 tokens: 27 us against 33).  Sampling
+// from the target, with half the bytes per node, is the better one at every size (87 requests of 128256 tokens 68 us
+// against 104, 64 of 50257 27 against 37).
 static int walk_batch_cluster(const VerifyArgs& a, int requests) {
   if (a.temperature == 0.f) return vwk::kCl;
-  if (a.V > vwk::kClBatch * vwk::kTh * 32) return requests * vwk::kCl <= 4 * device_sm_count() ? vwk::kCl : 0;
+  const bool sample = (a.flags & SEQ_VERIFY_TARGET_SAMPLE) != 0;
+  if (a.V > vwk::kClBatch * vwk::kTh * 32) return sample || requests * vwk::kCl <= 4 * device_sm_count() ? vwk::kCl : 0;
   if (requests * vwk::kCl > device_sm_count()) return vwk::kClBatch;
-  static int side_by_side[6][64];  // per kernel shape and device: clusters of 16, + 1; 0 = not asked yet
+  static int side_by_side[9][64];  // per kernel shape and device: clusters of 16, + 1; 0 = not asked yet
   const int slice = (((a.V + vwk::kCl - 1) / vwk::kCl) + 3) & ~3;
-  const int shape = (slice <= vwk::kTh * 8 ? 0 : slice <= vwk::kTh * 16 ? 1 : 2) + ((a.flags & SEQ_VERIFY_LOGITS_BF16) ? 3 : 0);
+  const int shape = (slice <= vwk::kTh * 8 ? 0 : slice <= vwk::kTh * 16 ? 1 : 2) + (sample ? 6 : (a.flags & SEQ_VERIFY_LOGITS_BF16) ? 3 : 0);
   int dev = 0, n = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return vwk::kCl;
   if (dev >= 0 && dev < 64) n = __atomic_load_n(&side_by_side[shape][dev], __ATOMIC_ACQUIRE);
