@@ -386,22 +386,23 @@ def seq_tree_verify_batch(parent, tokens, target_logits, draft_logits, temperatu
     """R requests in one launch.  parent, tokens [R, n]; target_logits, draft_logits [R, n, V]; uniforms [R, n+1];
     residual_out [R, V] and next_child_out [R, n] optional.  Returns path [R, n], path_len [R], bonus_token [R]."""
     R, n, V = target_logits.shape
-    dev = target_logits.device
-    for t, nm in ((parent, "parent"), (tokens, "tokens"), (uniforms, "uniforms"), (target_logits, "target_logits"),
-                  (draft_logits, "draft_logits"), (residual_out, "residual_out"), (next_child_out, "next_child_out")):
-        if t is not None and (t.shape[0] != R or t.stride(-1) != 1):
-            raise ValueError(f"{nm}: one entry per request, innermost dimension contiguous")
+    for t in (parent, tokens, uniforms, target_logits, draft_logits, residual_out, next_child_out):
+        if t is not None and (t.shape[0] != R or t.stride()[-1] != 1):
+            raise ValueError("one entry per request, innermost dimension contiguous: all of parent, tokens, uniforms, "
+                             "target_logits, draft_logits, residual_out, next_child_out")
     request, row, _ = target_logits.stride()
     draft_request, draft_row, _ = draft_logits.stride() if draft_logits is not None else (request, 0, 1)
     if draft_request != request:
         raise ValueError("target_logits and draft_logits must have the same stride between requests")
-    if parent.stride(0) != tokens.stride(0) or parent.stride(0) != n or (next_child_out is not None and next_child_out.stride(0) != n):
+    if tokens.stride(0) != n or parent.stride(0) != n or (next_child_out is not None and next_child_out.stride(0) != n):
         raise ValueError("parent, tokens and next_child_out must be [R, n] contiguous")
     ldt = target_logits.dtype
     if ldt is not torch.float32 and ldt is not torch.bfloat16:
         raise ValueError("target_logits must be float32 or bfloat16")
-    path = torch.empty((R, n), dtype=torch.int32, device=dev)
-    path_len, bonus = torch.empty((2, R), dtype=torch.int32, device=dev).unbind(0)  # (every launch writes both)
+    # (parent is [R, n] contiguous and, by the check below, int32 on the device; three allocations in its image take half
+    # the time of torch.empty and views)
+    path = torch.empty_like(parent)
+    path_len, bonus = parent.new_empty((R,)), parent.new_empty((R,))
     flags = ((SEQ_VERIFY_SPECINFER if specinfer else 0) | (SEQ_VERIFY_TARGET_SAMPLE if target_sample else 0) |
              (SEQ_VERIFY_LOGITS_BF16 if ldt is torch.bfloat16 else 0))
     p = VerifyBatchParams(
