@@ -98,7 +98,9 @@ int seq_tree_mask_from_parents(const int32_t* parent, int32_t n, uint32_t* mask_
  * over j in [0, prefix_len)  and  j = prefix_len + a for every a whose bit is
  * set in row i of mask_bits.  Scores, softmax and accumulation are fp32; with
  * 16-bit inputs the probabilities are rounded to the input type before the
- * P.V product on the tensor-core path.
+ * P.V product on the tensor-core path, except for groups of query heads that
+ * do not divide 128: there what the rounding leaves enters the product too,
+ * as a second value of the input type.
  *
  * Layouts (strides in ELEMENTS, innermost head_dim contiguous):
  *   q, out        element (i,h,c) at i*stride_tok + h*stride_head + c

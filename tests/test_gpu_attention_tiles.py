@@ -29,6 +29,21 @@ def test_groups_that_do_not_divide_the_tile(hkv, group, n, L, kernel):
     G.check_attention(_inputs(hkv, group, n, L, "bf16"), kernel=kernel)
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "fp16"])
+@pytest.mark.parametrize("kernel", [B.KERNEL_AUTO, B.KERNEL_TENSOR_CORE_STREAM, B.KERNEL_TENSOR_CORE_GRID])
+@pytest.mark.parametrize("hkv,group,n,L", [(2, 5, 30, 700), (1, 3, 50, 150), (1, 12, 25, 63), (1, 100, 3, 1200)])
+def test_probabilities_are_not_rounded_once_for_groups_that_do_not_divide_the_tile(hkv, group, n, L, dtype, kernel):
+    """The output is no further from fp64 than its own rounding puts it.  P as two pieces is off by 2^-17 at most (bfloat16;
+    half 2^-22), far below the output's 2^-9 (2^-12): 2 % of margin covers it.  P rounded once is off by as much as the
+    output is, independently: 25 to 40 % more."""
+    ai = _inputs(hkv, group, n, L, dtype)
+    out, _, status = G.run_attention(ai, kernel)
+    ref, _, _ = O.tree_attention(ai.q, ai.k_cache, ai.v_cache, ai.parent, L)
+    rounded = torch.from_numpy(ref).to(ai.q.dtype).double().numpy()
+    assert status == 0
+    assert np.linalg.norm(out.double().cpu().numpy() - ref) < 1.02 * np.linalg.norm(rounded - ref)
+
+
 @pytest.mark.parametrize("hkv,n,L", [(60, 2, 1250), (40, 3, 1100), (32, 2, 1030), (24, 3, 1590), (16, 4, 3000), (1, 5, 2200), (1, 4, 4000)])
 def test_clusters_of_every_size(hkv, n, L):
     """Where the device runs 74, 44, 36, 28, 21, 14 and 14 clusters of 2 to 8 CTAs side by side, these take one size each."""
