@@ -399,10 +399,9 @@ def seq_tree_verify_batch(parent, tokens, target_logits, draft_logits, temperatu
     ldt = target_logits.dtype
     if ldt is not torch.float32 and ldt is not torch.bfloat16:
         raise ValueError("target_logits must be float32 or bfloat16")
-    # (parent is [R, n] contiguous and, by the check below, int32 on the device; three allocations in its image take half
-    # the time of torch.empty and views)
-    path = torch.empty_like(parent)
-    path_len, bonus = parent.new_empty((R,)), parent.new_empty((R,))
+    # (parent is, by the check below, int32 on the device; three allocations of its kind take half the time of torch.empty
+    # and views.  Its own shape says nothing: a view of fewer columns of an [R, n] buffer passes the checks above)
+    path, path_len, bonus = parent.new_empty((R, n)), parent.new_empty((R,)), parent.new_empty((R,))
     flags = ((SEQ_VERIFY_SPECINFER if specinfer else 0) | (SEQ_VERIFY_TARGET_SAMPLE if target_sample else 0) |
              (SEQ_VERIFY_LOGITS_BF16 if ldt is torch.bfloat16 else 0))
     p = VerifyBatchParams(
