@@ -80,8 +80,9 @@ struct DsShared {
 
 // Ranks the first `count` entries of the list against each other - larger score first, then lower token -, leaves the k
 // best in order at its front, their number in sh.count and, once there are k, the last one's score in sh.tau.  Entries
-// without a chance (-inf) drop out.  All threads call it after a barrier behind the last write to the list.
-__device__ __forceinline__ void ds_compact(DsShared& sh, int count, int k) {
+// without a chance (-inf) drop out.  All threads call it after a barrier behind the last write to the list.  The number is
+// also returned: a thread that read sh.count afterwards could find what a warp ahead of it has listed since.
+__device__ __forceinline__ int ds_compact(DsShared& sh, int count, int k) {
   const int tid = threadIdx.x;
   if (count <= kDsThreads / 2) {
     // a short list: two, four or eight threads share an entry's comparisons
@@ -104,7 +105,7 @@ __device__ __forceinline__ void ds_compact(DsShared& sh, int count, int k) {
     }
     if (tid == 0) sh.count = min(total, k);
     __syncthreads();
-    return;
+    return min(total, k);
   }
   float2 mine[kDsList / kDsThreads];
   int rank[kDsList / kDsThreads];
@@ -137,6 +138,7 @@ __device__ __forceinline__ void ds_compact(DsShared& sh, int count, int k) {
     }
   if (tid == 0) sh.count = min(total, k);
   __syncthreads();
+  return min(total, k);
 }
 
 // The bound a token has to pass: the threshold less what the bounds' rounding may cost (31 ulp of place in the first step,
@@ -244,8 +246,7 @@ __global__ void __launch_bounds__(kDsThreads) draft_sample_kernel(const DraftSam
       sh.list[j].x = ds_score(lrow[t], urow[t], a.inv_T, unused);
     }
     __syncthreads();
-    ds_compact(sh, count, a.k);
-    ranked = sh.count;
+    ranked = ds_compact(sh, count, a.k);
     cut = ds_cut(sh.tau);
   };
   for (int t0 = kDsStep, step = 1; t0 < cnt; t0 += kDsStep, ++step) {
@@ -267,11 +268,11 @@ __global__ void __launch_bounds__(kDsThreads) draft_sample_kernel(const DraftSam
       __syncthreads();
       const int count = sh.count;
       __syncthreads();
-      ds_compact(sh, count, a.k);
+      ranked = ds_compact(sh, count, a.k);
     }
   }
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  int have = sh.count;
+  int have = ranked;
   if (a.parts > 1) {
     cg::this_cluster().barrier_wait();  // the first CTA runs: its shared memory may be written
     float2* to = cg::this_cluster().map_shared_rank(sh.cand, 0) + part * a.k;
@@ -309,8 +310,7 @@ __global__ void __launch_bounds__(kDsThreads) draft_sample_kernel(const DraftSam
     __syncthreads();
     const int count = sh.count;
     __syncthreads();
-    ds_compact(sh, count, a.k);
-    have = sh.count;
+    have = ds_compact(sh, count, a.k);
   }
   for (int j = tid; j < a.k; j += kDsThreads) a.out[(int64_t)row * a.k + j] = j < have ? __float_as_int(sh.list[j].y) : -1;
 }

@@ -55,3 +55,25 @@ def test_rows_with_few_tokens_in_the_running(finite):
         assert (got[r] >= 0).sum() == min(k, finite)
         if finite == 0 or ref["min_rel_gap"] >= 1e-4:
             assert got[r].tolist() == ref["tokens"].tolist()
+
+
+@pytest.mark.parametrize("rows,V,k", [(378, 128256, 9), (300, 130000, 64), (9, 131072, 33)])
+def test_rankings_between_steps_keep_every_listed_token(rows, V, k):
+    """Rows of many steps, ranked after the 2nd, 4th, 8th, 16th and 32nd while warps that are ahead list the next step's
+    tokens: the same tokens on every one of twenty calls, and those of a sort in double precision."""
+    d = _dev()
+    g = torch.Generator(device=d)
+    g.manual_seed(k)
+    logits = torch.randn((rows, V), device=d, generator=g) * 3
+    u = torch.rand((rows, V), device=d, generator=g)
+    first = B.seq_tree_draft_sample(logits, 0.6, u, k).clone()
+    for _ in range(19):
+        assert torch.equal(B.seq_tree_draft_sample(logits, 0.6, u, k), first)
+    clear = 0
+    for r in range(rows):
+        score = logits[r].double() / float(np.float32(0.6)) - torch.log(-torch.log(u[r].double()))
+        best = torch.topk(torch.where(u[r] > 0, score, torch.full_like(score, float("-inf"))), k + 1)
+        if (best.values[:-1] - best.values[1:]).min() > 1e-4:
+            clear += 1
+            assert first[r].tolist() == best.indices[:k].tolist(), r
+    assert clear >= rows // 2
