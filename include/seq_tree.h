@@ -273,8 +273,10 @@ enum {
   SEQ_VERIFY_SCHED_NODES = 32,
   /* target_logits and draft_logits hold bfloat16 instead of fp32 (what a 16-bit language-model head writes; half the
    * bytes per visited node).  Every value is widened to fp32 exactly and the arithmetic is unchanged.  Row strides
-   * stay in elements (multiples of 4), rows 8-byte aligned.  One request at T > 0 in the default mode or with
-   * SEQ_VERIFY_SPECINFER, on the walk schedule; anything else returns SEQ_ERR_UNSUPPORTED. */
+   * stay in elements (multiples of 4), rows 8-byte aligned.  Requests alone or in batches of any size, at T = 0 and at
+   * T > 0 in the default mode or with SEQ_VERIFY_SPECINFER, on the walk schedule, vocabularies up to 131072; anything
+   * else (the every-node hook, the node-parallel schedule, sampling from the target at T > 0) returns
+   * SEQ_ERR_UNSUPPORTED. */
   SEQ_VERIFY_LOGITS_BF16 = 8
 };
 

@@ -183,8 +183,8 @@ static int verify_launch(const seq_tree_verify_params* p, int batch, int64_t tre
     if (!fits8 && (!fits16 || batch > 0 || (p->flags & SEQ_VERIFY_ALL_NODES))) return SEQ_ERR_UNSUPPORTED;
   }
 
-  // 16-bit logits: served by the walk with its rows in registers only (default mode and the variant without the draft
-  // update, T > 0, one request, a device that places a cluster of 16)
+  // 16-bit logits: served by the walk with its rows in registers only (T = 0; at T > 0 the default mode and the variant
+  // without the draft update; one request or a batch; a device that places a cluster of 16)
   const bool bf16 = (p->flags & SEQ_VERIFY_LOGITS_BF16) != 0;
   if (bf16 && ((p->flags & SEQ_VERIFY_SCHED_NODES) || ((p->flags & SEQ_VERIFY_TARGET_SAMPLE) && p->temperature > 0.f) || !verify_walk_supported(p->vocab, p->flags, p->temperature)))
     return SEQ_ERR_UNSUPPORTED;

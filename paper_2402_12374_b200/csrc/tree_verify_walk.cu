@@ -1072,15 +1072,16 @@ int launch_verify_walk(const VerifyArgs& a, cudaStream_t stream) { return walk_l
 // / 86).  Larger vocabularies need 16 CTAs and are served in turns: 10 / 32 requests of 128256 tokens 29 / 68 us against 41
 // / 71, 48 requests 99 against 92.  Greedy walks keep 16 CTAs (64 requests of 32000 tokens: 27 us against 33).  Sampling
 // from the target, with half the bytes per node, is the better one at every size (87 requests of 128256 tokens 68 us
-// against 104, 64 of 50257 27 against 37).
+// against 104, 64 of 50257 27 against 37).  16-bit logits always stay here: the shared-memory walk does not read them.
 static int walk_batch_cluster(const VerifyArgs& a, int requests) {
   if (a.temperature == 0.f) return vwk::kCl;
   const bool sample = (a.flags & SEQ_VERIFY_TARGET_SAMPLE) != 0;
-  if (a.V > vwk::kClBatch * vwk::kTh * 32) return sample || requests * vwk::kCl <= 4 * device_sm_count() ? vwk::kCl : 0;
+  const bool bf16 = (a.flags & SEQ_VERIFY_LOGITS_BF16) != 0;
+  if (a.V > vwk::kClBatch * vwk::kTh * 32) return sample || bf16 || requests * vwk::kCl <= 4 * device_sm_count() ? vwk::kCl : 0;
   if (requests * vwk::kCl > device_sm_count()) return vwk::kClBatch;
   static int side_by_side[9][64];  // per kernel shape and device: clusters of 16, + 1; 0 = not asked yet
   const int slice = (((a.V + vwk::kCl - 1) / vwk::kCl) + 3) & ~3;
-  const int shape = (slice <= vwk::kTh * 8 ? 0 : slice <= vwk::kTh * 16 ? 1 : 2) + (sample ? 6 : (a.flags & SEQ_VERIFY_LOGITS_BF16) ? 3 : 0);
+  const int shape = (slice <= vwk::kTh * 8 ? 0 : slice <= vwk::kTh * 16 ? 1 : 2) + (sample ? 6 : bf16 ? 3 : 0);
   int dev = 0, n = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return vwk::kCl;
   if (dev >= 0 && dev < 64) n = __atomic_load_n(&side_by_side[shape][dev], __ATOMIC_ACQUIRE);

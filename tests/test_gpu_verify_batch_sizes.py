@@ -56,3 +56,9 @@ def test_large_batches(R, V, n, mode, bf16):
         t, u, cdf = int(bonus[r].item()), float(vi.uniforms[n]), np.cumsum(ref["residual"])
         assert ref["residual"][t] > 0 and (t == 0 or cdf[t - 1] - 1e-5 <= u) and u < cdf[t] + 1e-5
     assert clear >= R - 2
+
+
+@pytest.mark.parametrize("R", [37, 38, 60])
+def test_bf16_batches_beyond_what_the_shared_memory_walk_would_take(R):
+    """From 38 requests (148 SMs) a vocabulary above 65536 is the shared-memory walk's in fp32; it has no 16-bit form."""
+    test_large_batches(R, 65540, 3, "sequoia", True)
