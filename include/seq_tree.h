@@ -61,7 +61,8 @@ enum {
   SEQ_DEV_BAD_TOKEN = 2,   /* token id outside [0,vocab): the child is rejected, R and D untouched */
   SEQ_DEV_NONFINITE = 4,   /* NaN or +inf logit on a visited row */
   SEQ_DEV_DEGENERATE = 8,  /* sum max(R-D,0) == 0 after a rejection (impossible in exact arithmetic): R kept */
-  SEQ_DEV_TIMEOUT = 16,    /* a bounded on-chip wait ran out; outputs of that call are undefined */
+  SEQ_DEV_TIMEOUT = 16,    /* a bounded on-chip wait ran out; outputs of that call are undefined, but for the verification's
+                              path_len and bonus_token: 0 and -1, or what had been decided */
   SEQ_DEV_BAD_PATH = 32,   /* seq_tree_kv_commit: path not a root-to-node path (see there); nothing was moved */
   SEQ_DEV_BAD_LENGTH = 64  /* *prefix_len_dev outside [0, prefix_len]: clamped into that range */
 };

@@ -222,7 +222,7 @@ __device__ __forceinline__ void send4(uint32_t to, uint32_t bar, float4 v) {  //
                ::"r"(to), "r"(__float_as_uint(v.x)), "r"(__float_as_uint(v.y)), "r"(__float_as_uint(v.z)), "r"(__float_as_uint(v.w)), "r"(bar) : "memory");
 }
 // False when the bounded wait ran out (the same for the whole warp, after SEQ_DEV_TIMEOUT and a pause that lets the stores
-// on their way to and from this CTA land): the warp leaves the kernel.
+// on their way to and from this CTA land): the warp leaves the kernel, through timed_out().
 __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, int32_t* dev_status) {
   uint32_t done = 0;
 #pragma unroll 1
@@ -236,6 +236,11 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, int32_t*
     for (int it = 0; it < 1000; ++it) __nanosleep(1000);
   }
   return done;
+}
+// What a request that was given up leaves behind: no path and no token.  (Every CTA of the cluster gets here, the others
+// because this one's entries stay out, and each writes the same; what a thread had decided before is overwritten or not.)
+__device__ __forceinline__ void timed_out(const VerifyArgs& a) {
+  if ((threadIdx.x & 31) == 0) { *a.path_len = 0; *a.bonus = -1; }
 }
 // Before anything else: the mbarriers, and this CTA's arrival at the one cluster barrier.  exchange_ready() waits for it:
 // from there on every CTA is resident and its mbarriers count.
@@ -540,7 +545,7 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
     };
     if (n_kids > 0) take_kids(0);
     WTRACE(leader, 12);
-    if (!exchange_pull<CL>(c, x, a.dev_status)) return;
+    if (!exchange_pull<CL>(c, x, a.dev_status)) return timed_out(a);
     WTRACE(leader, 14);
     float Mp = -INFINITY, Mq = -INFINITY;
 #pragma unroll
@@ -649,7 +654,7 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
         load_row<NCH, kBf16>(c, tbase + (int64_t)nxt * a.target_stride * kEsz, pn);
         if (nxt_has_kids) load_row<NCH, kBf16>(c, dbase + (int64_t)nxt * a.draft_stride * kEsz, qn);
       }
-      if (!exchange_pull<CL>(c, x, a.dev_status)) return;
+      if (!exchange_pull<CL>(c, x, a.dev_status)) return timed_out(a);
       WTRACE(leader, 18);
       float zsum = 0.f, zdsum = 0.f;
 #pragma unroll
@@ -808,7 +813,7 @@ __global__ void __launch_bounds__(kTh, 1) tree_verify_greedy_kernel(const Verify
     const int first_kid = pick[2];
     if (first_kid != 0x7fffffff) load_row<NCH, kBf16>(c, tbase + (int64_t)first_kid * a.target_stride * kEsz, pn);
     Exch<kCl> t;
-    if (!exchange_pull<kCl>(c, t, a.dev_status)) return;
+    if (!exchange_pull<kCl>(c, t, a.dev_status)) return timed_out(a);
     key = INT_MIN; idx = 0x7fffffff;
 #pragma unroll
     for (int m = 0; m < kCl * kWarps / 32; ++m) {  // entries in vocabulary order: the first of equal keys stays
@@ -932,7 +937,7 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
     const int first_kid = pick[2];
     if (first_kid != 0x7fffffff) load_row<NCH, false>(c, tbase + (int64_t)first_kid * a.target_stride * 4, pn);
     Exch<CL> x;
-    if (!exchange_pull<CL>(c, x, a.dev_status)) return;
+    if (!exchange_pull<CL>(c, x, a.dev_status)) return timed_out(a);
     float Mp = -INFINITY;
 #pragma unroll
     for (int m = 0; m < kPPL; ++m) Mp = fmaxf(Mp, x.e[m].x);
@@ -963,7 +968,7 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
         const int found = __reduce_max_sync(0xffffffffu, mine);
         if (c.lane < CL) send4(c.remote + (uint32_t)offsetof(Shared, drawn) + 16u * buf, c.remote + bar, make_float4(__int_as_float(found), 0.f, 0.f, 0.f));
       }
-      if (!bar_wait(c.local + bar, (dn >> 1) & 1u, a.dev_status)) return;
+      if (!bar_wait(c.local + bar, (dn >> 1) & 1u, a.dev_status)) return timed_out(a);
       if (c.tid == 0) bar_arm(c.local + bar, sizeof(float4));
       token = __float_as_int(sh->drawn[buf].x);
       ++dn;
