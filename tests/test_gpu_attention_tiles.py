@@ -69,3 +69,14 @@ def test_single_precision_with_the_length_in_device_memory():
     assert int(st.item()) == 0
     ref, _, _ = O.tree_attention(ai.q, ai.k_cache[:, :L + n], ai.v_cache[:, :L + n], ai.parent, L)
     assert np.abs(out.double().cpu().numpy() - ref).max() < 1e-5
+
+
+@pytest.mark.parametrize("hkv,group,n,L", [(8, 5, 100, 500), (32, 1, 64, 1024)])
+def test_single_precision_sums_over_keys_stay_short(hkv, group, n, L):
+    """Relative error against fp64 below six units of 2^-24.  A score's two chains of 64 products leave about four (the same
+    whatever the prefix), 32-key sums and their few additions one; one chain over 600 or 1088 keys adds three and more."""
+    ai = _inputs(hkv, group, n, L, "fp32")
+    out, _, status = G.run_attention(ai)
+    ref, _, _ = O.tree_attention(ai.q, ai.k_cache, ai.v_cache, ai.parent, L)
+    assert status == 0
+    assert np.linalg.norm(out.double().cpu().numpy() - ref) < 6 * 2.0 ** -24 * np.linalg.norm(ref)
