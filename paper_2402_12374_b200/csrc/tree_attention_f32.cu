@@ -14,7 +14,7 @@
 //
 // What bounds it: multiply-adds and shared-memory reads side by side (12 16-byte loads per 128 FMA slots at RPT = 8) for
 // 32 rows and more, the K/V stream below.  32 heads, 64 nodes, a prefix of 1024: one CTA per (node, head), which re-read
-// K and V for each, took 331 us; this one 45 (the FMAs alone would take 16).  Rows fetched by cp.async from the computing
+// K and V for each, took 331 us; this one 46 (the FMAs alone would take 16).  Rows fetched by cp.async from the computing
 // warps: 58; by row-sized bulk copies: 71 (about 70 cycles for each 512 bytes).
 #include <type_traits>
 
@@ -48,6 +48,7 @@ struct F32Smem {
   float q[kF32Warps * RPT][kHeadDim];
   float p[kF32Warps * RPT][kF32Keys];
   uint64_t k_full, v_full;  // one phase per tile
+  uint32_t seen[kF32Warps][4];  // by group of the tile: the keys that some row of the warp sees (groups of tree keys)
 };
 
 __device__ __forceinline__ uint32_t f32_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -72,6 +73,11 @@ __device__ __forceinline__ uint64_t f32_fma2(uint64_t a, uint64_t b, uint64_t c)
 __device__ __forceinline__ uint64_t f32_mul2(uint64_t a, uint64_t b) {
   uint64_t d;
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t f32_add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
 __device__ __forceinline__ uint64_t f32_pair(float lo, float hi) {
@@ -136,7 +142,7 @@ __device__ __forceinline__ uint32_t f32_window(const uint32_t* row, int wpr, int
 // One tile of NJ groups of 32 keys for one warp: scores, softmax step, and (when the caller has made sure that V is in
 // place) the product with V.
 template <int RPT>
-struct F32Row { float m[RPT], l[RPT], alpha[RPT]; ulonglong2 o[RPT]; };  // running maximum (the whole row's), this lane's share of the sum, what the output so far is to be scaled by, output (two packed pairs)
+struct F32Row { float m[RPT], l[RPT]; ulonglong2 o[RPT]; };  // running maximum (the whole row's), this lane's share of the sum, output (two packed pairs)
 
 template <int RPT, int NJ>
 __device__ __forceinline__ void f32_softmax(F32Smem<RPT>& sm, F32Row<RPT>& st, int row0, int lane, float (&s)[RPT][NJ]) {
@@ -162,49 +168,58 @@ __device__ __forceinline__ void f32_softmax(F32Smem<RPT>& sm, F32Row<RPT>& st, i
     }
     st.l[i] = fmaf(st.l[i], alpha, sum);
     st.m[i] = mx[i];
-    st.alpha[i] = alpha;
+    const uint64_t alpha2 = f32_pair(alpha, alpha);
+    st.o[i].x = f32_mul2(st.o[i].x, alpha2);
+    st.o[i].y = f32_mul2(st.o[i].y, alpha2);
   }
   __syncwarp();
 }
 
-// O = alpha O + P V over `keys` keys.  Each 32 of them are summed by themselves and then added: relative error of the output
-// against fp64, 64 nodes on 1024 keys: 4.8e-7 with one chain over all of a CTA's keys, 2.8e-7 so (a CTA per node and head,
-// four chains: 3.9e-7), for 43.4 -> 45.4 us.
-template <int RPT>
-__device__ __forceinline__ void f32_pv(const F32Smem<RPT>& sm, F32Row<RPT>& st, int row0, int lane, int keys) {
-  const uint8_t* vcol = sm.v + (lane >> 3) * 4096;  // this lane's quarter of head_dim
+// O += P V over group `grp` of 32 keys of the tile, summed by themselves and then added: relative error of the output against
+// fp64, 64 nodes on 1024 keys: 4.8e-7 with one chain over all of a CTA's keys, 2.8e-7 so (a CTA per node and head, four
+// chains: 3.9e-7), for 43.4 -> 45.4 us.
+//
+// kTree: the group reaches into the tree's keys, of which a row sees few.  A product is left out where p is 0, so that what
+// another branch's row of V holds - infinities and NaN too - never reaches a row, and four keys that no row of the warp sees
+// (`seen`, a bit for each key) are passed over: 64 nodes on 1024 keys 45.4 -> 46.4 us, 128 on 128 40.2 -> 36.8, 768 on none
+// 84 -> 73 (branches in place of the predicates: 51.6, 44 and 100).
+template <int RPT, bool kTree>
+__device__ __forceinline__ void f32_pv(const F32Smem<RPT>& sm, F32Row<RPT>& st, int row0, int lane, int grp, uint32_t seen) {
+  const uint8_t* vcol = sm.v + (lane >> 3) * 4096 + grp * kF32GroupBytes;  // this lane's quarter of head_dim
+  ulonglong2 t[RPT];
+#pragma unroll
+  for (int i = 0; i < RPT; ++i) t[i] = make_ulonglong2(0ull, 0ull);
 #pragma unroll 1
-  for (int grp = 0; grp < keys; grp += 32) {
-    ulonglong2 t[RPT];
+  for (int c = 0; c < 32; c += 4) {
+    if (kTree && !((seen >> c) & 15u)) continue;
+    const uint8_t* at = vcol + c * 128;
+    const int word = (lane ^ c) & 7;  // (c is a multiple of 4: key c + e has swizzle (c & 7) + e)
+    ulonglong2 vv[4];
+    float4 p[RPT];
 #pragma unroll
-    for (int i = 0; i < RPT; ++i) t[i] = make_ulonglong2(0ull, 0ull);
-#pragma unroll 1
-    for (int c = 0; c < 32; c += 4) {
-      const uint8_t* at = vcol + (grp >> 5) * kF32GroupBytes + c * 128;
-      const int word = (lane ^ c) & 7;  // (c is a multiple of 4: key c + e has swizzle (c & 7) + e)
-      ulonglong2 vv[4];
-      float4 p[RPT];
+    for (int e = 0; e < 4; ++e) vv[e] = *reinterpret_cast<const ulonglong2*>(at + e * 128 + ((word ^ e) << 4));
 #pragma unroll
-      for (int e = 0; e < 4; ++e) vv[e] = *reinterpret_cast<const ulonglong2*>(at + e * 128 + ((word ^ e) << 4));
+    for (int i = 0; i < RPT; ++i) p[i] = *reinterpret_cast<const float4*>(&sm.p[row0 + i][32 * grp + c]);
 #pragma unroll
-      for (int i = 0; i < RPT; ++i) p[i] = *reinterpret_cast<const float4*>(&sm.p[row0 + i][grp + c]);
+    for (int e = 0; e < 4; ++e)
 #pragma unroll
-      for (int e = 0; e < 4; ++e)
-#pragma unroll
-        for (int i = 0; i < RPT; ++i) {
-          const float pe = e == 0 ? p[i].x : e == 1 ? p[i].y : e == 2 ? p[i].z : p[i].w;
-          const uint64_t pp = f32_pair(pe, pe);
+      for (int i = 0; i < RPT; ++i) {
+        const float pe = e == 0 ? p[i].x : e == 1 ? p[i].y : e == 2 ? p[i].z : p[i].w;
+        const uint64_t pp = f32_pair(pe, pe);
+        if (kTree) {
+          asm("{\n\t.reg .pred s;\n\tsetp.neu.f32 s, %4, 0f00000000;\n\t"
+              "@s fma.rn.f32x2 %0, %5, %2, %0;\n\t@s fma.rn.f32x2 %1, %5, %3, %1;\n\t}"
+              : "+l"(t[i].x), "+l"(t[i].y) : "l"(vv[e].x), "l"(vv[e].y), "f"(pe), "l"(pp));
+        } else {
           t[i].x = f32_fma2(pp, vv[e].x, t[i].x);
           t[i].y = f32_fma2(pp, vv[e].y, t[i].y);
         }
-    }
+      }
+  }
 #pragma unroll
-    for (int i = 0; i < RPT; ++i) {
-      const float scale = grp == 0 ? st.alpha[i] : 1.f;
-      const uint64_t s2 = f32_pair(scale, scale);
-      st.o[i].x = f32_fma2(st.o[i].x, s2, t[i].x);
-      st.o[i].y = f32_fma2(st.o[i].y, s2, t[i].y);
-    }
+  for (int i = 0; i < RPT; ++i) {
+    st.o[i].x = f32_add2(st.o[i].x, t[i].x);
+    st.o[i].y = f32_add2(st.o[i].y, t[i].y);
   }
 }
 
@@ -286,14 +301,21 @@ tree_attention_f32_kernel(const __grid_constant__ CUtensorMap k_map, const __gri
       if (more && threadIdx.x == 0) request(&k_map, sm.k, &sm.k_full, grp + 4);
       if (warp_live) {
         if ((grp + NJ) * 32 > L) {  // the tile reaches into the tree's keys (or past the end)
+          uint32_t seen[NJ] = {};
 #pragma unroll
           for (int i = 0; i < RPT; ++i) {
             const int node = min((R0 + row0 + i) / a.group, a.n - 1);
             const uint32_t* mrow = a.mask_bits + (size_t)node * a.mask_wpr;
 #pragma unroll
-            for (int j = 0; j < NJ; ++j)
-              if (!((f32_window(mrow, a.mask_wpr, node + 1, (grp + j) * 32 - L) >> lane) & 1u)) s[i][j] = -INFINITY;
+            for (int j = 0; j < NJ; ++j) {
+              const uint32_t bits = f32_window(mrow, a.mask_wpr, node + 1, (grp + j) * 32 - L);
+              if (!((bits >> lane) & 1u)) s[i][j] = -INFINITY;
+              seen[j] |= bits;
+            }
           }
+#pragma unroll
+          for (int j = 0; j < NJ; ++j)
+            if (lane == j) sm.seen[warp][j] = seen[j];
         }
         f32_softmax<RPT, NJ>(sm, st, row0, lane, s);
       }
@@ -303,14 +325,13 @@ tree_attention_f32_kernel(const __grid_constant__ CUtensorMap k_map, const __gri
     else if (nj == 2) tile(std::integral_constant<int, 2>());
     else tile(std::integral_constant<int, 1>());
     f32_wait(&sm.v_full, phase, a.dev_status);
-    if (a.L_dev != nullptr && (grp + nj) * 32 > n_keys) {
-      // the maps of this mode cover the whole cache: rows past the tree may hold anything, and 0 * NaN is not 0
-      for (int r = n_keys - grp * 32 + warp; r < nj * 32; r += kF32Warps)
-        *reinterpret_cast<float4*>(sm.v + (r >> 5) * kF32GroupBytes + (lane >> 3) * 4096 + (r & 31) * 128 + (lane & 7) * 16) =
-            make_float4(0.f, 0.f, 0.f, 0.f);
-      __syncthreads();
+    if (warp_live) {
+#pragma unroll 1
+      for (int j = 0; j < nj; ++j) {
+        if ((grp + j + 1) * 32 <= L) f32_pv<RPT, false>(sm, st, row0, lane, j, 0u);
+        else f32_pv<RPT, true>(sm, st, row0, lane, j, sm.seen[warp][j]);
+      }
     }
-    if (warp_live) f32_pv<RPT>(sm, st, row0, lane, 32 * nj);
     __syncthreads();  // everyone has read V
     if (more && threadIdx.x == 0) request(&v_map, sm.v, &sm.v_full, grp + 4);
   }

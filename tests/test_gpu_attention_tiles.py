@@ -80,3 +80,25 @@ def test_single_precision_sums_over_keys_stay_short(hkv, group, n, L):
     ref, _, _ = O.tree_attention(ai.q, ai.k_cache, ai.v_cache, ai.parent, L)
     assert status == 0
     assert np.linalg.norm(out.double().cpu().numpy() - ref) < 6 * 2.0 ** -24 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+@pytest.mark.parametrize("hkv,group,n,L", [(2, 1, 40, 70), (2, 3, 9, 0), (1, 1, 5, 3000), (1, 8, 70, 33)])
+def test_single_precision_rows_do_not_depend_on_other_branches(hkv, group, n, L, bad):
+    """A key and value row that holds infinities or NaN reaches the node's own row and its descendants', no other one."""
+    d = G.dev()
+    ai = _inputs(hkv, group, n, L, "fp32")
+    parent = ai.parent.numpy()
+    victim = 1
+    sees = np.zeros(n, dtype=bool)
+    for i in range(n):
+        sees[i] = i == victim or (parent[i] >= 0 and sees[parent[i]])
+    mask, _, _ = G.gpu_mask(parent)
+    q, k, v = ai.q.to(d), ai.k_cache.to(d), ai.v_cache.to(d)
+    want = B.seq_tree_attention(q, k, v, mask, L).clone()
+    k[:, L + victim], v[:, L + victim] = bad, bad
+    got = B.seq_tree_attention(q, k, v, mask, L)
+    torch.cuda.synchronize()
+    assert 0 < sees.sum() < n
+    assert torch.equal(got[~sees], want[~sees])
+    assert not torch.isfinite(got[sees]).any()
