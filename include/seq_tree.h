@@ -131,7 +131,9 @@ int seq_tree_mask_from_parents(const int32_t* parent, int32_t n, uint32_t* mask_
  * workspace: at least seq_tree_attention_workspace_bytes(p) bytes, 256-byte
  * aligned, device; contents undefined before and after.  The size depends on
  * the shape and on p->kernel and may be 0 (workspace may then be NULL): the
- * CUDA-core kernel keeps the partial results of its key-range splits there,
+ * CUDA-core kernels keep the partial results of their key-range splits there
+ * (the fp32 one makes do with less, in fewer splits, down to none for most
+ * shapes: a workspace sized for the longest prefix serves every shorter one),
  * the tensor-core kernel the pieces of the query tiles that its CTAs share
  * when there are more (tile, kv head) units than SMs (about 19 MB then).  A
  * call with a workspace that is too small returns SEQ_ERR_WORKSPACE and

@@ -75,6 +75,11 @@ static int choose_kernel(const seq_tree_attention_params& p) {
   return 2;
 }
 
+// Bytes of the CUDA-core kernels' partial results.
+static size_t cuda_core_workspace(const seq_tree_attention_params& p, int splits) {
+  return splits > 1 ? split_workspace_bytes(splits, p.num_q_heads, p.n_tree) : 0;
+}
+
 }  // namespace seqtree
 
 using namespace seqtree;
@@ -84,8 +89,11 @@ extern "C" size_t seq_tree_attention_workspace_bytes(const seq_tree_attention_pa
   const int which = choose_kernel(*p);
   if (which == 0) return 0;
   if (which == 2) return umma_workspace_bytes(*p);  // only its stream mode (more units than SMs) needs one
-  const int splits = which == 3 ? f32_splits(*p) : simt_default_splits(*p);
-  size_t bytes = splits > 1 ? split_workspace_bytes(splits, p->num_q_heads, p->n_tree) : 0;
+  size_t bytes = cuda_core_workspace(*p, simt_default_splits(*p));
+  if (which == 3) {
+    const size_t plan = cuda_core_workspace(*p, f32_splits(*p));
+    bytes = plan > bytes ? plan : bytes;
+  }
   return (bytes + 255) & ~(size_t)255;
 }
 
@@ -95,12 +103,20 @@ extern "C" int seq_tree_attention(const seq_tree_attention_params* p, void* stre
   const int which = choose_kernel(*p);
   if (which == 0) return SEQ_ERR_UNSUPPORTED;
   if (which == 2) return launch_attention_umma(*p, umma_default_splits(*p), (cudaStream_t)stream);
-  const int splits = which == 3 ? f32_splits(*p) : simt_default_splits(*p);
-  if (splits > 1) {
-    if (p->workspace == nullptr || p->workspace_bytes < split_workspace_bytes(splits, p->num_q_heads, p->n_tree))
-      return SEQ_ERR_WORKSPACE;
-    if (reinterpret_cast<uintptr_t>(p->workspace) % 256 != 0) return SEQ_ERR_INVALID_ARG;
+  const int splits = simt_default_splits(*p);
+  size_t need = cuda_core_workspace(*p, splits), lent = p->workspace != nullptr ? p->workspace_bytes : 0;
+  const bool aligned = reinterpret_cast<uintptr_t>(p->workspace) % 256 == 0;
+  if (which == 3) {
+    // The fp32 kernel's best split of the key range is not monotone in the prefix length, and asks for more than the kernel
+    // before it did: it makes do with what it is lent, from the smaller of the two needs on, so that a workspace sized for
+    // the longest prefix serves every shorter one.
+    const size_t plan = cuda_core_workspace(*p, f32_splits(*p));
+    need = plan < need ? plan : need;
   }
-  if (which == 3) return launch_attention_f32(*p, ~(size_t)0, (cudaStream_t)stream);
+  if (need > 0) {
+    if (lent < need) return SEQ_ERR_WORKSPACE;
+    if (!aligned) return SEQ_ERR_INVALID_ARG;
+  }
+  if (which == 3) return launch_attention_f32(*p, aligned ? lent : 0, (cudaStream_t)stream);
   return launch_attention_simt(*p, splits, (cudaStream_t)stream);
 }

@@ -102,3 +102,36 @@ def test_single_precision_rows_do_not_depend_on_other_branches(hkv, group, n, L,
     assert 0 < sees.sum() < n
     assert torch.equal(got[~sees], want[~sees])
     assert not torch.isfinite(got[sees]).any()
+
+
+@pytest.mark.parametrize("hkv,group,n,cap", [(2, 2, 8, 8192), (8, 8, 64, 8192), (8, 5, 100, 8192)])
+def test_single_precision_workspace_of_the_longest_prefix_serves_every_shorter_one(hkv, group, n, cap):
+    """The plan's own need rises and falls with the prefix length: every length of a decoding run, in steps of 32, is taken
+    with the workspace of the longest one, and a few that would like more of it agree with the oracle."""
+    d = G.dev()
+    ai = _inputs(hkv, group, n, cap, "fp32")
+    mask, _, _ = G.gpu_mask(ai.parent.numpy())
+    q, k, v = ai.q.to(d), ai.k_cache.to(d), ai.v_cache.to(d)
+    longest = B.AttentionCall(q, k, v, mask, cap)
+    short = 0
+    for L in range(0, cap, 32):
+        own = B.AttentionCall(q, k, v, mask, L, workspace=torch.empty(0, dtype=torch.uint8, device=d))
+        call = B.AttentionCall(q, k, v, mask, L, workspace=longest.workspace)
+        out = call.run()  # (refused: raises)
+        if own.workspace_bytes_needed > longest.workspace_bytes_needed and short < 3:
+            short += 1
+            ref, _, _ = O.tree_attention(ai.q, ai.k_cache[:, :L + n], ai.v_cache[:, :L + n], ai.parent, L)
+            assert np.abs(out.double().cpu().numpy() - ref).max() < 1e-5
+    torch.cuda.synchronize()
+
+
+def test_single_precision_without_a_workspace():
+    """Shapes with rows for every SM never needed one; the split of the key range is then left out."""
+    d = G.dev()
+    ai = _inputs(32, 1, 64, 1000, "fp32")
+    mask, _, _ = G.gpu_mask(ai.parent.numpy())
+    call = B.AttentionCall(ai.q.to(d), ai.k_cache.to(d), ai.v_cache.to(d), mask, 1000, workspace=torch.empty(0, dtype=torch.uint8, device=d))
+    out = call.run()
+    torch.cuda.synchronize()
+    ref, _, _ = O.tree_attention(ai.q, ai.k_cache, ai.v_cache, ai.parent, 1000)
+    assert np.abs(out.double().cpu().numpy() - ref).max() < 1e-5
