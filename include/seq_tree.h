@@ -135,9 +135,10 @@ int seq_tree_mask_from_parents(const int32_t* parent, int32_t n, uint32_t* mask_
  * (the fp32 one makes do with less, in fewer splits, down to none for most
  * shapes: a workspace sized for the longest prefix serves every shorter one),
  * the tensor-core kernel the pieces of the query tiles that its CTAs share
- * when there are more (tile, kv head) units than SMs (about 19 MB then).  A
- * call with a workspace that is too small returns SEQ_ERR_WORKSPACE and
- * launches nothing.  Two calls that run concurrently need a workspace each.
+ * when there are more (tile, kv head) units than SMs (about 19 MB then; with
+ * kernel = 0 a group of heads that does not divide 128 does without).  A call
+ * with a workspace that is too small returns SEQ_ERR_WORKSPACE and launches
+ * nothing.  Two calls that run concurrently need a workspace each.
  * The results do not depend on the order in which CTAs finish: a call
  * repeated on the same inputs returns the same bits.
  */

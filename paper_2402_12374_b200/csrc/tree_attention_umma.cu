@@ -1250,9 +1250,13 @@ int launch_attention_umma(const seq_tree_attention_params& p, int splits, cudaSt
   a.blocks_per_head_host = 0; a.total_blocks_host = 0;
   a.L_dev = p.prefix_len_dev; a.L_count = p.prefix_len_dev_count; a.zero_tail = p.prefix_len_dev != nullptr ? 1 : 0;
   a.ws_count = nullptr; a.ws_ml = nullptr; a.ws_o = nullptr;
+  const bool lent = p.workspace != nullptr && p.workspace_bytes >= stream_count_bytes(p) + stream_ml_bytes() + stream_o_bytes();
+  // (groups that do not divide 128 used to run on the CUDA cores, which ask for nothing at these sizes: without a workspace
+  // they take the grid schedule instead, 500 nodes on 4600 keys of 40/8 heads 99 us against 67)
+  if (!lent && p.kernel == 0 && kTileM % G != 0) a.stream = 0;
   if (a.stream) {
     const size_t cnt_bytes = stream_count_bytes(p);
-    if (p.workspace == nullptr || p.workspace_bytes < cnt_bytes + stream_ml_bytes() + stream_o_bytes()) return SEQ_ERR_WORKSPACE;
+    if (!lent) return SEQ_ERR_WORKSPACE;
     if (reinterpret_cast<uintptr_t>(p.workspace) % 256 != 0) return SEQ_ERR_INVALID_ARG;
     for (int t = 0; t < tiles; ++t) {
       const int i1 = (t + 1) * nodes_per_tile < p.n_tree ? (t + 1) * nodes_per_tile : p.n_tree;

@@ -135,3 +135,22 @@ def test_single_precision_without_a_workspace():
     torch.cuda.synchronize()
     ref, _, _ = O.tree_attention(ai.q, ai.k_cache, ai.v_cache, ai.parent, 1000)
     assert np.abs(out.double().cpu().numpy() - ref).max() < 1e-5
+
+
+@pytest.mark.parametrize("hkv,group,n,L", [(8, 5, 500, 4600), (50, 3, 126, 2100)])
+def test_groups_that_do_not_divide_the_tile_without_a_workspace(hkv, group, n, L):
+    """More tiles than SMs and many keys: the plan would like a workspace; without one the same tiles run one per CTA."""
+    d = G.dev()
+    ai = _inputs(hkv, group, n, L, "bf16")
+    mask, _, st = G.gpu_mask(ai.parent.numpy())
+    q, k, v = ai.q.to(d), ai.k_cache.to(d), ai.v_cache.to(d)
+    call = B.AttentionCall(q, k, v, mask, L, workspace=torch.empty(0, dtype=torch.uint8, device=d), dev_status=st)
+    assert call.workspace_bytes_needed > 0
+    got, want = call.run(), B.seq_tree_attention(q, k, v, mask, L, dev_status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    rows = [0, 1, n // 2, n - 1]
+    G.check_attention(ai, rows=rows)
+    assert (got.float() - want.float()).abs().max() < 2e-2  # (both within half a unit of the exact rows, which are below 2)
+    with pytest.raises(RuntimeError):
+        B.AttentionCall(q, k, v, mask, L, workspace=torch.empty(0, dtype=torch.uint8, device=d), kernel=B.KERNEL_TENSOR_CORE_STREAM).run()
