@@ -142,8 +142,8 @@ __device__ __forceinline__ int ds_compact(DsShared& sh, int count, int k) {
 }
 
 // The bound a token has to pass: the threshold less what the bounds' rounding may cost (31 ulp of place in the first step,
-// a few ulp of the approximations).
-__device__ __forceinline__ float ds_cut(float tau) { return fminf(tau - 1e-3f - 1e-5f * fminf(fabsf(tau), 1e30f), 3e38f); }
+// a few ulp of the approximations: below 4e-6 of it at every magnitude).
+__device__ __forceinline__ float ds_cut(float tau) { return fminf(tau - 1e-3f - 1e-5f * fminf(fabsf(tau), 3e38f), 3e38f); }
 
 template <bool kVec>
 __global__ void __launch_bounds__(kDsThreads) draft_sample_kernel(const DraftSampleArgs a) {

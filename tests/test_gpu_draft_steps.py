@@ -77,3 +77,19 @@ def test_rankings_between_steps_keep_every_listed_token(rows, V, k):
             clear += 1
             assert first[r].tolist() == best.indices[:k].tolist(), r
     assert clear >= rows // 2
+
+
+@pytest.mark.parametrize("T", [1e-28, 1e-31, 1e-33, 1e-36, 2e-38])
+def test_scores_of_any_magnitude(T):
+    """At such temperatures the uniforms do not matter any more (logit / T in single precision swallows them): the draw is the
+    order of the logits.  At 2e-38 the scores of the largest ones are infinite: equal, in token order."""
+    rng = np.random.default_rng(5)
+    rows, V, k = 64, 5000, 4
+    logits = (3 * rng.standard_normal((rows, V))).astype(np.float32)
+    u = (rng.random((rows, V)) * 0.9 + 0.05).astype(np.float32)
+    d = _dev()
+    got = B.seq_tree_draft_sample(torch.from_numpy(logits).to(d), T, torch.from_numpy(u).to(d), k).cpu().numpy()
+    with np.errstate(over="ignore"):
+        score = logits * (np.float32(1) / np.float32(T))
+    want = np.argsort(-score, axis=1, kind="stable")[:, :k]
+    assert (got == want).all()
