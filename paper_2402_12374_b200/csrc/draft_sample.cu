@@ -14,8 +14,8 @@
 // (each thread scores the token with its best bound; the k-th largest of the bests of 64 or 128 groups of threads); after
 // that only tokens whose bound passes the threshold are listed.  Whenever the steps done have doubled (about k tokens pass
 // in that time), and at the end, the listed tokens are scored and ranked against each other, the k best stay and the
-// threshold becomes the k-th score itself.  A list that overflows (long runs of equal scores) sends the part through the
-// same ranking 256 tokens at a time.  The parts of a row are a thread-block cluster (up to 8): each pushes its k best into
+// threshold becomes the k-th score itself.  A list that overflows (long runs of equal scores, rows in ascending order) leaves
+// the rest of the part to k block-wide arg-max rounds per step.  The parts of a row are a thread-block cluster (up to 8): each pushes its k best into
 // the first CTA's shared memory, which ranks them in the same way.  No workspace, one launch.
 //
 // What bounds it: the two streams of logits and uniforms from HBM.  378 rows of 128256 tokens, k = 9: k block-wide arg-max
@@ -23,6 +23,7 @@
 // bandwidth of 6.55 TB/s; k = 32: 72).  A few short rows are bound by the chain of steps, rankings and the cluster: 5 us.
 #include <cooperative_groups.h>
 #include <float.h>
+#include <limits.h>
 #include <math.h>
 
 #include "common.cuh"
@@ -69,6 +70,9 @@ __device__ __forceinline__ float ds_score(float logit, float u, float inv_T, boo
   if (!(u > 0.f && u < 1.f)) return -INFINITY;
   return logit * inv_T - __logf(ds_neg_log(u));
 }
+
+// float -> int of the same order
+__device__ __forceinline__ int ds_ordered(float x) { const int b = __float_as_int(x); return b ^ ((b >> 31) & 0x7fffffff); }
 
 struct DsShared {
   float2 list[kDsList];  // (score, token bits); behind the ranked ones, tokens not scored yet
@@ -234,9 +238,10 @@ __global__ void __launch_bounds__(kDsThreads) draft_sample_kernel(const DraftSam
   list_passing(0, cut);
 
   // ---- the other steps: bounds against the threshold, a ranking every few of them
-  int ranked = 0;  // entries at the list's front that carry their score
+  int ranked = 0;  // entries at the list's front that carry their score: the best of the tokens before `next`
+  int next = 0;
   bool overflow = false;
-  auto rank_list = [&]() {
+  auto rank_list = [&](int seen) {
     __syncthreads();
     const int count = sh.count;
     overflow |= count > kDsList;
@@ -247,30 +252,73 @@ __global__ void __launch_bounds__(kDsThreads) draft_sample_kernel(const DraftSam
     }
     __syncthreads();
     ranked = ds_compact(sh, count, a.k);
+    next = seen;
     cut = ds_cut(sh.tau);
   };
   for (int t0 = kDsStep, step = 1; t0 < cnt; t0 += kDsStep, ++step) {
     const float best = bounds(false);
     if (t0 + kDsStep < cnt) fetch(t0 + kDsStep);
     if (best > cut) list_passing(t0, cut);
-    if ((step & (step + 1)) == 0) rank_list();
-  }
-  rank_list();
-  if (bad) dev_flag(a.dev_status, SEQ_DEV_NONFINITE);
-  if (overflow) {
-    __syncthreads();
-    if (tid == 0) { sh.count = 0; sh.tau = -INFINITY; }
-    __syncthreads();
-    for (int t0 = 0; t0 < cnt; t0 += kDsThreads) {
-      const int t = t0 + tid;
-      const float s = t < cnt ? ds_score(lrow[t], urow[t], a.inv_T, unused) : -INFINITY;
-      if (s > -INFINITY && s >= sh.tau) sh.list[atomicAdd(&sh.count, 1)] = make_float2(s, __int_as_float(t));
-      __syncthreads();
-      const int count = sh.count;
-      __syncthreads();
-      ranked = ds_compact(sh, count, a.k);
+    if ((step & (step + 1)) == 0) {
+      rank_list(t0 + kDsStep);
+      if (overflow) break;
     }
   }
+  if (!overflow) rank_list(cnt);
+  if (overflow) {
+    // Too many tokens in the running.  From the first step that is not ranked on, the step's k best are found by k arg-max
+    // rounds - each thread keeps its scores and its best, whoever loses the best looks for the next one - and ranked
+    // with those of the steps before.  A token has to beat the k-th of those: an equal one comes later in the order.  (378
+    // rows of 128256 equal or ascending tokens, k = 9: 130 and 241 us; ranking 256 tokens at a time took 10 ms.)
+    int2* w_best = reinterpret_cast<int2*>(sh.top);  // [2][kDsWarps], used in turn
+    int turn = 0;
+    if (ranked < a.k && tid == 0) sh.tau = -INFINITY;
+    __syncthreads();
+    fetch(next);
+    for (int t0 = next; t0 < cnt; t0 += kDsStep) {
+      const float tau = sh.tau;
+      float best = -INFINITY;
+      int at = 0;
+#pragma unroll
+      for (int e = 0; e < kDsE; ++e) {
+        const float s = ds_score(x[e], u[e], a.inv_T, bad);
+        ub[e] = s > tau ? s : -INFINITY;
+        if (ub[e] > best) { best = ub[e]; at = e; }
+      }
+      if (t0 + kDsStep < cnt) fetch(t0 + kDsStep);
+      int found = 0;
+      for (; found < a.k; ++found, ++turn) {
+        const bool any = best > -INFINITY;
+        const int mine = token_of(t0, at);
+        auto argmax = [](int key, int token) {  // over the warp: the larger key, then the lower token
+          const int m = __reduce_max_sync(0xffffffffu, key);
+          return make_int2(m, __reduce_min_sync(0xffffffffu, key == m ? token : INT_MAX));
+        };
+        int2 w = argmax(any ? ds_ordered(best) : INT_MIN, any ? mine : INT_MAX);
+        if (lane == 0) w_best[(turn & 1) * kDsWarps + warp] = w;
+        __syncthreads();
+        w = w_best[(turn & 1) * kDsWarps + lane % kDsWarps];
+        w = argmax(w.x, w.y);
+        if (w.y == INT_MAX) break;
+        if (any && mine == w.y) {
+          sh.list[ranked + found] = make_float2(best, __int_as_float(mine));
+          best = -INFINITY;
+          const int gone = at;
+#pragma unroll
+          for (int e = 0; e < kDsE; ++e) {
+            if (e == gone) ub[e] = -INFINITY;
+            if (ub[e] > best) { best = ub[e]; at = e; }
+          }
+        }
+      }
+      ++turn;  // (the round that ended the step read one of the two as well)
+      if (found > 0) {
+        __syncthreads();
+        ranked = ds_compact(sh, ranked + found, a.k);
+      }
+    }
+  }
+  if (bad) dev_flag(a.dev_status, SEQ_DEV_NONFINITE);
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   int have = ranked;
   if (a.parts > 1) {

@@ -93,3 +93,46 @@ def test_scores_of_any_magnitude(T):
         score = logits * (np.float32(1) / np.float32(T))
     want = np.argsort(-score, axis=1, kind="stable")[:, :k]
     assert (got == want).all()
+
+
+@pytest.mark.parametrize("rows,V,k", [(3, 40000, 64), (2, 33333, 1), (450, 20001, 9), (5, 131072, 33)])
+def test_lists_that_overflow_behind_ranked_steps(rows, V, k):
+    """Equal uniforms, so that the draw is the order of the logits, lower token first: noise for a third of the row, then
+    a staircase of runs of 37 equal logits that rises above it, the last third level with its top; the k-th token lies in
+    a run.  A NaN behind the overflow is flagged."""
+    rng = np.random.default_rng(V)
+    logits = np.empty((rows, V), np.float32)
+    third = V // 3
+    logits[:, :third] = rng.standard_normal((rows, third))
+    logits[:, third:] = 2.0 + np.minimum(np.arange(V - third), third) // 37 / 64.0
+    want = np.argsort(-logits, axis=1, kind="stable")[:, :k]
+    logits[0, V - 1] = np.nan
+    d = _dev()
+    st = torch.zeros(1, dtype=torch.int32, device=d)
+    got = B.seq_tree_draft_sample(torch.from_numpy(logits).to(d), 0.7, torch.full((rows, V), 0.5, device=d), k, dev_status=st).cpu().numpy()
+    assert (got == want).all()
+    assert int(st.item()) == B.SEQ_DEV_NONFINITE
+
+
+@pytest.mark.parametrize("order", ["equal", "ascending"])
+def test_no_order_of_a_row_costs_many_times_another(order):
+    """378 rows of 128256 tokens: two to four times the time of random rows (160 times when a list that overflowed was ranked 256
+    tokens at a time)."""
+    d = _dev()
+    rows, V, k = 378, 128256, 9
+    u = torch.rand((rows, V), device=d)
+    half = torch.full((rows, V), 0.5, device=d)
+    x = torch.zeros((rows, V), device=d) if order == "equal" else torch.linspace(0, 400, V, device=d).repeat(rows, 1)
+
+    def ms(logits, uniforms):
+        best = float("inf")
+        for _ in range(4):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            B.seq_tree_draft_sample(logits, 0.6, uniforms, k)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1))
+        return best
+
+    assert ms(x, half) < 10 * ms(torch.randn((rows, V), device=d), u)
