@@ -10,9 +10,10 @@
 // the histograms with the masses' sums, the tokens of the cut's bin; every CTA then finds the cut by itself and writes its
 // slice.  The histogram covers the exponent arguments below 15 first - tokens below 2^-15 of the most probable one, most of
 // the vocabulary, only enter the sum - and the rest, in two more rounds, in the rare case that the cut is not among them.
-// One CTA takes the row through global memory instead (four passes, or seven with a radix select on the logit bits, 11 + 11
-// + 10) where the vocabulary is larger, and where more than 1024 tokens share the cut's bin (flat rows, long runs of equal
-// logits).
+// Where more than 512 tokens share the cut's bin (flat rows, long runs of equal logits) the bin is cut up by the logit bits,
+// 9 at a time, until few tokens are left or all are equal (tp_refine).  Larger vocabularies: one CTA takes the row through
+// global memory, in four passes, or with more than 1024 tokens in the cut's bin in seven with a radix select on the logit
+// bits (11 + 11 + 10).
 //
 // What bounds it: the chain of exchanges for a few rows, HBM for many.  64 rows of 32000 tokens: 29.7 us with one CTA of
 // 1024 threads per row reading it four times and adding every token to the histogram, 13.2 so (about a dozen exchanges and
@@ -365,7 +366,10 @@ __global__ void __launch_bounds__(kTpThreads) top_p_row_kernel(const TopPArgs a)
 constexpr int kTpBins = 768;           // bins of one round of the histogram, 24 groups of 32
 constexpr int kTpRounds = 3;           // 2048 bins in rounds, most probable first (the last one is shorter)
 constexpr int kTpMaxCluster = 8, kTpMaxSlice = 16384;
-constexpr int kTpFastCand = 512;       // tokens of the cut's bin that are ordered here (more: the row goes to one CTA)
+// Tokens of the cut's bin that are ordered by their running masses (more: tp_refine; with 1024, rows of deviation 0.5 below
+// take 408 us instead of 452, ordinary ones 208 instead of 193, for the room), and from how many on each CTA of the cluster
+// looks at its own ones only.
+constexpr int kTpFastCand = 512, kTpAlone = 128;
 constexpr int kTpQueue = 64;           // per warp: tokens of the round's bins waiting to be added by a full warp
 struct TpFast {
   // Two limbs of 20 and 21 bits per bin, added without a return value; from 4096 tokens in one bin on they could wrap, and
@@ -373,13 +377,15 @@ struct TpFast {
   uint32_t limb[2][kTpBins];
   unsigned long long coarse[32];       // masses of the groups of bins; [24] all tokens' mass, [25] the round's tokens' (both exact)
   unsigned long long stage[kTpMaxCluster][32];  // what was read from the cluster's CTAs
-  unsigned long long part[2][kTpWarps];
+  __align__(16) unsigned long long part[2][kTpWarps];
   float queue[kTpWarps][kTpQueue];
   __align__(16) ulonglong2 cand[kTpFastCand];  // this CTA's tokens of the cut's bin (read by the other CTAs)
   __align__(16) ulonglong2 all[kTpFastCand];   // the cluster's
   unsigned long long tau_comp;
   int32_t max;                         // the row's maximum as an ordered integer (every CTA of the cluster adds its warps')
   int32_t ncand;
+  uint32_t kmin, kmax;                 // tp_refine: range of the keys in question (every CTA of the cluster adds its warps')
+  uint32_t klo, khi;                   // ... and what is left of it
   __align__(16) float x[4];            // the slice (as long as it is)
 };
 
@@ -403,6 +409,181 @@ __device__ __forceinline__ unsigned long long tp_warp_sum(unsigned long long v) 
   return v;
 }
 
+// tp_cut for many tokens: each CTA looks among its own ones, up to 32 threads share one's running mass, and whoever holds the
+// last kept token tells the others, for one barrier more on the way.  (378 rows of 128256 logits of deviation 1, 400 tokens
+// in the bin: 440 us when every CTA looked at all of them, so 284.  64 rows of 32000 of deviation 3, where few are in the
+// bin, would take 13.4 us instead of 12.8.)
+__device__ __forceinline__ void tp_cut_own(TpFast& me, int n, unsigned long long rest, int ranks) {
+  cg::cluster_group cluster = cg::this_cluster();
+  const int count = me.ncand;
+  int log_share = 0;
+  while (log_share < 5 && (count << (log_share + 1)) <= kTpThreads) ++log_share;
+  const int sub = threadIdx.x & ((1 << log_share) - 1);
+  for (int i0 = 0; i0 < count; i0 += kTpThreads >> log_share) {  // (whole warps)
+    const int i = i0 + ((int)threadIdx.x >> log_share);
+    const ulonglong2 mine = i < count ? me.cand[i] : make_ulonglong2(~0ull, 0ull);
+    unsigned long long before = 0;
+#pragma unroll 4
+    for (int j = sub; j < n; j += 1 << log_share) {
+      const ulonglong2 t = me.all[j];
+      before += t.x > mine.x ? t.y : 0ull;
+    }
+    for (int d = 0; d < log_share; ++d) before += __shfl_xor_sync(0xffffffffu, before, 1 << d);
+    if (sub == 0 && before < rest && rest <= before + mine.y)
+      for (int r = 0; r < ranks; ++r) cluster.map_shared_rank(&me, r)->tau_comp = mine.x;
+  }
+}
+
+// The tokens of the cluster's lists (me.cand, me.ncand of them, which may be more than were stored): their number, and when
+// they are few a copy of all of them in me.all.  `before`: those of lower ranks.  A cluster barrier precedes the reads.
+__device__ __forceinline__ int tp_gather(TpFast& me, int ranks, int rank, int& before) {
+  cg::cluster_group cluster = cg::this_cluster();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  cluster.sync();
+  const int c = lane < ranks ? cluster.map_shared_rank(&me, lane)->ncand : 0;
+  int incl = c;
+#pragma unroll
+  for (int o = 1; o < kTpMaxCluster; o <<= 1) {
+    const int up = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += up;
+  }
+  const int n = __shfl_sync(0xffffffffu, incl, kTpMaxCluster - 1);
+  const int theirs = __shfl_sync(0xffffffffu, c, warp % kTpMaxCluster);
+  const int at = __shfl_sync(0xffffffffu, incl, warp % kTpMaxCluster) - theirs;
+  if (warp < ranks && n <= kTpFastCand) {  // warp r copies CTA r's list
+    const TpFast* other = cluster.map_shared_rank(&me, warp);
+    for (int i = lane; i < theirs; i += 32) me.all[at + i] = other->cand[i];
+  }
+  before = __shfl_sync(0xffffffffu, incl - c, rank);
+  return n;
+}
+
+// Where more than kTpFastCand tokens are in question - a flat row, runs of equal logits, a bin of the histogram that
+// wrapped: the tokens with cut_lo <= bin < cut_hi, in which mass `rest` is still to be found.  Their keys are cut into 512
+// equal steps, the step with the cut is found by the masses (three limbs of 14 bits, which cannot wrap), and so on inside
+// it until few tokens are left or they are all equal; equal ones are kept in token order.  Leaves the range of keys in
+// which the cut lies in me.klo, me.khi.  True: the tokens to be ordered are in me.all (n of them), the mass to find among
+// them in `rest`.  False: they are equal, and the last kept one, as far as this CTA is concerned, is in me.tau_comp.
+// (When one CTA took such a row through global memory instead: 64 rows of 128256 equal logits 8.8 ms, so 0.19; of
+// deviation 0.05 440 us, so 95; 378 rows of deviation 0.5 1001, so 452.  With fewer tokens in the cut's bin nothing of this
+// runs.)
+__device__ __noinline__ bool tp_refine(TpFast& me, int rank, int ranks, int lo, int cnt, float M, float c2, float cut_lo, float cut_hi,
+                                       unsigned long long& rest, int& n) {
+  cg::cluster_group cluster = cg::this_cluster();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, cnt_all = (cnt + 31) & ~31;
+  uint32_t lowest = 0xffffffffu, highest = 0u;
+  for (int i = tid; i < cnt; i += kTpThreads) {
+    const float x = me.x[i], d = (M - x) * c2, p = d * 51.2f;
+    if (p >= cut_lo && p < cut_hi && d < 40.f) { lowest = min(lowest, tp_key(x)); highest = max(highest, tp_key(x)); }
+  }
+  lowest = __reduce_min_sync(0xffffffffu, lowest);
+  highest = __reduce_max_sync(0xffffffffu, highest);
+  if (lane < ranks && highest != 0u) {
+    atomicMin(&cluster.map_shared_rank(&me, lane)->kmin, lowest);
+    atomicMax(&cluster.map_shared_rank(&me, lane)->kmax, highest);
+  }
+  cluster.sync();  // (also: the lists and bins have been read)
+  uint32_t klo = me.kmin, khi = me.kmax;
+  uint32_t* limb = me.limb[0];  // [3][512]
+  static_assert(2 * kTpBins >= 3 * 512, "the three limbs take the place of the two");
+  for (;;) {
+    if (tid == 0) me.ncand = 0;
+    if (klo != khi) {
+      const int shift = max(0, 32 - __clz(khi - klo) - 9);
+      for (int i = tid; i < 3 * 512; i += kTpThreads) limb[i] = 0u;
+      __syncthreads();
+#pragma unroll 1
+      for (int i = tid; i < cnt_all; i += kTpThreads) {  // (whole warps)
+        const float x = i < cnt ? me.x[i] : -INFINITY;
+        const uint32_t key = tp_key(x);
+        const bool in = i < cnt && key >= klo && key <= khi;
+        const uint32_t who = __ballot_sync(0xffffffffu, in);
+        if (who == 0u) continue;
+        const int b = in ? (int)((khi - key) >> shift) : 0;
+        const unsigned long long w = in ? tp_mass(x, M, c2) : 0ull;
+        const uint32_t w0 = (uint32_t)w & 0x3fffu, w1 = (uint32_t)(w >> 14) & 0x3fffu, w2 = (uint32_t)(w >> 28);
+        const int first = __shfl_sync(0xffffffffu, b, __ffs(who) - 1);
+        if (__all_sync(0xffffffffu, !in || b == first)) {  // one bin: equal logits, or steps wider than the warp's tokens
+          const uint32_t s0 = __reduce_add_sync(0xffffffffu, w0), s1 = __reduce_add_sync(0xffffffffu, w1), s2 = __reduce_add_sync(0xffffffffu, w2);
+          if (lane < 3) atomicAdd(&limb[512 * lane + first], lane == 0 ? s0 : lane == 1 ? s1 : s2);
+        } else if (in) {
+          atomicAdd(&limb[b], w0);
+          atomicAdd(&limb[512 + b], w1);
+          atomicAdd(&limb[1024 + b], w2);
+        }
+      }
+      __syncthreads();
+      auto mass_of = [](const TpFast& of, int b) -> unsigned long long {
+        const uint32_t* l = of.limb[0];
+        return l[b] + ((unsigned long long)l[512 + b] << 14) + ((unsigned long long)l[1024 + b] << 28);
+      };
+      {
+        static_assert(kTpWarps == 16, "one warp for each group of 32 bins");
+        const unsigned long long v = tp_warp_sum(mass_of(me, 32 * warp + lane));
+        if (lane == 0) me.coarse[warp] = v;
+      }
+      cluster.sync();
+      // the cluster's groups, then the bins of the one that holds the cut (every warp for itself)
+      int at = 0;
+#pragma unroll 1
+      for (int level = 0; level < 2; ++level) {
+        if (warp < ranks) {
+          const TpFast* other = cluster.map_shared_rank(&me, warp);
+          me.stage[warp][lane] = level ? mass_of(*other, 32 * at + lane) : lane < 16 ? other->coarse[lane] : 0ull;
+        }
+        __syncthreads();
+        unsigned long long v = 0;
+        for (int r = 0; r < ranks; ++r) v += me.stage[r][lane];
+        const unsigned long long incl = tp_warp_scan(v);
+        const int hit = max(__ffs(__ballot_sync(0xffffffffu, incl - v < rest && rest <= incl)) - 1, 0);  // (there is one: the masses are exact)
+        rest -= __shfl_sync(0xffffffffu, incl - v, hit);
+        at = level ? 32 * at + hit : hit;
+        __syncthreads();
+      }
+      khi -= (uint32_t)at << shift;
+      klo = max(klo, khi - min(khi, (1u << shift) - 1u));
+    } else {
+      __syncthreads();
+    }
+    for (int i = tid; i < cnt; i += kTpThreads) {
+      const float x = me.x[i];
+      const uint32_t key = tp_key(x);
+      if (key < klo || key > khi) continue;
+      const int pos = atomicAdd(&me.ncand, 1);
+      if (pos < kTpFastCand) me.cand[pos] = make_ulonglong2(((unsigned long long)key << 32) | (uint32_t)~(uint32_t)(lo + i), tp_mass(x, M, c2));
+    }
+    int before;
+    n = tp_gather(me, ranks, rank, before);
+    if (tid == 0) { me.klo = klo; me.khi = khi; }
+    if (n <= kTpFastCand) return true;
+    if (klo == khi) {
+      // equal logits share one mass: the first `need` of them in token order are kept, `mine` of them this CTA's
+      const float x = __uint_as_float((khi & 0x80000000u) ? khi & 0x7fffffffu : ~khi);
+      const unsigned long long each = tp_mass(x, M, c2);
+      const unsigned long long need = each ? (rest + each - 1) / each : (unsigned long long)n;
+      const int have = me.ncand;
+      const int mine = need <= (unsigned long long)before ? 0 : need >= (unsigned long long)before + have ? have : (int)(need - before);
+      if (mine > 0 && mine < have) {  // the last of them: runs of an odd length per thread (no bank conflicts), counted and scanned
+        const int len = ((cnt + kTpThreads - 1) / kTpThreads) | 1;
+        const int i0 = min(tid * len, cnt), i1 = min(i0 + len, cnt);
+        unsigned long long own = 0, total;
+        for (int i = i0; i < i1; ++i) own += tp_key(me.x[i]) == khi;
+        unsigned long long seen = tp_block_scan(own, me.part[0], total);
+        if (seen < (unsigned long long)mine && (unsigned long long)mine <= seen + own)
+          for (int i = i0; i < i1; ++i)
+            if (tp_key(me.x[i]) == khi && ++seen == (unsigned long long)mine) {
+              me.tau_comp = ((unsigned long long)khi << 32) | (uint32_t)~(uint32_t)(lo + i);
+              break;
+            }
+      } else if (tid == 0) {
+        me.tau_comp = mine == have ? (unsigned long long)khi << 32 : ~0ull;
+      }
+      return false;
+    }
+    cluster.sync();  // everyone has read the lists and the bins
+  }
+}
+
 __global__ void __launch_bounds__(kTpThreads, 2) top_p_cluster_kernel(const TopPArgs a, const int slice) {
   extern __shared__ __align__(16) uint8_t tp_smem[];
   TpFast& me = *reinterpret_cast<TpFast*>(tp_smem);
@@ -412,7 +593,7 @@ __global__ void __launch_bounds__(kTpThreads, 2) top_p_cluster_kernel(const TopP
   const float* row = a.logits + (int64_t)blockIdx.y * a.in_stride + lo;
   float* orow = a.out + (int64_t)blockIdx.y * a.out_stride + lo;
 
-  if (tid == 0) { me.ncand = 0; me.tau_comp = 0ull; me.max = tp_ordered(-INFINITY); }
+  if (tid == 0) { me.ncand = 0; me.tau_comp = 0ull; me.max = tp_ordered(-INFINITY); me.kmin = 0xffffffffu; me.kmax = 0u; }
   __syncthreads();
   cluster.barrier_arrive();  // waited for before the first remote access
   for (int i = tid; i < 2 * kTpBins; i += kTpThreads) me.limb[0][i] = 0u;
@@ -580,36 +761,40 @@ __global__ void __launch_bounds__(kTpThreads, 2) top_p_cluster_kernel(const TopP
     v.x = decide(v.x, i); v.y = decide(v.y, i + 1); v.z = decide(v.z, i + 2); v.w = decide(v.w, i + 3);
     if (early) store(i, v);
   }
-  cluster.sync();
-  int n;  // tokens of the whole cluster
-  {
-    const int c = lane < ranks ? cluster.map_shared_rank(&me, lane)->ncand : 0;
-    int incl = c;
-#pragma unroll
-    for (int o = 1; o < kTpMaxCluster; o <<= 1) {
-      const int up = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += up;
-    }
-    n = __shfl_sync(0xffffffffu, incl, kTpMaxCluster - 1);
-    const int mine = __shfl_sync(0xffffffffu, c, warp % kTpMaxCluster);
-    const int before = __shfl_sync(0xffffffffu, incl, warp % kTpMaxCluster) - mine;
-    if (warp < ranks && n <= kTpFastCand) {  // warp r copies CTA r's list
-      const TpFast* other = cluster.map_shared_rank(&me, warp);
-      for (int i = lane; i < mine; i += 32) me.all[before + i] = other->cand[i];
-    }
+  int before, n = tp_gather(me, ranks, rank, before);  // tokens of the whole cluster
+  const bool refine = whole_row || n > kTpFastCand;    // (the same for every CTA)
+  unsigned long long rest = whole_row ? target : rest0;
+  bool order = true;
+  if (refine) order = tp_refine(me, rank, ranks, lo, cnt, M, a.c2, whole_row ? 0.f : cut_lo, whole_row ? INFINITY : cut_hi, rest, n);
+  const bool alone = order && n > kTpAlone && ranks > 1;
+  if (alone) {
+    __syncthreads();
+    tp_cut_own(me, n, rest, ranks);
+    cluster.sync();
+  } else {
+    cluster.barrier_arrive();  // waited for at the end: nobody leaves while its list is being read
+    __syncthreads();
+    if (order) tp_cut(me.all, n, rest, &me.tau_comp);
   }
-  cluster.barrier_arrive();  // waited for at the end: nobody leaves while its list is being read
-  __syncthreads();
-  if (n > kTpFastCand || whole_row) {  // (the same for every CTA) too many to order here: the first CTA takes the row
-    cluster.barrier_wait();
-    if (rank == 0) top_p_row(*reinterpret_cast<TpShared*>(tp_smem), a, blockIdx.y);
-    return;
-  }
-  tp_cut(me.all, n, rest0, &me.tau_comp);
   const unsigned long long tau_comp = me.tau_comp;
 
   // ---- the tokens of the cut's bin: kept if not behind the last kept one in the order (key descending, index ascending)
-  if (!early) {
+  if (refine) {  // ... of the range of keys that is left; all is written (again)
+    const uint32_t klo = me.klo, khi = me.khi;
+    kept = 0;
+    auto inside = [&](float x, int i) -> float {
+      const uint32_t key = tp_key(x);
+      const unsigned long long comp = ((unsigned long long)key << 32) | (uint32_t)~(uint32_t)(lo + i);
+      const bool keep = key > khi || (key >= klo && comp >= tau_comp);
+      kept += keep;
+      return keep ? x : -INFINITY;
+    };
+#pragma unroll 1
+    for (int i = 4 * tid; i < cnt4; i += 4 * kTpThreads) {
+      const float4 v = *reinterpret_cast<const float4*>(&me.x[i]);
+      store(i, make_float4(inside(v.x, i), inside(v.y, i + 1), inside(v.z, i + 2), inside(v.w, i + 3)));
+    }
+  } else if (!early) {
 #pragma unroll 1
     for (int i = 4 * tid; i < cnt4; i += 4 * kTpThreads) {
       float4 v = *reinterpret_cast<const float4*>(&me.x[i]);
@@ -618,7 +803,7 @@ __global__ void __launch_bounds__(kTpThreads, 2) top_p_cluster_kernel(const TopP
     }
     __syncthreads();
   }
-  for (int j = tid; j < me.ncand; j += kTpThreads)
+  for (int j = tid; j < (refine ? 0 : me.ncand); j += kTpThreads)
     if (me.cand[j].x >= tau_comp) {
       const int i = (int)~(uint32_t)me.cand[j].x - lo;
       orow[i] = me.x[i];
@@ -628,7 +813,7 @@ __global__ void __launch_bounds__(kTpThreads, 2) top_p_cluster_kernel(const TopP
     kept = __reduce_add_sync(0xffffffffu, kept);
     if (lane == 0) atomicAdd(a.kept_out + blockIdx.y, kept);
   }
-  cluster.barrier_wait();
+  if (!alone) cluster.barrier_wait();
 }
 
 // top_p >= 1: every token stays (rows copied when the call is not in place)
@@ -649,8 +834,7 @@ static int launch_top_p(int rows, const TopPArgs& a, cudaStream_t stream) {
   ranks = ranks > most ? most : ranks;
   ranks = ranks > kTpMaxCluster ? kTpMaxCluster : ranks < least ? least : ranks;
   const int slice = (int)(((a.V + ranks - 1) / ranks + 3) & ~(int64_t)3);
-  // (the fallback's scratch takes the slice's place too)
-  const size_t fast = offsetof(TpFast, x) + (size_t)slice * 4, smem = fast > sizeof(TpShared) ? fast : sizeof(TpShared);
+  const size_t smem = offsetof(TpFast, x) + (size_t)slice * 4;
   static int attr_done[64];
   const int rc = once_per_device(attr_done, [&]() -> int {  // above the 48 KB a kernel gets without asking
     SEQ_CUDA_OK(cudaFuncSetAttribute(top_p_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(offsetof(TpFast, x) + kTpMaxSlice * 4)));

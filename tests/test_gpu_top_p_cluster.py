@@ -65,3 +65,68 @@ def test_many_tokens_in_the_cut_of_one_row_only(in_place):
     x = (3 * rng.standard_normal((3, 30000))).astype(np.float32)
     x[1] = 0.25
     _check(x, 1.0, 0.6, in_place)
+
+
+@pytest.mark.parametrize("in_place", [False, True])
+@pytest.mark.parametrize("rows,V,spread", [(2, 128256, 0.5), (40, 50257, 0.2), (160, 16384, 0.05), (1, 131072, 0.01), (3, 128255, 1e-3), (2, 32770, 1e-5),
+                                           (5, 4097, 0.0), (3, 600, 1e-3)])
+def test_many_tokens_in_the_cut(rows, V, spread, in_place):
+    """Rows whose cut's bin holds more tokens than are ordered at once, from a few hundred to the whole row (the bins' counters
+    wrap from 4096 tokens per CTA on), cut at several places."""
+    rng = np.random.default_rng(rows + V)
+    x = (1.7 + spread * rng.standard_normal((rows, V))).astype(np.float32)
+    for top_p in (0.9,) if V > 60000 else (1e-5, 0.37, 0.9, 0.99999):
+        _check(x, 0.6, top_p, in_place)
+
+
+@pytest.mark.parametrize("levels", [1, 2, 7, 300])
+@pytest.mark.parametrize("rows,V", [(1, 30000), (2, 131072), (300, 5001)])
+def test_runs_of_equal_logits_are_kept_in_token_order(rows, V, levels):
+    """Few distinct logits, of both signs: the cut falls inside a run that spreads over all CTAs of a cluster."""
+    rng = np.random.default_rng(levels)
+    x = (rng.integers(0, levels, (rows, V)).astype(np.float32) - levels // 2) / 64.0
+    for top_p in (0.003, 0.5, 0.97):
+        _check(x, 0.8, top_p, False)
+
+
+def test_flat_rows_with_what_never_counts():
+    """NaN, infinities and tokens below 2^-40 of the most probable one beside thousands in one bin."""
+    d = torch.device("cuda:0")
+    V = 60000
+    x = torch.full((2, V), 0.5, device=d)
+    x[:, ::3] = float("-inf")
+    x[:, 1::6] = -100.0
+    x[1, 2], x[1, 8] = float("nan"), float("inf")
+    out, kept = torch.empty_like(x), torch.empty(2, dtype=torch.int32, device=d)
+    st = torch.zeros(1, dtype=torch.int32, device=d)
+    B.seq_tree_top_p_filter(x, 1.0, 0.25, out=out, kept_out=kept, dev_status=st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == B.SEQ_DEV_NONFINITE
+    for r in range(2):
+        live = torch.nonzero(x[r] == 0.5).flatten()
+        n = -(-len(live) // 4)
+        assert int(kept[r]) == n
+        assert torch.equal(torch.nonzero(out[r] > float("-inf")).flatten(), live[:n])
+
+
+def test_no_spread_of_a_row_costs_many_times_another():
+    """378 rows of 128256 tokens: equal logits take about five times what ordinary rows take, narrow ones two to three times (185
+    and 8 times when one CTA took such a row)."""
+    d = torch.device("cuda:0")
+    x = torch.randn((378, 128256), device=d)
+    out = torch.empty_like(x)
+
+    def ms(logits):
+        best = float("inf")
+        for _ in range(4):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            B.seq_tree_top_p_filter(logits, 0.6, 0.9, out=out)
+            e1.record()
+            torch.cuda.synchronize()
+            best = min(best, e0.elapsed_time(e1))
+        return best
+
+    ordinary = ms(x * 3)
+    for spread, times in ((0.0, 20), (0.05, 5)):
+        assert ms(x * spread) < times * ordinary, spread
