@@ -29,8 +29,9 @@ namespace cg = cooperative_groups;
 
 namespace seqtree {
 
-constexpr int kTpThreads = 512;
+constexpr int kTpThreads = 512;      // per CTA of a cluster
 constexpr int kTpWarps = kTpThreads / 32;
+constexpr int kTpRowThreads = 1024;  // of the one CTA that takes a row of a larger vocabulary
 constexpr float kTpScale = 1099511627776.f;  // 2^40
 constexpr int kTpCand = 1024;  // tokens of the cut's bin that are ordered in shared memory (more: radix select)
 
@@ -49,8 +50,8 @@ struct TpShared {
   // compare-and-swap loop): mass = lo + hi * 2^21 + top * 2^53, carries moved up when an add wraps
   uint32_t lo[2048], hi[2048], top[2048];
   uint32_t count[1024];
-  __align__(16) unsigned long long warp_tot[kTpWarps];
-  float warp_max[kTpWarps];
+  __align__(16) unsigned long long warp_tot[kTpRowThreads / 32];
+  float warp_max[kTpRowThreads / 32];
   // results of a level's search
   uint32_t sel_bin; unsigned long long sel_above; unsigned long long sel_mass; uint32_t sel_count;
   int32_t tie_limit;
@@ -82,7 +83,7 @@ __device__ __forceinline__ unsigned long long tp_mass(float x, float M, float c2
 template <typename F>
 __device__ __forceinline__ void tp_for_each(const float* row, int V, F f) {
   const int V4 = V & ~3;
-  constexpr int kStride = kTpThreads * 4;
+  constexpr int kStride = kTpRowThreads * 4;
   int i = threadIdx.x * 4;
   for (; i + 3 * kStride < V4; i += 4 * kStride) {
     float4 x[4];
@@ -106,10 +107,11 @@ __device__ __forceinline__ void tp_for_each(const float* row, int V, F f) {
         f(j, x[k].x); f(j + 1, x[k].y); f(j + 2, x[k].z); f(j + 3, x[k].w);
       }
   }
-  for (int t = V4 + threadIdx.x; t < V; t += kTpThreads) f(t, row[t]);
+  for (int t = V4 + threadIdx.x; t < V; t += kTpRowThreads) f(t, row[t]);
 }
 
 // Exclusive prefix sum over the block's threads in thread order; every thread also gets the total.
+template <int kThreads>
 __device__ __forceinline__ unsigned long long tp_block_scan(unsigned long long v, unsigned long long* warp_tot, unsigned long long& total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned long long inc = v;
@@ -123,7 +125,7 @@ __device__ __forceinline__ unsigned long long tp_block_scan(unsigned long long v
   __syncthreads();
   unsigned long long before = 0, all = 0;
 #pragma unroll
-  for (int w = 0; w < kTpWarps; w += 2) {
+  for (int w = 0; w < kThreads / 32; w += 2) {
     const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(&warp_tot[w]);
     if (w < warp) before += t.x;
     if (w + 1 < warp) before += t.y;
@@ -135,13 +137,13 @@ __device__ __forceinline__ unsigned long long tp_block_scan(unsigned long long v
 
 // Among `bins` bins of sh.hist taken from the highest index down, finds the one in which the running mass reaches
 // `target` (> 0, <= the bins' total); leaves its index, the mass above it, its own mass (and token count when
-// `with_count`) in sh.sel_*.  bins is 2048 or 1024: four or two bins per thread.
+// `with_count`) in sh.sel_*.  bins is 2048 or 1024: two or one per thread.
 __device__ __forceinline__ void tp_find_crossing(TpShared& sh, int bins, unsigned long long target, bool with_count) {
-  const int per = bins / kTpThreads;
+  const int per = bins / kTpRowThreads;
   const int hi = bins - 1 - (int)threadIdx.x * per;  // this thread's highest bin
   unsigned long long mine = 0, total;
   for (int b = 0; b < per; ++b) mine += sh.hist[hi - b];
-  unsigned long long above = tp_block_scan(mine, sh.warp_tot, total);
+  unsigned long long above = tp_block_scan<kTpRowThreads>(mine, sh.warp_tot, total);
   if (above < target && target <= above + mine) {
     for (int b = 0; b < per; ++b) {
       const unsigned long long m = sh.hist[hi - b];
@@ -164,8 +166,9 @@ __device__ __forceinline__ int tp_lbin(float x, float M, float c2) {
 
 // Among n tokens of the cut's bin, (key and index, mass) each, finds the last kept one: the first, in descending order, at
 // which the running mass reaches `rest`.  No sort: a token's running mass is the sum over those before it.
+template <int kThreads>
 __device__ __forceinline__ void tp_cut(const ulonglong2* tokens, int n, unsigned long long rest, unsigned long long* tau_comp) {
-  for (int i = threadIdx.x; i < n; i += kTpThreads) {
+  for (int i = threadIdx.x; i < n; i += kThreads) {
     const ulonglong2 mine = tokens[i];
     unsigned long long before = 0;
 #pragma unroll 4
@@ -178,14 +181,18 @@ __device__ __forceinline__ void tp_cut(const ulonglong2* tokens, int n, unsigned
   __syncthreads();
 }
 
-// One row by one CTA through global memory.
-__device__ __noinline__ void top_p_row(TpShared& sh, const TopPArgs& a, int row_index) {
+// One row by one CTA through global memory.  (64 rows of 151936 tokens: 85 us; with 512 threads,
+// and half the loads in flight, 132.)
+__global__ void __launch_bounds__(kTpRowThreads, 1) top_p_row_kernel(const TopPArgs a) {
+  extern __shared__ __align__(16) uint8_t tp_smem[];
+  TpShared& sh = *reinterpret_cast<TpShared*>(tp_smem);
+  const int row_index = blockIdx.x;
   const float* row = a.logits + (int64_t)row_index * a.in_stride;
   float* orow = a.out + (int64_t)row_index * a.out_stride;
   const int V = a.V, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
   // ---- the row maximum (NaN / +inf flagged and read as -inf), histogram cleared meanwhile
-  for (int i = threadIdx.x; i < 2048; i += kTpThreads) { sh.lo[i] = 0u; sh.hi[i] = 0u; sh.top[i] = 0u; }
+  for (int i = threadIdx.x; i < 2048; i += kTpRowThreads) { sh.lo[i] = 0u; sh.hi[i] = 0u; sh.top[i] = 0u; }
   if (threadIdx.x == 0) { sh.bad = 0; sh.kept = 0; sh.tie_limit = INT_MAX; sh.ncand = 0; sh.tau_comp = 0ull; }
   int bad = 0;
   float m = -INFINITY;
@@ -195,7 +202,7 @@ __device__ __noinline__ void top_p_row(TpShared& sh, const TopPArgs& a, int row_
   __syncthreads();
   float M = -INFINITY;
 #pragma unroll 1
-  for (int w = 0; w < kTpWarps; ++w) M = fmaxf(M, sh.warp_max[w]);
+  for (int w = 0; w < kTpRowThreads / 32; ++w) M = fmaxf(M, sh.warp_max[w]);
   if (bad) sh.bad = 1;
   if (M == -INFINITY) {  // no token with any mass: nothing to keep
     tp_for_each(row, V, [&](int i, float) { orow[i] = -INFINITY; });
@@ -228,15 +235,15 @@ __device__ __noinline__ void top_p_row(TpShared& sh, const TopPArgs& a, int row_
     }
   });
   __syncthreads();
-  for (int i = threadIdx.x; i < 2048; i += kTpThreads)
+  for (int i = threadIdx.x; i < 2048; i += kTpRowThreads)
     sh.hist[i] = (unsigned long long)sh.lo[i] + ((unsigned long long)sh.hi[i] << 21) + ((unsigned long long)sh.top[i] << 53);
   __syncthreads();
   unsigned long long target;
   {
     // the whole mass, then the mass the nucleus has to reach (rounded up, at least one unit)
     unsigned long long mine = 0, S;
-    for (int i = threadIdx.x; i < 2048; i += kTpThreads) mine += sh.hist[i];
-    tp_block_scan(mine, sh.warp_tot, S);
+    for (int i = threadIdx.x; i < 2048; i += kTpRowThreads) mine += sh.hist[i];
+    tp_block_scan<kTpRowThreads>(mine, sh.warp_tot, S);
     const double want = ceil(a.top_p * (double)S);
     target = want < 1.0 ? 1ull : (want >= (double)S ? S : (unsigned long long)want);
   }
@@ -262,11 +269,11 @@ __device__ __noinline__ void top_p_row(TpShared& sh, const TopPArgs& a, int row_
   uint32_t tau = 0;          // fallback only: key of the least probable kept token
   bool exact = ncand <= kTpCand;
   if (exact) {
-    tp_cut(cand, ncand, rest0, &sh.tau_comp);
+    tp_cut<kTpRowThreads>(cand, ncand, rest0, &sh.tau_comp);
   } else {
     // ---- many tokens in one bin (a flat row, runs of equal logits): radix select on the key bits inside the bin
     __syncthreads();
-    for (int i = threadIdx.x; i < 2048; i += kTpThreads) sh.hist[i] = 0ull;
+    for (int i = threadIdx.x; i < 2048; i += kTpRowThreads) sh.hist[i] = 0ull;
     __syncthreads();
     tp_for_each(row, V, [&](int, float x) {
       int b2 = 0;
@@ -278,7 +285,7 @@ __device__ __noinline__ void top_p_row(TpShared& sh, const TopPArgs& a, int row_
     const uint32_t p0 = sh.sel_bin;
     const unsigned long long above0 = sh.sel_above;
     __syncthreads();
-    for (int i = threadIdx.x; i < 2048; i += kTpThreads) sh.hist[i] = 0ull;
+    for (int i = threadIdx.x; i < 2048; i += kTpRowThreads) sh.hist[i] = 0ull;
     __syncthreads();
     tp_for_each(row, V, [&](int, float x) {
       int b2 = 0;
@@ -291,7 +298,7 @@ __device__ __noinline__ void top_p_row(TpShared& sh, const TopPArgs& a, int row_
     const uint32_t p1 = (p0 << 11) | sh.sel_bin;
     const unsigned long long above1 = above0 + sh.sel_above;
     __syncthreads();
-    for (int i = threadIdx.x; i < 1024; i += kTpThreads) { sh.hist[i] = 0ull; sh.count[i] = 0u; }
+    for (int i = threadIdx.x; i < 1024; i += kTpRowThreads) { sh.hist[i] = 0ull; sh.count[i] = 0u; }
     __syncthreads();
     tp_for_each(row, V, [&](int, float x) {
       int b2 = 0;
@@ -315,7 +322,7 @@ __device__ __noinline__ void top_p_row(TpShared& sh, const TopPArgs& a, int row_
     if (need < ties) {
       // the cut falls inside a run of equal logits: contiguous chunks per thread, a scan of the tie counts, and the
       // thread whose chunk holds the need-th tie finds its index
-      const int len = (V + kTpThreads - 1) / kTpThreads;
+      const int len = (V + kTpRowThreads - 1) / kTpRowThreads;
       const int lo = min((int)threadIdx.x * len, V), hi = min(lo + len, V);
       unsigned long long cnt = 0;
       for (int i = lo; i < hi; ++i) {
@@ -323,7 +330,7 @@ __device__ __noinline__ void top_p_row(TpShared& sh, const TopPArgs& a, int row_
         cnt += tp_key(tp_clean(row[i], b2)) == tau;
       }
       unsigned long long total;
-      const unsigned long long before = tp_block_scan(cnt, sh.warp_tot, total);
+      const unsigned long long before = tp_block_scan<kTpRowThreads>(cnt, sh.warp_tot, total);
       if (before < need && need <= before + cnt) {
         unsigned long long seen = before;
         for (int i = lo; i < hi; ++i) {
@@ -355,11 +362,6 @@ __device__ __noinline__ void top_p_row(TpShared& sh, const TopPArgs& a, int row_
     if (a.kept_out != nullptr) a.kept_out[row_index] = sh.kept;
     if (sh.bad) dev_flag(a.dev_status, SEQ_DEV_NONFINITE);
   }
-}
-
-__global__ void __launch_bounds__(kTpThreads) top_p_row_kernel(const TopPArgs a) {
-  extern __shared__ __align__(16) uint8_t tp_smem[];
-  top_p_row(*reinterpret_cast<TpShared*>(tp_smem), a, blockIdx.x);
 }
 
 // One row by one cluster, the CTA's slice in shared memory.
@@ -568,7 +570,7 @@ __device__ __noinline__ bool tp_refine(TpFast& me, int rank, int ranks, int lo, 
         const int i0 = min(tid * len, cnt), i1 = min(i0 + len, cnt);
         unsigned long long own = 0, total;
         for (int i = i0; i < i1; ++i) own += tp_key(me.x[i]) == khi;
-        unsigned long long seen = tp_block_scan(own, me.part[0], total);
+        unsigned long long seen = tp_block_scan<kTpThreads>(own, me.part[0], total);
         if (seen < (unsigned long long)mine && (unsigned long long)mine <= seen + own)
           for (int i = i0; i < i1; ++i)
             if (tp_key(me.x[i]) == khi && ++seen == (unsigned long long)mine) {
@@ -774,7 +776,7 @@ __global__ void __launch_bounds__(kTpThreads, 2) top_p_cluster_kernel(const TopP
   } else {
     cluster.barrier_arrive();  // waited for at the end: nobody leaves while its list is being read
     __syncthreads();
-    if (order) tp_cut(me.all, n, rest, &me.tau_comp);
+    if (order) tp_cut<kTpThreads>(me.all, n, rest, &me.tau_comp);
   }
   const unsigned long long tau_comp = me.tau_comp;
 
@@ -843,7 +845,7 @@ static int launch_top_p(int rows, const TopPArgs& a, cudaStream_t stream) {
   });
   if (rc != SEQ_OK) return rc;
   if (!cluster) {
-    top_p_row_kernel<<<rows, kTpThreads, sizeof(TpShared), stream>>>(a);
+    top_p_row_kernel<<<rows, kTpRowThreads, sizeof(TpShared), stream>>>(a);
     SEQ_CUDA_OK(cudaGetLastError());
     return SEQ_OK;
   }

@@ -130,3 +130,28 @@ def test_no_spread_of_a_row_costs_many_times_another():
     ordinary = ms(x * 3)
     for spread, times in ((0.0, 20), (0.05, 5)):
         assert ms(x * spread) < times * ordinary, spread
+
+
+@pytest.mark.parametrize("spread,top_p", [(3.0, 0.9), (0.5, 0.37), (0.0, 0.6), (1e-3, 0.97)])
+@pytest.mark.parametrize("V", [131073, 151936])
+def test_rows_larger_than_a_cluster(V, spread, top_p):
+    """One CTA per row, with and without the radix select."""
+    x = (0.3 + spread * np.random.default_rng(V).standard_normal((3, V))).astype(np.float32)
+    _check(x, 0.8, top_p, V == 151936)
+
+
+def test_rows_larger_than_a_cluster_keep_enough_loads_in_flight():
+    """A row of 131073 tokens on one CTA of 1024 threads takes about 72 us; on 512 threads it took 104."""
+    d = torch.device("cuda:0")
+    x = 3 * torch.randn((64, 131076), device=d)[:, :131073]
+    x, out = torch.empty((64, 131076), device=d)[:, :131073].copy_(x), torch.empty((64, 131076), device=d)[:, :131073]
+    best = float("inf")
+    for _ in range(6):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record()
+        for _ in range(5):
+            B.seq_tree_top_p_filter(x, 0.6, 0.9, out=out)
+        e1.record()
+        torch.cuda.synchronize()
+        best = min(best, e0.elapsed_time(e1) / 5 * 1e3)
+    assert best < 100
