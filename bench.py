@@ -476,7 +476,7 @@ def top_p_leg(cfg, ver_h, T, dev, stream, peaks, top_p=0.9) -> dict:
             "gpu_launches_per_call": 1,
             "roofline": {"bound": "hbm", "achieved": gbs, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                          "frac": gbs / peaks["hbm_gbs"], "algorithmic_bytes": nbytes, "traffic": None},
-            "note": "every row read once and written once (the four re-reads of the select come from L2); outside the timed step"}
+            "note": "every row read once and written once (the passes in between are over shared memory); outside the timed step"}
 
 
 def verify_batch_leg(cfg, parent, ver_h, T, dev, stream) -> dict:
@@ -527,7 +527,7 @@ def verify_batch_leg(cfg, parent, ver_h, T, dev, stream) -> dict:
         raise RuntimeError(f"verify_batch: dev_status {int(status.item())}, {same} of {R} bonus tokens equal to single launches")
     return {"requests": R, "us_per_launch": us_b, "us_per_request": us_b / R, "us_per_request_single_launches": us_s / R,
             "gpu_launches_per_call": 1, "bonus_tokens_equal_to_single_launches": f"{same}/{R}",
-            "note": "one cluster per request: of 16 CTAs (rows in registers) while the batch fits the GPU side by side, else of 8; outside the timed step"}
+            "note": "one cluster per request: of 16 CTAs while the batch fits the GPU side by side, else of 8; rows in registers but for large batches beyond 65536 tokens; outside the timed step"}
 
 
 def attention_batch_leg(cfg, parent, attn_h, dev, stream, peaks) -> dict:

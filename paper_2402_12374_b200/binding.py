@@ -314,7 +314,7 @@ class VerifyCall:
                  path=None, path_len=None, bonus_token=None, residual_out=None, next_child_out=None,
                  all_nodes: bool = False, dev_status=None, specinfer: bool = False, target_sample: bool = False,
                  schedule: str = "auto", workspace=None):
-        """schedule: "auto" (node-parallel where it applies), "walk" or "nodes" (forced)."""
+        """schedule: "auto" (the walk), "walk" or "nodes" (the node-parallel one, where it applies)."""
         n, V = target_logits.shape
         dev = target_logits.device
         if path is None:

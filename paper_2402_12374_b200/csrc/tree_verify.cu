@@ -1,5 +1,5 @@
 // seq_tree_verify: entry points, argument checks and the choice of kernel; and the walk of Algorithm 2 from the root
-// with its rows in SHARED memory (sampling from the target at T > 0, the every-node hook, batches of requests, and
+// with its rows in SHARED memory (the every-node hook, vocabularies beyond 131072, large batches beyond 65536 tokens, and
 // devices that cannot place a cluster of 16 CTAs).  The default walk keeps its rows in registers
 // (tree_verify_walk.cu); the node-parallel schedule is tree_verify_nodes.cu.
 //
