@@ -50,6 +50,36 @@ def test_clusters_of_every_size(hkv, n, L):
     G.check_attention(_inputs(hkv, 1, n, L, "bf16"))
 
 
+def _launched_cluster_size(hkv, n, L):
+    """CTAs along the key range of the attention's launch, read off a captured graph (the grid's z extent)."""
+    from cuda.bindings import driver
+
+    d = G.dev()
+    ai = _inputs(hkv, 1, n, L, "bf16")
+    call = B.AttentionCall(ai.q.to(d), ai.k_cache.to(d), ai.v_cache.to(d), None, L, parent=ai.parent.to(d))
+    call.run()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call.run()
+    raw = driver.CUgraph(graph.raw_cuda_graph())
+    _, _, count = driver.cuGraphGetNodes(raw)
+    assert count == 1
+    rc, nodes, _ = driver.cuGraphGetNodes(raw, count)
+    assert rc == driver.CUresult.CUDA_SUCCESS
+    rc, params = driver.cuGraphKernelNodeGetParams(nodes[0])
+    assert rc == driver.CUresult.CUDA_SUCCESS
+    return params.gridDimZ
+
+
+def test_the_shapes_above_take_clusters_of_every_size():
+    """Should the plan's constants or the device's occupancy move, the test above would go on passing without its purpose."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the shapes are chosen for 148 SMs")
+    sizes = [_launched_cluster_size(*shape) for shape in [(60, 2, 1250), (40, 3, 1100), (32, 2, 1030), (24, 3, 1590), (16, 4, 3000), (1, 5, 2200), (1, 4, 4000)]]
+    assert set(sizes) == set(range(2, 9)), sizes
+
+
 @pytest.mark.parametrize("hkv,group,n,L", [(1, 1, 1, 0), (2, 1, 8, 31), (1, 1, 9, 119), (1, 2, 8, 128), (2, 3, 11, 97), (1, 1, 32, 96), (1, 1, 33, 224),
                                            (2, 4, 16, 255), (1, 5, 13, 64), (3, 1, 65, 63), (1, 150, 2, 40), (1, 1, 1, 3000)])
 def test_single_precision_tiles(hkv, group, n, L):
