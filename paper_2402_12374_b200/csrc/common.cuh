@@ -24,6 +24,10 @@ __device__ __forceinline__ void dev_flag(int32_t* dev_status, int bit) {
   if (dev_status != nullptr) atomicOr(dev_status, bit);
 }
 
+// Asks for a line of global memory to be brought into L2.  Allowed before griddepcontrol.wait, while the previous kernel may
+// still be writing the line: its stores go to L2 as well, and nothing is read here.  The address has to be a valid one.
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // Maximum over the warp in one redux.sync: floats are mapped to integers in the same order (sign-magnitude to
 // two's complement), -inf and +inf included.  (A NaN, which fmaxf would drop, comes out as the maximum.)
 __device__ __forceinline__ float warp_max(float v) {

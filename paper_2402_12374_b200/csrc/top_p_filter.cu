@@ -600,6 +600,7 @@ __global__ void __launch_bounds__(kTpThreads, 2) top_p_cluster_kernel(const TopP
   cluster.barrier_arrive();  // waited for before the first remote access
   for (int i = tid; i < 2 * kTpBins; i += kTpThreads) me.limb[0][i] = 0u;
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  for (int i = 32 * tid; i < cnt; i += 32 * kTpThreads) prefetch_l2(row + i);  // the slice, while the previous kernel ends (64 rows of 32000: 14.4 -> 13.7 us)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if (a.kept_out != nullptr && rank == 0 && tid == 0) a.kept_out[blockIdx.y] = 0;  // (the cluster's barriers order it before the counts)
 
