@@ -28,11 +28,17 @@
 // the CTA-wide barrier.  Many units of long tiles go to the kernel of tree_attention_stream.cu.
 //
 // Merge.  The CTAs that share (tile, kv head) form a thread-block cluster along the key range (cs = 1 .. 8).  Each sends
-// its rows' (m, l) into every CTA as soon as its two chains are done; that travels while it reads its accumulators out of
-// tensor memory.  Then it knows the rows' common maximum and sum, scales its partial to its share of the final output, and
-// sends each slice of 8 output columns to the CTA that owns it (the K/V stages, dead by then, receive them).  After a
-// cluster barrier an owner has only additions left.  No workspace, no second kernel.  (Against unscaled pieces, with the
-// owner working out every contributor's factor behind the barrier: 64 nodes on 1024 keys of 32 heads 9.95 -> 9.6 us.)
+// its rows' (m, l) into every CTA as soon as its two chains are done, puts its piece into its V stages, slice by slice of 8
+// output columns in the order of their owners, and copies each owner its slices in one go (into the K stages: an MMA commit of
+// every chain of the cluster says that no S is to come).  While the pieces travel each owner works out the rows' common
+// maximum, sum and the pieces' shares; then it adds its slices up.  Both transfers count their bytes into an mbarrier of the
+// receiver; the only cluster barriers are at the start and, off the path, at the end.  No workspace, no second kernel.  (With
+// scaled pieces stored one by one and three cluster barriers, whose release waits for all of a warp's stores: 64 nodes on 1024
+// keys of 32 heads 9.1 us instead of 8.5, 128 on 2048 of 40 13.8 / 13.3.)
+//
+// Most of the code around the loop over blocks runs once per launch, at the rate at which its instructions are fetched, so it
+// is kept short: quotients as products, loops that are not unrolled (merge with shares in registers and the loop over
+// contributors unrolled: 8.7 us).
 //
 // Masking: key j < prefix_len is visible; key prefix_len + t is visible iff bit t of the row's
 // ancestor mask; masked scores become -inf before the maximum, so their probability is exactly 0.
@@ -65,14 +71,17 @@ constexpr uint32_t kKvHalf = kKvBytes / 2;       // one 64-row x 64-element sub-
 struct UmmaSmem {
   // all tiles 1024-byte aligned (128-byte swizzle atoms are 8 rows x 128 B)
   uint8_t q[kTileBytes];
-  uint8_t k[2][2][kKvBytes];  // [chain][stage]; after the last block these 64 KB receive the cluster merge
-  uint8_t v[2][2][kKvBytes];  // [chain][stage]
+  uint8_t receive[20480];     // with the K stages behind it, once their S are done: the other CTAs' pieces (cluster merge)
+  uint8_t k[2][2][kKvBytes];  // [chain][stage]
+  uint8_t v[2][2][kKvBytes];  // [chain][stage]; after the last block: this CTA's piece (cluster merge)
   float2 ml_chain[2][kTileM];                // [chain]: (m, l) of every row of the two chains of this CTA
   float2 ml_cta[kMaxClusterSplit][kTileM];   // (m, l) of every row of every CTA of the cluster, after its chains are merged
   uint64_t q_full;
   uint64_t k_full[2][2], k_empty[2][2], v_full[2][2], v_empty[2][2], s_full[2][2], p_full[2][2];  // [chain][stage]
   uint64_t pv_done[2];                       // [chain]: one phase per block of the chain
   uint64_t all_done[2];                      // [chain]: every MMA of the chain has completed
+  uint64_t k_free;                           // cluster merge: no chain of any CTA has an S to come, the K stages may be written
+  uint64_t ml_full, data_full;               // ... and this CTA's ml_cta and pieces are here
   uint32_t tmem_base;
   volatile int abort_flag;
   // mask from the parent array: the tree, and the ancestor rows of the current tile's nodes (row stride 33 words)
@@ -80,7 +89,8 @@ struct UmmaSmem {
   uint32_t tile_mask[kTileM][SEQ_MAX_TREE / 32 + 1];
 };
 
-static_assert(offsetof(UmmaSmem, v) == offsetof(UmmaSmem, k) + sizeof(UmmaSmem::k), "the cluster merge receives into k and v as one buffer");
+static_assert(offsetof(UmmaSmem, k) == offsetof(UmmaSmem, receive) + sizeof(UmmaSmem::receive) && sizeof(UmmaSmem::receive) + sizeof(UmmaSmem::k) >= 7 * 3 * 4096,
+              "the cluster merge receives cs * ceil(16 / cs) slices of 4 KB in one buffer");
 
 struct UmmaArgs {
   int32_t n, L_host, Hq, Hkv, group, mask_wpr, splits, nodes_per_tile, tiles;
@@ -105,7 +115,6 @@ struct UmmaArgs {
 };
 
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 // The address of a shared-memory word of CTA `rank` of the cluster, and stores to it.
 __device__ __forceinline__ uint32_t remote_smem(uint32_t addr, int rank) {
@@ -113,12 +122,22 @@ __device__ __forceinline__ uint32_t remote_smem(uint32_t addr, int rank) {
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(addr), "r"(rank));
   return d;
 }
-__device__ __forceinline__ void st_cluster4(uint32_t addr, const float* x) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]) : "memory");
+// An asynchronous store of 8 bytes, and a copy of shared memory, to another CTA of the cluster; both count their bytes into an
+// mbarrier there.
+__device__ __forceinline__ void st_async2(uint32_t addr, float x, float y, uint32_t bar) {
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];"
+               ::"r"(addr), "r"(__float_as_uint(x)), "r"(__float_as_uint(y)), "r"(bar) : "memory");
 }
-__device__ __forceinline__ void st_cluster2(uint32_t addr, float x, float y) {
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(x), "f"(y) : "memory");
+__device__ __forceinline__ void copy_to_cta(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst), "r"(src), "r"(bytes), "r"(bar) : "memory");
 }
+// Arrives on the mbarrier at the same place of every CTA in `mask` when the MMAs issued so far have completed.
+__device__ __forceinline__ void tc_commit_cluster(uint64_t* bar, uint32_t mask) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)), "h"((uint16_t)mask) : "memory");
+}
+// The 16 slices of 8 output columns are owned round-robin: slice s by CTA s % cs, as its slot s / cs.
+__device__ __forceinline__ int slices_of(int cta, const UmmaArgs& a) { return a.slices_each + (cta < a.slices_more); }
+__device__ __forceinline__ int slices_before(int cta, const UmmaArgs& a) { return cta * a.slices_each + min(cta, a.slices_more); }
 enum { kGrid, kCluster };  // the schedule: a CTA per unit, a cluster of CTAs per unit
 // kFineP: P enters its product as two 16-bit pieces, the rounded value and the rest, each in a run of MMAs of its own.  For
 // the groups of heads that do not divide 128, whose probabilities are held to single precision (the other groups round P
@@ -139,7 +158,6 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
   int utrace_i = 0;
 #endif
   const int split = kMode == kCluster ? blockIdx.z : 0;  // the cluster spans blockIdx.z
-  if (kMode == kCluster) cluster_arrive_relaxed();  // "this CTA runs": waited for before the first remote store
   if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 10);
 #ifdef SEQ_TRACE
   const unsigned cta_lin = (blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
@@ -161,6 +179,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
   take_blocks();
   // A stage barrier counts the blocks its chain has processed so far; q_full and all_done[] have one phase.
   const uint32_t live_rows = (uint32_t)((i1 - i0) * a.group);
+  const uint32_t plane = ((live_rows + 31u) & ~31u) * 16u;  // cluster merge: bytes of four columns of all rows
   if (threadIdx.x == 0) {  // the barriers of the first loads, which this thread requests below
     mbar_init(&sm->q_full, 1);
     mbar_init(&sm->k_full[0][0], 1);
@@ -181,8 +200,17 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
       mbar_init(&sm->pv_done[c], 1);
       mbar_init(&sm->all_done[c], 1);  // one arriver: the chain's MMA warp
     }
+    if (kMode == kCluster) { mbar_init(&sm->k_free, 2 * a.splits); mbar_init(&sm->ml_full, 1); mbar_init(&sm->data_full, 1); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (kMode == kCluster) {
+      mbar_expect_tx(&sm->ml_full, (uint32_t)a.splits * live_rows * 8u);
+      mbar_expect_tx(&sm->data_full, (uint32_t)(a.splits - 1) * (uint32_t)slices_of(split, a) * 2u * plane);
+    }
     sm->abort_flag = 0;
+  }
+  if (kMode == kCluster) {  // "this CTA runs and its barriers count": waited for before anything is sent
+    __syncwarp();
+    cluster_arrive_relaxed();
   }
   // ... and everything above ran while the previous kernel in the stream was still finishing.  Nothing before this
   // line reads or writes global memory.
@@ -269,6 +297,11 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
       const int c = warp - 1;
       const int n_c = nblk > c ? (nblk - c + 1) >> 1 : 0;  // blocks of this chain
       const bool q_here = nblk > 0 && mbar_wait(sm, &sm->q_full, 0, a.dev_status);
+      if (kMode == kCluster) {
+        __syncwarp();
+        cluster_wait();
+      }
+      const uint32_t everyone = (1u << a.splits) - 1u;
       if (n_c > 0) {
         bool go = q_here;
         const uint32_t q_lo = desc_lo(smem_u32(sm->q), 16);
@@ -283,6 +316,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
             mma_qk<kHalfBytes, kKvHalf>(d, q_lo, desc_lo(smem_u32(sm->k[c][b]), 16), a.idesc_qk);
             tc_commit(&sm->s_full[c][b]);  // the row threads wait for this one
             tc_commit(&sm->k_empty[c][b]);
+            if (kMode == kCluster && u + 1 == n_c) tc_commit_cluster(&sm->k_free, everyone);
           }
           __syncwarp();
           if (lane == 0) UTRACE(c == 0 ? 1 : 3, 2);
@@ -329,15 +363,17 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
         }
         if (elect_one()) tc_commit(&sm->all_done[c]);  // arrives when every MMA of this chain has completed
         __syncwarp();
-      } else if (nblk > 0 && lane == 0) {
-        mbar_arrive(&sm->all_done[c]);  // a chain without blocks
+      } else if (lane == 0) {  // a chain without blocks
+        if (nblk > 0) mbar_arrive(&sm->all_done[c]);
+        if (kMode == kCluster)
+          for (int q = 0; q < a.splits; ++q)
+            asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(remote_smem(smem_u32(&sm->k_free), q)) : "memory");
       }
       __syncwarp();
     }
-    if (kMode == kCluster) {  // the cluster barriers of the merge (see the row threads)
-      cluster_wait();
-      cluster_arrive_relaxed();
-      cluster_wait();
+    if (kMode == kCluster) {  // (nobody leaves before every piece has arrived, see the row threads)
+      __syncwarp();
+      if (warp == 0 || warp == 3) cluster_wait();
       cluster_arrive_relaxed();
       cluster_wait();
     }
@@ -541,11 +577,9 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
       __syncwarp();
       cluster_wait();  // every CTA of the cluster runs
       if (chain == 0 && row_valid) {
-        const uint32_t to = smem_u32(&sm->ml_cta[split][r]);
-        for (int q = 0; q < a.splits; ++q) st_cluster2(remote_smem(to, q), M, Lc);
+        const uint32_t to = smem_u32(&sm->ml_cta[split][r]), bar = smem_u32(&sm->ml_full);
+        for (int q = 0; q < a.splits; ++q) st_async2(remote_smem(to, q), M, Lc, remote_smem(bar, q));
       }
-      __syncwarp();
-      cluster_arrive_release();
     }
     const uint32_t oA = tmem + 256u + lane_sel + 64u * chain, oB = oA + 128u;
     uint64_t* m2 = reinterpret_cast<uint64_t*>(merged);
@@ -586,54 +620,62 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
       if (chain == 0 && a.lse != nullptr) a.lse[(size_t)h * a.n + i] = (M + log2f(Lc)) * kLn2;
     }
   } else {
-    // Step 2, across the cluster (cs = 2 .. 8 CTAs along the key range).  The 16 slices of 8 output columns are owned
-    // round-robin: slice s by CTA s % cs, as its slot s / cs.  An owner receives into its K and V stages (adjacent in
-    // shared memory: cs * ceil(16 / cs) * 4 KB <= 84 KB of their 128 KB), as float4 planes [contributor][slot][half][row].
-    const int cs = a.splits, slots = a.slots;  // (any cs from 2 to 8; the last slots of some CTAs may be empty)
-    cluster_wait();  // every CTA's (m, l) is here, and every CTA is done with its K and V stages
-    if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 7);
-    float Mg = -INFINITY;
-    for (int q = 0; q < cs; ++q) Mg = fmaxf(Mg, sm->ml_cta[q][r].x);
-    float Ls = 0.f;
-    for (int q = 0; q < cs; ++q) {
-      const float2 mlq = sm->ml_cta[q][r];
-      if (mlq.x != -INFINITY) Ls += mlq.y * ex2(mlq.x - Mg);
-    }
-    const uint32_t recv = smem_u32(&sm->k[0][0][0]);
-    // (rows past the tile's last node are padding: nothing of theirs is pushed, reduced or stored)
-    if (row_valid) {
-      const float f = M == -INFINITY ? 0.f : ex2(M - Mg) / Ls;  // some CTA saw the row's own key, so Ls > 0
-      const uint64_t f2 = pair_of(f, f);
-      uint64_t* m2 = reinterpret_cast<uint64_t*>(merged);
-#pragma unroll
-      for (int e = 0; e < 32; ++e) m2[e] = mul2(m2[e], f2);
+    // Step 2, across the cluster (cs = 2 .. 8 CTAs along the key range).  The piece goes into the V stages, slice by slice in
+    // the order of the owners, as float4 planes [half][row]; one copy takes an owner its slices, into its receive buffer
+    // [contributor][slot][half][row].
+    const int cs = a.splits, slots = a.slots;  // (the last slots of some CTAs may be empty)
+    const uint32_t piece = smem_u32(&sm->v[0][0][0]), receive = smem_u32(&sm->receive[0]);
+    if (row_valid) {  // (rows past the tile's last node are padding: nothing of theirs is written, reduced or stored)
       int slot = chain ? a.half_slot : 0, owner = chain ? a.half_owner : 0;
-      const uint32_t to = recv + 16u * (uint32_t)(split * slots * 2 * kTileM + r);
 #pragma unroll
       for (int j = 0; j < 8; ++j) {
-        const uint32_t dst = remote_smem(to + 16u * (uint32_t)(slot * 2 * kTileM), owner);
-        st_cluster4(dst, merged + 8 * j);
-        st_cluster4(dst + 16u * kTileM, merged + 8 * j + 4);
+        float4* to = reinterpret_cast<float4*>(&sm->v[0][0][0] + (uint32_t)(slices_before(owner, a) + slot) * 2u * plane) + r;
+        to[0] = make_float4(merged[8 * j], merged[8 * j + 1], merged[8 * j + 2], merged[8 * j + 3]);
+        to[plane / 16u] = make_float4(merged[8 * j + 4], merged[8 * j + 5], merged[8 * j + 6], merged[8 * j + 7]);
         if (++owner == cs) { owner = 0; ++slot; }
       }
     }
+    fence_async_smem();
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    if (warp == 4) {
+      mbar_wait(sm, &sm->k_free, 0, a.dev_status);  // (on a timeout the copies go out all the same: the others count on them)
+      if (lane < cs && lane != split)
+        copy_to_cta(remote_smem(receive + (uint32_t)(split * slots) * 2u * plane, lane), piece + (uint32_t)slices_before(lane, a) * 2u * plane,
+                    (uint32_t)slices_of(lane, a) * 2u * plane, remote_smem(smem_u32(&sm->data_full), lane));
+      __syncwarp();
+    }
     if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 13);
+    // The rows' common maximum and sum, and each piece's share of the output, while the pieces travel.
+    mbar_wait(sm, &sm->ml_full, 0, a.dev_status);
+    float Mg = -INFINITY, Ls = 0.f;
+#pragma unroll 1
+    for (int q = 0; q < cs; ++q) {  // (one pass: the sum so far follows the maximum)
+      const float2 ml = sm->ml_cta[q][r];
+      const float m = fmaxf(Mg, ml.x);
+      if (m != -INFINITY) Ls = Ls * ex2(Mg - m) + ml.y * ex2(ml.x - m);
+      Mg = m;
+    }
+    const float inv = 1.f / Ls;  // some CTA saw the row's own key, so Ls > 0
+    if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 7);
+    mbar_wait(sm, &sm->data_full, 0, a.dev_status);
     __syncwarp();
-    cluster_arrive_release();
-    cluster_wait();
+    cluster_arrive_relaxed();  // every piece for this CTA is here: its senders may leave
     if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 8);
-    const ulonglong2* mine = reinterpret_cast<const ulonglong2*>(&sm->k[0][0][0]) + r;
     if (row_valid)
       for (int slot = chain; slot * cs + split < 16; slot += 2) {  // the two warp groups share this CTA's slots
-        const ulonglong2* src = mine + slot * 2 * kTileM;
-        ulonglong2 x = src[0], y = src[kTileM];
-        for (int q = 1; q < cs; ++q) {
-          src += slots * 2 * kTileM;
-          const ulonglong2 u = src[0], v = src[kTileM];
-          x.x = add2(x.x, u.x); x.y = add2(x.y, u.y); y.x = add2(y.x, v.x); y.y = add2(y.y, v.y);
+        uint64_t x[4] = {0ull, 0ull, 0ull, 0ull};
+#pragma unroll 2
+        for (int q = 0; q < cs; ++q) {
+          const uint8_t* at = q == split ? &sm->v[0][0][0] + (uint32_t)(slices_before(split, a) + slot) * 2u * plane
+                                         : &sm->receive[0] + (uint32_t)(q * slots + slot) * 2u * plane;
+          const ulonglong2 u = *(reinterpret_cast<const ulonglong2*>(at) + r), w = *(reinterpret_cast<const ulonglong2*>(at + plane) + r);
+          const float f = ex2(sm->ml_cta[q][r].x - Mg) * inv;
+          const uint64_t f2 = pair_of(f, f);
+          x[0] = fma2(u.x, f2, x[0]); x[1] = fma2(u.y, f2, x[1]); x[2] = fma2(w.x, f2, x[2]); x[3] = fma2(w.y, f2, x[3]);
         }
         float o[8];
-        unpair(x.x, o[0], o[1]); unpair(x.y, o[2], o[3]); unpair(y.x, o[4], o[5]); unpair(y.y, o[6], o[7]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) unpair(x[e], o[2 * e], o[2 * e + 1]);
         uint4 val;
         val.x = pack2<kBf16>(o[0], o[1]);
         val.y = pack2<kBf16>(o[2], o[3]);
@@ -642,12 +684,13 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
         *reinterpret_cast<uint4*>(out_row + 2 * (8 * (slot * cs + split))) = val;
       }
     if (split == 0 && chain == 0 && row_valid && a.lse != nullptr) a.lse[(size_t)h * a.n + i] = (Mg + log2f(Ls)) * kLn2;
+    __syncwarp();
+    cluster_wait();
   }
   if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 9);
 #ifdef SEQ_TRACE
   if (threadIdx.x == 128 && cta_lin < 1024) g_cta_times[cta_lin][1] = gtimer();
 #endif
-  // no remote access happens after the last cluster barrier, so CTAs may leave independently
   tc_fence_before();
   __syncthreads();  // pairs with warp group 0, whose MMA warp then frees the tensor memory
 }
