@@ -15,11 +15,18 @@
 // global memory, in four passes, or with more than 1024 tokens in the cut's bin in seven with a radix select on the logit
 // bits (11 + 11 + 10).
 //
-// What bounds it: the chain of exchanges for a few rows, HBM for many.  64 rows of 32000 tokens: 29.7 us with one CTA of
-// 1024 threads per row reading it four times and adding every token to the histogram, 13.2 so (about a dozen exchanges and
-// barriers of 0.5 to 1 us each around 4 us of passes); one row 28.6 -> 8.0; 127 rows of 128256 89 -> 81.
+// What bounds it: the chain of exchanges for a few rows, instruction issue for many (75 instructions for each token, 58 % of
+// the issue slots, at 512 rows of 32000).  64 rows of 32000 tokens: 29.7 us with one CTA of 1024 threads per row reading it
+// four times and adding every token to the histogram, 13.6 with a cluster per row that worked out every token's bin in two
+// passes and queued the histogram's tokens by votes, 12.5 so: estimates to a margin tell most tokens off, their mass is taken
+// without a branch, the histogram's tokens wait in lists of the threads' own.  127 rows of 128256 71 -> 61 us, 378 192 -> 168,
+// 300 of 50257 68 -> 61; at temperature 1, where a third of the tokens are in the histogram, 127 rows 87.6 -> 84.9 and 512 of
+// 32000 62.7 -> 63.0.  (Exact limits found by a search over the floats: 15.0; a warp's queue instead of lists: 13.4; lists of
+// 16: 378 rows 180.)
 #include <climits>
 #include <cstddef>
+
+#include <type_traits>
 
 #include <cooperative_groups.h>
 
@@ -40,6 +47,7 @@ struct TopPArgs {
   float* out; int64_t out_stride;
   int32_t V;
   float c2;       // log2(e) / T
+  float bin_width;  // of a first-level bin, in logits (rounded: for estimates)
   double top_p;
   int32_t* kept_out; int32_t* dev_status;
 };
@@ -372,7 +380,7 @@ constexpr int kTpMaxCluster = 8, kTpMaxSlice = 16384;
 // take 408 us instead of 452, ordinary ones 208 instead of 193, for the room), and from how many on each CTA of the cluster
 // looks at its own ones only.
 constexpr int kTpFastCand = 512, kTpAlone = 128;
-constexpr int kTpQueue = 64;           // per warp: tokens of the round's bins waiting to be added by a full warp
+constexpr int kTpList = 8;             // per thread: tokens of the round's bins waiting to be added
 struct TpFast {
   // Two limbs of 20 and 21 bits per bin, added without a return value; from 4096 tokens in one bin on they could wrap, and
   // then the bins' total is not the exact sum of the round's masses any more.
@@ -380,8 +388,7 @@ struct TpFast {
   unsigned long long coarse[32];       // masses of the groups of bins; [24] all tokens' mass, [25] the round's tokens' (both exact)
   unsigned long long stage[kTpMaxCluster][32];  // what was read from the cluster's CTAs
   __align__(16) unsigned long long part[2][kTpWarps];
-  float queue[kTpWarps][kTpQueue];
-  __align__(16) ulonglong2 cand[kTpFastCand];  // this CTA's tokens of the cut's bin (read by the other CTAs)
+  __align__(16) ulonglong2 cand[kTpFastCand];  // this CTA's tokens of the cut's bin (read by the other CTAs); before that the threads' lists
   __align__(16) ulonglong2 all[kTpFastCand];   // the cluster's
   unsigned long long tau_comp;
   int32_t max;                         // the row's maximum as an ordered integer (every CTA of the cluster adds its warps')
@@ -390,6 +397,9 @@ struct TpFast {
   uint32_t klo, khi;                   // ... and what is left of it
   __align__(16) float x[4];            // the slice (as long as it is)
 };
+
+static_assert(offsetof(TpFast, all) == offsetof(TpFast, cand) + sizeof(TpFast::cand) && sizeof(TpFast::cand) + sizeof(TpFast::all) >= kTpList * kTpThreads * 4,
+              "the threads' lists take the place of both token lists");
 
 // float <-> int of the same order
 __device__ __forceinline__ int tp_ordered(float x) { const int b = __float_as_int(x); return b ^ ((b >> 31) & 0x7fffffff); }
@@ -608,7 +618,9 @@ __global__ void __launch_bounds__(kTpThreads, 2) top_p_cluster_kernel(const TopP
   int bad = 0;
   float m = -INFINITY;
   auto take = [&](int i, float4 v) {
-    v.x = tp_clean(v.x, bad); v.y = tp_clean(v.y, bad); v.z = tp_clean(v.z, bad); v.w = tp_clean(v.w, bad);
+    if (!((v.x + v.y) + (v.z + v.w) < INFINITY)) {  // a NaN or +inf among them (or a sum beyond the largest number)
+      v.x = tp_clean(v.x, bad); v.y = tp_clean(v.y, bad); v.z = tp_clean(v.z, bad); v.w = tp_clean(v.w, bad);
+    }
     m = fmaxf(fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)), m);
     *reinterpret_cast<float4*>(&me.x[i]) = v;
   };
@@ -642,44 +654,60 @@ __global__ void __launch_bounds__(kTpThreads, 2) top_p_cluster_kernel(const TopP
   unsigned long long target = 0, above_round = 0, rest0 = 0;
   int B0 = -1;            // the bin in which the cut falls, and the mass still to find inside it
   bool wrapped = false;
-  float* queue = me.queue[warp];
+  // Where a bin begins among the logits, to a margin of 4e-6, eight times what the rounding of a bin's number can be off: one
+  // comparison tells most tokens off, and only for the others is the bin itself worked out.  (The margin is never 0.)
+  auto margin = [&](float x) { return fmaf(4e-6f, fabsf(M) + fabsf(x), 1e-30f); };
   for (int round = 0, bin0 = 0; round < kTpRounds; ++round, bin0 += kTpBins) {
     const float first = (float)bin0, last = fminf(first + (float)kTpBins, 2048.f);
+    const float x_last = M - last * a.bin_width, x_first = M - first * a.bin_width;
+    const float t_low = x_last - margin(x_last), t_high = x_first + margin(x_first);
     unsigned long long sum = 0;
     uint32_t small = 0;  // tokens behind the first round's bins: below 2^25 each, 32 of them at most
-    int waiting = 0;
-    auto add = [&](float x) {  // a token of the round's bins
-      const float d = (M - x) * a.c2;
-      const unsigned long long w = __float2ull_rn(tp_ex2(-d) * kTpScale);
-      const int b = (int)(d * 51.2f) - bin0;
-      sum += w;
-      atomicAdd(&me.limb[0][b], (uint32_t)w & 0xfffffu);
-      const uint32_t high = (uint32_t)(w >> 20);
-      if (high) atomicAdd(&me.limb[1][b], high);
-    };
-    // Few tokens of a warp are in the round's bins, but often one is: they queue up, and a full warp of them is added at once.
-    auto see = [&](float x) {
+    auto add = [&](float x) {  // a token that may be one of the round's bins
       const float d = (M - x) * a.c2, p = d * 51.2f;
-      const bool in = p >= first && p < last && d < 40.f;
-      if (round == 0 && !in && d < 40.f) small += __float2uint_rn(tp_ex2(-d) * kTpScale);
-      const uint32_t who = __ballot_sync(0xffffffffu, in);
-      if (in) queue[waiting + __popc(who & ((1u << lane) - 1u))] = x;
-      waiting += __popc(who);
-      if (waiting >= 32) {
-        __syncwarp();
-        waiting -= 32;
-        add(queue[waiting + lane]);
-        __syncwarp();
+      const unsigned long long w = __float2ull_rn(tp_ex2(-d) * kTpScale);
+      if (p >= first && p < last && d < 40.f) {
+        const int b = (int)p - bin0;
+        sum += w;
+        atomicAdd(&me.limb[0][b], (uint32_t)w & 0xfffffu);
+        const uint32_t high = (uint32_t)(w >> 20);
+        if (high) atomicAdd(&me.limb[1][b], high);
+      } else if (round == 0 && d < 40.f) {
+        small += (uint32_t)w;
       }
     };
+    // The round's tokens wait in a list of the thread's own, so that the lanes of a warp add theirs side by side.
+    float* const list = reinterpret_cast<float*>(me.cand) + tid;
+    float* end = list;
+    auto flush = [&]() {
+      for (float* t = list; __any_sync(0xffffffffu, t < end); t += kTpThreads)
+        if (t < end) add(*t);
+      end = list;
+    };
+    auto pass = [&](auto opening) {
 #pragma unroll 1
-    for (int i0 = 0; i0 < cnt4; i0 += 4 * kTpThreads) {  // (whole warps take part: the queue is theirs)
-      const int i = i0 + 4 * tid;
-      const float4 v = i < cnt4 ? *reinterpret_cast<const float4*>(&me.x[i]) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-      see(v.x); see(v.y); see(v.z); see(v.w);
-    }
-    __syncwarp();
-    if (lane < waiting) add(queue[lane]);
+      for (int i0 = 0; i0 < cnt4; i0 += 4 * kTpThreads) {  // (whole warps take part)
+        const int i = i0 + 4 * tid;
+        const float4 v = i < cnt4 ? *reinterpret_cast<const float4*>(&me.x[i]) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+        if (__any_sync(0xffffffffu, end > list + (kTpList - 4) * kTpThreads)) flush();
+        const float x[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const bool listed = x[e] >= t_low && (decltype(opening)::value || x[e] < t_high);
+          if (decltype(opening)::value) {  // (no branch: the sum is taken of all of them, 0 for those that do not count)
+            const float d = (M - x[e]) * a.c2;
+            const uint32_t w = __float2uint_rn(tp_ex2(-d) * kTpScale);
+            small += !listed && d < 40.f ? w : 0u;
+          }
+          if (listed) {
+            *end = x[e];
+            end += kTpThreads;
+          }
+        }
+      }
+    };
+    if (round == 0) pass(std::true_type()); else pass(std::false_type());
+    flush();
     const unsigned long long sum_all = tp_warp_sum(sum + small), sum_round = tp_warp_sum(sum);
     if (lane == 0) { me.part[0][warp] = sum_all; me.part[1][warp] = sum_round; }
     __syncthreads();
@@ -758,10 +786,19 @@ __global__ void __launch_bounds__(kTpThreads, 2) top_p_cluster_kernel(const TopP
       if (i + 2 < cnt) orow[i + 2] = v.z;
     }
   };
+  // from t_keep on a more probable bin, below t_drop a less probable one
+  const float x_lo = M - cut_lo * a.bin_width, x_hi = M - cut_hi * a.bin_width, t_keep = x_lo + margin(x_lo), t_drop = x_hi - margin(x_hi);
 #pragma unroll 1
-  for (int i = 4 * tid; i < cnt4; i += 4 * kTpThreads) {
+  for (int i = 4 * tid; i < (whole_row ? 0 : cnt4); i += 4 * kTpThreads) {
     float4 v = *reinterpret_cast<const float4*>(&me.x[i]);
-    v.x = decide(v.x, i); v.y = decide(v.y, i + 1); v.z = decide(v.z, i + 2); v.w = decide(v.w, i + 3);
+    const bool k0 = v.x >= t_keep, k1 = v.y >= t_keep, k2 = v.z >= t_keep, k3 = v.w >= t_keep;
+    const float near = fmaxf(fmaxf(k0 ? -INFINITY : v.x, k1 ? -INFINITY : v.y), fmaxf(k2 ? -INFINITY : v.z, k3 ? -INFINITY : v.w));
+    if (near >= t_drop) {  // one of the four is in the bin, or so close to it that its own bin has to tell
+      v.x = decide(v.x, i); v.y = decide(v.y, i + 1); v.z = decide(v.z, i + 2); v.w = decide(v.w, i + 3);
+    } else {
+      kept += k0 + k1 + k2 + k3;
+      v = make_float4(k0 ? v.x : -INFINITY, k1 ? v.y : -INFINITY, k2 ? v.z : -INFINITY, k3 ? v.w : -INFINITY);
+    }
     if (early) store(i, v);
   }
   int before, n = tp_gather(me, ranks, rank, before);  // tokens of the whole cluster
@@ -891,6 +928,7 @@ extern "C" int seq_tree_top_p_filter(const seq_tree_top_p_params* p, void* strea
   a.out = p->out; a.out_stride = p->out_row_stride;
   a.V = p->vocab;
   a.c2 = kLog2e / p->temperature;
+  a.bin_width = 1.f / (51.2f * a.c2);
   a.top_p = (double)p->top_p;
   a.kept_out = p->kept_out; a.dev_status = p->dev_status;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
