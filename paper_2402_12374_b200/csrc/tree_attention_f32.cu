@@ -189,7 +189,7 @@ __device__ __forceinline__ void f32_pv(const F32Smem<RPT>& sm, F32Row<RPT>& st, 
   ulonglong2 t[RPT];
 #pragma unroll
   for (int i = 0; i < RPT; ++i) t[i] = make_ulonglong2(0ull, 0ull);
-#pragma unroll 1
+#pragma unroll 2  // (the next four keys' operands on their way: 64 nodes on 1024 keys of 32 heads 46.85 -> 44.75 us, one node on 2000 21.2 -> 19.5)
   for (int c = 0; c < 32; c += 4) {
     if (kTree && !((seen >> c) & 15u)) continue;
     const uint8_t* at = vcol + c * 128;
