@@ -29,7 +29,7 @@
 //
 // Merge.  The CTAs that share (tile, kv head) form a thread-block cluster along the key range (cs = 1 .. 8).  Each sends
 // its rows' (m, l) into every CTA as soon as its two chains are done, puts its piece into its V stages, slice by slice of 8
-// output columns in the order of their owners, and copies each owner its slices in one go (into the K stages: an MMA commit of
+// output columns, and copies each owner its run of slices in one go (into the K stages: an MMA commit of
 // every chain of the cluster says that no S is to come).  While the pieces travel each owner works out the rows' common
 // maximum, sum and the pieces' shares; then it adds its slices up.  Both transfers count their bytes into an mbarrier of the
 // receiver; the only cluster barriers are at the start and, off the path, at the end.  No workspace, no second kernel.  (With
@@ -68,6 +68,11 @@ constexpr int kMaxClusterSplit = 8;
 constexpr uint32_t kKvBytes = kBlockN * 128 * 2; // a K or V tile: 64 keys x 128 elements
 constexpr uint32_t kKvHalf = kKvBytes / 2;       // one 64-row x 64-element sub-tile of K or V
 
+// Tiles of up to so many rows store their output a row per thread, 16 bytes at a time; beyond, where every such store of a
+// warp touches 32 lines, the way through shared memory is the shorter one.  (16 rows 5.3 us against 5.85, 64 rows 5.85 / 6.1, 80
+// rows 4.85 / 5.05; 100 rows 6.85 / 6.7, 256 nodes on 2048 keys of 52 heads 23.2 / 22.35.)
+constexpr uint32_t kDirectRows = 80;
+
 struct UmmaSmem {
   // all tiles 1024-byte aligned (128-byte swizzle atoms are 8 rows x 128 B)
   uint8_t q[kTileBytes];
@@ -104,7 +109,6 @@ struct UmmaArgs {
   uint32_t group_magic;   // x / group = x * group_magic >> 16 for x < 128
   uint32_t split_magic;   // x / splits = high word of x * split_magic for x < 2^29 (splits > 1)
   int32_t slots, slices_each, slices_more;  // ceil(16 / splits), 16 / splits, 16 % splits
-  int32_t half_slot, half_owner;            // 8 / splits, 8 % splits
   float scale_log2;
   uint32_t idesc_qk, idesc_pv;
   const uint32_t* mask_bits;
@@ -135,7 +139,7 @@ __device__ __forceinline__ void copy_to_cta(uint32_t dst, uint32_t src, uint32_t
 __device__ __forceinline__ void tc_commit_cluster(uint64_t* bar, uint32_t mask) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(smem_u32(bar)), "h"((uint16_t)mask) : "memory");
 }
-// The 16 slices of 8 output columns are owned round-robin: slice s by CTA s % cs, as its slot s / cs.
+// Of the 16 slices of 8 output columns each CTA owns a run.
 __device__ __forceinline__ int slices_of(int cta, const UmmaArgs& a) { return a.slices_each + (cta < a.slices_more); }
 __device__ __forceinline__ int slices_before(int cta, const UmmaArgs& a) { return cta * a.slices_each + min(cta, a.slices_more); }
 enum { kGrid, kCluster };  // the schedule: a CTA per unit, a cluster of CTAs per unit
@@ -435,7 +439,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
     }
     asm volatile("bar.sync 1, 256;" ::: "memory");
   }
-  const uint32_t* mrow = a.mask_bits != nullptr ? a.mask_bits + (size_t)min(i, a.n - 1) * a.mask_wpr : sm->tile_mask[r_node];
+  const uint32_t* mrow = a.mask_bits + (size_t)min(i, a.n - 1) * a.mask_wpr;  // (the caller's mask, if there is one)
   const int mask_wpr = a.mask_bits != nullptr ? a.mask_wpr : (a.n + 31) >> 5;
   const float sc = a.scale_log2;
 
@@ -464,8 +468,25 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
     const bool masked = kb + kBlockN > L;  // the block reaches into the tree keys (or past the end)
     uint32_t vis[2] = {0xFFFFFFFFu, 0xFFFFFFFFu};
     if (masked) {
-      vis[0] = mask_window(mrow, mask_wpr, a.n, kb - L);
-      vis[1] = mask_window(mrow, mask_wpr, a.n, kb - L + 32);
+      // 64 bits of the row from tree index kb - L on; negative indices are prefix keys (visible)
+      const int t = kb - L, w0 = t >> 5;  // (floor)
+      uint32_t word[3];
+#pragma unroll
+      for (int x = 0; x < 3; ++x) word[x] = w0 + x < 0 ? 0xFFFFFFFFu : 0u;
+      if (a.mask_bits != nullptr) {
+#pragma unroll
+        for (int x = 0; x < 3; ++x)
+          if ((uint32_t)(w0 + x) < (uint32_t)mask_wpr) word[x] = mrow[w0 + x];
+      } else {
+#pragma unroll
+        for (int x = 0; x < 3; ++x)
+          if ((uint32_t)(w0 + x) < (uint32_t)mask_wpr) word[x] = sm->tile_mask[r_node][w0 + x];
+      }
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        const int live = a.n - t - 32 * x;  // tree indices >= n do not exist, whatever the mask words hold there
+        vis[x] = __funnelshift_r(word[x], word[x + 1], t & 31) & (live >= 32 ? 0xFFFFFFFFu : live <= 0 ? 0u : (1u << live) - 1u);
+      }
     }
     tc_wait_ld();
     if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 2);
@@ -606,34 +627,43 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
   }
   uint8_t* out_row = reinterpret_cast<uint8_t*>(a.out) + 2 * ((int64_t)i * a.o_stride_tok + (int64_t)h * a.o_stride_head);
   if (kMode != kCluster) {
-    if (row_valid) {
-      const float inv = 1.f / Lc;  // the row saw at least its own key, so Lc > 0
+    const float inv = 1.f / Lc;  // the row saw at least its own key, so Lc > 0
+    auto words = [&](int j) -> uint4 {  // columns 8j .. 8j+7 of the thread's 64
+      const float* x = merged + 8 * j;
+      return make_uint4(pack2<kBf16>(x[0] * inv, x[1] * inv), pack2<kBf16>(x[2] * inv, x[3] * inv), pack2<kBf16>(x[4] * inv, x[5] * inv), pack2<kBf16>(x[6] * inv, x[7] * inv));
+    };
+    if (live_rows <= kDirectRows) {
+      if (row_valid) {
 #pragma unroll
-      for (int e = 0; e < 64; e += 8) {
-        uint4 val;
-        val.x = pack2<kBf16>(merged[e] * inv, merged[e + 1] * inv);
-        val.y = pack2<kBf16>(merged[e + 2] * inv, merged[e + 3] * inv);
-        val.z = pack2<kBf16>(merged[e + 4] * inv, merged[e + 5] * inv);
-        val.w = pack2<kBf16>(merged[e + 6] * inv, merged[e + 7] * inv);
-        *reinterpret_cast<uint4*>(out_row + 2 * (64 * chain + e)) = val;
+        for (int j = 0; j < 8; ++j) *reinterpret_cast<uint4*>(out_row + 128 * chain + 16 * j) = words(j);
       }
-      if (chain == 0 && a.lse != nullptr) a.lse[(size_t)h * a.n + i] = (M + log2f(Lc)) * kLn2;
+    } else {
+      // Out through this warp's 32 rows of the Q tile, where 16 bytes of 32 rows turn into 128 bytes of four.
+      uint8_t* stage = sm->q + (uint32_t)chain * kHalfBytes + (uint32_t)quad * 4096u;
+      if (row_valid) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) *reinterpret_cast<uint4*>(stage + lane * 128 + ((j ^ (lane & 7)) << 4)) = words(j);
+      }
+      __syncwarp();
+      const int64_t mine = row_valid ? out_row - reinterpret_cast<uint8_t*>(a.out) : -1;  // (strides are positive)
+      uint8_t* const column = reinterpret_cast<uint8_t*>(a.out) + 128 * chain + 16 * (lane & 7);
+#pragma unroll 1
+      for (int row = lane >> 3; row < 32; row += 4) {
+        const int64_t at = __shfl_sync(0xffffffffu, mine, row);
+        if (at >= 0) *reinterpret_cast<uint4*>(column + at) = *reinterpret_cast<const uint4*>(stage + row * 128 + (((lane & 7) ^ (row & 7)) << 4));
+      }
     }
+    if (chain == 0 && row_valid && a.lse != nullptr) a.lse[(size_t)h * a.n + i] = (M + log2f(Lc)) * kLn2;
   } else {
-    // Step 2, across the cluster (cs = 2 .. 8 CTAs along the key range).  The piece goes into the V stages, slice by slice in
-    // the order of the owners, as float4 planes [half][row]; one copy takes an owner its slices, into its receive buffer
+    // Step 2, across the cluster (cs = 2 .. 8 CTAs along the key range).  The piece goes into the V stages, slice by slice, as
+    // float4 planes [half][row]; one copy takes an owner its slices, into its receive buffer
     // [contributor][slot][half][row].
-    const int cs = a.splits, slots = a.slots;  // (the last slots of some CTAs may be empty)
+    const int cs = a.splits, slots = a.slots;  // (the last slot of some CTAs may be empty)
     const uint32_t piece = smem_u32(&sm->v[0][0][0]), receive = smem_u32(&sm->receive[0]);
     if (row_valid) {  // (rows past the tile's last node are padding: nothing of theirs is written, reduced or stored)
-      int slot = chain ? a.half_slot : 0, owner = chain ? a.half_owner : 0;
+      float4* to = reinterpret_cast<float4*>(&sm->v[0][0][0] + (uint32_t)chain * 16u * plane) + r;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        float4* to = reinterpret_cast<float4*>(&sm->v[0][0][0] + (uint32_t)(slices_before(owner, a) + slot) * 2u * plane) + r;
-        to[0] = make_float4(merged[8 * j], merged[8 * j + 1], merged[8 * j + 2], merged[8 * j + 3]);
-        to[plane / 16u] = make_float4(merged[8 * j + 4], merged[8 * j + 5], merged[8 * j + 6], merged[8 * j + 7]);
-        if (++owner == cs) { owner = 0; ++slot; }
-      }
+      for (int j = 0; j < 16; ++j) to[(uint32_t)j * (plane / 16u)] = make_float4(merged[4 * j], merged[4 * j + 1], merged[4 * j + 2], merged[4 * j + 3]);
     }
     fence_async_smem();
     asm volatile("bar.sync 1, 256;" ::: "memory");
@@ -657,16 +687,19 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
     }
     const float inv = 1.f / Ls;  // some CTA saw the row's own key, so Ls > 0
     if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 7);
+    // the two warp groups share this CTA's slices
+    const int owned = slices_of(split, a), before = slices_before(split, a);
+    const int first_slot = chain ? (owned + 1) >> 1 : 0, end_slot = chain ? owned : (owned + 1) >> 1;
     mbar_wait(sm, &sm->data_full, 0, a.dev_status);
     __syncwarp();
     cluster_arrive_relaxed();  // every piece for this CTA is here: its senders may leave
     if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 8);
     if (row_valid)
-      for (int slot = chain; slot * cs + split < 16; slot += 2) {  // the two warp groups share this CTA's slots
+      for (int slot = first_slot; slot < end_slot; ++slot) {
         uint64_t x[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll 2
         for (int q = 0; q < cs; ++q) {
-          const uint8_t* at = q == split ? &sm->v[0][0][0] + (uint32_t)(slices_before(split, a) + slot) * 2u * plane
+          const uint8_t* at = q == split ? &sm->v[0][0][0] + (uint32_t)(before + slot) * 2u * plane
                                          : &sm->receive[0] + (uint32_t)(q * slots + slot) * 2u * plane;
           const ulonglong2 u = *(reinterpret_cast<const ulonglong2*>(at) + r), w = *(reinterpret_cast<const ulonglong2*>(at + plane) + r);
           const float f = ex2(sm->ml_cta[q][r].x - Mg) * inv;
@@ -681,7 +714,7 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
         val.y = pack2<kBf16>(o[2], o[3]);
         val.z = pack2<kBf16>(o[4], o[5]);
         val.w = pack2<kBf16>(o[6], o[7]);
-        *reinterpret_cast<uint4*>(out_row + 2 * (8 * (slot * cs + split))) = val;
+        *reinterpret_cast<uint4*>(out_row + 2 * (8 * (before + slot))) = val;
       }
     if (split == 0 && chain == 0 && row_valid && a.lse != nullptr) a.lse[(size_t)h * a.n + i] = (Mg + log2f(Ls)) * kLn2;
     __syncwarp();
@@ -826,7 +859,6 @@ int launch_attention_umma(const seq_tree_attention_params& p, int splits, cudaSt
   a.group_magic = (uint32_t)((65536 + G - 1) / G);
   a.split_magic = (uint32_t)((((uint64_t)1 << 32) / (uint64_t)splits) + 1);
   a.slots = (15 + splits) / splits; a.slices_each = 16 / splits; a.slices_more = 16 % splits;
-  a.half_slot = 8 / splits; a.half_owner = 8 % splits;
   const float scale = p.softmax_scale > 0.f ? p.softmax_scale : 0.08838834764831845f;
   a.scale_log2 = scale * kLog2e;
   const uint32_t fmt = p.dtype == SEQ_BF16 ? 1u : 0u;

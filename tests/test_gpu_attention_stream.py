@@ -1,0 +1,79 @@
+"""The tensor-core attention's stream schedule where its two chains share an accumulator and a reference maximum, and the
+outputs that leave through shared memory."""
+from __future__ import annotations
+
+import dataclasses
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import oracle as O
+from paper_2402_12374_b200 import binding as B
+from paper_2402_12374_b200 import workloads as W
+from tests import gpu_util as G
+
+pytestmark = pytest.mark.gpu
+
+
+def _inputs(hkv, group, n, L, dtype, seed=3):
+    cfg = dataclasses.replace(W.CONFIGS["tiny"], num_q_heads=hkv * group, num_kv_heads=hkv, prefix_len=L, n_tree=n, max_depth=14, max_fanout=8)
+    return W.make_attention_inputs(cfg, seed, dtype=dtype, extra_capacity=9)
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp16"])
+@pytest.mark.parametrize("step", [64, 128, 192])
+@pytest.mark.parametrize("hkv,group,n,L", [(2, 1, 30, 700), (1, 8, 20, 1000), (1, 5, 30, 450)])
+def test_scores_that_rise_along_the_keys(hkv, group, n, L, step, dtype):
+    """Every `step` keys the scores of all rows rise by 12 (17 in powers of two, beyond the 8 a reference lets pass): the
+    reference moves in one chain's turn, in the other's, or in both, and the accumulator is rescaled.  The output is then all
+    but decided by the last keys, to the output type's rounding of V (2e-2 covers four of bfloat16's)."""
+    ai = _inputs(hkv, group, n, L, dtype)
+    u = torch.ones(128) / 128 ** 0.5
+    total = L + n
+    rise = 12.0 * torch.floor(torch.arange(total) / step)
+    q = (0.3 * ai.q.float() - (0.3 * ai.q.float() @ u)[..., None] * u + 16.0 * u).to(ai.q.dtype)
+    k = ai.k_cache.float().clone()
+    k[:, :total] = 0.3 * k[:, :total]
+    k[:, :total] -= (k[:, :total] @ u)[..., None] * u
+    k[:, :total] += (rise * 128 ** 0.5 / 16.0)[None, :, None] * u
+    if dtype == "fp16" and float(k.abs().max()) > 6e4:
+        pytest.skip("keys beyond half precision")
+    ai = dataclasses.replace(ai, q=q, k_cache=k.to(ai.k_cache.dtype))
+    ref, _, _ = O.tree_attention(ai.q, ai.k_cache, ai.v_cache, ai.parent, L)
+    for kernel in (B.KERNEL_TENSOR_CORE_STREAM, B.KERNEL_TENSOR_CORE_GRID):
+        out, _, status = G.run_attention(ai, kernel)
+        assert status == 0
+        assert np.abs(out.double().cpu().numpy() - ref).max() < 2e-2
+
+
+@pytest.mark.parametrize("hkv,group,n,L", [(1, 1, 1, 0), (1, 1, 1, 63), (1, 1, 1, 64), (1, 1, 3, 126), (1, 8, 17, 190), (2, 4, 33, 64), (3, 1, 129, 0),
+                                           (1, 2, 65, 319), (8, 8, 40, 1500)])
+def test_pairs_of_blocks(hkv, group, n, L):
+    """One block, one pair, an odd block behind pairs, pieces of every size; mask given and derived from the tree."""
+    ai = _inputs(hkv, group, n, L, "bf16")
+    G.check_attention(ai, kernel=B.KERNEL_TENSOR_CORE_STREAM)
+    d = G.dev()
+    mask, _, st = G.gpu_mask(ai.parent.numpy())
+    args = (ai.q.to(d), ai.k_cache.to(d), ai.v_cache.to(d))
+    given = B.seq_tree_attention(*args, mask, L, kernel=B.KERNEL_TENSOR_CORE_STREAM)
+    derived = B.seq_tree_attention(*args, None, L, parent=ai.parent.to(d), kernel=B.KERNEL_TENSOR_CORE_STREAM, dev_status=st)
+    assert torch.equal(given, derived) and int(st.item()) == 0
+
+
+@pytest.mark.parametrize("kernel", [B.KERNEL_TENSOR_CORE_STREAM, B.KERNEL_TENSOR_CORE_GRID])
+@pytest.mark.parametrize("hkv,group,n", [(1, 1, 80), (1, 1, 81), (2, 8, 10), (2, 8, 11), (1, 5, 17), (1, 1, 128), (1, 3, 43), (1, 1, 200)])
+def test_outputs_with_strides_of_their_own(hkv, group, n, kernel):
+    """Rows of the output apart from each other, around the number of rows from which they leave through shared memory;
+    nothing between them is touched."""
+    d, L = G.dev(), 20
+    ai = _inputs(hkv, group, n, L, "fp16")
+    mask, _, st = G.gpu_mask(ai.parent.numpy())
+    Hq = hkv * group
+    buf = torch.full((n, Hq + 1, 128 + 8), 7.0, dtype=torch.float16, device=d)
+    out = buf[:, :Hq, :128]
+    B.seq_tree_attention(ai.q.to(d), ai.k_cache.to(d), ai.v_cache.to(d), mask, L, out=out, dev_status=st, kernel=kernel)
+    ref, _, _ = O.tree_attention(ai.q, ai.k_cache, ai.v_cache, ai.parent, L)
+    assert int(st.item()) == 0
+    assert np.abs(out.double().cpu().numpy() - ref).max() < G.ATTN_TOL[torch.float16]
+    assert bool((buf[:, Hq] == 7.0).all()) and bool((buf[:, :, 128:] == 7.0).all())
