@@ -737,7 +737,7 @@ bool umma_supported(const seq_tree_attention_params& p) {
 // How the tiles are spread over the SMs.  Grid schedule: one CTA (or a cluster of `splits` CTAs along the key
 // range) per (tile, kv head), in as many waves as that takes.  Stream schedule: one CTA per SM, each with an equal range of the
 // flattened block space and share the tiles that a range boundary cuts.  p.kernel = 3 / 4 force one of them.
-struct UmmaPlan { int splits; bool stream; };
+struct UmmaPlan { int splits; bool stream, optional; };  // optional: without a workspace, the grid schedule
 constexpr size_t kUmmaSmemBytes = sizeof(UmmaSmem) + 1024;
 // Clusters of cs CTAs that the device runs at a time (one CTA fills an SM).  Asked once per device and size; without a
 // device, or where the question fails, what the SMs would hold.
@@ -781,9 +781,9 @@ static UmmaPlan umma_plan(const seq_tree_attention_params& p) {
   const bool can_stream = tiles <= kMaxStreamTiles && p.prefix_len_dev_count <= 1 && (double)units * (nblk + kStreamTileCost) < 2147483648.0;
   const int kNumSMs = device_sm_count();
 #ifdef SEQ_TRACE
-  if (const char* e = getenv("SEQ_DEBUG_SPLITS")) return {atoi(e), false};  // debug builds only
+  if (const char* e = getenv("SEQ_DEBUG_SPLITS")) return {atoi(e), false, false};  // debug builds only
 #endif
-  if (p.kernel == 3 && can_stream) return {1, true};
+  if (p.kernel == 3 && can_stream) return {1, true, false};
   // More units than SMs.  Measured over batches of the paper's shapes (5 to 32 requests stacked as heads): plain
   // waves of one CTA per unit win by 5-50 % when tiles are short (a tile cut by a range boundary costs a trip
   // through the workspace, and every CTA starts and finishes two tiles more), the stream schedule wins by 5-15 %
@@ -791,25 +791,34 @@ static UmmaPlan umma_plan(const seq_tree_attention_params& p) {
   if (p.kernel != 4 && can_stream && units > kNumSMs) {
     const long waves = (units + kNumSMs - 1) / kNumSMs;
     const bool last_wave_thin = units * 10 <= waves * kNumSMs * 6;
-    if (nblk >= 32 && (last_wave_thin || nblk >= 72)) return {1, true};
+    if (nblk >= 32 && (last_wave_thin || nblk >= 72)) return {1, true, false};
   }
-  // Otherwise the split with the lowest estimate.  Microseconds per wave, fitted to launches of 72 shapes (8 to 768 nodes,
-  // prefixes of 100 to 8000 keys, 8 to 384 units) with every split forced: 0.45 per block of a CTA's key range, 4.7 fixed,
-  // and the merge across the cluster, which grows with the pieces that an owner's threads add up one after the other
-  // (ceil(ceil(16 / cs) / 2) * cs, hence 4 below 3).  What a wave holds is asked of the device: a cluster lies in one
+  // Otherwise the split with the lowest estimate.  Microseconds per wave, fitted to launches of 110 shapes (1 to 256 nodes,
+  // prefixes of 32 to 8192 keys, 8 to 148 units) with every split forced: 0.45 per block of a CTA's key range, 5 fixed, and
+  // the merge across the cluster.  (Picks within 0.25 % of the best split on the average and 4 % at worst; with the figures of
+  // the merge that stored its pieces one by one, 2.3 to 4.2, 2 % and 34 %: 4 nodes on 350 keys of 64/8 heads 6.05 -> 5.6 us,
+  // 8 on 1024 7.25 -> 6.6.)  What a wave holds is asked of the device: a cluster lies in one
   // GPC, so the SMs left over in each are lost to it (74, 44, 36, 28, 21, 14 and 14 clusters of 2 to 8 CTAs were seen, where
   // 148 / cs had been assumed; 24 units of 17 blocks 17.3 -> 10.1 us, 16 of 48 21.8 -> 12.5, 48 of 66 34.7 -> 23.3).
-  static const double kMerge[kMaxClusterSplit + 1] = {0.0, 0.0, 2.25, 3.2, 2.8, 3.5, 3.8, 4.2, 4.2};
+  static const double kMerge[kMaxClusterSplit + 1] = {0.0, 0.0, 1.45, 2.0, 1.7, 2.3, 2.05, 1.8, 1.8};
   int best = 1;
   double best_cost = -1.0;
   for (int cs = 1; cs <= kMaxClusterSplit && cs <= nblk; ++cs) {
     const int room = clusters_side_by_side(cs);
     if (room == 0) continue;
     const long waves = (units + room - 1) / room;
-    const double cost = (double)waves * (0.45 * ((nblk + cs - 1) / cs) + 4.7 + kMerge[cs]);
+    const double cost = (double)waves * (0.45 * ((nblk + cs - 1) / cs) + 5.0 + kMerge[cs]);
     if (best_cost < 0 || cost < best_cost - 1e-9) { best = cs; best_cost = cost; }
   }
-  return {best, false};
+  // ... against that of the stream schedule: 0.4 per block of an SM's range, 7 per tile it starts or finishes, 7 fixed (3 to 8
+  // % off over 20 shapes of 96 to 384 units).  192 units of 44 blocks 49.5 -> 44.5 us, of 67 blocks 69.7 / 57.9, 96 of 134
+  // 68.3 / 55.9.  Not where K and V are more than L2 holds: the tiles of a head, in step when they start together, each fetch
+  // them anew (104 units of 132 blocks, 220 MB: 66 us in one wave, 84 as a stream).  These calls were served without a
+  // workspace before there was this rule, and without one they still are.
+  const double kv_bytes = 4.0 * ((double)p.prefix_len + p.n_tree) * kHeadDim * p.num_kv_heads;
+  const double stream_cost = 0.4 * units * nblk / kNumSMs + 7.0 * ((double)units / kNumSMs + 1.0) + 7.0;
+  if (p.kernel != 4 && can_stream && nblk >= 24 && kv_bytes < 120e6 && stream_cost < 0.96 * best_cost) return {best, true, true};
+  return {best, false, false};
 }
 
 int umma_default_splits(const seq_tree_attention_params& p) { return umma_plan(p).splits; }
@@ -848,7 +857,9 @@ int launch_attention_umma(const seq_tree_attention_params& p, int splits, cudaSt
   // (groups that do not divide 128 used to run on the CUDA cores, which ask for nothing at these sizes: without a workspace
   // they take the grid schedule instead, 500 nodes on 4600 keys of 40/8 heads 99 us against 67)
   const bool lent = p.workspace != nullptr && p.workspace_bytes >= stream_workspace_bytes(p);
-  if (umma_plan(p).stream && (lent || p.kernel != 0 || kTileM % G == 0)) return launch_attention_stream(p, stream);
+  const bool aligned = reinterpret_cast<uintptr_t>(p.workspace) % 256 == 0;
+  const UmmaPlan plan = umma_plan(p);
+  if (plan.stream && (plan.optional ? lent && aligned : lent || p.kernel != 0 || kTileM % G == 0)) return launch_attention_stream(p, stream);
 
   CUtensorMap q_map, k_map, v_map;
   if (!attention_maps(p, 2, &q_map, &k_map, &v_map)) return SEQ_ERR_CUDA;

@@ -1,5 +1,5 @@
-"""The tensor-core attention's stream schedule where its two chains share an accumulator and a reference maximum, and the
-outputs that leave through shared memory."""
+"""The tensor-core attention's stream schedule where its two chains share an accumulator and a reference maximum, the outputs
+that leave through shared memory, and the calls whose schedule depends on a workspace."""
 from __future__ import annotations
 
 import dataclasses
@@ -77,3 +77,23 @@ def test_outputs_with_strides_of_their_own(hkv, group, n, kernel):
     assert int(st.item()) == 0
     assert np.abs(out.double().cpu().numpy() - ref).max() < G.ATTN_TOL[torch.float16]
     assert bool((buf[:, Hq] == 7.0).all()) and bool((buf[:, :, 128:] == 7.0).all())
+
+
+def test_a_stream_that_is_only_the_faster_choice_needs_no_workspace():
+    """96 units of 131 blocks: streamed where a workspace is lent, served by the grid schedule where none (or a short or
+    misaligned one) is."""
+    d = G.dev()
+    n, L = 384, 8000
+    ai = _inputs(8, 4, n, L, "bf16")
+    parent = ai.parent.to(d)
+    args = (ai.q.to(d), ai.k_cache.to(d), ai.v_cache.to(d))
+    call = B.AttentionCall(*args, None, L, parent=parent)
+    streamed = call.run().clone()
+    forced = B.seq_tree_attention(*args, None, L, parent=parent, kernel=B.KERNEL_TENSOR_CORE_GRID)
+    assert (streamed.float() - forced.float()).norm() < 5e-3 * forced.float().norm()  # two roundings of P to bfloat16
+    if call.workspace_bytes_needed == 0:
+        pytest.skip("not streamed on this device")
+    backing = torch.empty(call.workspace_bytes_needed + 256, dtype=torch.uint8, device=d)
+    for lent in (backing[:0], backing[:4096], backing[8:8 + call.workspace_bytes_needed]):
+        got = B.seq_tree_attention(*args, None, L, parent=parent, workspace=lent)
+        assert torch.equal(got, forced)
