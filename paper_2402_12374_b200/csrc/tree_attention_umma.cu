@@ -811,13 +811,14 @@ static UmmaPlan umma_plan(const seq_tree_attention_params& p) {
     if (best_cost < 0 || cost < best_cost - 1e-9) { best = cs; best_cost = cost; }
   }
   // ... against that of the stream schedule: 0.4 per block of an SM's range, 7 per tile it starts or finishes, 7 fixed (3 to 8
-  // % off over 20 shapes of 96 to 384 units).  192 units of 44 blocks 49.5 -> 44.5 us, of 67 blocks 69.7 / 57.9, 96 of 134
-  // 68.3 / 55.9.  Not where K and V are more than L2 holds: the tiles of a head, in step when they start together, each fetch
-  // them anew (104 units of 132 blocks, 220 MB: 66 us in one wave, 84 as a stream).  These calls were served without a
-  // workspace before there was this rule, and without one they still are.
+  // % off over 20 shapes of 96 to 384 units).  192 units of 67 blocks 69.7 -> 57.9 us, 96 of 134 68.3 -> 55.9; taken where
+  // it is an eighth lower, because a caller has 19 MB of workspace to find for it (the first time 0.2 ms).  Not where K and V
+  // are more than L2 holds: the tiles of a head, in step when they start together, each fetch them anew (104 units of 132
+  // blocks, 220 MB: 66 us in one wave, 84 as a stream).  These calls were served without a workspace before there was this
+  // rule, and without one they still are.
   const double kv_bytes = 4.0 * ((double)p.prefix_len + p.n_tree) * kHeadDim * p.num_kv_heads;
   const double stream_cost = 0.4 * units * nblk / kNumSMs + 7.0 * ((double)units / kNumSMs + 1.0) + 7.0;
-  if (p.kernel != 4 && can_stream && nblk >= 24 && kv_bytes < 120e6 && stream_cost < 0.96 * best_cost) return {best, true, true};
+  if (p.kernel != 4 && can_stream && nblk >= 24 && kv_bytes < 120e6 && stream_cost < 0.88 * best_cost) return {best, true, true};
   return {best, false, false};
 }
 
