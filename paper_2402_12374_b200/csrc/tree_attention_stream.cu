@@ -171,11 +171,14 @@ tree_attention_stream_kernel(const __grid_constant__ CUtensorMap q_map, const __
     blocks_per_head = sum;
     total_blocks = sum * a.Hkv;
   }
-  // where the range of CTA x starts: total_blocks * x / gridDim.x
-  const int per_cta = total_blocks / (int)gridDim.x, left_over = total_blocks - per_cta * (int)gridDim.x;
-  auto cta_lo = [&](int x) { return per_cta * x + (left_over * x) / (int)gridDim.x; };
-  range_lo = cta_lo(blockIdx.x);
-  range_hi = cta_lo(blockIdx.x + 1);
+  // where the range of CTA x starts: total_blocks * x / ctas.  The launch was planned for the longest prefix; a short one can
+  // have fewer positions than the grid has CTAs.  The CTAs that share a cut tile are counted from the ranges and each of them
+  // has to arrive, so none of those may be empty: the first `ctas` have one each, the others none.
+  const int ctas = min((int)gridDim.x, total_blocks);
+  const int per_cta = total_blocks / ctas, left_over = total_blocks - per_cta * ctas;
+  auto cta_lo = [&](int x) { return per_cta * x + (left_over * x) / ctas; };
+  range_lo = cta_lo(min((int)blockIdx.x, ctas));
+  range_hi = cta_lo(min((int)blockIdx.x + 1, ctas));
   if (a.mask_bits == nullptr)
     for (int t = threadIdx.x; t < a.n; t += kUmmaThreads) sm->parent[t] = a.parent[t];
   if (a.rows < kTileM) {  // rows no copy writes (the group does not divide 128): zeros, so that their scores are finite
@@ -538,7 +541,7 @@ tree_attention_stream_kernel(const __grid_constant__ CUtensorMap q_map, const __
   if (piece) {
     t0 = g * blocks_per_head + sm->tile_prefix[sg.slot_in_head] + kStreamTileCost;
     const int t1 = t0 + sg.nblk_tile;
-    c_first = min((int)((float)t0 / (float)total_blocks * (float)gridDim.x), (int)gridDim.x - 1);  // the CTA whose range holds block t0 ...
+    c_first = min((int)((float)t0 / (float)total_blocks * (float)ctas), ctas - 1);  // the CTA whose range holds block t0 ...
     while (cta_lo(c_first + 1) <= t0) ++c_first;                      // ... exactly
     while (cta_lo(c_first) > t0) --c_first;
     c_last = c_first;
@@ -761,8 +764,7 @@ int launch_attention_stream(const seq_tree_attention_params& p, cudaStream_t str
   SEQ_CUDA_OK(cudaLaunchKernelEx(&zero, zero_words_kernel, a.ws_count, words));
 
   cudaLaunchConfig_t cfg = {};
-  // One CTA per SM, but never more CTAs than positions in the layout: a range must not be empty
-  // (the CTAs that share a cut tile are counted from the ranges, and each of them has to arrive).
+  // One CTA per SM, but no more than positions in the layout (of the longest prefix: see the kernel).
   const int sms = device_sm_count();
   cfg.gridDim = dim3(a.total_blocks_host < sms ? a.total_blocks_host : sms);
   cfg.blockDim = dim3(kUmmaThreads);

@@ -97,3 +97,28 @@ def test_a_stream_that_is_only_the_faster_choice_needs_no_workspace():
     for lent in (backing[:0], backing[:4096], backing[8:8 + call.workspace_bytes_needed]):
         got = B.seq_tree_attention(*args, None, L, parent=parent, workspace=lent)
         assert torch.equal(got, forced)
+
+
+@pytest.mark.parametrize("kernel", [B.KERNEL_AUTO, B.KERNEL_TENSOR_CORE_STREAM])
+@pytest.mark.parametrize("hq,hkv,n,bound", [(64, 8, 16, 20000), (32, 8, 16, 18432), (32, 4, 16, 13312), (8, 1, 3, 9000)])
+def test_lengths_in_device_memory_far_below_the_bound(hq, hkv, n, bound, kernel):
+    """A launch planned for a long prefix that meets a short one: the layout then has fewer positions than the grid has CTAs,
+    and every tile is written all the same (the output starts as NaN)."""
+    d = G.dev()
+    ai = _inputs(hkv, hq // hkv, n, bound, "bf16")
+    q, k, v, parent = ai.q.to(d), ai.k_cache.to(d), ai.v_cache.to(d), ai.parent.to(d)
+    st = torch.zeros(1, dtype=torch.int32, device=d)
+    length = torch.zeros(1, dtype=torch.int32, device=d)
+    out = torch.empty_like(q)
+    call = B.AttentionCall(q, k, v, None, bound, parent=parent, out=out, dev_status=st, kernel=kernel, prefix_len_dev=length)
+    for L in (0, 64, 100, 200, 300, 500, 600, 1000, bound):
+        length.fill_(L)
+        out.fill_(float("nan"))
+        call.run()
+        if L < bound:
+            ref = O.tree_attention(ai.q, ai.k_cache[:, :L + n], ai.v_cache[:, :L + n], ai.parent, L)[0]
+        else:  # (the oracle would take its time)
+            ref = B.seq_tree_attention(q, k, v, None, L, parent=parent, kernel=B.KERNEL_TENSOR_CORE_GRID).double().cpu().numpy()
+        err = np.abs(out.double().cpu().numpy() - ref).max()
+        assert err < G.ATTN_TOL[torch.bfloat16], f"prefix {L}: {err}"  # (NaN is not below it)
+    assert int(st.item()) == 0
