@@ -435,7 +435,9 @@ tree_attention_stream_kernel(const __grid_constant__ CUtensorMap q_map, const __
       uint64_t sm2[2] = {pair_of(0.f, 0.f), pair_of(0.f, 0.f)};
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        if (c == 2) second_half();
+        // (with kFineP the first store already goes to columns that the second half is read from, and nothing but a wait orders
+        // a store to tensor memory behind a load)
+        if (c == (kFineP ? 0 : 2)) second_half();
         uint32_t packed[16], rest[16];
 #pragma unroll
         for (int e = 0; e < 16; ++e) {  // two scores at a time: one packed multiply-add, two exponentials, one packed add

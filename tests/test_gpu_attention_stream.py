@@ -61,6 +61,21 @@ def test_pairs_of_blocks(hkv, group, n, L):
     assert torch.equal(given, derived) and int(st.item()) == 0
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "fp16"])
+@pytest.mark.parametrize("hkv,group,n,L", [(2, 5, 26, 1500), (2, 3, 43, 2000), (1, 5, 100, 3001), (3, 3, 128, 900)])
+def test_groups_that_do_not_divide_a_tile_on_long_prefixes(hkv, group, n, L, dtype):
+    """Their probabilities enter the product in two pieces, the second stored where scores of the same pair are read from: on
+    unmasked pairs the output is as good as the exact one rounded to its type.  The two pieces leave 2^-16 (bfloat16) or 2^-22
+    (half) of a probability at most, single precision less: a thirty-second of a unit in the last place covers them."""
+    ai = _inputs(hkv, group, n, L, dtype)
+    ref, _, _ = O.tree_attention(ai.q, ai.k_cache, ai.v_cache, ai.parent, L)
+    out, _, status = G.run_attention(ai, B.KERNEL_TENSOR_CORE_STREAM)
+    assert status == 0
+    rounded = torch.from_numpy(ref).to(out.dtype).double().numpy()
+    unit = 2.0 ** (-7 if dtype == "bf16" else -10)
+    assert np.linalg.norm(out.double().cpu().numpy() - ref) < np.linalg.norm(rounded - ref) + unit / 32 * np.linalg.norm(ref)
+
+
 @pytest.mark.parametrize("kernel", [B.KERNEL_TENSOR_CORE_STREAM, B.KERNEL_TENSOR_CORE_GRID])
 @pytest.mark.parametrize("hkv,group,n", [(1, 1, 80), (1, 1, 81), (2, 8, 10), (2, 8, 11), (1, 5, 17), (1, 1, 128), (1, 3, 43), (1, 1, 200)])
 def test_outputs_with_strides_of_their_own(hkv, group, n, kernel):
