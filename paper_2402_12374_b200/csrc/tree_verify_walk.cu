@@ -146,10 +146,11 @@ __device__ __forceinline__ void load_row(const Ctx& c, const void* row_v, RawRow
     }
   }
 }
-// The lines that load_row will read, asked for before the previous kernel has ended: the tree's arrays, node 0's rows and those
-// of node 1, the root's first child (whose rows the walk requests before it knows whether it needs them).  768 nodes x 128256
-// tokens 17.6 -> 17.3 us in a row of calls on rows that are not in L2, 16 requests of 64 x 32000 20.85 -> 20.4, greedy
-// 128 x 32000 5.0 -> 4.85.
+// The lines that load_row will read, asked for before the previous kernel has ended: the tree's arrays, node 0's rows and the
+// target row of node 1, the root's first child (which the walk requests before it knows whether it needs it).  Not node 1's
+// draft row: it need not exist if node 1 is a leaf, and the tree is not known yet.  In calls on several sets of inputs in turn
+// 768 nodes x 128256 tokens 18.6 -> 18.4 us, 16 requests of 64 x 32000 21.5 -> 21.15, greedy 128 x 32000 5.23 -> 5.18; with
+// node 1's draft row the same.
 template <int NCH, bool kBf16>
 __device__ __forceinline__ void prefetch_row(const Ctx& c, const void* row) {
   constexpr int kEsz = kBf16 ? 2 : 4, kLine = 128 / kEsz;  // elements of a line
@@ -441,7 +442,6 @@ __global__ void __launch_bounds__(kTh, CL == kClBatch && NCH <= 4 ? 2 : 1) tree_
   if (a.n > 1) {
     prefetch_row<NCH, kBf16>(c, dbase);
     prefetch_row<NCH, kBf16>(c, tbase + a.target_stride * kEsz);
-    prefetch_row<NCH, kBf16>(c, dbase + a.draft_stride * kEsz);
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
   WTRACE(leader, 1);

@@ -582,3 +582,23 @@ def test_tensor_core_attention_clusters_of_odd_sizes(heads):
         again = call.run()
         torch.cuda.synchronize()
         assert int(st.item()) == 0 and torch.equal(first, again)
+
+
+@pytest.mark.parametrize("mode", ["default", "specinfer", "bf16"])
+@pytest.mark.parametrize("V", [4096, 32000, 128256])
+def test_verify_without_draft_rows_for_leaves(V, mode):
+    """A tree of depth one needs the root's draft row alone: a draft matrix of one row gives what one of all rows gives."""
+    d, n = G.dev(), 5
+    for seed in range(4):
+        vi = W.make_verify_inputs(W.CONFIGS["tiny"], 0.6, seed, parent=W.star_tree(n), vocab=V)
+        st = torch.zeros(1, dtype=torch.int32, device=d)
+        dt = torch.bfloat16 if mode == "bf16" else torch.float32
+        target, draft = vi.target_logits.to(d, dt), vi.draft_logits.to(d, dt)
+        got = []
+        for rows in (draft, draft[:1].clone()):
+            residual = torch.empty(V, dtype=torch.float32, device=d)
+            nxt = torch.empty(n, dtype=torch.int32, device=d)
+            path, plen, bonus = B.seq_tree_verify(vi.parent.to(d), vi.tokens.to(d), target, rows, 0.6, vi.uniforms.to(d),
+                                                  residual_out=residual, next_child_out=nxt, dev_status=st, specinfer=mode == "specinfer")
+            got.append((path[:int(plen)].tolist(), int(bonus), nxt.tolist(), residual))
+        assert got[0][:3] == got[1][:3] and torch.equal(got[0][3], got[1][3]) and int(st.item()) == 0
