@@ -738,6 +738,7 @@ bool umma_supported(const seq_tree_attention_params& p) {
 // range) per (tile, kv head), in as many waves as that takes.  Stream schedule: one CTA per SM, each with an equal range of the
 // flattened block space and share the tiles that a range boundary cuts.  p.kernel = 3 / 4 force one of them.
 struct UmmaPlan { int splits; bool stream, optional; };  // optional: without a workspace, the grid schedule
+constexpr long kOptionalStreamUnits = 48;  // (see umma_plan)
 constexpr size_t kUmmaSmemBytes = sizeof(UmmaSmem) + 1024;
 // Clusters of cs CTAs that the device runs at a time (one CTA fills an SM).  Asked once per device and size; without a
 // device, or where the question fails, what the SMs would hold.
@@ -811,14 +812,23 @@ static UmmaPlan umma_plan(const seq_tree_attention_params& p) {
     if (best_cost < 0 || cost < best_cost - 1e-9) { best = cs; best_cost = cost; }
   }
   // ... against that of the stream schedule: 0.4 per block of an SM's range, 7 per tile it starts or finishes, 7 fixed (3 to 8
-  // % off over 20 shapes of 96 to 384 units).  192 units of 67 blocks 69.7 -> 57.9 us, 96 of 134 68.3 -> 55.9; taken where
-  // it is an eighth lower, because a caller has 19 MB of workspace to find for it (the first time 0.2 ms).  Not where K and V
-  // are more than L2 holds: the tiles of a head, in step when they start together, each fetch them anew (104 units of 132
-  // blocks, 220 MB: 66 us in one wave, 84 as a stream).  These calls were served without a workspace before there was this
-  // rule, and without one they still are.
+  // % off over 20 shapes of 96 to 384 units).  192 units of 84 blocks 76 -> 65.5 us, 96 of 131 65 -> 56; taken where it is an
+  // eighth lower, because a caller has 19 MB of workspace to find for it (the first time 0.2 ms).  These calls were served
+  // without a workspace before there was this rule, and without one they still are.  It holds
+  // - from 48 units on (48 of 200 blocks 52 -> 49 us, 52 of 300 92 -> 64, 80 of 200 73 -> 65): with fewer a tile has more than
+  //   three pieces and one CTA adds them all up, which the estimate knows nothing of (1 unit of 200 blocks 19 us in a cluster,
+  //   237 as a stream; 8 of 300 26 / 53; 16 of 500 46 / 53; 32 of 500 64 / 67);
+  // - for a length given by the host: one in device memory is planned for at its largest, and the stream is the slower one of
+  //   the two well below that (96 units planned for 128 blocks: 64 / 54 us there, 37 / 39 at half of it, 12 / 23 at 500 keys);
+  // - where L2 holds K and V: the tiles of a head, in step when they start together, each fetch them anew from memory (80 units
+  //   of 450 blocks, 118 MB: 149 us in one wave, 155 as a stream; 104 of 132, 220 MB: 66 / 84; 312 of 67, 114 MB: 99 / 90).
+  // Over 537 shapes of 48 to 400 units and 24 to 450 blocks no pick of the stream by this rule is more than 3 % slower than the
+  // grid schedule.
   const double kv_bytes = 4.0 * ((double)p.prefix_len + p.n_tree) * kHeadDim * p.num_kv_heads;
   const double stream_cost = 0.4 * units * nblk / kNumSMs + 7.0 * ((double)units / kNumSMs + 1.0) + 7.0;
-  if (p.kernel != 4 && can_stream && nblk >= 24 && kv_bytes < 120e6 && stream_cost < 0.88 * best_cost) return {best, true, true};
+  if (p.kernel != 4 && can_stream && units >= kOptionalStreamUnits && p.prefix_len_dev == nullptr && nblk >= 24 && kv_bytes < 115e6 &&
+      stream_cost < 0.88 * best_cost)
+    return {best, true, true};
   return {best, false, false};
 }
 

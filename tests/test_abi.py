@@ -225,3 +225,32 @@ def test_attention_schedule_choice_is_visible_through_the_workspace_size(lib):
     assert shape(128, 2048, 6 * 40, 6 * 40) == 0   # 240 units: waves
     assert shape(64, 1024, 8 * 32, 8 * 32, kernel=3) > 0 and shape(768, 4096, 64, 8, kernel=4) == 0
     assert shape(64, 1024, 32, 32, kernel=3) > 0   # forced even where one wave would do
+
+
+def test_a_workspace_is_asked_for_only_where_the_stream_schedule_was_measured_faster(lib):
+    """Up to one tile per SM: from 48 (tile, kv head) units on, with the length given by the host and K and V within L2."""
+    from paper_2402_12374_b200 import binding as B
+
+    fake = 0x1000  # never dereferenced
+
+    def need(hq, hkv, n, blocks, **kw):
+        p = B.AttentionParams()
+        L = 64 * blocks - n
+        p.n_tree, p.prefix_len, p.num_q_heads, p.num_kv_heads, p.head_dim, p.dtype = n, L, hq, hkv, 128, B.SEQ_BF16
+        p.q = p.k_cache = p.v_cache = p.out = p.parent = fake
+        p.q_stride_tok = p.o_stride_tok = hq * 128
+        p.q_stride_head = p.o_stride_head = 128
+        p.kv_stride_tok, p.kv_stride_head, p.kv_capacity = 128, (L + n) * 128, L + n
+        for k, v in kw.items():
+            setattr(p, k, v)
+        return lib.seq_tree_attention_workspace_bytes(C.byref(p))
+
+    for hkv in (1, 2, 4, 8):
+        for tiles in (1, 2, 3, 4, 5):  # up to 40 units
+            for blocks in (50, 100, 200, 300, 500, 1000, 3000):
+                assert need(8 * hkv, hkv, 16 * tiles, blocks) == 0, (hkv, tiles, blocks)
+    assert need(64, 8, 208, 200) > 0                                                # 104 units
+    assert need(64, 8, 208, 200, prefix_len_dev=fake, prefix_len_dev_count=1) == 0  # ... with the length in device memory
+    assert need(64, 8, 208, 460) == 0                                               # 120 MB of keys and values
+    assert need(64, 8, 32, 300, kernel=B.KERNEL_TENSOR_CORE_STREAM) > 0
+    assert need(64, 8, 768, 76) > 0 and need(64, 8, 768, 76, prefix_len_dev=fake, prefix_len_dev_count=1) > 0  # 384 units
