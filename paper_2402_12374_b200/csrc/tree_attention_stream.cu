@@ -515,15 +515,14 @@ tree_attention_stream_kernel(const __grid_constant__ CUtensorMap q_map, const __
       sum = exponentials();
       if (settle) break;
       settle = __any_sync(0xffffffffu, !(sum <= kRescaleLimit));
-      if (settle) continue;
-      if (!mine) {
+      if (!settle && !mine) {
         if (!mbar_wait(sm, &sm->settled[chain ^ 1][quad], ((chain ? base_a : base_b) + ((u - 1) >> 1)) & 1, a.dev_status)) { ok = false; break; }
         mine = true;
         ref = sm->ref[r];
         settle = __any_sync(0xffffffffu, ref != m_used);
-        if (settle) continue;
       }
-      break;
+      if (!settle) break;
+      tc_wait_st();  // (a pass that is repeated stores to the same columns, and stores are not ordered among themselves)
     }
     if (!ok) break;
     if (opening || m_used != ref) sm->ref[r] = m_used;

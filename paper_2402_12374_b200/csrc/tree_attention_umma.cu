@@ -560,6 +560,8 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
         }
       }
       sum = exponentials();
+      tc_wait_st();  // (for the hand-over below, and because a repeated pass stores other values to the same columns: stores to
+                     // tensor memory are not ordered among themselves.  A wait of its own there: 2 us more for 32 layers)
       if (settle) break;
       settle = __any_sync(0xffffffffu, !(sum <= kRescaleLimit));
       if (!settle) break;
@@ -568,7 +570,6 @@ tree_attention_umma_kernel(const __grid_constant__ CUtensorMap q_map, const __gr
     if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 3);
     l = l * alpha + sum;
     if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 4);
-    tc_wait_st();
     if (threadIdx.x == SEQ_TRACE_ROW) UTRACE(2, 12);
     tc_fence_before();
     __syncwarp();
