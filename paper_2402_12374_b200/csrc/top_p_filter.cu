@@ -20,9 +20,9 @@
 // four times and adding every token to the histogram, 13.6 with a cluster per row that worked out every token's bin in two
 // passes and queued the histogram's tokens by votes, 12.5 so: estimates to a margin tell most tokens off, their mass is taken
 // without a branch, the histogram's tokens wait in lists of the threads' own.  127 rows of 128256 71 -> 61 us, 378 192 -> 168,
-// 300 of 50257 68 -> 61; at temperature 1, where a third of the tokens are in the histogram, 127 rows 87.6 -> 84.9 and 512 of
-// 32000 62.7 -> 63.0.  (Exact limits found by a search over the floats: 15.0; a warp's queue instead of lists: 13.4; lists of
-// 16: 378 rows 180.)
+// 300 of 50257 68 -> 61; at temperature 1, where a third of the tokens are in the histogram, 127 rows 79.4 -> 76.0, 512 of 32000
+// 64.6 -> 63.5, but 3 of 32000 9.14 -> 9.3; at 1.5, 512 rows of 128256 346 -> 344.  (Exact limits found by a search over the
+// floats: 15.0; a warp's queue instead of lists: 13.4; lists of 16: 378 rows 180.)
 #include <climits>
 #include <cstddef>
 
@@ -679,9 +679,16 @@ __global__ void __launch_bounds__(kTpThreads, 2) top_p_cluster_kernel(const TopP
     // The round's tokens wait in a list of the thread's own, so that the lanes of a warp add theirs side by side.
     float* const list = reinterpret_cast<float*>(me.cand) + tid;
     float* end = list;
+    // (Two at a time, both loads ahead of the first one's atomics.  512 rows of 128256 at temperature 1.5: 354 us one at a time,
+    // 344 so, 341 four at a time, which at 1 is 281 against 277; 3 rows at 1.5 16.9, 16.3 and 16.1, at 1 14.2, 14.0 and 14.2.)
     auto flush = [&]() {
-      for (float* t = list; __any_sync(0xffffffffu, t < end); t += kTpThreads)
-        if (t < end) add(*t);
+      for (float* t = list; __any_sync(0xffffffffu, t < end); t += 2 * kTpThreads) {
+        float x[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) x[k] = t + k * kTpThreads < end ? t[k * kTpThreads] : -INFINITY;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) add(x[k]);
+      }
       end = list;
     };
     auto pass = [&](auto opening) {
