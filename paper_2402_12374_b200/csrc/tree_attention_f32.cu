@@ -189,7 +189,8 @@ __device__ __forceinline__ void f32_pv(const F32Smem<RPT>& sm, F32Row<RPT>& st, 
   ulonglong2 t[RPT];
 #pragma unroll
   for (int i = 0; i < RPT; ++i) t[i] = make_ulonglong2(0ull, 0ull);
-#pragma unroll 2  // (the next four keys' operands on their way: 64 nodes on 1024 keys of 32 heads 46.85 -> 44.75 us, one node on 2000 21.2 -> 19.5)
+#pragma unroll (RPT < 8 ? 2 : 1)  // (the next four keys' operands on their way.  64 nodes on 1024 keys of 32 heads, RPT 4, 46.9 -> 44.8 us, one
+  // node on 2000, RPT 1, 20.5 -> 18.8; with 8 rows a step has loads enough of its own: 85 nodes on 104 keys of 64/8 31.6 -> 32.9)
   for (int c = 0; c < 32; c += 4) {
     if (kTree && !((seen >> c) & 15u)) continue;
     const uint8_t* at = vcol + c * 128;
