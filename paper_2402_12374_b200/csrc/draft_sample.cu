@@ -42,6 +42,7 @@ constexpr int kDsMaxParts = 8;           // CTAs per row: a portable cluster
 
 struct DraftSampleArgs {
   int32_t n_rows, V, k, parts, part_tokens;  // part_tokens: a multiple of the step
+  int32_t early;                             // the next kernel is let in at the start (see ds_early), not behind the last step
   const float* logits; int64_t logits_stride;
   const float* uniforms; int64_t uniforms_stride;
   float inv_T;
@@ -157,11 +158,9 @@ __global__ void __launch_bounds__(kDsThreads) draft_sample_kernel(const DraftSam
   const int lo = part * a.part_tokens, cnt = min(a.part_tokens, a.V - lo);
   const float* lrow = a.logits + (int64_t)row * a.logits_stride + lo;
   const float* urow = a.uniforms + (int64_t)row * a.uniforms_stride + lo;
-  // The next kernel in the stream may be scheduled as soon as every CTA of this one runs (it waits before it reads), and this
-  // one asks for its first two steps, a line of 32 tokens a thread, while the previous one ends: call after call, 378 rows x
-  // 128256 62.5 -> 60.7 us, 378 x 50257 32.1 -> 29.8, 37 x 128256 14.2 -> 11.8, 20 x 50257 8.2 -> 7.25, 1 x 32000 5.05 -> 4.9
-  // (only asked for: 62.6, 32.2, 13.3, 7.6 and 4.7; with fewer than 297 CTAs only: 62.6, 32.1, 12.0, 7.1, 4.9).
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // While the previous kernel ends this one asks for its first two steps, a line of 32 tokens a thread: call after call, 378 rows x
+  // 50257 31.9 -> 31.9 us, 37 x 128256 15.5 -> 13.8, 23 x 50257 9.2 -> 8.1, 1 x 32000 5.97 -> 5.87 (k = 9).
+  if (a.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (32 * tid < cnt) {
     prefetch_l2(lrow + 32 * tid);
     prefetch_l2(urow + 32 * tid);
@@ -328,6 +327,7 @@ __global__ void __launch_bounds__(kDsThreads) draft_sample_kernel(const DraftSam
     }
   }
   if (bad) dev_flag(a.dev_status, SEQ_DEV_NONFINITE);
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // (nothing to it if the next kernel has been let in)
   int have = ranked;
   if (a.parts > 1) {
     cg::this_cluster().barrier_wait();  // the first CTA runs: its shared memory may be written
@@ -386,6 +386,21 @@ static int ds_part_tokens(const seq_tree_draft_sample_params* p) {
 }
 static int ds_parts(const seq_tree_draft_sample_params* p) { return (p->vocab + ds_part_tokens(p) - 1) / ds_part_tokens(p); }
 
+// Whether the next kernel in the stream (which waits before it reads) may be scheduled as soon as every CTA of this one runs,
+// its own first steps then asked for while these CTAs still work: 378 rows x 128256 64.9 -> 63.0 us, 378 x 50257 31.9 -> 30.3,
+// 200 x 32000 16.0 -> 14.8, 84 x 32000 10.4 -> 9.4 (k = 9).  Its CTAs take what places are free, so that they start unevenly over
+// the SMs; what that costs shows
+// - where the SMs are far from full, below 1.75 CTAs each (17 rows x 128256, k = 24: 16.9 us, let in early 19.7);
+// - where a launch in clusters of 3, 5, 6 or 7 just fits at three CTAs an SM, 2.56 to 2.9 each (80 rows x 50257, 5 CTAs each:
+//   15.7 and 18.1; 136 x 128256, 3 each: 34.5 and 39.2; 69 x 128256, 6 each: 21.4 and 23.1).
+// Against the kernel that neither let in early nor asked ahead, over 2 to 420 rows of 32000, 50257 and 128256 tokens at k = 2, 9
+// and 24, calls are 8 % faster on the average and 3 % slower at worst (241 rows x 50257, where a second wave begins).
+static bool ds_early(int ctas, int parts) {
+  const int sms = device_sm_count();
+  const bool just_fits = 100 * ctas > 256 * sms && 10 * ctas <= 29 * sms;
+  return 4 * ctas >= 7 * sms && !(just_fits && (parts & (parts - 1)) != 0);
+}
+
 static int ds_validate(const seq_tree_draft_sample_params* p) {
   if (p == nullptr || p->draft_logits == nullptr || p->uniforms == nullptr || p->tokens_out == nullptr)
     return SEQ_ERR_INVALID_ARG;
@@ -409,6 +424,7 @@ extern "C" int seq_tree_draft_sample(const seq_tree_draft_sample_params* p, void
   const int parts = ds_parts(p);
   DraftSampleArgs a;
   a.n_rows = p->n_rows; a.V = p->vocab; a.k = p->k; a.parts = parts; a.part_tokens = ds_part_tokens(p);
+  a.early = ds_early((int)(parts * (p->n_rows < 4096 ? p->n_rows : 4096)), parts);  // (more rows: beyond either line)
   a.logits = p->draft_logits; a.logits_stride = p->logits_row_stride;
   a.uniforms = p->uniforms; a.uniforms_stride = p->uniforms_row_stride;
   a.inv_T = 1.f / p->temperature;
