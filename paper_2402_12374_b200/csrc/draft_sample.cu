@@ -391,13 +391,13 @@ static int ds_parts(const seq_tree_draft_sample_params* p) { return (p->vocab + 
 // 200 x 32000 16.0 -> 14.8, 84 x 32000 10.4 -> 9.4 (k = 9).  Its CTAs take what places are free, so that they start unevenly over
 // the SMs; what that costs shows
 // - where the SMs are far from full, below 1.75 CTAs each (17 rows x 128256, k = 24: 16.9 us, let in early 19.7);
-// - where a launch in clusters of 3, 5, 6 or 7 just fits at three CTAs an SM, 2.56 to 2.9 each (80 rows x 50257, 5 CTAs each:
+// - where a launch in clusters of 3, 5, 6 or 7 just fits at three CTAs an SM, 2.63 to 2.9 each (80 rows x 50257, 5 CTAs each:
 //   15.7 and 18.1; 136 x 128256, 3 each: 34.5 and 39.2; 69 x 128256, 6 each: 21.4 and 23.1).
 // Against the kernel that neither let in early nor asked ahead, over 2 to 420 rows of 32000, 50257 and 128256 tokens at k = 2, 9
 // and 24, calls are 8 % faster on the average and 3 % slower at worst (241 rows x 50257, where a second wave begins).
 static bool ds_early(int ctas, int parts) {
   const int sms = device_sm_count();
-  const bool just_fits = 100 * ctas > 256 * sms && 10 * ctas <= 29 * sms;
+  const bool just_fits = 100 * ctas > 263 * sms && 10 * ctas <= 29 * sms;
   return 4 * ctas >= 7 * sms && !(just_fits && (parts & (parts - 1)) != 0);
 }
 
