@@ -802,15 +802,19 @@ static UmmaPlan umma_plan(const seq_tree_attention_params& p) {
   // 8 on 1024 7.25 -> 6.6.)  What a wave holds is asked of the device: a cluster lies in one
   // GPC, so the SMs left over in each are lost to it (74, 44, 36, 28, 21, 14 and 14 clusters of 2 to 8 CTAs were seen, where
   // 148 / cs had been assumed; 24 units of 17 blocks 17.3 -> 10.1 us, 16 of 48 21.8 -> 12.5, 48 of 66 34.7 -> 23.3).
+  // A merge of tiles of more than 64 rows takes 0.75 to 1.1 us longer (32 units of 6 blocks, 128 rows: 7.8 us in one CTA, 8.4 in
+  // four; 64 rows: 7.45 and 6.9), which decides between one CTA and a cluster up to 8 blocks: 32 units of 6 to 7 blocks 8.45 -> 7.8
+  // and 9.05 -> 8.5.
   static const double kMerge[kMaxClusterSplit + 1] = {0.0, 0.0, 1.45, 2.0, 1.7, 2.3, 2.05, 1.8, 1.8};
+  const double wide = (p.n_tree < nodes_per_tile ? p.n_tree : nodes_per_tile) * G > 64 ? 0.9 : 0.0;
   int best = 1;
-  double best_cost = -1.0;
+  double best_cost = -1.0, grid_cost = 0.0;  // grid_cost: as the rule for the stream below was fitted, whatever the tiles' rows
   for (int cs = 1; cs <= kMaxClusterSplit && cs <= nblk; ++cs) {
     const int room = clusters_side_by_side(cs);
     if (room == 0) continue;
     const long waves = (units + room - 1) / room;
-    const double cost = (double)waves * (0.45 * ((nblk + cs - 1) / cs) + 5.0 + kMerge[cs]);
-    if (best_cost < 0 || cost < best_cost - 1e-9) { best = cs; best_cost = cost; }
+    const double plain = (double)waves * (0.45 * ((nblk + cs - 1) / cs) + 5.0 + kMerge[cs]), cost = plain + (cs > 1 ? waves * wide : 0.0);
+    if (best_cost < 0 || cost < best_cost - 1e-9) { best = cs; best_cost = cost; grid_cost = plain; }
   }
   // ... against that of the stream schedule: 0.4 per block of an SM's range, 7 per tile it starts or finishes, 7 fixed (3 to 8
   // % off over 20 shapes of 96 to 384 units).  192 units of 84 blocks 76 -> 65.5 us, 96 of 131 65 -> 56; taken where it is an
@@ -828,7 +832,7 @@ static UmmaPlan umma_plan(const seq_tree_attention_params& p) {
   const double kv_bytes = 4.0 * ((double)p.prefix_len + p.n_tree) * kHeadDim * p.num_kv_heads;
   const double stream_cost = 0.4 * units * nblk / kNumSMs + 7.0 * ((double)units / kNumSMs + 1.0) + 7.0;
   if (p.kernel != 4 && can_stream && units >= kOptionalStreamUnits && p.prefix_len_dev == nullptr && nblk >= 24 && kv_bytes < 115e6 &&
-      stream_cost < 0.88 * best_cost)
+      stream_cost < 0.88 * grid_cost)
     return {best, true, true};
   return {best, false, false};
 }
