@@ -104,14 +104,21 @@ def test_a_stream_that_is_only_the_faster_choice_needs_no_workspace():
     args = (ai.q.to(d), ai.k_cache.to(d), ai.v_cache.to(d))
     call = B.AttentionCall(*args, None, L, parent=parent)
     streamed = call.run().clone()
+    if torch.cuda.get_device_properties(d).multi_processor_count != 148:
+        pytest.skip("the rule's figures are those of 148 SMs")
+    assert call.workspace_bytes_needed > 0
+    stream = B.seq_tree_attention(*args, None, L, parent=parent, kernel=B.KERNEL_TENSOR_CORE_STREAM)
     forced = B.seq_tree_attention(*args, None, L, parent=parent, kernel=B.KERNEL_TENSOR_CORE_GRID)
+    assert torch.equal(streamed, stream) and not torch.equal(streamed, forced)
     assert (streamed.float() - forced.float()).norm() < 5e-3 * forced.float().norm()  # two roundings of P to bfloat16
-    if call.workspace_bytes_needed == 0:
-        pytest.skip("not streamed on this device")
     backing = torch.empty(call.workspace_bytes_needed + 256, dtype=torch.uint8, device=d)
     for lent in (backing[:0], backing[:4096], backing[8:8 + call.workspace_bytes_needed]):
         got = B.seq_tree_attention(*args, None, L, parent=parent, workspace=lent)
         assert torch.equal(got, forced)
+    # with the length in device memory, which may be far below the bound that the launch is planned for, the grid schedule
+    length = torch.tensor([L], dtype=torch.int32, device=d)
+    replayed = B.AttentionCall(*args, None, L, parent=parent, prefix_len_dev=length)
+    assert replayed.workspace_bytes_needed == 0 and torch.equal(replayed.run(), forced)
 
 
 @pytest.mark.parametrize("kernel", [B.KERNEL_AUTO, B.KERNEL_TENSOR_CORE_STREAM])
