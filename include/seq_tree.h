@@ -134,11 +134,16 @@ int seq_tree_mask_from_parents(const int32_t* parent, int32_t n, uint32_t* mask_
  * CUDA-core kernels keep the partial results of their key-range splits there
  * (the fp32 one makes do with less, in fewer splits, down to none for most
  * shapes: a workspace sized for the longest prefix serves every shorter one),
- * the tensor-core kernel the pieces of the query tiles that its CTAs share
- * when there are more (tile, kv head) units than SMs (about 19 MB then; with
- * kernel = 0 a group of heads that does not divide 128 does without).  A call
- * with a workspace that is too small returns SEQ_ERR_WORKSPACE and launches
- * nothing.  Two calls that run concurrently need a workspace each.
+ * the tensor-core kernel, in its stream schedule, the pieces of the query tiles
+ * that its CTAs share (about 19 MB).  That schedule is taken for more
+ * (tile, kv head) units than SMs with long tiles: a workspace that is too small
+ * then returns SEQ_ERR_WORKSPACE and launches nothing (but with kernel = 0 a
+ * group of heads that does not divide 128 does without).  It is also taken,
+ * with kernel = 0 or 2, for some calls of 48 units and more for which it is only
+ * the faster of two: they report the size as well, but without a workspace, or with
+ * one that is too small or not aligned, they run the grid schedule instead and
+ * succeed; the two schedules' results differ by rounding.  A call writes the
+ * workspace it is lent: two calls that can run concurrently need one each.
  * The results do not depend on the order in which CTAs finish: a call
  * repeated on the same inputs returns the same bits.
  */
@@ -161,7 +166,7 @@ typedef struct {
   size_t workspace_bytes;
   int32_t* dev_status;
   int32_t kernel; /* 0 = choose; 1 = force the CUDA-core kernel; 2 = force the tensor-core kernel; 3, 4 = the tensor-core
-                     kernel with its stream / grid schedule forced (tuning and tests; results do not depend on it) */
+                     kernel with its stream / grid schedule forced (tuning and tests; results differ by rounding) */
   const int32_t* parent; /* nullable, [n_tree] int32, device: see "mask from the parent array" above */
   /* nullable, device: the prefix length as the previous step's seq_tree_kv_commit left it.  When given, the kernels
    * read the length from there and prefix_len is only the LARGEST value it can take (it sizes the launch, the

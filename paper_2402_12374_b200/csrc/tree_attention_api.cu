@@ -88,7 +88,7 @@ extern "C" size_t seq_tree_attention_workspace_bytes(const seq_tree_attention_pa
   if (validate_attention_params(p) != SEQ_OK) return 0;
   const int which = choose_kernel(*p);
   if (which == 0) return 0;
-  if (which == 2) return umma_workspace_bytes(*p);  // only its stream mode (more units than SMs) needs one
+  if (which == 2) return umma_workspace_bytes(*p);  // only its stream schedule asks for one, in some calls as an option (umma_plan)
   size_t bytes = cuda_core_workspace(*p, simt_default_splits(*p));
   if (which == 3) {
     const size_t plan = cuda_core_workspace(*p, f32_splits(*p));

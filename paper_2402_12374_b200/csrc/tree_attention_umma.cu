@@ -817,7 +817,7 @@ static UmmaPlan umma_plan(const seq_tree_attention_params& p) {
     if (best_cost < 0 || cost < best_cost - 1e-9) { best = cs; best_cost = cost; grid_cost = plain; }
   }
   // ... against that of the stream schedule: 0.4 per block of an SM's range, 7 per tile it starts or finishes, 7 fixed (3 to 8
-  // % off over 20 shapes of 96 to 384 units).  192 units of 84 blocks 76 -> 65.5 us, 96 of 131 65 -> 56; taken where it is an
+  // % off over 20 shapes of 96 to 384 units).  320 units of 67 blocks 99 -> 82 us, 104 of 200 95 -> 79; taken where it is an
   // eighth lower, because a caller has 19 MB of workspace to find for it (the first time 0.2 ms).  These calls were served
   // without a workspace before there was this rule, and without one they still are.  It holds
   // - from 48 units on (48 of 200 blocks 52 -> 49 us, 52 of 300 92 -> 64, 80 of 200 73 -> 65): with fewer a tile has more than
