@@ -20,9 +20,9 @@
 // (see the row threads).
 //
 // What bounds it: shared memory.  A pair of blocks costs 512 cycles of writes by TMA, 512 of Q and K read by S, 256 of V read by
-// P V, 1280 of about 1430; the exponentials take 1024 of them, the products as many.  768 nodes on 4096 keys of 64/8 heads
-// 119 -> 104 us (in a long loop, under the power cap, 131 -> 115), on 8192 keys 225 -> 183, 384 nodes on 2048 keys of 52 heads
-// 39.8 -> 38.2.  Of that, the scores of a pair read in two halves, the second while the first is worked on: 107 -> 104; the
+// P V, 1280 of about 1430; the exponentials take 1024 of them, the products as many.  Calls on several inputs in turn, against
+// the kernel with chains of 64 keys: 768 nodes on 4096 keys of 64/8 heads 136.7 -> 124.6 us (bursts of 40, before the power cap
+// sets in, 119 -> 104), on 8192 keys 243 -> 201, 384 nodes on 2048 keys of 52 heads 41.3 -> 40.0.  Of that, in bursts, the scores of a pair read in two halves, the second while the first is worked on: 107 -> 104; the
 // output through shared memory and Q in two buffers: a tile's end 9000 -> 7000 cycles.  Without gain: a quarter of the
 // exponentials as polynomials on the FMA pipe (120 -> 125), P rounded by integer arithmetic (124), the ancestor rows derived
 // by the V producer (118 -> 121), the next pair's scores read ahead of this one's hand-over (104 -> 111).
