@@ -872,16 +872,51 @@ __global__ void top_p_copy_kernel(const TopPArgs a) {
   if (threadIdx.x == 0 && a.kept_out != nullptr) a.kept_out[blockIdx.x] = a.V;
 }
 
+// Clusters of `ranks` CTAs, with the largest slice's shared memory, that the device runs at a time.  Asked once per device and
+// size; without a device, or where the question fails, what the SMs would hold at two CTAs each.
+static int tp_clusters_side_by_side(int ranks) {
+  const int all = 2 * device_sm_count() / ranks;
+  static int known[kTpMaxCluster + 1][64];  // + 1; 0 = not asked yet
+  int dev = 0;
+  if (ranks == 1 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) { cudaGetLastError(); return all; }
+  int n = __atomic_load_n(&known[ranks][dev], __ATOMIC_ACQUIRE);
+  if (n == 0) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ranks);
+    cfg.blockDim = dim3(kTpThreads);
+    cfg.dynamicSmemBytes = offsetof(TpFast, x) + kTpMaxSlice * 4;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)ranks;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, top_p_cluster_kernel, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = all;
+    }
+    ++n;
+    __atomic_store_n(&known[ranks][dev], n, __ATOMIC_RELEASE);
+  }
+  return n - 1;
+}
+
 // CTAs per row: as many as let the rows' clusters run side by side (two CTAs per SM), of at least 4096 tokens each and 8 at
 // most; at least what keeps a slice within 16384 tokens.  A row of more than 8 x 16384 tokens goes to one CTA.
+// What runs side by side is asked of the device, as a cluster lies in one GPC (33, 37, 45, 56, 71 and 93 clusters of 8 to 3 CTAs
+// were seen, 2 * 148 / ranks had been assumed), and three places are left free: in a row of calls the next one's clusters
+// come in as these leave, and where all places are needed they get between (45 rows of 32000 in clusters of 6: 13.4 us or 17.5
+// from one build to the next; in clusters of 5 12.1).  One place where a step down makes the slices a third longer and more
+// (70 rows at temperature 1 in clusters of 4 15.1, of 3 16.9).  36 rows of 32000 19.2 -> 11.6 us, 58 20.0 -> 12.3, 98 22.7 -> 16.1, 48 of
+// 50257 21.8 -> 13.8; no room for a tenth of the rows: 66 rows at temperature 1 16.9 instead of 14.7.
 static int launch_top_p(int rows, const TopPArgs& a, cudaStream_t stream) {
   const int least = (a.V + kTpMaxSlice - 1) / kTpMaxSlice, most = (a.V + 4095) / 4096;
   const bool cluster = least <= kTpMaxCluster;
   int64_t ranks = 2 * (int64_t)device_sm_count() / rows;
   ranks = ranks > most ? most : ranks;
   ranks = ranks > kTpMaxCluster ? kTpMaxCluster : ranks < least ? least : ranks;
-  const int slice = (int)(((a.V + ranks - 1) / ranks + 3) & ~(int64_t)3);
-  const size_t smem = offsetof(TpFast, x) + (size_t)slice * 4;
+  // (the attributes first: the question below asks for the shared memory of the largest slice)
   static int attr_done[64];
   const int rc = once_per_device(attr_done, [&]() -> int {  // above the 48 KB a kernel gets without asking
     SEQ_CUDA_OK(cudaFuncSetAttribute(top_p_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(offsetof(TpFast, x) + kTpMaxSlice * 4)));
@@ -889,6 +924,9 @@ static int launch_top_p(int rows, const TopPArgs& a, cudaStream_t stream) {
     return SEQ_OK;
   });
   if (rc != SEQ_OK) return rc;
+  while (cluster && ranks > least && tp_clusters_side_by_side((int)ranks) < (int64_t)rows + (ranks > 4 ? 3 : 1)) --ranks;
+  const int slice = (int)(((a.V + ranks - 1) / ranks + 3) & ~(int64_t)3);
+  const size_t smem = offsetof(TpFast, x) + (size_t)slice * 4;
   if (!cluster) {
     top_p_row_kernel<<<rows, kTpRowThreads, sizeof(TpShared), stream>>>(a);
     SEQ_CUDA_OK(cudaGetLastError());

@@ -155,3 +155,18 @@ def test_rows_larger_than_a_cluster_keep_enough_loads_in_flight():
         torch.cuda.synchronize()
         best = min(best, e0.elapsed_time(e1) / 5 * 1e3)
     assert best < 100
+
+
+@pytest.mark.parametrize("rows", [30, 31, 34, 35, 42, 43, 53, 54, 70, 71, 92, 93, 148])
+def test_row_counts_that_change_the_clusters_side_by_side(rows):
+    """Around the numbers of rows at which a row gets fewer CTAs because its clusters would not all be placed: every row as it
+    comes out alone, bit for bit (the masses are integers, so the number of CTAs does not enter the result)."""
+    d = torch.device("cuda:0")
+    g = torch.Generator(device=d)
+    g.manual_seed(rows)
+    x = 3 * torch.randn((rows, 32000), device=d, generator=g)
+    kept = torch.empty(rows, dtype=torch.int32, device=d)
+    out = B.seq_tree_top_p_filter(x, 0.8, 0.9, kept_out=kept)
+    for r in range(rows):
+        one = torch.empty(1, dtype=torch.int32, device=d)
+        assert torch.equal(B.seq_tree_top_p_filter(x[r:r + 1], 0.8, 0.9, kept_out=one), out[r:r + 1]) and int(one) == int(kept[r])
