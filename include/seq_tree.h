@@ -12,8 +12,9 @@
  *     device that is current when the call is made.  The library allocates
  *     no device memory and never synchronises the host.  Between calls it keeps
  *     only per-device facts that it looks up once (a driver entry point, the
- *     SM count, whether a 16-CTA cluster can be placed, function attributes
- *     already set, the address of the built-in scratch array) and up to 1024
+ *     SM count, whether a 16-CTA cluster can be placed and how many smaller
+ *     ones side by side, function attributes already set, the address of the
+ *     built-in scratch array) and up to 1024
  *     tensor maps it has encoded, keyed by the arguments of the encode (pointer,
  *     extents, strides), so that a repeated launch makes no driver call; those
  *     lookups are guarded, so calls may come from several host threads.
